@@ -1,0 +1,1316 @@
+// Variant (iii)(a) in arrival order: the main path of a step.
+//
+// Edges of the hit graph are symmetric (8-adjacent or same pixel, |dToA| <=
+// dt), so joining hits needs no time order inside a tile, only that each hit
+// meets every hit it can be joined to.  A stream is nearly time ordered
+// (Section 3.1), so those lie a short way around it.  No sort, no sorted
+// copies and no gather are needed; a record is read from DRAM once.
+//
+//   k_arrival_tile   one CTA per time tile: tile j owns the hits of its ToA
+//                    interval [cut j, cut j+1), picked from its TILE positions
+//                    and a margin on both sides, and sees the hits of the dt
+//                    before it.  Links in shared memory, pairs that join an
+//                    earlier tile's hit go to a list, and every tile cluster's
+//                    features are reduced.
+//   k_arrival_cross  joins tile clusters over the listed pairs, closes the
+//                    segments (watermark), and proves that every hit found its
+//                    tile and every tile the hits before it; if not, the step
+//                    takes the time-sorted path (link.cu).
+//   k_arrival_roots  adds each tile cluster's features to its cluster's.
+//   k_arrival_labels labels, closed flags and label flags per hit.
+//   k_arrival_emit   records in label order; streaming: finalised hits, the
+//                    carry of open hits and the stream state.
+//
+// Small steps (at most SMALL_TILES tiles) work for any order, so that they
+// need no sorted path behind them: k_arrival_small owns hits by position and
+// looks back over earlier positions, and k_arrival_redo joins the tiles that
+// did not look far enough with every earlier tile.
+//
+// Owning by time keeps events whole: arrival disorder spreads an event's hits
+// over a thousand positions, and tiles of positions would cut a quarter of
+// the events into fragments (256x256 stream, 64 Mi hits: 522 tile clusters and
+// 320 pairs across per tile by position, against 3.45 M clusters in all, 210
+// per tile).
+//
+// Tile clusters are numbered c = tile * TILE + (index among the tile's
+// clusters), so that everything kept per cluster (32-byte RootSlot, first and
+// last ToA, union-find parent) is dense and a hit's cluster is one 32-bit c.
+#include "tpc_internal.cuh"
+
+namespace tpc {
+
+constexpr int AT = 512;                          // threads of the tile kernels (64 registers, two CTAs per SM)
+constexpr int AW = AT / 32;
+constexpr uint32_t A_MARGIN = 1024;              // positions around the tile read at once
+constexpr int A_ITEMS = (TILE + 2 * A_MARGIN) / AT;   // records per thread
+constexpr int A_GROUP = 4;                       // ... in flight together
+constexpr uint32_t A_STEP = TILE / ACHUNKS;      // positions per further round
+constexpr int A_HPER = (A_STEP + AT - 1) / AT;
+constexpr uint32_t A_ENT = 5632;                 // hits staged: a tile's own and the earlier ones
+constexpr int A_PER = A_ENT / AT;
+constexpr uint32_t A_WORDS = 2304;               // 256 rows of nine 30-pixel words
+constexpr uint32_t A_XTRA = 1024;                // unions beyond each hit's first
+constexpr uint32_t A_CROSS = 1024;               // pairs across tiles
+constexpr uint32_t A_LATER = 2048;               // hits beside cells of several hits
+constexpr uint32_t A_FAR = 1024;                 // hits found beyond the margins
+constexpr int A_JUMPS = 5;                       // path-shortening passes over the tile's forest
+constexpr int A_ROUNDS = 4;                      // further rounds on each side
+constexpr int A_BACK_ROUNDS = 16;                // rounds back of a small step's tiles
+constexpr uint32_t A_NONE = 0x7FFFu;             // no hit
+constexpr uint32_t A_MULTI = 0x8000u;            // head flag: the cell holds several hits
+static_assert(A_WORDS <= 4096, "word indices take 12 bits");
+static_assert(A_ITEMS * AT == TILE + 2 * (int)A_MARGIN && A_PER * AT == (int)A_ENT && A_ITEMS % A_GROUP == 0, "whole rounds");
+
+// A cell is a pixel column x of a row (y mod R).  Occupied cells are found by
+// a bitmap (30 pixels per word, the outer two bits repeating the neighbour
+// words' border pixels, so that the three cells x-1..x+1 of a row are always
+// in one word), and numbered by rank: word.y holds the occupied cells before
+// the word, so a cell's slot is word.y + the set bits below it and the cells
+// of a row's neighbourhood have consecutive slots.  head[slot] is a hit of
+// the cell; further hits (a pixel hit more than once, or rows that share a
+// cell on sensors taller than R) hang on next[].  110 KB: two CTAs per SM.
+struct ArrivalShared {
+    uint2 word[A_WORDS];         // bits; cells before the word (minus the repeated low bit)
+    uint16_t head[A_ENT];
+    uint16_t next[A_ENT];
+    uint32_t key[A_ENT];         // ToA - base
+    uint32_t code[A_ENT];        // cell and row: (y / R) << 17 | word << 5 | bit
+    uint16_t par[A_ENT];         // forest over the tile's own hits
+    uint32_t xtra[A_XTRA];       // unions beyond each hit's first (k << 16 | j)
+    uint32_t cross[A_CROSS];     // pairs across tiles (own << 16 | earlier)
+    uint16_t later[A_LATER];     // hits beside cells of several hits
+    uint16_t far[A_FAR];         // hits beyond the margins: position - window start
+    uint32_t red[4][AW];
+    uint32_t cnt[2][AW], turn[2][AW];
+    unsigned long long m64[2][AW];
+    uint32_t cut[2];
+    uint32_t nent, nown, ntail, nxtra, ncross, nlater, nroots, tsum, flag;
+    // After the links, in the place of what is no longer needed:
+    __device__ uint16_t *tot() { return head; }                                   // [A_ENT] ToT per entry
+    __device__ uint16_t *pos() { return next; }                                   // [A_ENT] position per entry
+    __device__ uint16_t *id() { return reinterpret_cast<uint16_t *>(xtra); }      // [A_ENT] cluster of each tile root
+    __device__ uint32_t *sums() { return reinterpret_cast<uint32_t *>(word); }    // [2 * A_WORDS] feature sums
+};
+static_assert((A_XTRA + A_CROSS) * 4 + A_LATER * 2 >= A_ENT * 2, "cluster indices fit the lists");
+// Small steps stage every entry's position too.
+struct SmallShared {
+    ArrivalShared s;
+    uint16_t pos[A_ENT];
+};
+constexpr int A_SMEM = (int)sizeof(ArrivalShared), A_SMALL_SMEM = (int)sizeof(SmallShared);
+static_assert((unsigned long long)A_ENT * 0xFFFFu < (1ull << 32), "a tile's sum ToT fits 32 bits");
+
+// Time window of 32-bit keys: base = 2^28 ticks before the segment's first
+// hit.  A hit outside it (or a dt of 2^27 ticks and more) is "wide": a small
+// step takes keys relative to its smallest ToA instead, others the
+// time-sorted path.
+constexpr uint64_t A_GUARD = ARRIVAL_DT;
+
+__device__ __forceinline__ uint32_t absdiff(uint32_t a, uint32_t b) { return a > b ? a - b : b - a; }
+
+__device__ __forceinline__ uint32_t lanes_below() {
+    uint32_t m;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
+    return m;
+}
+
+// The cell grid of a W x H sensor: R rows (a power of two) of nw words.
+struct Cells {
+    uint32_t nw, rmask, rshift, nwords;   // words per row, R - 1, log2 R, words
+    bool alias;                           // rows share cells
+    __device__ Cells(uint32_t W, uint32_t H) {
+        nw = (W + 29u) / 30u;                              // <= 2185
+        rshift = 31u - __clz((int)(A_WORDS / nw));         // at least one row
+        while (rshift && (1u << (rshift - 1u)) >= H) --rshift;
+        rmask = (1u << rshift) - 1u;
+        nwords = nw << rshift;
+        alias = H > rmask + 1u;
+    }
+    // y / R < 64: a row holds W * R > 30 * A_WORDS / 4 pixels when rows share cells, of at most 2^20
+    __device__ __forceinline__ uint32_t code(uint32_t pix) const {
+        const uint32_t x = pix & 0xFFFFu, y = pix >> 16, wi = x / 30u;
+        return (y >> rshift) << 17 | ((y & rmask) * nw + wi) << 5 | (x - wi * 30u + 1u);
+    }
+    __device__ __forceinline__ void set(ArrivalShared &S, uint32_t code) const {
+        atomicOr(&S.word[(code >> 5) & 0xFFFu].x, 1u << (code & 31u));
+    }
+    __device__ __forceinline__ void pixel(uint32_t code, uint32_t magic, uint32_t &x, uint32_t &y) const {
+        const uint32_t word = (code >> 5) & 0xFFFu, row = nw == 1u ? word : __umulhi(word, magic);
+        x = (word - row * nw) * 30u + (code & 31u) - 1u;
+        y = (code >> 17 << rshift) + row;
+    }
+    // word / nw = umulhi(word, magic) for words < 2^12, nw > 1 (nw = 1 apart: the factor would be 2^32)
+    __device__ __forceinline__ uint32_t magic() const { return 0xFFFFFFFFu / nw + 1u; }
+    __device__ __forceinline__ void clear(ArrivalShared &S) const {
+        for (uint32_t i = threadIdx.x; i < (nwords + 1) / 2; i += AT)
+            reinterpret_cast<uint4 *>(S.word)[i] = make_uint4(0, 0, 0, 0);
+    }
+};
+
+// root of x with path halving (parents only move towards the root)
+__device__ __forceinline__ uint32_t arrival_root(volatile uint16_t *par, uint32_t x) {
+    while (true) {
+        const uint32_t p = par[x];
+        const uint32_t gp = par[p];
+        if (p == gp) return p;
+        par[x] = (uint16_t)gp;
+        x = gp;
+    }
+}
+
+// par[a]: a -> b if a is still a root (16-bit compare and swap)
+__device__ __forceinline__ bool arrival_hook(uint16_t *par, uint32_t a, uint32_t b) {
+    uint32_t *word = reinterpret_cast<uint32_t *>(par) + (a >> 1);
+    const uint32_t shift = (a & 1u) * 16u;
+    uint32_t old = *reinterpret_cast<volatile uint32_t *>(word);
+    while (((old >> shift) & 0xFFFFu) == a) {
+        const uint32_t seen = atomicCAS(word, old, (old & ~(0xFFFFu << shift)) | b << shift);
+        if (seen == old) return true;
+        old = seen;
+    }
+    return false;
+}
+
+// Links of the staged entries 0..n_e: cells numbered, heads and lists built,
+// then each pair of adjacent hits met once, by the hit that is later in raster
+// order (row above, left), on one pixel by the earlier hit.
+// own(e, key): whether an entry is the tile's own; near(a, b): two keys within
+// dt; join(e, own, j, own, linked): takes a pair; linked: e has a parent.
+template <class Own, class Near, class Join>
+__device__ __forceinline__ void arrival_links(ArrivalShared &S, const Cells &C, uint32_t n_e, Own own, Near near,
+                                              Join join) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __syncthreads();                // bits, keys and codes are in place
+    {   // repeat the border pixels in the neighbour words, and count the cells before each word
+        constexpr uint32_t PER = (A_WORDS + AT - 1) / AT;
+        const uint32_t i0 = tid * PER;
+        uint32_t bits[PER], sum = 0, col = i0 - i0 / C.nw * C.nw;
+        uint32_t before = i0 && i0 < C.nwords ? S.word[i0 - 1].x : 0u;
+#pragma unroll
+        for (uint32_t i = 0; i < PER; ++i) bits[i] = i0 + i < C.nwords ? S.word[i0 + i].x & 0x7FFFFFFEu : 0u;
+        const uint32_t after = i0 + PER < C.nwords ? S.word[i0 + PER].x : 0u;
+        uint32_t full[PER];
+#pragma unroll
+        for (uint32_t i = 0; i < PER; ++i) {
+            const uint32_t l = i ? bits[i - 1] : before, r = i + 1 < PER ? bits[i + 1] : after;
+            full[i] = bits[i] | (col ? (l >> 30) & 1u : 0u);
+            ++col;
+            if (col == C.nw) col = 0; else full[i] |= (r & 2u) << 30;
+            sum += __popc(bits[i]);
+        }
+        uint32_t x = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) S.cnt[0][warp] = x;
+        __syncthreads();
+        uint32_t run = x - sum + __reduce_add_sync(0xffffffffu, lane < warp ? S.cnt[0][lane] : 0u);
+#pragma unroll
+        for (uint32_t i = 0; i < PER; ++i) {
+            if (i0 + i < C.nwords) S.word[i0 + i] = make_uint2(full[i], run - (full[i] & 1u));
+            run += __popc(bits[i]);
+        }
+    }
+    __syncthreads();
+    uint32_t slots[A_PER];
+#pragma unroll
+    for (int q = 0; q < A_PER; ++q) {   // any hit of a cell becomes its head
+        const uint32_t e = q * AT + tid;
+        slots[q] = 0;
+        if (e < n_e) {
+            const uint32_t code = S.code[e];
+            const uint2 v = S.word[(code >> 5) & 0xFFFu];
+            slots[q] = v.y + __popc(v.x & ~(0xFFFFFFFFu << (code & 31u)));
+            S.head[slots[q]] = (uint16_t)e;
+            S.next[e] = (uint16_t)A_NONE;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < A_PER; ++q) {   // the others hang behind it
+        const uint32_t e = q * AT + tid;
+        if (e >= n_e) continue;
+        const uint32_t s = slots[q], h = S.head[s] & A_NONE;
+        if (h == e) continue;
+        uint32_t *half = reinterpret_cast<uint32_t *>(S.next) + (h >> 1);
+        const uint32_t shift = (h & 1u) * 16u;
+        uint32_t old = *reinterpret_cast<volatile uint32_t *>(half);
+        while (true) {
+            S.next[e] = (uint16_t)(old >> shift);
+            const uint32_t seen = atomicCAS(half, old, (old & ~(0xFFFFu << shift)) | e << shift);
+            if (seen == old) break;
+            old = seen;
+        }
+        S.head[s] = (uint16_t)(h | A_MULTI);
+    }
+    __syncthreads();
+
+    // heads of the cells around a hit (left, above left, above, above right)
+    // and of its own; up: y / R of the row above
+    auto around = [&](uint32_t code, uint32_t (&hd)[4], uint32_t &up) -> uint32_t {
+        const uint32_t word = (code >> 5) & 0xFFFu, bit = code & 31u;
+        const uint2 v0 = S.word[word];
+        const uint32_t s0 = v0.y + __popc(v0.x & ~(0xFFFFFFFFu << bit));
+        hd[0] = hd[1] = hd[2] = hd[3] = A_NONE;
+        if ((v0.x >> (bit - 1u)) & 1u) hd[0] = S.head[s0 - 1];
+        const bool wrap = word < C.nw;   // the grid's first row: the last one lies above it
+        up = (code >> 17) - (wrap ? 1u : 0u);
+        if (!wrap || code >> 17) {
+            const uint2 v1 = S.word[wrap ? word + C.nwords - C.nw : word - C.nw];
+            const uint32_t m = v1.x >> (bit - 1u);
+            const uint32_t s1 = v1.y + __popc(v1.x & ~(0xFFFFFFFFu << (bit - 1u)));
+            if (m & 1u) hd[1] = S.head[s1];
+            if (m & 2u) hd[2] = S.head[s1 + (m & 1u)];
+            if (m & 4u) hd[3] = S.head[s1 + __popc(m & 3u)];
+        }
+        return S.head[s0];
+    };
+    // Cells of several hits: on a neighbour pixel the latest hit at or before
+    // this one and the earliest after it (the others within dt are joined to
+    // those along their pixel), on the own pixel the next one.
+    auto crowded = [&](uint32_t e) {
+        const uint32_t code = S.code[e], key = S.key[e];
+        const bool mine = own(e, key);
+        bool linked = S.par[e] != e;
+        uint32_t hd[4], up;
+        const uint32_t self = around(code, hd, up);
+        uint32_t multi = self & A_MULTI ? 16u : 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) multi |= hd[i] & A_MULTI ? 1u << i : 0u;
+        while (multi) {
+            const int i = __ffs(multi) - 1;
+            multi &= multi - 1u;
+            const uint32_t row = i == 0 || i == 4 ? code >> 17 : up;
+            uint32_t j = (i == 4 ? self : i == 0 ? hd[0] : i == 1 ? hd[1] : i == 2 ? hd[2] : hd[3]) & A_NONE;
+            uint32_t jlo = A_NONE, jhi = A_NONE, klo = 0, khi = 0xFFFFFFFFu;
+            do {
+                const uint32_t k = S.key[j];
+                if (j != e && S.code[j] >> 17 == row) {
+                    if (k < key || (k == key && (i != 4 || j < e))) {
+                        if (k >= klo) { klo = k; jlo = j; }
+                    } else if (k < khi || (k == khi && j < jhi)) {
+                        khi = k;
+                        jhi = j;
+                    }
+                }
+                j = S.next[j];
+            } while (j != A_NONE);
+            if (i != 4 && jlo != A_NONE && near(key, klo)) join(e, mine, jlo, own(jlo, klo), linked);
+            if (jhi != A_NONE && near(khi, key)) join(e, mine, jhi, own(jhi, khi), linked);
+        }
+    };
+    for (uint32_t e = tid; e < n_e; e += AT) {
+        const uint32_t code = S.code[e], key = S.key[e];
+        uint32_t hd[4], up;
+        const uint32_t self = around(code, hd, up);
+        uint32_t kk[4];
+        bool ok[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            kk[i] = 0;
+            ok[i] = false;
+            if (hd[i] < A_NONE) {   // a cell with one hit
+                kk[i] = S.key[hd[i]];
+                ok[i] = near(key, kk[i]);
+                if (C.alias) ok[i] = ok[i] && S.code[hd[i]] >> 17 == (i ? up : code >> 17);
+            }
+        }
+        // A pair whose two hits are both within dt of a third neighbour's is
+        // left out: the third one's pairs imply it.
+        if (ok[2]) {
+            ok[0] = ok[0] && !near(kk[2], kk[0]);
+            ok[1] = ok[1] && !near(kk[2], kk[1]);
+            ok[3] = ok[3] && !near(kk[2], kk[3]);
+        } else if (ok[0]) {
+            ok[1] = ok[1] && !near(kk[0], kk[1]);
+        }
+        uint32_t todo = (ok[0] ? 1u : 0u) | (ok[1] ? 2u : 0u) | (ok[2] ? 4u : 0u) | (ok[3] ? 8u : 0u);
+        if (todo) {
+            const bool mine = own(e, key);
+            bool linked = false;
+            do {
+                const uint32_t low = todo & (0u - todo);
+                const uint32_t j = low == 1u ? hd[0] : low == 2u ? hd[1] : low == 4u ? hd[2] : hd[3];
+                const uint32_t k = low == 1u ? kk[0] : low == 2u ? kk[1] : low == 4u ? kk[2] : kk[3];
+                todo ^= low;
+                join(e, mine, j, own(j, k), linked);
+            } while (todo);
+        }
+        // a tenth of the hits lie beside crowded cells: they are taken up
+        // together afterwards, not by one lane of every warp
+        if ((self | hd[0] | hd[1] | hd[2] | hd[3]) & A_MULTI) {
+            const uint32_t k = atomicAdd(&S.nlater, 1u);
+            if (k < A_LATER) S.later[k] = (uint16_t)e; else crowded(e);
+        }
+    }
+    __syncthreads();
+    const uint32_t n_l = min(S.nlater, A_LATER);
+    for (uint32_t i = tid; i < n_l; i += AT) crowded(S.later[i]);
+}
+
+// A pair of own hits: e's first makes j its parent (always raster-earlier, or
+// the next hit of its pixel, so parents form no cycle), others are listed.
+__device__ __forceinline__ bool join_own(ArrivalShared &S, uint32_t e, uint32_t j, bool &linked) {
+    if (!linked) {
+        S.par[e] = (uint16_t)j;
+        linked = true;
+        return true;
+    }
+    const uint32_t k = atomicAdd(&S.nxtra, 1u);
+    if (k < A_XTRA) S.xtra[k] = e << 16 | j;
+    return k < A_XTRA;
+}
+
+// Components of the tile's own hits, their features, and each hit's cluster.
+// ToTs and positions (pos[e], from `origin`) of the entries are staged; the
+// caller's barrier is behind them and the links.
+template <class Own>
+__device__ __forceinline__ void arrival_clusters(const Work &w, const Seg &g, uint32_t t, ArrivalShared &S,
+                                                 const Cells &C, uint32_t n_e, Own own, const uint16_t *pos,
+                                                 uint32_t origin, uint64_t base) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    const uint32_t first_c = t * TILE;
+    volatile uint16_t *par = S.par;
+    // Raster-order parents chain along a track; every hit first jumps to its
+    // ancestors a few times (all hits at once, so paths shrink by half and
+    // more each time) before unions and finds walk what is left.  (An earlier
+    // tile's hits are their own parents.)
+#pragma unroll 1
+    for (int r = 0; r < A_JUMPS; ++r) {
+        uint32_t p[A_PER];
+#pragma unroll
+        for (int q = 0; q < A_PER; ++q) p[q] = q * AT + tid < n_e ? par[q * AT + tid] : 0u;
+#pragma unroll
+        for (int q = 0; q < A_PER; ++q) p[q] = q * AT + tid < n_e ? par[p[q]] : 0u;
+#pragma unroll
+        for (int q = 0; q < A_PER; ++q)
+            if (q * AT + tid < n_e) par[q * AT + tid] = (uint16_t)p[q];
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < min(S.nxtra, A_XTRA); i += AT) {
+        uint32_t a = S.xtra[i] >> 16, b = S.xtra[i] & 0xFFFFu;
+        while (true) {   // hook the larger root under the smaller
+            a = arrival_root(S.par, a);
+            b = arrival_root(S.par, b);
+            if (a == b) break;
+            if (a < b) { const uint32_t c = a; a = b; b = c; }
+            if (arrival_hook(S.par, a, b)) break;
+        }
+    }
+    __syncthreads();
+    // number the roots, and take every hit to its root's number
+    uint16_t *id = S.id();
+    uint32_t c[A_PER];
+#pragma unroll
+    for (int q = 0; q < A_PER; ++q) {
+        const uint32_t e = q * AT + tid;
+        c[q] = e < n_e ? par[e] : 0xFFFFFFFFu;
+        const bool root = c[q] == e && own(e, S.key[e]);
+        const uint32_t m = __ballot_sync(0xffffffffu, root);
+        if (m) {
+            uint32_t k = 0;
+            if (lane == 0) k = atomicAdd(&S.nroots, (uint32_t)__popc(m));
+            k = __shfl_sync(0xffffffffu, k, 0);
+            if (root) id[e] = (uint16_t)(k + __popc(m & lanes_below()));
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < A_PER; ++q) {
+        const uint32_t e = q * AT + tid;
+        if (e < n_e) {
+            const uint32_t key = S.key[e], p = par[c[q]];
+            if (!own(e, key)) {
+                c[q] = 0xFFFFFFFFu;
+                continue;
+            }
+            c[q] = id[p == c[q] ? p : arrival_root(par, p)];
+            const uint32_t at = origin + pos[e];
+            w.root_of[at] = first_c + c[q];
+            if (w.rkey) w.rkey[at] = key;
+        }
+    }
+    // Features per cluster, as many clusters at once as the space holds.
+    // Shared memory adds 32 bits natively and 64 by compare-and-swap loops:
+    // while the tile's whole ToT keeps every sum in bounds (4096 hits of the
+    // usual ToTs do, 40 times over) size and ToT share a word and the moments
+    // take one each; otherwise the moments carry into a second word.
+    uint32_t *A = S.sums();
+    const uint16_t *tots = S.tot();
+    const uint32_t nroots = S.nroots, tsum = S.tsum, magic = C.magic();
+    if (nroots > TILE) {   // more clusters than the tile has numbers (nearly every hit alone, more hits than positions)
+        if (tid == 0) atomicMax(&w.prob->raw_fail, RAW_COVER);
+        return;
+    }
+    const bool streaming = g.ss != nullptr;
+    const uint32_t reach = max(g.width, g.height);
+    const bool slim = tsum < (1u << 19) && (unsigned long long)tsum * reach < (1ull << 32);
+    static_assert(A_ENT < (1u << 13), "a size above a 19-bit sum ToT");
+    constexpr uint32_t PASS = 2 * A_WORDS / 8;
+    for (uint32_t r0 = 0; r0 < nroots; r0 += PASS) {
+        const uint32_t nr = min(nroots - r0, PASS);
+        for (uint32_t i = tid; i < nr; i += AT) {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) A[k * PASS + i] = 0;
+            A[6 * PASS + i] = A[7 * PASS + i] = 0xFFFFFFFFu;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < A_PER; ++q) {
+            const uint32_t i = c[q] - r0;
+            if (i < nr) {
+                const uint32_t e = q * AT + tid, tot = tots[e];
+                uint32_t x, y;
+                C.pixel(S.code[e], magic, x, y);
+                uint32_t *a = A + i;   // size (and ToT), ToT, x, carry, y, carry, first position, first key
+                if (slim) {
+                    atomicAdd(a, (1u << 19) + tot);
+                    atomicAdd(a + 2 * PASS, tot * x);
+                    atomicAdd(a + 4 * PASS, tot * y);
+                } else {
+                    const uint32_t vx = tot * x, vy = tot * y;
+                    atomicAdd(a, 1u);
+                    atomicAdd(a + PASS, tot);
+                    if (atomicAdd(a + 2 * PASS, vx) > ~vx) atomicAdd(a + 3 * PASS, 1u);
+                    if (atomicAdd(a + 4 * PASS, vy) > ~vy) atomicAdd(a + 5 * PASS, 1u);
+                }
+                atomicMin(a + 6 * PASS, (uint32_t)pos[e]);
+                atomicMin(a + 7 * PASS, S.key[e]);
+            }
+        }
+        __syncthreads();
+        for (uint32_t i = tid; i < nr; i += AT) {
+            const uint4 a = make_uint4(A[i], A[PASS + i], A[2 * PASS + i], A[3 * PASS + i]);
+            const uint4 b = make_uint4(A[4 * PASS + i], A[5 * PASS + i], A[6 * PASS + i], A[7 * PASS + i]);
+            const uint32_t cc = first_c + r0 + i;
+            uint4 *slot = reinterpret_cast<uint4 *>(w.rslot + cc);
+            slot[0] = make_uint4(slim ? a.x & 0x7FFFFu : a.y, 0u, a.z, a.w);
+            slot[1] = make_uint4(b.x, b.y, slim ? a.x >> 19 : a.x, origin + b.z);
+            w.rfirst[cc] = base + b.w;
+            w.gpar[cc] = cc;
+        }
+        if (streaming) {   // last ToAs, in the place of the first ones
+            __syncthreads();
+            for (uint32_t i = tid; i < nr; i += AT) A[7 * PASS + i] = 0;
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < A_PER; ++q)
+                if (c[q] - r0 < nr) atomicMax(&A[7 * PASS + c[q] - r0], S.key[q * AT + tid]);
+            __syncthreads();
+            for (uint32_t i = tid; i < nr; i += AT) w.rlast[first_c + r0 + i] = base + A[7 * PASS + i];
+        }
+        __syncthreads();
+    }
+    if (tid == 0) w.atile[t].nroots = nroots;
+}
+
+// Cut before tile j of a segment: the median ToA key of 32 hits around its
+// first position, the same for both tiles that need it (called by a warp).
+__device__ __forceinline__ uint32_t arrival_cut(const Seg &g, uint32_t j, uint64_t base, int lane) {
+    if (j == 0) return 0u;
+    if (j >= g.ntiles) return 0xFFFFFFFFu;   // above every key that is not wide
+    const uint32_t p = min(j * TILE - 512u + 32u * lane, g.n - 1u);
+    const uint32_t key = (uint32_t)(hit_toa(ld_hit(g.hits + p)) - base);
+    uint32_t rank = 0;
+#pragma unroll
+    for (int o = 1; o < 32; ++o) {
+        const int from = (lane + o) & 31;
+        const uint32_t k = __shfl_sync(0xffffffffu, key, from);
+        rank += k < key || (k == key && from < lane);
+    }
+    return __shfl_sync(0xffffffffu, key, __ffs(__ballot_sync(0xffffffffu, rank == 16u)) - 1);
+}
+
+__global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
+    extern __shared__ __align__(16) unsigned char a_raw[];
+    ArrivalShared &S = *reinterpret_cast<ArrivalShared *>(a_raw);
+    Prob &P = *w.prob;
+    const uint32_t nt = P.ntiles, nsegs = P.nsegs;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
+        const uint32_t si = nsegs == 1 ? 0u : w.tile_seg[t];
+        const Seg &g = w.seg[si];
+        if (t + gridDim.x < nt) {   // the next tile's records on their way to L2
+            const uint32_t t1 = t + gridDim.x;
+            const Seg &g1 = nsegs == 1 ? g : w.seg[w.tile_seg[t1]];
+            const uint32_t p = (t1 - g1.tile0) * TILE + tid * (128u / sizeof(tpc_hit));
+            if (p < g1.n) asm volatile("prefetch.global.L2 [%0];" ::"l"(g1.hits + p));
+        }
+        const uint32_t j = t - g.tile0, n = g.n, off = g.off, dt = g.dt, W = g.width, H = g.height;
+        const uint64_t base = g.raw_base;
+        const tpc_hit *hits = g.hits;
+        const Cells C(W, H);
+        // ---- records around the tile --------------------------------------
+        const int32_t p0 = (int32_t)(j * TILE) - (int32_t)A_MARGIN + tid;   // position (in the segment) of record 0
+        uint4 v[A_GROUP];
+#pragma unroll
+        for (int q = 0; q < A_GROUP; ++q) {
+            const int32_t p = p0 + q * AT;
+            if ((uint32_t)p < n) v[q] = ld_hit(hits + p);
+        }
+        if (tid == 0) {
+            S.flag = *reinterpret_cast<volatile uint32_t *>(&P.raw_fail);
+            S.nent = S.nown = S.ntail = S.nxtra = S.ncross = S.nlater = S.nroots = S.tsum = 0;
+        }
+        C.clear(S);
+        if (warp < 2) {
+            const uint32_t k = arrival_cut(g, j + warp, base, lane);
+            if (lane == 0) S.cut[warp] = k;
+        }
+        const uint32_t n_carry = g.n_carry, limit = (W - 1u) | (H - 1u) << 16;
+        __syncthreads();
+        const bool last = j + 1 == g.ntiles;
+        const uint32_t cut = S.cut[0], cut1 = S.cut[1];   // own keys: cut <= key < cut1
+        if (S.flag) return;           // the time-sorted path takes the step
+        if (cut1 < cut) {             // no time order to speak of
+            if (tid == 0) P.raw_fail = RAW_UNORDERED;
+            return;
+        }
+        const uint32_t lo = cut > dt ? cut - dt : 0u;             // earlier hits below it join nothing here
+        const uint32_t span = cut1 - lo;                          // kept keys: key - lo < span
+        const uint32_t tail = last ? 0xFFFFFFFFu : cut1 > dt ? cut1 - dt : 0u;   // own hits the next tile must see
+        const uint32_t guard = base ? ARRIVAL_DT : 0u;
+        uint32_t high = 0, bad = 0, kmin = 0xFFFFFFFFu, kmax = 0, cmin = 0xFFFFFFFFu;
+        uint32_t mine[A_ITEMS], staged = 0, own_sum = 0, tsum = 0, edge = 0;   // own_sum: own | tail << 16
+        // one record: its key and code; whether it is staged
+        auto look = [&](const uint4 &r, int32_t p, uint32_t &key, uint32_t &code) -> bool {
+            key = 0;
+            if ((uint32_t)p >= n) return false;   // (before the segment too)
+            const uint64_t rel = hit_toa(r) - base;
+            key = (uint32_t)rel;
+            high |= (uint32_t)(rel >> 32);
+            const uint32_t pix = __vminu2(r.x, limit);
+            bad |= pix ^ r.x;
+            kmin = min(kmin, key);
+            kmax = max(kmax, key);
+            if ((uint32_t)p >= n_carry) cmin = min(cmin, key);
+            code = C.code(pix);
+            return key - lo < span;
+        };
+#pragma unroll
+        for (int h = 0; h < A_ITEMS / A_GROUP; ++h) {
+            uint32_t key[A_GROUP], code[A_GROUP], mask[A_GROUP], sum = 0;
+#pragma unroll
+            for (int q = 0; q < A_GROUP; ++q) {
+                const int i = h * A_GROUP + q;
+                const bool kept = look(v[q], p0 + i * AT, key[q], code[q]);
+                mask[q] = __ballot_sync(0xffffffffu, kept);
+                sum += __popc(mask[q]);
+                mine[i] = hit_tot(v[q]);
+                if (kept) {
+                    staged |= 1u << i;
+                    if (key[q] >= cut) {
+                        own_sum += key[q] >= tail && !last ? 0x10001u : 1u;
+                        tsum += mine[i];
+                        if (i == A_ITEMS - 1) edge |= 2u;
+                    }
+                    if (i == 0) edge |= 1u;
+                }
+            }
+            if (h + 1 < A_ITEMS / A_GROUP) {
+#pragma unroll
+                for (int q = 0; q < A_GROUP; ++q) {
+                    const int32_t p = p0 + ((h + 1) * A_GROUP + q) * AT;
+                    if ((uint32_t)p < n) v[q] = ld_hit(hits + p);
+                }
+            }
+            uint32_t e0 = 0;
+            if (lane == 0) e0 = atomicAdd(&S.nent, sum);
+            e0 = __shfl_sync(0xffffffffu, e0, 0);
+#pragma unroll
+            for (int q = 0; q < A_GROUP; ++q) {
+                const int i = h * A_GROUP + q;
+                const uint32_t e = e0 + __popc(mask[q] & lanes_below());
+                if (((staged >> i) & 1u) && e < A_ENT) {
+                    S.key[e] = key[q];
+                    S.code[e] = code[q];
+                    S.par[e] = (uint16_t)e;
+                    C.set(S, code[q]);
+                    mine[i] |= e << 16;
+                }
+                e0 += __popc(mask[q]);
+            }
+        }
+        const bool given_up = tid == 0 && *reinterpret_cast<volatile uint32_t *>(&P.raw_fail) != 0;
+        own_sum = __reduce_add_sync(0xffffffffu, own_sum);
+        tsum = __reduce_add_sync(0xffffffffu, tsum);
+        kmin = __reduce_min_sync(0xffffffffu, kmin);
+        kmax = __reduce_max_sync(0xffffffffu, kmax);
+        cmin = __reduce_min_sync(0xffffffffu, cmin);
+        edge = __reduce_or_sync(0xffffffffu, edge | (bad ? 4u : 0u));
+        if (lane == 0) {
+            atomicAdd(&S.nown, own_sum & 0xFFFFu);
+            if (own_sum >> 16) atomicAdd(&S.ntail, own_sum >> 16);
+            atomicAdd(&S.tsum, tsum);
+            S.red[0][warp] = kmin;
+            S.red[1][warp] = kmax;
+            S.red[2][warp] = cmin;
+            S.red[3][warp] = edge;
+        }
+        const bool wide = high || kmin < guard || kmax > 0xFFFFFFFFu - ARRIVAL_DT;
+        if (__syncthreads_or((wide && kmin <= kmax) || given_up)) {   // (no hits: kmin > kmax)
+            if (tid == 0) atomicMax(&P.raw_fail, RAW_COVER);
+            return;
+        }
+        edge = __reduce_or_sync(0xffffffffu, S.red[3][min(lane, AW - 1)]);
+        // ---- hits beyond the margins: rounds while the outermost hits
+        // read still held some of the tile --------------------------
+        const uint32_t e_far = min(S.nent, A_ENT);
+        if (edge & 3u) __syncthreads();   // read by all before a round adds to it
+        const int32_t win = (int32_t)(j * TILE) - (int32_t)(A_MARGIN + A_ROUNDS * A_STEP);   // origin of positions
+#pragma unroll 1
+        for (int side = 0; side < 2; ++side) {
+            bool more = (edge >> side) & 1u;
+            int32_t a = side ? (int32_t)((j + 1) * TILE + A_MARGIN) : (int32_t)(j * TILE) - (int32_t)(A_MARGIN + A_STEP);
+#pragma unroll 1
+            for (int r = 0; more && r < A_ROUNDS && (side ? a < (int32_t)n : a + (int32_t)A_STEP > 0); ++r) {
+                bool outer = false;
+#pragma unroll 1
+                for (uint32_t u = tid; u < A_STEP; u += AT) {
+                    const int32_t p = a + (int32_t)u;
+                    uint32_t key, code;
+                    uint4 x = make_uint4(0, 0, 0, 0);
+                    if ((uint32_t)p < n) x = ld_hit(hits + p);
+                    if (!look(x, p, key, code)) continue;
+                    outer |= !side || key >= cut;
+                    const uint32_t e = atomicAdd(&S.nent, 1u);
+                    if (e < A_ENT && e - e_far < A_FAR) {
+                        S.key[e] = key;
+                        S.code[e] = code;
+                        S.par[e] = (uint16_t)e;
+                        S.far[e - e_far] = (uint16_t)(p - win);
+                        C.set(S, code);
+                    } else {
+                        S.flag = 1u;
+                    }
+                    if (key >= cut) {
+                        atomicAdd(&S.nown, 1u);
+                        atomicAdd(&S.tsum, hit_tot(x));
+                        if (key >= tail && !last) atomicAdd(&S.ntail, 1u);
+                    }
+                }
+                more = __syncthreads_or(outer);
+                a += side ? (int32_t)A_STEP : -(int32_t)A_STEP;
+            }
+        }
+        const uint32_t n_e = S.nent;
+        if (n_e > A_ENT || S.flag) {
+            if (tid == 0) atomicMax(&P.raw_fail, RAW_COVER);
+            return;
+        }
+        ATile &info = w.atile[t];
+        if (warp == 0) {
+            kmin = __reduce_min_sync(0xffffffffu, S.red[0][min(lane, AW - 1)]);
+            kmax = __reduce_max_sync(0xffffffffu, S.red[1][min(lane, AW - 1)]);
+            cmin = __reduce_min_sync(0xffffffffu, S.red[2][min(lane, AW - 1)]);
+            if (lane == 0) {
+                Seg &gw = w.seg[si];
+                atomicMin(reinterpret_cast<unsigned long long *>(&gw.toa_min), (unsigned long long)(base + kmin));
+                atomicMax(reinterpret_cast<unsigned long long *>(&gw.toa_max), (unsigned long long)(base + kmax));
+                if (cmin != 0xFFFFFFFFu)
+                    atomicMin(reinterpret_cast<unsigned long long *>(&gw.chunk_min), (unsigned long long)(base + cmin));
+                atomicAdd(&gw.n_owned, S.nown);
+                if (edge & 4u) atomicOr(&P.err, E_RANGE);
+                info.base = base;
+                info.cut = cut;
+                info.nhalo = n_e - S.nown;
+                info.ntail = S.ntail;
+            }
+        }
+        // ---- links -----------------------------------------------------------
+        auto own = [&](uint32_t, uint32_t key) { return key >= cut; };
+        // (keys keep 2^27 from both ends of 32 bits and dt is less: the sum wraps for no far pair)
+        const uint32_t dt2 = 2u * dt;
+        auto near = [&](uint32_t a, uint32_t b) { return a - b + dt <= dt2; };
+        arrival_links(S, C, n_e, own, near, [&](uint32_t e, bool me, uint32_t o, bool oo, bool &linked) {
+            if (me && oo) {
+                if (join_own(S, e, o, linked)) return;
+            } else if (me == oo) {
+                return;   // two earlier hits: an earlier tile's pair
+            }
+            const uint32_t k = atomicAdd(&S.ncross, 1u);   // (own pairs beyond their list too)
+            if (k < A_CROSS) S.cross[k] = me ? e << 16 | o : o << 16 | e;
+        });
+        __syncthreads();
+        // ---- positions and ToTs of the entries, where the lists were ---------
+        uint16_t *pos = S.pos(), *tot = S.tot();
+        const uint32_t nx = S.ncross;
+        if (nx > A_CROSS) {
+            if (tid == 0) atomicMax(&P.raw_fail, RAW_COVER);
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < A_ITEMS; ++i) {
+            if ((staged >> i) & 1u) {
+                pos[mine[i] >> 16] = (uint16_t)(p0 + i * AT - win);
+                tot[mine[i] >> 16] = (uint16_t)mine[i];
+            }
+        }
+        for (uint32_t e = e_far + tid; e < n_e; e += AT) {
+            pos[e] = S.far[e - e_far];
+            tot[e] = (uint16_t)hit_tot(ld_hit(hits + (win + (int32_t)S.far[e - e_far])));
+        }
+        __syncthreads();
+        for (uint32_t i = tid; i < nx; i += AT) {   // pairs across tiles, by position
+            const uint32_t x = S.cross[i];
+            w.xlist[(size_t)t * A_PAIRS + i] =
+                make_uint2(off + (uint32_t)(win + pos[x >> 16]), off + (uint32_t)(win + pos[x & 0xFFFFu]));
+        }
+        if (tid == 0) info.nx = nx;
+        arrival_clusters(w, g, t, S, C, n_e, own, pos, off + (uint32_t)win, base);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Small steps: tiles own their positions, whatever the order.
+
+// One tile.  DIRECT (k_arrival_redo): pairs are joined at once in the global
+// forest, every earlier position is looked at, nothing else is written.
+template <bool DIRECT>
+__device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShared &SS) {
+    ArrivalShared &S = SS.s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const Seg &g = w.seg[0];   // (a small step has one segment)
+    uint32_t begin, end;
+    tile_range(g, t, begin, end);
+    const uint32_t n_t = end - begin, dt = g.dt, W = g.width, H = g.height;
+    const tpc_hit *hits = g.hits;
+    const Cells C(W, H);
+    ATile &info = w.atile[t];
+    constexpr int OWN = (TILE + AT - 1) / AT;
+
+    // ---- the tile's own hits ---------------------------------------------
+    uint64_t base = g.raw_base;
+    const uint64_t low = base ? A_GUARD : 0, room = (1ull << 32) - A_GUARD - low;
+    bool wide = dt >= A_GUARD;
+    const uint32_t new0 = g.n_carry > begin ? g.n_carry - begin : 0;   // first new hit
+    uint32_t kmin, kmax, tots[OWN];
+    if (tid == 0) S.nxtra = S.ncross = S.nlater = S.nroots = S.tsum = 0;
+    C.clear(S);
+    __syncthreads();
+    for (int attempt = 0;; ++attempt) {
+        bool bad = false;
+        uint32_t cmin = 0xFFFFFFFFu;
+        kmin = 0xFFFFFFFFu;
+        if (tid < (int)ACHUNKS) S.cnt[1][tid] = 0;   // largest key of each chunk
+        __syncthreads();
+        uint4 v[OWN];
+#pragma unroll
+        for (int q = 0; q < OWN; ++q)
+            if (q * AT + tid < n_t) v[q] = ld_hit(hits + begin + q * AT + tid);
+#pragma unroll
+        for (int q = 0; q < OWN; ++q) {
+            const uint32_t e = q * AT + tid;
+            tots[q] = 0;
+            const uint32_t top = __reduce_max_sync(0xffffffffu, e < n_t ? (uint32_t)(hit_toa(v[q]) - base) : 0u);
+            if (lane == 0 && e < n_t) atomicMax(&S.cnt[1][e / A_STEP], top);   // (a warp's hits share a chunk)
+            if (e >= n_t) continue;
+            const uint64_t rel = hit_toa(v[q]) - base;
+            const uint32_t key = (uint32_t)rel, pix = clamp_pix(v[q].x, W, H), code = C.code(pix);
+            wide |= rel - low > room;
+            bad |= pix != v[q].x;
+            tots[q] = hit_tot(v[q]);
+            S.key[e] = key;
+            S.code[e] = code;
+            S.par[e] = (uint16_t)e;
+            SS.pos[e] = (uint16_t)(begin + e);
+            C.set(S, code);
+            kmin = min(kmin, key);
+            if (e >= new0) cmin = min(cmin, key);
+        }
+        if (!DIRECT && __any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&w.prob->err, E_RANGE);
+        kmin = __reduce_min_sync(0xffffffffu, kmin);
+        cmin = __reduce_min_sync(0xffffffffu, cmin);
+        if (lane == 0) { S.red[0][warp] = kmin; S.red[1][warp] = cmin; }
+        if (!__syncthreads_or(wide && attempt == 0)) break;
+        // keys relative to the segment's smallest ToA (which hold its ToAs
+        // unless they span 2^32 ticks: an error)
+        uint64_t m = ~0ull, mx = 0;
+        for (uint32_t i = tid; i < g.n; i += AT) {
+            const uint64_t a = hit_toa(ld_hit(hits + i));
+            m = a < m ? a : m;
+            mx = a > mx ? a : mx;
+        }
+        m = warp_min_u64(m);
+        mx = warp_max_u64(mx);
+        if (lane == 0) { S.m64[0][warp] = m; S.m64[1][warp] = mx; }
+        __syncthreads();
+        for (int q = 0; q < AW; ++q) {
+            m = S.m64[0][q] < m ? S.m64[0][q] : m;
+            mx = S.m64[1][q] > mx ? S.m64[1][q] : mx;
+        }
+        if (!DIRECT && tid == 0 && (mx - m) >> 32) atomicOr(&w.prob->err, E_SPAN);
+        base = m;
+    }
+    {
+        kmin = __reduce_min_sync(0xffffffffu, S.red[0][min(lane, AW - 1)]);
+        kmax = __reduce_max_sync(0xffffffffu, S.cnt[1][min(lane, (int)ACHUNKS - 1)]);
+    }
+    const uint32_t lo = kmin > dt ? kmin - dt : 0u;       // earlier hits below it join nothing here
+    const uint64_t hi = (uint64_t)kmax + dt;
+    if (!DIRECT && warp == 0) {
+        const uint32_t cmin = __reduce_min_sync(0xffffffffu, S.red[1][min(lane, AW - 1)]);
+        if (lane < (int)ACHUNKS) info.cmax[lane] = base + S.cnt[1][lane];
+        if (lane == 0) {
+            Seg &gw = w.seg[0];
+            atomicMin(reinterpret_cast<unsigned long long *>(&gw.toa_min), (unsigned long long)(base + kmin));
+            atomicMax(reinterpret_cast<unsigned long long *>(&gw.toa_max), (unsigned long long)(base + kmax));
+            if (new0 < n_t)
+                atomicMin(reinterpret_cast<unsigned long long *>(&gw.chunk_min), (unsigned long long)(base + cmin));
+            info.base = base;
+            info.lo = base + lo;
+        }
+    }
+
+    // ---- links, with the earlier hits in rounds of A_STEP positions --------
+    auto own = [&](uint32_t e, uint32_t) { return e < n_t; };
+    uint32_t h0 = begin;            // every position in [h0, begin) has been looked at
+    bool done = begin == 0, redo = false;
+    for (bool first = true;; first = false) {
+        if (!first) {               // the earlier hits so far are joined: the next ones beside the own hits
+            __syncthreads();
+            C.clear(S);
+            if (tid == 0) S.nlater = 0;
+            __syncthreads();
+            for (uint32_t e = tid; e < n_t; e += AT) C.set(S, S.code[e]);
+        }
+        uint32_t n_e = n_t;
+        for (uint32_t buf = 0; !done;) {
+            const uint32_t a = h0 - A_STEP;
+            if (DIRECT && w.atile[a / TILE].cmax[(a % TILE) / A_STEP] < base + lo) {
+                h0 = a;
+                done = h0 == 0;
+                continue;
+            }
+            uint32_t kk[A_HPER], pp[A_HPER], mask[A_HPER], sum = 0;
+#pragma unroll
+            for (int u = 0; u < A_HPER; ++u) {
+                const bool in = u * AT + tid < (int)A_STEP;
+                const uint4 v = ld_hit(hits + a + (in ? u * AT + tid : 0));
+                const uint64_t rel = hit_toa(v) - base;
+                kk[u] = (uint32_t)rel;
+                pp[u] = C.code(clamp_pix(v.x, W, H));
+                mask[u] = __ballot_sync(0xffffffffu, in && rel >= lo && rel <= hi);
+                sum += __popc(mask[u]);
+            }
+            if (lane == 0) S.turn[buf][warp] = sum | (mask[0] ? 0x80000000u : 0u);
+            __syncthreads();
+            const uint32_t c = lane < AW ? S.turn[buf][lane] : 0u;
+            buf ^= 1u;   // the next round's barrier separates this one's reads from the round after
+            const uint32_t total = __reduce_add_sync(0xffffffffu, c & 0x7FFFFFFFu);
+            const bool oldest = __any_sync(0xffffffffu, c >> 31);   // some of the oldest AT positions matter
+            if (n_e + total > A_ENT) break;   // no room beside the staged ones: join those first
+            uint32_t e = n_e + __reduce_add_sync(0xffffffffu, lane < warp ? c & 0x7FFFFFFFu : 0u);
+#pragma unroll
+            for (int u = 0; u < A_HPER; ++u) {
+                if ((mask[u] >> lane) & 1u) {
+                    const uint32_t i = e + __popc(mask[u] & lanes_below());
+                    S.key[i] = kk[u];
+                    S.code[i] = pp[u];
+                    S.par[i] = (uint16_t)i;
+                    SS.pos[i] = (uint16_t)(a + u * AT + tid);
+                    C.set(S, pp[u]);
+                }
+                e += __popc(mask[u]);
+            }
+            n_e += total;
+            h0 = a;
+            if (h0 == 0) done = true;
+            else if (!DIRECT && !oldest) done = true;
+            else if (!DIRECT && begin - h0 == A_BACK_ROUNDS * A_STEP) done = redo = true;
+        }
+        arrival_links(S, C, n_e, own, [&](uint32_t a, uint32_t b) { return absdiff(a, b) <= dt; },
+                      [&](uint32_t e, bool me, uint32_t o, bool oo, bool &linked) {
+            if (me && oo) {
+                if (!first || (!DIRECT && join_own(S, e, o, linked))) return;
+            } else if (me == oo) {
+                return;   // two earlier hits: an earlier tile's pair
+            }
+            const uint32_t a = SS.pos[e], b = SS.pos[o];
+            if (DIRECT) {
+                gunion(w.gpar, w.root_of[a], w.root_of[b]);
+            } else {
+                const uint32_t k = atomicAdd(&S.ncross, 1u);
+                if (k < A_PAIRS) w.xlist[(size_t)t * A_PAIRS + k] = make_uint2(a, b);
+            }
+        });
+        if (done) break;
+    }
+    __syncthreads();
+    if (DIRECT) return;
+    if (tid == 0) {
+        info.h0 = h0;
+        info.nx = S.ncross;
+        info.redo = redo ? 1u : 0u;
+    }
+    uint32_t tsum = 0;
+#pragma unroll
+    for (int q = 0; q < OWN; ++q) {
+        if (q * AT + tid < n_t) S.tot()[q * AT + tid] = (uint16_t)tots[q];
+        tsum += tots[q];
+    }
+    tsum = __reduce_add_sync(0xffffffffu, tsum);
+    if (lane == 0) atomicAdd(&S.tsum, tsum);
+    __syncthreads();
+    arrival_clusters(w, g, t, S, C, n_t, own, SS.pos, 0u, base);
+}
+
+__global__ void __launch_bounds__(AT) k_arrival_small(Work w) {
+    extern __shared__ __align__(16) unsigned char a_raw[];
+    SmallShared &S = *reinterpret_cast<SmallShared *>(a_raw);
+    const uint32_t nt = w.prob->ntiles;
+    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
+        __syncthreads();   // the arrays are free for the next tile
+        small_tile<false>(w, t, S);
+    }
+}
+
+// Tiles that did not look far enough back, or listed more pairs than their
+// list holds.
+__global__ void __launch_bounds__(AT) k_arrival_redo(Work w) {
+    extern __shared__ __align__(16) unsigned char a_raw[];
+    SmallShared &S = *reinterpret_cast<SmallShared *>(a_raw);
+    const uint32_t nt = w.prob->ntiles;
+    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
+        if (!w.atile[t].redo) continue;
+        __syncthreads();
+        small_tile<true>(w, t, S);
+    }
+}
+
+// Joins the listed pairs, and proves that the tiles cover the step: their
+// ToA intervals are disjoint, so every hit found its tile if the own hits add
+// up to all hits; and a tile saw every earlier hit within dt of its interval
+// if it counted as many of them as its predecessor counted own hits that
+// late (which are all there are, if dt reaches no further back than the
+// predecessor's interval).  A small step's tile that looked back to position
+// h0 is complete if every hit before h0 is earlier than its first by more
+// than dt.
+constexpr int AX = 256;
+
+__global__ void __launch_bounds__(AX) k_arrival_cross(Work w, int small, cudaGraphConditionalHandle sorted) {
+    Prob &P = *w.prob;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    bool lost = P.raw_fail != 0;
+    if (!small)
+        for (uint32_t s = tid; s < P.nsegs; s += AX) lost |= w.seg[s].n_owned != w.seg[s].n;
+    bool fail = __syncthreads_or(lost);
+    if (!fail) {
+        const uint32_t nt = P.ntiles;
+        for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
+            const ATile &info = w.atile[t];
+            if (warp == 0) {
+                const Seg &g = w.seg[w.tile_seg[t]];
+                if (small) {
+                    const uint32_t hc = info.h0 / A_STEP;   // chunks not looked at
+                    uint64_t m = 0;
+                    for (uint32_t i = lane; i < hc; i += 32) {
+                        const uint64_t c = w.atile[i / ACHUNKS].cmax[i % ACHUNKS];
+                        m = c > m ? c : m;
+                    }
+                    m = warp_max_u64(m);
+                    if (lane == 0 && ((hc && m >= info.lo) || info.nx > A_PAIRS)) w.atile[t].redo = 1u;
+                } else if (lane == 0 && t > g.tile0) {
+                    const ATile &prev = w.atile[t - 1];
+                    fail = info.nhalo != prev.ntail || (t - 1 > g.tile0 && info.cut < prev.cut + g.dt);
+                }
+            }
+            const uint32_t nx = min(info.nx, (uint32_t)A_PAIRS);
+            const uint2 *list = w.xlist + (size_t)t * A_PAIRS;
+            for (uint32_t i = tid; i < nx; i += AX) {
+                const uint2 p = list[i];
+                gunion(w.gpar, w.root_of[p.x], w.root_of[p.y]);
+            }
+            if (fail) break;   // (lane 0 of warp 0: its other tiles no longer matter)
+        }
+    }
+    if (fail && tid == 0) {
+        atomicMax(&P.raw_fail, RAW_COVER);
+        if (sorted) cudaGraphSetConditional(sorted, 1u);
+    }
+    if (blockIdx.x == 0)
+        for (uint32_t s = tid; s < P.nsegs; s += AX) seg_close(w.seg[s], P);
+}
+
+// Each tile cluster adds its features to its cluster's, and points straight
+// at it.  The finds write nothing on their way: a path halved with a parent
+// read before another thread's final store would undo that store.
+__global__ void __launch_bounds__(256) k_arrival_roots(Work w) {
+    const Prob &P = *w.prob;
+    if (P.raw_fail) return;
+    const uint32_t nt = P.ntiles;
+    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
+        const uint32_t nr = w.atile[t].nroots;
+        const bool streaming = w.seg[w.tile_seg[t]].ss != nullptr;
+        for (uint32_t i = threadIdx.x; i < nr; i += blockDim.x) {
+            const uint32_t c = t * TILE + i;
+            volatile uint32_t *par = w.gpar;
+            uint32_t r = c;
+            for (uint32_t p = par[r]; p != r; p = par[r]) r = p;
+            if (r == c) continue;
+            w.gpar[c] = r;
+            const RootSlot s = w.rslot[c];
+            RootSlot &d = w.rslot[r];
+            atomicAdd(&d.tot, s.tot);
+            atomicAdd(&d.wx, s.wx);
+            atomicAdd(&d.wy, s.wy);
+            atomicAdd(&d.size, s.size);
+            atomicMin(&d.min, s.min);
+            atomicMin(reinterpret_cast<unsigned long long *>(&w.rfirst[r]), (unsigned long long)w.rfirst[c]);
+            if (streaming)
+                atomicMax(reinterpret_cast<unsigned long long *>(&w.rlast[r]), (unsigned long long)w.rlast[c]);
+        }
+    }
+}
+
+// Labels of the hits at a tile's positions.  Their clusters are mostly tile
+// clusters of this time tile and the two beside it: those tiles' labels are
+// gathered once into shared memory (if they fit), then looked up per hit.
+constexpr uint32_t AL_CAP = 4096;
+
+__global__ void __launch_bounds__(256) k_arrival_labels(Work w) {
+    __shared__ uint32_t s_lab[AL_CAP];   // label position in the segment, closed flag
+    __shared__ uint32_t s_cnt[2];
+    const Prob &P = *w.prob;
+    if (P.raw_fail) return;
+    const uint32_t nt = P.ntiles;
+    const int lane = threadIdx.x & 31;
+    constexpr uint32_t CLOSED = 0x80000000u;   // a segment holds at most 2^31 - 1 hits
+    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
+        const Seg &g = w.seg[w.tile_seg[t]];
+        uint32_t begin, end;
+        tile_range(g, t, begin, end);
+        const uint32_t mode = g.close_mode, off = g.off;
+        const uint64_t mark = g.watermark;
+        auto label_of = [&](uint32_t c) -> uint32_t {
+            const uint32_t r = w.gpar[c];
+            const bool closed = mode == CLOSE_ALL || (mode == CLOSE_WM && w.rlast[r] <= mark);
+            return (w.rslot[r].min - off) | (closed ? CLOSED : 0u);
+        };
+        const uint32_t n0 = t > g.tile0 ? w.atile[t - 1].nroots : 0, n1 = w.atile[t].nroots;
+        const uint32_t n2 = t + 1 < g.tile0 + g.ntiles ? w.atile[t + 1].nroots : 0;
+        const bool table = n0 + n1 + n2 <= AL_CAP;
+        // c in [c0, c0 + n0), [c1, c1 + n1), [c2, c2 + n2): s_lab[c - c0], s_lab[n0 + c - c1], ...
+        const uint32_t c1 = t * TILE, c0 = c1 - TILE, c2 = c1 + TILE;
+        if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
+        if (table)
+            for (uint32_t i = threadIdx.x; i < n0 + n1 + n2; i += blockDim.x)
+                s_lab[i] = label_of(i < n0 ? c0 + i : i < n0 + n1 ? c1 + i - n0 : c2 + i - n0 - n1);
+        __syncthreads();
+        const bool direct = g.ss == nullptr;   // one-shot: every hit is final
+        uint32_t c_label = 0, c_closed = 0;
+        constexpr int ITEMS = TILE / 256;
+#pragma unroll 8
+        for (int q = 0; q < ITEMS; ++q) {
+            const uint32_t pos = begin + q * 256 + threadIdx.x;
+            bool is_label = false, closed = false;
+            if (pos < end) {
+                const uint32_t c = w.root_of[pos];
+                uint32_t v;
+                if (table && c - c1 < n1) v = s_lab[n0 + c - c1];
+                else if (table && c - c0 < n0) v = s_lab[c - c0];
+                else if (table && c - c2 < n2) v = s_lab[n0 + n1 + c - c2];
+                else v = label_of(c);
+                const uint32_t l = v & ~CLOSED;
+                closed = (v & CLOSED) != 0;
+                is_label = closed && l == pos - off;
+                const uint64_t lab = gidx_of(g, l);
+                if (direct) g.out_labels[pos - off] = lab;
+                else w.lab_tmp[pos] = lab;
+            }
+            const uint32_t bl = __ballot_sync(0xffffffffu, is_label);
+            const uint32_t bc = __ballot_sync(0xffffffffu, closed);
+            if (lane == 0) {
+                w.flag_label[pos >> 5] = bl;
+                w.flag_closed[pos >> 5] = bc;
+                c_label += __popc(bl);
+                c_closed += __popc(bc);
+            }
+        }
+        if (lane == 0) {
+            atomicAdd(&s_cnt[0], c_label);
+            atomicAdd(&s_cnt[1], c_closed);
+        }
+        __syncthreads();
+        if (threadIdx.x < 2) w.tile_cnt[threadIdx.x * P.tile_cap + t] = s_cnt[threadIdx.x];
+        __syncthreads();
+    }
+}
+
+// Records in label order (and, streaming, the finalised hits and the carry).
+// CTAs take contiguous tiles and sum the counts of their segment's earlier
+// tiles themselves: a sum over 16384 counts costs less than a launch and the
+// one-CTA scan it replaces.
+constexpr int AE = 256;
+
+__device__ uint32_t emit_sum(const uint32_t *cnt, uint32_t n, uint32_t *s_red) {
+    uint32_t m = 0;
+    for (uint32_t i = threadIdx.x; i < n; i += AE) m += cnt[i];
+    m = __reduce_add_sync(0xffffffffu, m);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    m = 0;
+    for (int q = 0; q < AE / 32; ++q) m += s_red[q];
+    return m;
+}
+
+// Exclusive prefix of the popcounts of a tile's 128 flag words.
+__device__ uint32_t emit_prefix(uint32_t bits, uint32_t *s_red) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t c = __popc(bits);
+    uint32_t x = c;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    __syncthreads();
+    if (lane == 31) s_red[warp] = x;
+    __syncthreads();
+    x -= c;
+    for (int q = 0; q < warp; ++q) x += s_red[q];
+    return x;
+}
+
+__device__ void emit_totals(Seg &g, Prob &P, uint32_t n_clusters, uint32_t n_final) {
+    g.n_clusters = n_clusters;
+    g.n_final = n_final;
+    g.n_open = g.n - n_final;
+    if (n_clusters > g.out_cap) atomicOr(&P.err, E_CAP);
+    if (!g.ss) return;
+    StreamState &ss = *g.ss;
+    if (g.n_open > g.carry_cap) atomicOr(&P.err, E_CAP);
+    ss.n_carry = g.n_open <= g.carry_cap ? g.n_open : 0;
+    ss.seen_max = g.seen_after;
+    ss.has_seen = ss.has_seen || g.n != 0;
+    if (g.close_mode == CLOSE_WM) ss.watermark = g.watermark;
+}
+
+__global__ void __launch_bounds__(AE) k_arrival_emit(Work w, uint64_t *counts, uint32_t keep) {
+    __shared__ uint32_t s_red[AE / 32];
+    __shared__ uint16_t s_pos[TILE];
+    Prob &P = *w.prob;
+    if (P.raw_fail) return;
+    const uint32_t nt = P.ntiles, cap = P.tile_cap, per = (nt + gridDim.x - 1) / gridDim.x;
+    const uint32_t t0 = blockIdx.x * per, t1 = min(t0 + per, nt);
+    const uint32_t *cnt = w.tile_cnt;
+    if (blockIdx.x == 0)   // segments without hits
+        for (uint32_t s = threadIdx.x; s < P.nsegs; s += AE)
+            if (w.seg[s].ntiles == 0) emit_totals(w.seg[s], P, 0, 0);
+    uint32_t rec = 0, fin = 0, open_total = 0;
+    const Seg *cur = nullptr;
+    for (uint32_t t = t0; t < t1; ++t) {
+        const uint32_t si = w.tile_seg[t];
+        const Seg &g = w.seg[si];
+        uint32_t begin, end;
+        tile_range(g, t, begin, end);
+        if (cur != &g) {
+            cur = &g;
+            rec = emit_sum(cnt + g.tile0, t - g.tile0, s_red);
+            fin = emit_sum(cnt + cap + g.tile0, t - g.tile0, s_red);
+            if (g.ss) open_total = g.n - emit_sum(cnt + cap + g.tile0, g.ntiles, s_red);
+        }
+        const uint32_t nwords = (end - begin + 31) >> 5;
+        uint32_t bits = threadIdx.x < nwords ? w.flag_label[(begin >> 5) + threadIdx.x] : 0;
+        uint32_t k = emit_prefix(bits, s_red);
+        while (bits) {
+            const int b = __ffs(bits) - 1;
+            bits &= bits - 1;
+            s_pos[k++] = (uint16_t)((threadIdx.x << 5) + b);
+        }
+        __syncthreads();
+        const uint32_t n_rec = cnt[t];
+        for (uint32_t i = threadIdx.x; i < n_rec; i += AE) {
+            if (rec + i >= g.out_cap) break;
+            const uint32_t pos = begin + s_pos[i];
+            const uint32_t r = w.gpar[w.root_of[pos]];
+            const RootSlot s = w.rslot[r];
+            tpc_cluster out;
+            out.label = gidx_of(g, pos - g.off);
+            out.size = (int64_t)s.size;
+            out.sum_tot = (int64_t)s.tot;
+            out.first_toa = w.rfirst[r];
+            // fp32 quotient of the exact integer sums: three roundings, each
+            // at most 2^-24 relative (FP64 is a slow pipe on this GPU)
+            const float sw = (float)s.tot;
+            out.cx = (float)s.wx / sw;
+            out.cy = (float)s.wy / sw;
+            g.out_rec[rec + i] = out;
+        }
+        if (g.ss) {
+            const bool fits = open_total <= g.carry_cap;
+            const bool vw = threadIdx.x < nwords;
+            const uint32_t cl = vw ? w.flag_closed[(begin >> 5) + threadIdx.x] : 0;
+            uint32_t closed = fin + emit_prefix(cl, s_red);
+            if (vw) {
+                const uint32_t first = begin + (threadIdx.x << 5), last = min(first + 32, end);
+                for (uint32_t pos = first; pos < last; ++pos) {
+                    const uint32_t local = pos - g.off;
+                    if ((cl >> (pos - first)) & 1u) {
+                        if (closed < g.out_cap) {
+                            g.out_labels[closed] = w.lab_tmp[pos];
+                            if (g.out_index) g.out_index[closed] = gidx_of(g, local);
+                        }
+                        ++closed;
+                    } else if (fits) {
+                        const uint32_t dst = g.carry_cap - open_total + (local - closed);
+                        g.carry_out[dst] = g.hits[local];
+                        g.carry_gidx_out[dst] = gidx_of(g, local);
+                    }
+                }
+            }
+        }
+        rec += n_rec;
+        fin += cnt[cap + t];
+        if (t + 1 == g.tile0 + g.ntiles && threadIdx.x == 0) {
+            emit_totals(w.seg[si], P, rec, fin);
+            if (counts) {   // tpc_cluster_static's result words
+                counts[0] = rec;
+                counts[1] = P.err & keep;
+            }
+        }
+        __syncthreads();   // s_pos is rewritten for the next tile
+    }
+}
+
+cudaError_t init_arrival_attributes() {
+    cudaError_t e = cudaFuncSetAttribute(k_arrival_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_arrival_small, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMALL_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_arrival_redo, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMALL_SMEM);
+    return e;
+}
+
+// A small step has at most SMALL_TILES tiles.
+static int grid_of(int fit, bool small) { return small && fit > (int)SMALL_TILES ? (int)SMALL_TILES : fit; }
+
+// Links and the decision; `sorted` (0: none) is the conditional node that
+// holds the time-sorted path.
+void launch_arrival_link(const Work &w, bool small, cudaGraphConditionalHandle sorted, const Launch &L) {
+    if (small) {
+        k_arrival_small<<<SMALL_TILES, AT, A_SMALL_SMEM, L.stream>>>(w);
+        L.mark("k_arrival_small");
+    } else {
+        k_arrival_tile<<<L.fit(k_arrival_tile, AT, A_SMEM, G_LINK), AT, A_SMEM, L.stream>>>(w);
+        L.mark("k_arrival_tile");
+    }
+    k_arrival_cross<<<grid_of(L.fit(k_arrival_cross, AX, 0, G_LINK), small), AX, 0, L.stream>>>(w, small, sorted);
+    L.mark("k_arrival_cross");
+    if (small) {
+        k_arrival_redo<<<SMALL_TILES, AT, A_SMALL_SMEM, L.stream>>>(w);
+        L.mark("k_arrival_redo");
+    }
+}
+
+void launch_arrival_output(const Work &w, bool small, uint64_t *counts, uint32_t keep, const Launch &L) {
+    k_arrival_roots<<<grid_of(L.fit(k_arrival_roots, 256, 0, G_ACC), small), 256, 0, L.stream>>>(w);
+    L.mark("k_arrival_roots");
+    k_arrival_labels<<<grid_of(L.fit(k_arrival_labels, 256, 0, G_OUT), small), 256, 0, L.stream>>>(w);
+    L.mark("k_arrival_labels");
+    k_arrival_emit<<<grid_of(L.fit(k_arrival_emit, AE, 0, G_OUT), small), AE, 0, L.stream>>>(w, counts, keep);
+    L.mark("k_arrival_emit");
+}
+
+}  // namespace tpc

@@ -892,6 +892,7 @@ cudaError_t init_kernel_attributes() {
         e = cudaFuncSetAttribute(k_tile_link_table, cudaFuncAttributeMaxDynamicSharedMemorySize, TAB_SMEM);
     if (e == cudaSuccess) e = init_features_attributes();
     if (e == cudaSuccess) e = init_variants_attributes();
+    if (e == cudaSuccess) e = init_arrival_attributes();
     return e == cudaSuccess ? init_sortfast_attributes() : e;
 }
 

@@ -9,8 +9,8 @@
 // working memory comes from the fixed array below, which every GPU that
 // loads the library holds until the process exits.
 //
-// The kernels are the library's own (the same launch sequence as
-// tpc_flush); only the source of their scratch differs.  Every call shares
+// The kernels are the library's own (those of a small tpc_flush); only the
+// source of their scratch differs.  Every call shares
 // the one array and leaves its last contents behind: nothing in it has to
 // start at zero, because each call first rewrites the segment and problem
 // descriptors and every other array is fully written before it is read.
@@ -33,9 +33,8 @@ constexpr size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // byte offsets of every work array inside the scratch array
 struct Layout {
-    size_t seg, prob, tile_seg, redo, border_list, keys0, keys1, vals0, vals1, spix, stot, parent, root_of,
-        slot, flag_label, flag_closed,
-        tile_cnt, tile_base, hist, segtot, total;
+    size_t seg, prob, tile_seg, root_of, gpar, rslot, rfirst, xlist, flag_label, flag_closed, tile_cnt, atile, atmax,
+        total;
 };
 
 constexpr Layout make_layout() {
@@ -44,23 +43,16 @@ constexpr Layout make_layout() {
     l.seg = o; o += align256(sizeof(Seg));
     l.prob = o; o += align256(sizeof(Prob));
     l.tile_seg = o; o += align256(NA_TILES * 4);
-    l.redo = o; o += align256(NA_TILES * 4);
-    l.border_list = o; o += align256(NA_TILES * 4);
-    l.keys0 = o; o += align256(NA_POS * 4);
-    l.keys1 = o; o += align256(NA_POS * 4);
-    l.vals0 = o; o += align256(NA_POS * 4);
-    l.vals1 = o; o += align256(NA_POS * 4);
-    l.spix = o; o += align256(NA_POS * 4);
-    l.stot = o; o += align256(NA_POS * 2);
-    l.parent = o; o += align256(NA_POS * 4);
     l.root_of = o; o += align256(NA_POS * 4);
-    l.slot = o; o += align256(NA_POS * sizeof(Slot));
+    l.gpar = o; o += align256(NA_POS * 4);
+    l.rslot = o; o += align256(NA_POS * sizeof(RootSlot));
+    l.rfirst = o; o += align256(NA_POS * 8);
+    l.xlist = o; o += align256((size_t)NA_TILES * A_PAIRS * sizeof(uint2));
     l.flag_label = o; o += align256((NA_POS / 32 + 1) * 4);
     l.flag_closed = o; o += align256((NA_POS / 32 + 1) * 4);
     l.tile_cnt = o; o += align256(2 * NA_TILES * 4);
-    l.tile_base = o; o += align256(2 * NA_TILES * 4);
-    l.hist = o; o += align256((size_t)RADIX * NA_TILES * 4);
-    l.segtot = o; o += align256((size_t)MAX_SEGS * RADIX * 4);
+    l.atile = o; o += align256(NA_TILES * sizeof(ATile));
+    l.atmax = o; o += align256(NA_TILES * 4);
     l.total = o;
     return l;
 }
@@ -102,14 +94,6 @@ __global__ void k_na_begin(Work w, Seg s, uint32_t tile_cap, uint32_t pos_cap) {
     *w.prob = p;
 }
 
-// counts[1] keeps the public bits only (TPC_STATIC_E_*); with no record
-// buffer (record_cap == 0) the caller asked for labels alone, so more
-// clusters than records is not an error then.
-__global__ void k_na_end(Work w, uint64_t *counts, uint32_t keep) {
-    counts[0] = w.seg[0].n_clusters;
-    counts[1] = w.prob->err & keep;
-}
-
 __global__ void k_na_empty(uint64_t *counts) {
     counts[0] = 0;
     counts[1] = 0;
@@ -144,24 +128,16 @@ extern "C" int tpc_cluster_static(const tpc_hit *hits, size_t n, uint32_t width,
     w.seg = reinterpret_cast<Seg *>(base + NA.seg);
     w.prob = reinterpret_cast<Prob *>(base + NA.prob);
     w.tile_seg = reinterpret_cast<uint32_t *>(base + NA.tile_seg);
-    w.redo = reinterpret_cast<uint32_t *>(base + NA.redo);
-    w.border_list = reinterpret_cast<uint32_t *>(base + NA.border_list);
-    w.keys[0] = reinterpret_cast<uint32_t *>(base + NA.keys0);
-    w.keys[1] = reinterpret_cast<uint32_t *>(base + NA.keys1);
-    w.vals[0] = reinterpret_cast<uint32_t *>(base + NA.vals0);
-    w.vals[1] = reinterpret_cast<uint32_t *>(base + NA.vals1);
-    w.spix = reinterpret_cast<uint32_t *>(base + NA.spix);
-    w.stot = reinterpret_cast<uint16_t *>(base + NA.stot);
-    w.parent = reinterpret_cast<uint32_t *>(base + NA.parent);
     w.root_of = reinterpret_cast<uint32_t *>(base + NA.root_of);
-    w.slot = reinterpret_cast<Slot *>(base + NA.slot);
-    w.lab_tmp = nullptr;   // streaming only
+    w.gpar = reinterpret_cast<uint32_t *>(base + NA.gpar);
+    w.rslot = reinterpret_cast<RootSlot *>(base + NA.rslot);
+    w.rfirst = reinterpret_cast<uint64_t *>(base + NA.rfirst);
+    w.xlist = reinterpret_cast<uint2 *>(base + NA.xlist);
     w.flag_label = reinterpret_cast<uint32_t *>(base + NA.flag_label);
     w.flag_closed = reinterpret_cast<uint32_t *>(base + NA.flag_closed);
     w.tile_cnt = reinterpret_cast<uint32_t *>(base + NA.tile_cnt);
-    w.tile_base = reinterpret_cast<uint32_t *>(base + NA.tile_base);
-    w.hist = reinterpret_cast<uint32_t *>(base + NA.hist);
-    w.segtot = reinterpret_cast<uint32_t *>(base + NA.segtot);
+    w.atile = reinterpret_cast<ATile *>(base + NA.atile);
+    w.atmax = reinterpret_cast<uint32_t *>(base + NA.atmax);
 
     Seg s{};
     s.hits = hits;
@@ -178,18 +154,14 @@ extern "C" int tpc_cluster_static(const tpc_hit *hits, size_t n, uint32_t width,
 
     const Launch L{sms * 4, st, nullptr, sms};
     k_na_begin<<<1, 1, 0, st>>>(w, s, NA_TILES, NA_POS);
-    launch_setup(w, 1, L);
-    launch_sort_fast(w, L);
-    launch_seg_finalize(w, L);
-    launch_make_keys(w, L);
-    for (int pass = 0; pass < 4; ++pass) launch_radix_pass(w, pass, L);
-    launch_gather(w, L);
-    launch_link(w, L);
-    launch_features(w, L);
-    launch_outputs(w, L);
+    // counts[1] keeps the public bits only; with no record buffer
+    // (record_cap == 0) the caller asked for labels alone, so more clusters
+    // than records is not an error then
     static_assert(E_RANGE == TPC_STATIC_E_RANGE && E_SPAN == TPC_STATIC_E_SPAN && E_CAP == TPC_STATIC_E_CAP,
                   "public error bits");
     const uint32_t keep = TPC_STATIC_E_RANGE | TPC_STATIC_E_SPAN | (record_cap ? TPC_STATIC_E_CAP : 0u);
-    k_na_end<<<1, 1, 0, st>>>(w, counts, keep);
+    launch_setup(w, 1, L, true);
+    launch_arrival_link(w, true, 0, L);
+    launch_arrival_output(w, true, counts, keep, L);
     return cudaGetLastError() == cudaSuccess ? TPC_OK : TPC_ERR_CUDA;
 }

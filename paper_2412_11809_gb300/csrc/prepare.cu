@@ -9,7 +9,7 @@ namespace tpc {
 // fill the tile -> segment table.  Streaming segments pick up the carry left
 // by the previous step: it sits right-aligned in the carry region of their
 // input buffer, immediately followed by the new chunk.
-__global__ void k_setup(Work w, int nsegs) {
+__global__ void k_setup(Work w, int nsegs, uint32_t arrival) {
     __shared__ uint32_t s_tile0[MAX_SEGS + 1];
     if (threadIdx.x == 0) {
         uint32_t off = 0, tile = 0;
@@ -24,7 +24,10 @@ __global__ void k_setup(Work w, int nsegs) {
                 g.carry_gidx = nullptr;
             }
             g.n = g.n_carry + g.n_new;
-            g.fast_base = fast_key_base(g);
+            const uint64_t t0 = g.n ? hit_toa(ld_hit(g.hits)) : 0;
+            g.fast_base = fast_key_base(t0);
+            g.raw_base = t0 > ARRIVAL_BACK ? t0 - ARRIVAL_BACK : 0;
+            g.n_owned = 0;
             g.off = off;
             g.tile0 = tile;
             g.ntiles = (g.n + TILE - 1) / TILE;
@@ -49,6 +52,8 @@ __global__ void k_setup(Work w, int nsegs) {
         p.redo_count = 0;
         p.border_count = 0;
         p.merge_count = 0;
+        p.raw = arrival;
+        p.raw_fail = 0;
         p.err = 0;
         p.ntiles = tile;
         if (tile > p.tile_cap || off > p.pos_cap) {
@@ -73,10 +78,7 @@ __global__ void k_setup(Work w, int nsegs) {
 // relative to fast_key_base; if a ToA lies outside 2^32 ticks of that base,
 // or the check found the tiles out of order, every segment takes the
 // general sort with keys relative to its minimum ToA) and the streaming
-// watermark.  A later hit j satisfies toa_j > seen_max - max_disorder (the
-// t-ordered property, Section 3.1), and can join hit i only if
-// toa_j - toa_i <= dt, so every cluster whose last ToA <=
-// seen_max - max_disorder - dt is final.
+// watermark (seg_close).
 __global__ void k_seg_finalize(Work w) {
     __shared__ uint32_t s_fallback;
     const uint32_t nsegs = w.prob->nsegs;
@@ -87,9 +89,7 @@ __global__ void k_seg_finalize(Work w) {
         uint32_t passes = 0;
         if (g.n) {
             uint64_t span = g.toa_max - g.toa_min;
-            if (span >> 32) {
-                atomicOr(&w.prob->err, E_SPAN);
-            } else if (span) {
+            if (span && !(span >> 32)) {
                 uint32_t bits = 64 - __clzll((long long)span);
                 passes = (bits + RADIX_BITS - 1) / RADIX_BITS;
             }
@@ -98,27 +98,7 @@ __global__ void k_seg_finalize(Work w) {
         }
         g.npasses = passes;
         atomicMax(&w.prob->lsd_passes, passes);   // used only by the general sort
-        if (!g.ss) {
-            g.close_mode = CLOSE_ALL;   // one-shot: the end of the stream
-            continue;
-        }
-        StreamState &ss = *g.ss;
-        const uint64_t md = g.max_disorder;   // ~0: a flush of a streaming context
-        if (md != ~0ull && g.n_new && ss.has_seen && ss.seen_max >= md &&
-            g.chunk_min <= ss.seen_max - md)
-            atomicOr(&w.prob->err, E_LATE);
-        uint64_t seen = ss.has_seen ? ss.seen_max : 0;
-        if (g.n && g.toa_max > seen) seen = g.toa_max;
-        g.seen_after = seen;
-        const uint64_t lag = md + (uint64_t)g.dt;
-        if (md == ~0ull) {
-            g.close_mode = CLOSE_ALL;
-        } else if (lag >= md && seen >= lag) {
-            g.close_mode = CLOSE_WM;
-            g.watermark = seen - lag;
-        } else {
-            g.close_mode = CLOSE_NONE;
-        }
+        seg_close(g, *w.prob);
     }
     __syncthreads();
     const uint32_t fallback = s_fallback;
@@ -194,8 +174,8 @@ __global__ void __launch_bounds__(256) k_gather(Work w) {
     }
 }
 
-void launch_setup(const Work &w, int nsegs, const Launch &L) {
-    k_setup<<<1, 1024, 0, L.stream>>>(w, nsegs);
+void launch_setup(const Work &w, int nsegs, const Launch &L, bool arrival) {
+    k_setup<<<1, 1024, 0, L.stream>>>(w, nsegs, arrival);
     L.mark("k_setup");
 }
 void launch_seg_finalize(const Work &w, const Launch &L) {

@@ -146,6 +146,13 @@ __global__ void __launch_bounds__(LS_THREADS, 3) k_tile_sort(Work w) {
             atomicMax(reinterpret_cast<unsigned long long *>(&gw.toa_max), (unsigned long long)tmax);
             atomicMin(reinterpret_cast<unsigned long long *>(&gw.chunk_min), (unsigned long long)cmin);
         }
+        if (P.raw_fail == RAW_UNORDERED) {   // only the extremes and the range check: the general sort orders the hits
+            bool out = false;
+            for (uint32_t j = threadIdx.x; j < n_t; j += LS_THREADS)
+                out |= (S.pix[j] & 0xFFFFu) >= g.width || (S.pix[j] >> 16) >= g.height;
+            if (__syncthreads_or(out) && threadIdx.x == 0) atomicOr(&w.prob->err, E_RANGE);
+            continue;
+        }
         const uint32_t span = kmax - kmin;
         const int passes = span ? (32 - __clz(span) + LS_BITS - 1) / LS_BITS : 0;
 
@@ -269,7 +276,7 @@ __global__ void __launch_bounds__(LS_THREADS) k_tile_merge(Work w) {
     LmShared<BIG ? (uint32_t)TILE : 2 * MERGE_BAND> &S =
         *reinterpret_cast<LmShared<BIG ? (uint32_t)TILE : 2 * MERGE_BAND> *>(lm_raw);
     const Prob &P = *w.prob;
-    const uint32_t nt = BIG ? P.merge_count : P.ntiles;   // the big kernel: the listed borders
+    const uint32_t nt = P.raw_fail == RAW_UNORDERED ? 0u : BIG ? P.merge_count : P.ntiles;   // BIG: the listed borders
     for (uint32_t u = blockIdx.x; u < nt; u += gridDim.x) {
         const uint32_t t = BIG ? w.redo[u] : u;
         const Seg &g = w.seg[w.tile_seg[t]];
@@ -351,8 +358,8 @@ __global__ void __launch_bounds__(LS_THREADS) k_tile_merge(Work w) {
 __global__ void __launch_bounds__(256) k_sort_check(Work w) {
     const Prob &P = *w.prob;
     const uint32_t nt = P.ntiles;
-    bool bad = false;
-    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += gridDim.x * blockDim.x) {
+    bool bad = P.raw_fail == RAW_UNORDERED;
+    for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; !bad && t < nt; t += gridDim.x * blockDim.x) {
         const Seg &g = w.seg[w.tile_seg[t]];
         uint32_t begin, end;
         tile_range(g, t, begin, end);

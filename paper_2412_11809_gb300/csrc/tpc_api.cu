@@ -3,7 +3,11 @@
 //
 // A processing step (tpc_flush, a streaming tpc_push, or tpc_batch_flush)
 // enqueues the same fixed kernel sequence on one CUDA stream:
-//   setup -> tile sort -> tile merge -> sort check -> segment finalize ->
+//   setup -> arrival-order tiles -> cross pairs -> [the time-sorted path] ->
+//   roots -> labels -> emit,
+// where the time-sorted path runs only if the cross kernel found that the
+// arrival-order one does not cover the step (a conditional graph node):
+//   tile sort -> tile merge -> sort check -> segment finalize ->
 //   (general-order fallback: keys -> radix passes 0..3 -> gather) ->
 //   table link -> tile link (redo tiles) -> border fast -> border link ->
 //   accumulate (finds the roots) -> labels -> tile scan -> records ->
@@ -181,10 +185,12 @@ struct Workspace {
         w.redo = mem.alloc<uint32_t>(T, e);
         w.border_list = mem.alloc<uint32_t>(T, e);
         w.keys[0] = mem.alloc<uint32_t>(P, e);
-        w.keys[1] = mem.alloc<uint32_t>(P, e);
-        w.vals[0] = mem.alloc<uint32_t>(P, e);
-        w.vals[1] = mem.alloc<uint32_t>(P, e);
-        w.spix = mem.alloc<uint32_t>(P, e);
+        w.rfirst = mem.alloc<uint64_t>(P, e);   // one block for the pair keys[1], vals[1]
+        w.keys[1] = reinterpret_cast<uint32_t *>(w.rfirst);
+        w.vals[1] = w.keys[1] + P;
+        w.rlast = mem.alloc<uint64_t>(P, e);    // and one for vals[0], spix
+        w.vals[0] = reinterpret_cast<uint32_t *>(w.rlast);
+        w.spix = w.vals[0] + P;
         w.stot = mem.alloc<uint16_t>(P, e);
         w.parent = mem.alloc<uint32_t>(P, e);
         w.root_of = mem.alloc<uint32_t>(P, e);
@@ -196,6 +202,12 @@ struct Workspace {
         w.tile_base = mem.alloc<uint32_t>(2 * T, e);
         w.hist = mem.alloc<uint32_t>((size_t)RADIX * T, e);
         w.segtot = mem.alloc<uint32_t>((size_t)MAX_SEGS * RADIX, e);
+        w.gpar = w.parent;
+        w.rslot = reinterpret_cast<RootSlot *>(w.slot);
+        w.xlist = reinterpret_cast<uint2 *>(w.lab_tmp);
+        w.rkey = w.keys[0];
+        w.atile = reinterpret_cast<ATile *>(w.hist);
+        w.atmax = w.tile_base;
         if (e == cudaSuccess) {
             Prob p{};
             p.tile_cap = (uint32_t)T;
@@ -292,6 +304,12 @@ __global__ void k_iota_u64(uint64_t *out, uint64_t base, size_t n) {
 
 }  // namespace
 
+// Path of a one-shot (a) or streaming step: in arrival order with the
+// time-sorted path behind it, in arrival order alone (small steps), or
+// time-sorted from the start (launch choices that name a sorted link kernel,
+// time windows the arrival-order keys cannot hold).
+enum StepMode { STEP_ARRIVAL, STEP_SMALL, STEP_SORTED };
+
 struct tpc_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -364,6 +382,7 @@ struct tpc_ctx {
     // graph of the step sequence
     cudaGraphExec_t graph = nullptr;
     int graph_nsegs = 0;
+    StepMode graph_mode{};         // the path the graph starts on
     uint64_t graph_gen = 0;        // workspace generation the graph was captured on
     int graph_grid = 0;
     Tuning graph_tune{};           // launch choices the graph was captured with
@@ -445,8 +464,8 @@ cudaError_t upload_segs(tpc_ctx *c, const Work &w, const Seg *segs, int nsegs, c
     return cudaEventRecord(c->seg_ev[slot], st);
 }
 
-void enqueue_kernels(const Work &w, int nsegs, const Launch &L) {
-    launch_setup(w, nsegs, L);
+// The time-sorted path, after the set-up.
+void enqueue_sorted(const Work &w, const Launch &L) {
     launch_sort_fast(w, L);
     launch_seg_finalize(w, L);
     launch_make_keys(w, L);
@@ -457,19 +476,81 @@ void enqueue_kernels(const Work &w, int nsegs, const Launch &L) {
     launch_outputs(w, L);
 }
 
-// Run the fixed kernel sequence, from a CUDA graph captured on first use
-// (and re-captured when the workspace or the segment count changes).
-cudaError_t run_step(tpc_ctx *owner, Workspace &ws, int nsegs, cudaStream_t st, Tracer *tr = nullptr) {
+// A whole step on the capturing stream L.stream: the arrival-order path and,
+// in a conditional node that its cross kernel switches on, the time-sorted
+// path for the steps it cannot cover.
+cudaError_t capture_step(const Work &w, int nsegs, StepMode mode, const Launch &L) {
+    launch_setup(w, nsegs, L, mode != STEP_SORTED);
+    if (mode == STEP_SORTED) {
+        enqueue_sorted(w, L);
+        return cudaGetLastError();
+    }
+    const bool small = mode == STEP_SMALL;
+    cudaGraphConditionalHandle cond = 0;
+    cudaStreamCaptureStatus status;
+    cudaGraph_t graph = nullptr;
+    cudaError_t e = cudaStreamGetCaptureInfo(L.stream, &status, nullptr, &graph, nullptr, nullptr, nullptr);
+    if (e == cudaSuccess && !small) e = cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault);
+    if (e != cudaSuccess) return e;
+    launch_arrival_link(w, small, cond, L);
+    if (!small) {
+        const cudaGraphNode_t *deps = nullptr;
+        const cudaGraphEdgeData *edges = nullptr;
+        size_t ndeps = 0;
+        e = cudaStreamGetCaptureInfo(L.stream, &status, nullptr, &graph, &deps, &edges, &ndeps);
+        if (e != cudaSuccess) return e;
+        cudaGraphNodeParams p{};
+        p.type = cudaGraphNodeTypeConditional;
+        p.conditional.handle = cond;
+        p.conditional.type = cudaGraphCondTypeIf;
+        p.conditional.size = 1;
+        cudaGraphNode_t node = nullptr;
+        e = cudaGraphAddNode(&node, graph, deps, edges, ndeps, &p);
+        if (e != cudaSuccess) return e;
+        cudaStream_t body;
+        e = cudaStreamCreateWithFlags(&body, cudaStreamNonBlocking);
+        if (e != cudaSuccess) return e;
+        e = cudaStreamBeginCaptureToGraph(body, p.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                          cudaStreamCaptureModeThreadLocal);
+        if (e == cudaSuccess) {
+            Launch B = L;
+            B.stream = body;
+            enqueue_sorted(w, B);
+            cudaGraph_t same = nullptr;
+            e = cudaStreamEndCapture(body, &same);
+        }
+        cudaStreamDestroy(body);
+        if (e != cudaSuccess) return e;
+        e = cudaStreamUpdateCaptureDependencies(L.stream, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
+        if (e != cudaSuccess) return e;
+    }
+    launch_arrival_output(w, small, nullptr, 0, L);
+    return cudaGetLastError();
+}
+
+// One step of a context: its kernel sequence, from a CUDA graph captured on
+// first use (and re-captured when the workspace, the segment count or the
+// path changes).
+cudaError_t run_step(tpc_ctx *owner, Workspace &ws, int nsegs, StepMode mode, cudaStream_t st, Tracer *tr = nullptr) {
     Launch L{grid_of(owner), st, nullptr, owner->sms, owner->ctas_per_sm};
     L.tune = owner->tune;
     if (tr) {   // kernels one by one with an event after each (no graph)
         cudaEventRecord(tr->ev[0], st);
         Launch T = L;
         T.tr = tr;
-        enqueue_kernels(ws.w, nsegs, T);
+        launch_setup(ws.w, nsegs, T, mode != STEP_SORTED);
+        uint32_t sorted = mode == STEP_SORTED;
+        if (!sorted) {
+            launch_arrival_link(ws.w, mode == STEP_SMALL, 0, T);
+            cudaError_t e = cudaMemcpyAsync(&sorted, &ws.w.prob->raw_fail, sizeof(sorted), cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            if (e != cudaSuccess) return e;
+        }
+        if (sorted) enqueue_sorted(ws.w, T);
+        else launch_arrival_output(ws.w, mode == STEP_SMALL, nullptr, 0, T);
         return cudaGetLastError();
     }
-    if (!owner->graph || owner->graph_nsegs != nsegs || owner->graph_gen != ws.gen ||
+    if (!owner->graph || owner->graph_nsegs != nsegs || owner->graph_mode != mode || owner->graph_gen != ws.gen ||
         owner->graph_grid != L.grid || std::memcmp(&owner->graph_tune, &owner->tune, sizeof(Tuning)) != 0) {
         if (owner->graph) {
             cudaGraphExecDestroy(owner->graph);
@@ -483,8 +564,9 @@ cudaError_t run_step(tpc_ctx *owner, Workspace &ws, int nsegs, cudaStream_t st, 
         if (e == cudaSuccess) {
             Launch C = L;
             C.stream = cap_st;
-            enqueue_kernels(ws.w, nsegs, C);
-            e = cudaStreamEndCapture(cap_st, &g);
+            e = capture_step(ws.w, nsegs, mode, C);
+            const cudaError_t end = cudaStreamEndCapture(cap_st, &g);
+            if (e == cudaSuccess) e = end;
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&owner->graph, g, 0);
         if (g) cudaGraphDestroy(g);
@@ -494,11 +576,19 @@ cudaError_t run_step(tpc_ctx *owner, Workspace &ws, int nsegs, cudaStream_t st, 
             return e;
         }
         owner->graph_nsegs = nsegs;
+        owner->graph_mode = mode;
         owner->graph_gen = ws.gen;
         owner->graph_grid = L.grid;
         owner->graph_tune = owner->tune;
     }
     return cudaGraphLaunch(owner->graph, st);
+}
+
+// The path of a step over these segments; positions: at least its hits.
+StepMode step_mode(const Seg *segs, int nsegs, size_t positions) {
+    for (int i = 0; i < nsegs; ++i)
+        if (segs[i].link_general || segs[i].dt >= ARRIVAL_DT) return STEP_SORTED;
+    return nsegs == 1 && positions <= (size_t)SMALL_TILES * TILE ? STEP_SMALL : STEP_ARRIVAL;
 }
 
 // Outputs of a one-shot step: the caller's bound buffers, else the
@@ -655,7 +745,7 @@ int stream_step(tpc_ctx *c, size_t n, bool close_all) {
     s.carry_cap = (uint32_t)c->carry_cap;
     s.n_new = (uint32_t)n;
     if (upload_segs(c, c->ws.w, &s, 1, c->stream) != cudaSuccess) return TPC_ERR_CUDA;
-    if (run_step(c, c->ws, 1, c->stream) != cudaSuccess) return TPC_ERR_CUDA;
+    if (run_step(c, c->ws, 1, step_mode(&s, 1, positions), c->stream) != cudaSuccess) return TPC_ERR_CUDA;
     c->scur = in;
     c->pushed += n;
     c->carry_ub = close_all ? 0 : positions;
@@ -663,6 +753,45 @@ int stream_step(tpc_ctx *c, size_t n, bool close_all) {
     c->res_prob = c->ws.w.prob;
     c->has_result = true;
     c->res_streaming = true;
+    return TPC_OK;
+}
+
+// tpc_forest of a step on the arrival-order path, whose union-find runs over
+// tile clusters: the (ToA, input) order from the kept keys (a stable radix
+// sort on the host), every hit's parent its cluster's earliest hit.
+int forest_of_arrival(tpc_ctx *c, const Seg &g, uint32_t *parent, uint32_t *input_pos) {
+    const size_t n = g.n, tiles = (n + TILE - 1) / TILE;
+    const Work &w = c->ws.w;
+    try {
+        std::vector<uint32_t> cluster(n), key(n), gpar(tiles * TILE), a(n), first(tiles * TILE, 0xFFFFFFFFu);
+        std::vector<ATile> at(tiles);
+        std::vector<uint64_t> toa(n);
+        if (cudaMemcpy(cluster.data(), w.root_of, n * 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
+            cudaMemcpy(key.data(), w.rkey, n * 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
+            cudaMemcpy(gpar.data(), w.gpar, tiles * TILE * 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
+            cudaMemcpy(at.data(), w.atile, tiles * sizeof(ATile), cudaMemcpyDeviceToHost) != cudaSuccess)
+            return TPC_ERR_CUDA;
+        uint64_t lowest = ~0ull;
+        for (size_t i = 0; i < n; ++i) {
+            toa[i] = at[i / TILE].base + key[i];
+            lowest = std::min(lowest, toa[i]);
+            a[i] = (uint32_t)i;
+        }
+        for (int shift = 0; shift < 32; shift += 16) {   // a step's ToAs span less than 2^32 ticks
+            std::vector<size_t> start(65537, 0);
+            for (size_t i = 0; i < n; ++i) ++start[(((toa[i] - lowest) >> shift) & 0xFFFF) + 1];
+            for (int d = 0; d < 65536; ++d) start[d + 1] += start[d];
+            for (size_t i = 0; i < n; ++i) input_pos[start[((toa[a[i]] - lowest) >> shift) & 0xFFFF]++] = a[i];
+            std::copy(input_pos, input_pos + n, a.begin());
+        }
+        for (size_t s = 0; s < n; ++s) {
+            const size_t root = gpar[cluster[a[s]]];
+            if (first[root] == 0xFFFFFFFFu) first[root] = (uint32_t)s;
+            parent[s] = first[root];
+        }
+    } catch (const std::bad_alloc &) {
+        return TPC_ERR_NOMEM;
+    }
     return TPC_OK;
 }
 
@@ -938,7 +1067,7 @@ static int flush_impl(tpc_ctx *c, Tracer *tr) {
     s.gidx_base = c->pushed;
     s.n_new = (uint32_t)n;
     if (upload_segs(c, c->ws.w, &s, 1, c->stream) != cudaSuccess) return TPC_ERR_CUDA;
-    if (run_step(c, c->ws, 1, c->stream, tr) != cudaSuccess) return TPC_ERR_CUDA;
+    if (run_step(c, c->ws, 1, step_mode(&s, 1, n), c->stream, tr) != cudaSuccess) return TPC_ERR_CUDA;
     c->res_base = c->pushed;
     c->pushed += n;
     c->pending = 0;
@@ -1106,7 +1235,7 @@ int tpc::batch_step(tpc_ctx **ctxs, int n, bool consume) {
         segs[k] = s;
     }
     if (upload_segs(lead, lead->ws.w, segs.data(), n, lead->stream) != cudaSuccess) return TPC_ERR_CUDA;
-    if (run_step(lead, lead->ws, n, lead->stream) != cudaSuccess) return TPC_ERR_CUDA;
+    if (run_step(lead, lead->ws, n, step_mode(segs.data(), n, positions), lead->stream) != cudaSuccess) return TPC_ERR_CUDA;
     for (int k = 0; k < n; ++k) {   // each context keeps its own copy of its results
         tpc_ctx *c = ctxs[perm[k]];
         if (cudaMemcpyAsync(c->own_res_seg, lead->ws.w.seg + k, sizeof(Seg), cudaMemcpyDeviceToDevice,
@@ -1155,6 +1284,7 @@ int tpc_forest(tpc_ctx *c, uint32_t *parent, uint32_t *input_pos, size_t cap, si
     if (n > cap) return TPC_ERR_CAP;
     if (!n) return TPC_OK;
     if (!parent || !input_pos) return TPC_ERR_ARG;
+    if (r.prob.raw && !r.prob.raw_fail) return forest_of_arrival(c, r.seg, parent, input_pos);
     // the sorted order lives in the buffer the step's last sort pass wrote
     const uint32_t sel = r.prob.npasses & 1u;
     if (cudaMemcpy(parent, c->ws.w.parent + r.seg.off, n * sizeof(uint32_t), cudaMemcpyDeviceToHost) !=

@@ -29,6 +29,15 @@ constexpr int RADIX_BITS = 8;
 constexpr int RADIX = 1 << RADIX_BITS;
 constexpr uint32_t MAX_PIXELS = 1u << 20;   // width*height bound (packed smem keys)
 
+// Arrival-order path (arrival.cu): chunks per tile whose ToA maxima it keeps,
+// pairs across tiles listed per tile, the tiles of a small step (one that
+// needs no time-sorted path behind it).
+constexpr uint32_t ACHUNKS = 4;
+constexpr uint32_t A_PAIRS = TILE;
+constexpr uint32_t SMALL_TILES = 16;
+constexpr uint32_t ARRIVAL_DT = 1u << 27;   // a time window this wide takes the time-sorted path
+constexpr uint64_t ARRIVAL_BACK = 1ull << 28;   // key base before the segment's first hit
+
 enum ErrBits : uint32_t {
     E_RANGE = 1u,     // hit outside the sensor
     E_SPAN = 2u,      // ToA span of a segment >= 2^32
@@ -77,6 +86,8 @@ struct Seg {
     uint64_t toa_min, toa_max;
     uint64_t key_base;         // sort keys are ToA - key_base (32 bits)
     uint64_t fast_base;        // the tile sort's key base (fast_key_base, set by k_setup)
+    uint64_t raw_base;         // the arrival-order path's key base (set by k_setup)
+    uint32_t n_owned;          // arrival-order path: hits that found their tile
     uint64_t chunk_min;        // min ToA of the new hits
     uint64_t watermark;        // CLOSE_WM: close clusters whose last ToA <= watermark
     uint64_t seen_after;       // streaming: max ToA seen after this step
@@ -100,7 +111,35 @@ struct Prob {
     uint32_t redo_count;   // tiles the table-mode link left to the general link kernel
     uint32_t border_count; // tile borders k_border_fast left to k_border_link
     uint32_t merge_count;  // tile borders k_tile_merge left to its whole-window form (listed in redo)
+    uint32_t raw;          // the step starts on the arrival-order path
+    uint32_t raw_fail;     // ... which could not cover it (RawFail): the time-sorted path takes it
 };
+
+enum RawFail : uint32_t {
+    RAW_COVER = 1u,        // a tile's hits did not fit, lay too far around it or too far in time
+    RAW_UNORDERED = 2u,    // tiles out of order in time: the general sort
+};
+
+// One tile of the arrival-order path.
+struct ATile {
+    uint64_t base;             // its keys are ToA - base
+    uint32_t nroots, nx;       // clusters of the tile; pairs across tiles
+    uint32_t cut;              // first key of its interval
+    uint32_t nhalo, ntail;     // earlier hits it saw; own hits the next tile must see
+    // small steps:
+    uint32_t h0;               // positions from h0 on were looked at
+    uint64_t lo;               // smallest ToA an earlier hit may have and join one of its hits
+    uint64_t cmax[ACHUNKS];    // largest ToA of each quarter of its positions
+    uint32_t redo;             // to be joined with every earlier tile
+};
+
+// Feature sums of one tile cluster (at a cluster's root: of the cluster).
+struct __align__(16) RootSlot {
+    unsigned long long tot, wx, wy;   // sum ToT, sum ToT*x, sum ToT*y
+    uint32_t size;
+    uint32_t min;                     // smallest position
+};
+static_assert(sizeof(RootSlot) == 32, "one sector per root");
 
 // Feature sums of one cluster, kept at its root's sorted position.  One
 // 40-byte record (8-byte aligned, so exactly two 32-byte sectors) instead of
@@ -135,7 +174,18 @@ struct Work {
     uint32_t *tile_base;       // [2][tile_cap] exclusive per-segment prefix
     uint32_t *hist;            // [RADIX][tile_cap]
     uint32_t *segtot;          // [MAX_SEGS][RADIX]
+    // Arrival-order path: its arrays take the place of the sorted path's
+    // (either path writes all it reads).  c = tile * TILE + index in the tile.
+    uint32_t *gpar;            // (parent) per c: union-find over tile clusters (root_of: c per position)
+    RootSlot *rslot;           // (slot) per c
+    uint64_t *rfirst, *rlast;  // (keys[1] + vals[1], vals[0] + spix) per c: first and last ToA
+    uint2 *xlist;              // (lab_tmp) [tile][A_PAIRS] positions to join across tiles
+    uint32_t *rkey;            // (keys[0]) per position: ToA - the tile's base; may be null
+    ATile *atile;              // (hist) per tile
+    uint32_t *atmax;           // (tile_base) per tile: largest key
 };
+static_assert(sizeof(ATile) <= RADIX * sizeof(uint32_t) && A_PAIRS * sizeof(uint2) <= TILE * sizeof(uint64_t) &&
+              sizeof(RootSlot) <= sizeof(Slot), "arrival-order arrays fit the sorted path's");
 
 // Extra arrays of the (b)/(c) variants (single-segment steps only).
 struct VarWork {
@@ -273,9 +323,37 @@ __device__ __forceinline__ uint64_t warp_max_u64(uint64_t v) {
 // before the segment's first hit.  Its keys are exact when every ToA lies
 // within 2^31 ticks of that hit (checked once the extremes are known; the
 // general sort, with base = minimum ToA, takes over otherwise).
-__device__ __forceinline__ uint64_t fast_key_base(const Seg &g) {
-    const uint64_t t0 = g.n ? hit_toa(ld_hit(g.hits)) : 0;
+__device__ __forceinline__ uint64_t fast_key_base(uint64_t t0) {
     return t0 > (1ull << 31) ? t0 - (1ull << 31) : 0;
+}
+
+// Once a segment's ToA extremes are known: its ToA span check and, streaming,
+// the watermark.  A later hit j satisfies toa_j > seen_max - max_disorder (the
+// t-ordered property, Section 3.1), and can join hit i only if
+// toa_j - toa_i <= dt, so every cluster whose last ToA <=
+// seen_max - max_disorder - dt is final.
+__device__ __forceinline__ void seg_close(Seg &g, Prob &P) {
+    if (g.n && (g.toa_max - g.toa_min) >> 32) atomicOr(&P.err, E_SPAN);
+    if (!g.ss) {
+        g.close_mode = CLOSE_ALL;   // one-shot: the end of the stream
+        return;
+    }
+    const StreamState &ss = *g.ss;
+    const uint64_t md = g.max_disorder;   // ~0: a flush of a streaming context
+    if (md != ~0ull && g.n_new && ss.has_seen && ss.seen_max >= md && g.chunk_min <= ss.seen_max - md)
+        atomicOr(&P.err, E_LATE);
+    uint64_t seen = ss.has_seen ? ss.seen_max : 0;
+    if (g.n && g.toa_max > seen) seen = g.toa_max;
+    g.seen_after = seen;
+    const uint64_t lag = md + (uint64_t)g.dt;
+    if (md == ~0ull) {
+        g.close_mode = CLOSE_ALL;
+    } else if (lag >= md && seen >= lag) {
+        g.close_mode = CLOSE_WM;
+        g.watermark = seen - lag;
+    } else {
+        g.close_mode = CLOSE_NONE;
+    }
 }
 
 // Pixel clamped into the sensor.  The tile sort reports hits outside it
@@ -345,7 +423,10 @@ struct Launch {
 
 cudaError_t init_kernel_attributes();   // once per process and device, before capture
 cudaError_t init_variants_attributes();
-void launch_setup(const Work &w, int nsegs, const Launch &L);
+void launch_setup(const Work &w, int nsegs, const Launch &L, bool arrival = false);
+cudaError_t init_arrival_attributes();
+void launch_arrival_link(const Work &w, bool small, cudaGraphConditionalHandle sorted, const Launch &L);
+void launch_arrival_output(const Work &w, bool small, uint64_t *counts, uint32_t keep, const Launch &L);
 void launch_seg_finalize(const Work &w, const Launch &L);
 void launch_make_keys(const Work &w, const Launch &L);
 void launch_sort_fast(const Work &w, const Launch &L);
