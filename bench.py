@@ -58,6 +58,11 @@ HIT_DTYPE_NP = np.dtype([("x", "<u2"), ("y", "<u2"), ("tot", "<u2"), ("reserved"
 # (records 16 B, keys/positions/pixels/parents 4 B, labels 8 B); the cluster
 # record bytes are charged per cluster.  Used for the dominant kernel's roofline.
 KERNEL_BYTES_PER_HIT = {
+    # arrival order: read the record; write the hit's tile cluster and its key
+    "k_arrival_tile": 16 + 8, "k_arrival_small": 16 + 8,
+    # read the tile cluster, write the label
+    "k_arrival_labels": 4 + 8,
+    # the time-sorted path (steps the arrival-order path cannot cover):
     # in-tile sort (also the load, range check and ToA extremes): read the
     # record; write key, position, pixel (4 each), ToT (2)
     "k_tile_sort": 16 + 14,
@@ -84,10 +89,10 @@ def path_bytes_per_hit(n_hits: int, n_clusters: int) -> float:
 
 
 # Device-code sources: every kernel of a processing step with its launch
-# configuration.  The launch order lives in the API file's enqueue_kernels(),
+# configuration.  The launch order lives in the API file's capture_step(),
 # hashed on its own; the rest of that file (context bookkeeping, checkpoints)
 # and the host-side buffer filling are not part of any kernel.
-KERNEL_SOURCES = ("features.cu", "link.cu", "noalloc.cu", "prepare.cu", "radix.cu", "sortfast.cu",
+KERNEL_SOURCES = ("arrival.cu", "features.cu", "link.cu", "noalloc.cu", "prepare.cu", "radix.cu", "sortfast.cu",
                   "tpc_internal.cuh")   # variants.cu: (b)/(c) kernels, never launched by the step
 
 
@@ -100,7 +105,7 @@ def kernel_source_sha() -> str:
     for f in KERNEL_SOURCES:
         h.update(open(os.path.join(csrc, f), "rb").read())
     api = open(os.path.join(csrc, "tpc_api.cu")).read()
-    start = api.index("void enqueue_kernels(")
+    start = api.index("cudaError_t capture_step(")
     h.update(api[start:api.index("\n}\n", start)].encode())
     return h.hexdigest()[:16]
 
