@@ -43,17 +43,16 @@ constexpr int AT = 512;                          // threads of the tile kernels 
 constexpr int AW = AT / 32;
 constexpr uint32_t A_MARGIN = 1024;              // positions around the tile read at once
 constexpr int A_ITEMS = (TILE + 2 * A_MARGIN) / AT;   // records per thread
-constexpr int A_GROUP = 4;                       // ... in flight together
+constexpr int A_GROUP = 2;                       // ... looked at while the next ones are in flight
 constexpr uint32_t A_STEP = TILE / ACHUNKS;      // positions per further round
 constexpr int A_HPER = (A_STEP + AT - 1) / AT;
 constexpr uint32_t A_ENT = 5632;                 // hits staged: a tile's own and the earlier ones
 constexpr int A_PER = A_ENT / AT;
 constexpr uint32_t A_WORDS = 2304;               // 256 rows of nine 30-pixel words
-constexpr uint32_t A_XTRA = 1024;                // unions beyond each hit's first
-constexpr uint32_t A_CROSS = 1024;               // pairs across tiles
+constexpr uint32_t A_XTRA = 2048;                // unions beyond each hit's first
 constexpr uint32_t A_LATER = 2048;               // hits beside cells of several hits
 constexpr uint32_t A_FAR = 1024;                 // hits found beyond the margins
-constexpr int A_JUMPS = 5;                       // path-shortening passes over the tile's forest
+constexpr int A_JUMPS = 2;                       // path-shortening passes over the tile's forest
 constexpr int A_ROUNDS = 4;                      // further rounds on each side
 constexpr int A_BACK_ROUNDS = 16;                // rounds back of a small step's tiles
 constexpr uint32_t A_NONE = 0x7FFFu;             // no hit
@@ -73,11 +72,9 @@ struct ArrivalShared {
     uint2 word[A_WORDS];         // bits; cells before the word (minus the repeated low bit)
     uint16_t head[A_ENT];
     uint16_t next[A_ENT];
-    uint32_t key[A_ENT];         // ToA - base
-    uint32_t code[A_ENT];        // cell and row: (y / R) << 17 | word << 5 | bit
-    uint16_t par[A_ENT];         // forest over the tile's own hits
+    uint2 kc[A_ENT];             // key (ToA - base) and code
+    uint16_t par[A_ENT];         // forest over the hits
     uint32_t xtra[A_XTRA];       // unions beyond each hit's first (k << 16 | j)
-    uint32_t cross[A_CROSS];     // pairs across tiles (own << 16 | earlier)
     uint16_t later[A_LATER];     // hits beside cells of several hits
     uint16_t far[A_FAR];         // hits beyond the margins: position - window start
     uint32_t red[4][AW];
@@ -91,7 +88,12 @@ struct ArrivalShared {
     __device__ uint16_t *id() { return reinterpret_cast<uint16_t *>(xtra); }      // [A_ENT] cluster of each tile root
     __device__ uint32_t *sums() { return reinterpret_cast<uint32_t *>(word); }    // [2 * A_WORDS] feature sums
 };
-static_assert((A_XTRA + A_CROSS) * 4 + A_LATER * 2 >= A_ENT * 2, "cluster indices fit the lists");
+static_assert(A_XTRA * 4 + A_LATER * 2 >= A_ENT * 2, "cluster indices fit the lists");
+
+// Code of a hit: word << 5 | bit of its cell, (y / R) << 17, and whether it is
+// the tile's own (otherwise an earlier tile's).
+constexpr uint32_t C_OWN = 1u << 31, C_CELL = C_OWN - 1u;
+
 // Small steps stage every entry's position too.
 struct SmallShared {
     ArrivalShared s;
@@ -114,12 +116,14 @@ __device__ __forceinline__ uint32_t lanes_below() {
     return m;
 }
 
-// The cell grid of a W x H sensor: R rows (a power of two) of nw words.
+// The cell grid of a W x H sensor: R rows (a power of two) of nw words.  A
+// row's last word never uses its 30th pixel, so that no word repeats a pixel of
+// another row.
 struct Cells {
     uint32_t nw, rmask, rshift, nwords;   // words per row, R - 1, log2 R, words
     bool alias;                           // rows share cells
     __device__ Cells(uint32_t W, uint32_t H) {
-        nw = (W + 29u) / 30u;                              // <= 2185
+        nw = W / 30u + 1u;                                 // <= 2185
         rshift = 31u - __clz((int)(A_WORDS / nw));         // at least one row
         while (rshift && (1u << (rshift - 1u)) >= H) --rshift;
         rmask = (1u << rshift) - 1u;
@@ -129,7 +133,9 @@ struct Cells {
     // y / R < 64: a row holds W * R > 30 * A_WORDS / 4 pixels when rows share cells, of at most 2^20
     __device__ __forceinline__ uint32_t code(uint32_t pix) const {
         const uint32_t x = pix & 0xFFFFu, y = pix >> 16, wi = x / 30u;
-        return (y >> rshift) << 17 | ((y & rmask) * nw + wi) << 5 | (x - wi * 30u + 1u);
+        uint32_t c = ((y & rmask) * nw + wi) * 32u + (x - wi * 30u) + 1u;
+        if (alias) c |= y >> rshift << 17;
+        return c;
     }
     __device__ __forceinline__ void set(ArrivalShared &S, uint32_t code) const {
         atomicOr(&S.word[(code >> 5) & 0xFFFu].x, 1u << (code & 31u));
@@ -137,7 +143,7 @@ struct Cells {
     __device__ __forceinline__ void pixel(uint32_t code, uint32_t magic, uint32_t &x, uint32_t &y) const {
         const uint32_t word = (code >> 5) & 0xFFFu, row = nw == 1u ? word : __umulhi(word, magic);
         x = (word - row * nw) * 30u + (code & 31u) - 1u;
-        y = (code >> 17 << rshift) + row;
+        y = ((code & C_CELL) >> 17 << rshift) + row;
     }
     // word / nw = umulhi(word, magic) for words < 2^12, nw > 1 (nw = 1 apart: the factor would be 2^32)
     __device__ __forceinline__ uint32_t magic() const { return 0xFFFFFFFFu / nw + 1u; }
@@ -174,41 +180,151 @@ __device__ __forceinline__ bool arrival_hook(uint16_t *par, uint32_t a, uint32_t
 // Links of the staged entries 0..n_e: cells numbered, heads and lists built,
 // then each pair of adjacent hits met once, by the hit that is later in raster
 // order (row above, left), on one pixel by the earlier hit.
-// own(e, key): whether an entry is the tile's own; near(a, b): two keys within
-// dt; join(e, own, j, own, linked): takes a pair; linked: e has a parent.
-template <class Own, class Near, class Join>
-__device__ __forceinline__ void arrival_links(ArrivalShared &S, const Cells &C, uint32_t n_e, Own own, Near near,
-                                              Join join) {
+// near(a, b): two keys within dt; join(e, j, linked): takes a pair; linked: e
+// has been joined before.  ALIAS: rows share cells.
+template <bool ALIAS, class Near, class Join>
+__device__ __forceinline__ void arrival_pairs(ArrivalShared &S, const Cells &C, uint32_t n_e, Near near, Join join) {
+    const int tid = threadIdx.x;
+    // Heads of the cells left, above left, above and above right (A_NONE: none)
+    // and of the own cell; up: y / R of the row above.
+    auto around = [&](uint32_t code, uint32_t (&hd)[4], uint32_t &up) -> uint32_t {
+        const uint32_t word = (code >> 5) & 0xFFFu, bit = code & 31u;
+        const uint2 v0 = S.word[word];
+        const uint32_t s0 = v0.y + __popc(v0.x & ~(0xFFFFFFFFu << bit));
+        const uint32_t self = S.head[s0];
+        hd[0] = hd[1] = hd[2] = hd[3] = A_NONE;
+        if ((v0.x >> (bit - 1u)) & 1u) hd[0] = S.head[s0 - 1];
+        const bool wrap = word < C.nw;   // the grid's first row: its last one lies above it
+        up = (code & C_CELL) >> 17;
+        const bool top = wrap && up == 0u;   // the sensor's first row
+        up -= wrap ? 1u : 0u;
+        const uint2 v1 = S.word[wrap ? word + C.nwords - C.nw : word - C.nw];
+        const uint32_t m = top ? 0u : v1.x >> (bit - 1u);
+        uint32_t s1 = v1.y + __popc(v1.x & ~(0xFFFFFFFFu << (bit - 1u)));
+        if (m & 1u) hd[1] = S.head[s1];
+        s1 += m & 1u;
+        if (m & 2u) hd[2] = S.head[s1];
+        s1 += (m >> 1) & 1u;
+        if (m & 4u) hd[3] = S.head[s1];
+        return self;
+    };
+    // Cells of several hits: on a neighbour pixel the latest hit at or before
+    // this one and the earliest after it (the others within dt are joined to
+    // those along their pixel), on the own pixel the next one.
+    auto crowded = [&](uint32_t e) {
+        const uint2 me = S.kc[e];
+        const uint32_t code = me.y & C_CELL, key = me.x;
+        bool linked = S.par[e] != e;
+        uint32_t hd[4], up;
+        const uint32_t self = around(code, hd, up);
+        uint32_t multi = self & A_MULTI ? 16u : 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) multi |= hd[i] & A_MULTI ? 1u << i : 0u;
+        while (multi) {
+            const int i = __ffs(multi) - 1;
+            multi &= multi - 1u;
+            const uint32_t row = i == 0 || i == 4 ? code >> 17 : up;
+            uint32_t j = (i == 4 ? self : i == 0 ? hd[0] : i == 1 ? hd[1] : i == 2 ? hd[2] : hd[3]) & A_NONE;
+            uint32_t jlo = A_NONE, jhi = A_NONE, klo = 0, khi = 0xFFFFFFFFu;
+            do {
+                const uint2 o = S.kc[j];
+                if (j != e && (!ALIAS || (o.y & C_CELL) >> 17 == row)) {
+                    if (o.x < key || (o.x == key && (i != 4 || j < e))) {
+                        if (o.x >= klo) { klo = o.x; jlo = j; }
+                    } else if (o.x < khi || (o.x == khi && j < jhi)) {
+                        khi = o.x;
+                        jhi = j;
+                    }
+                }
+                j = S.next[j];
+            } while (j != A_NONE);
+            if (i != 4 && jlo != A_NONE && near(key, klo)) join(e, jlo, linked);
+            if (jhi != A_NONE && near(khi, key)) join(e, jhi, linked);
+        }
+    };
+#pragma unroll 1
+    for (uint32_t e = tid; e < n_e; e += AT) {
+        const uint2 me = S.kc[e];
+        const uint32_t code = me.y & C_CELL, key = me.x;
+        uint32_t hd[4], up;
+        const uint32_t flags = around(code, hd, up);
+        uint32_t kk[4] = {0, 0, 0, 0};
+        bool ok[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (ALIAS) {
+                uint2 o = make_uint2(0, 0);
+                if (hd[i] < A_NONE) o = S.kc[hd[i]];   // a cell with one hit
+                kk[i] = o.x;
+                ok[i] = hd[i] < A_NONE && near(key, o.x) && (o.y & C_CELL) >> 17 == (i ? up : code >> 17);
+            } else {
+                if (hd[i] < A_NONE) kk[i] = S.kc[hd[i]].x;
+                ok[i] = hd[i] < A_NONE && near(key, kk[i]);
+            }
+        }
+        // A pair whose two hits are both within dt of a third neighbour's is
+        // left out: the third one's pairs imply it.
+        const bool by2 = ok[2];
+        ok[1] = ok[1] && !(by2 && near(kk[2], kk[1])) && !(!by2 && ok[0] && near(kk[0], kk[1]));
+        ok[0] = ok[0] && !(by2 && near(kk[2], kk[0]));
+        ok[3] = ok[3] && !(by2 && near(kk[2], kk[3]));
+        // the first of them, for all lanes at once; a second one is rare
+        const uint32_t j = by2 ? hd[2] : ok[0] ? hd[0] : ok[1] ? hd[1] : hd[3];
+        bool linked = by2 || ok[0] || ok[1] || ok[3];
+        if (linked) {
+            bool none = false;
+            join(e, j, none);
+        }
+        uint32_t more = (ok[0] && by2 ? 1u : 0u) | (ok[1] && (by2 || ok[0]) ? 2u : 0u) |
+                        (ok[3] && (by2 || ok[0] || ok[1]) ? 8u : 0u);
+        while (more) {
+            const uint32_t low = more & (0u - more);
+            more ^= low;
+            join(e, low == 1u ? hd[0] : low == 2u ? hd[1] : hd[3], linked);
+        }
+        // a tenth of the hits lie beside crowded cells: they are taken up
+        // together afterwards, not by one lane of every warp
+        if ((flags | hd[0] | hd[1] | hd[2] | hd[3]) & A_MULTI) {
+            const uint32_t k = atomicAdd(&S.nlater, 1u);
+            if (k < A_LATER) S.later[k] = (uint16_t)e;
+        }
+    }
+    __syncthreads();
+    const uint32_t listed = S.nlater;
+    if (listed <= A_LATER)
+        for (uint32_t i = tid; i < listed; i += AT) crowded(S.later[i]);
+    else   // (more than the list holds: all of them, those without such cells have nothing to do)
+        for (uint32_t e = tid; e < n_e; e += AT) crowded(e);
+}
+
+template <class Near, class Join>
+__device__ __forceinline__ void arrival_links(ArrivalShared &S, const Cells &C, uint32_t n_e, Near near, Join join) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    __syncthreads();                // bits, keys and codes are in place
+    __syncthreads();                // bits and entries are in place
     {   // repeat the border pixels in the neighbour words, and count the cells before each word
         constexpr uint32_t PER = (A_WORDS + AT - 1) / AT;
         const uint32_t i0 = tid * PER;
-        uint32_t bits[PER], sum = 0, col = i0 - i0 / C.nw * C.nw;
-        uint32_t before = i0 && i0 < C.nwords ? S.word[i0 - 1].x : 0u;
+        uint32_t bits[PER], sum = 0;
+        const uint32_t before = i0 && i0 < C.nwords ? S.word[i0 - 1].x : 0u;
 #pragma unroll
-        for (uint32_t i = 0; i < PER; ++i) bits[i] = i0 + i < C.nwords ? S.word[i0 + i].x & 0x7FFFFFFEu : 0u;
+        for (uint32_t i = 0; i < PER; ++i) bits[i] = i0 + i < C.nwords ? S.word[i0 + i].x : 0u;
         const uint32_t after = i0 + PER < C.nwords ? S.word[i0 + PER].x : 0u;
-        uint32_t full[PER];
 #pragma unroll
-        for (uint32_t i = 0; i < PER; ++i) {
-            const uint32_t l = i ? bits[i - 1] : before, r = i + 1 < PER ? bits[i + 1] : after;
-            full[i] = bits[i] | (col ? (l >> 30) & 1u : 0u);
-            ++col;
-            if (col == C.nw) col = 0; else full[i] |= (r & 2u) << 30;
-            sum += __popc(bits[i]);
-        }
+        for (uint32_t i = 0; i < PER; ++i) sum += __popc(bits[i]);
         uint32_t x = sum;
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
         if (lane == 31) S.cnt[0][warp] = x;
+        if (tid == 0) S.nlater = 0;
         __syncthreads();
-        uint32_t run = x - sum + __reduce_add_sync(0xffffffffu, lane < warp ? S.cnt[0][lane] : 0u);
+        uint32_t run = x - sum + __reduce_add_sync(0xffffffffu, lane < warp ? S.cnt[0][min(lane, AW - 1)] : 0u);
 #pragma unroll
         for (uint32_t i = 0; i < PER; ++i) {
-            if (i0 + i < C.nwords) S.word[i0 + i] = make_uint2(full[i], run - (full[i] & 1u));
+            const uint32_t l = i ? bits[i - 1] : before, r = i + 1 < PER ? bits[i + 1] : after;
+            const uint32_t low = (l >> 30) & 1u;
+            if (i0 + i < C.nwords) S.word[i0 + i] = make_uint2(bits[i] | low | (r & 2u) << 30, run - low);
             run += __popc(bits[i]);
         }
     }
@@ -219,11 +335,12 @@ __device__ __forceinline__ void arrival_links(ArrivalShared &S, const Cells &C, 
         const uint32_t e = q * AT + tid;
         slots[q] = 0;
         if (e < n_e) {
-            const uint32_t code = S.code[e];
+            const uint32_t code = S.kc[e].y;
             const uint2 v = S.word[(code >> 5) & 0xFFFu];
             slots[q] = v.y + __popc(v.x & ~(0xFFFFFFFFu << (code & 31u)));
             S.head[slots[q]] = (uint16_t)e;
             S.next[e] = (uint16_t)A_NONE;
+            S.par[e] = (uint16_t)e;
         }
     }
     __syncthreads();
@@ -245,144 +362,47 @@ __device__ __forceinline__ void arrival_links(ArrivalShared &S, const Cells &C, 
         S.head[s] = (uint16_t)(h | A_MULTI);
     }
     __syncthreads();
-
-    // heads of the cells around a hit (left, above left, above, above right)
-    // and of its own; up: y / R of the row above
-    auto around = [&](uint32_t code, uint32_t (&hd)[4], uint32_t &up) -> uint32_t {
-        const uint32_t word = (code >> 5) & 0xFFFu, bit = code & 31u;
-        const uint2 v0 = S.word[word];
-        const uint32_t s0 = v0.y + __popc(v0.x & ~(0xFFFFFFFFu << bit));
-        hd[0] = hd[1] = hd[2] = hd[3] = A_NONE;
-        if ((v0.x >> (bit - 1u)) & 1u) hd[0] = S.head[s0 - 1];
-        const bool wrap = word < C.nw;   // the grid's first row: the last one lies above it
-        up = (code >> 17) - (wrap ? 1u : 0u);
-        if (!wrap || code >> 17) {
-            const uint2 v1 = S.word[wrap ? word + C.nwords - C.nw : word - C.nw];
-            const uint32_t m = v1.x >> (bit - 1u);
-            const uint32_t s1 = v1.y + __popc(v1.x & ~(0xFFFFFFFFu << (bit - 1u)));
-            if (m & 1u) hd[1] = S.head[s1];
-            if (m & 2u) hd[2] = S.head[s1 + (m & 1u)];
-            if (m & 4u) hd[3] = S.head[s1 + __popc(m & 3u)];
-        }
-        return S.head[s0];
-    };
-    // Cells of several hits: on a neighbour pixel the latest hit at or before
-    // this one and the earliest after it (the others within dt are joined to
-    // those along their pixel), on the own pixel the next one.
-    auto crowded = [&](uint32_t e) {
-        const uint32_t code = S.code[e], key = S.key[e];
-        const bool mine = own(e, key);
-        bool linked = S.par[e] != e;
-        uint32_t hd[4], up;
-        const uint32_t self = around(code, hd, up);
-        uint32_t multi = self & A_MULTI ? 16u : 0u;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) multi |= hd[i] & A_MULTI ? 1u << i : 0u;
-        while (multi) {
-            const int i = __ffs(multi) - 1;
-            multi &= multi - 1u;
-            const uint32_t row = i == 0 || i == 4 ? code >> 17 : up;
-            uint32_t j = (i == 4 ? self : i == 0 ? hd[0] : i == 1 ? hd[1] : i == 2 ? hd[2] : hd[3]) & A_NONE;
-            uint32_t jlo = A_NONE, jhi = A_NONE, klo = 0, khi = 0xFFFFFFFFu;
-            do {
-                const uint32_t k = S.key[j];
-                if (j != e && S.code[j] >> 17 == row) {
-                    if (k < key || (k == key && (i != 4 || j < e))) {
-                        if (k >= klo) { klo = k; jlo = j; }
-                    } else if (k < khi || (k == khi && j < jhi)) {
-                        khi = k;
-                        jhi = j;
-                    }
-                }
-                j = S.next[j];
-            } while (j != A_NONE);
-            if (i != 4 && jlo != A_NONE && near(key, klo)) join(e, mine, jlo, own(jlo, klo), linked);
-            if (jhi != A_NONE && near(khi, key)) join(e, mine, jhi, own(jhi, khi), linked);
-        }
-    };
-    for (uint32_t e = tid; e < n_e; e += AT) {
-        const uint32_t code = S.code[e], key = S.key[e];
-        uint32_t hd[4], up;
-        const uint32_t self = around(code, hd, up);
-        uint32_t kk[4];
-        bool ok[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            kk[i] = 0;
-            ok[i] = false;
-            if (hd[i] < A_NONE) {   // a cell with one hit
-                kk[i] = S.key[hd[i]];
-                ok[i] = near(key, kk[i]);
-                if (C.alias) ok[i] = ok[i] && S.code[hd[i]] >> 17 == (i ? up : code >> 17);
-            }
-        }
-        // A pair whose two hits are both within dt of a third neighbour's is
-        // left out: the third one's pairs imply it.
-        if (ok[2]) {
-            ok[0] = ok[0] && !near(kk[2], kk[0]);
-            ok[1] = ok[1] && !near(kk[2], kk[1]);
-            ok[3] = ok[3] && !near(kk[2], kk[3]);
-        } else if (ok[0]) {
-            ok[1] = ok[1] && !near(kk[0], kk[1]);
-        }
-        uint32_t todo = (ok[0] ? 1u : 0u) | (ok[1] ? 2u : 0u) | (ok[2] ? 4u : 0u) | (ok[3] ? 8u : 0u);
-        if (todo) {
-            const bool mine = own(e, key);
-            bool linked = false;
-            do {
-                const uint32_t low = todo & (0u - todo);
-                const uint32_t j = low == 1u ? hd[0] : low == 2u ? hd[1] : low == 4u ? hd[2] : hd[3];
-                const uint32_t k = low == 1u ? kk[0] : low == 2u ? kk[1] : low == 4u ? kk[2] : kk[3];
-                todo ^= low;
-                join(e, mine, j, own(j, k), linked);
-            } while (todo);
-        }
-        // a tenth of the hits lie beside crowded cells: they are taken up
-        // together afterwards, not by one lane of every warp
-        if ((self | hd[0] | hd[1] | hd[2] | hd[3]) & A_MULTI) {
-            const uint32_t k = atomicAdd(&S.nlater, 1u);
-            if (k < A_LATER) S.later[k] = (uint16_t)e; else crowded(e);
-        }
-    }
-    __syncthreads();
-    const uint32_t n_l = min(S.nlater, A_LATER);
-    for (uint32_t i = tid; i < n_l; i += AT) crowded(S.later[i]);
+    if (C.alias) arrival_pairs<true>(S, C, n_e, near, join); else arrival_pairs<false>(S, C, n_e, near, join);
 }
 
-// A pair of own hits: e's first makes j its parent (always raster-earlier, or
-// the next hit of its pixel, so parents form no cycle), others are listed.
-__device__ __forceinline__ bool join_own(ArrivalShared &S, uint32_t e, uint32_t j, bool &linked) {
+// A pair: the hit's first makes the other its parent (always raster-earlier,
+// or the next hit of its pixel, so parents form no cycle), others are listed.
+__device__ __forceinline__ void join_hits(ArrivalShared &S, uint32_t e, uint32_t j, bool &linked) {
     if (!linked) {
         S.par[e] = (uint16_t)j;
         linked = true;
-        return true;
+        return;
     }
     const uint32_t k = atomicAdd(&S.nxtra, 1u);
     if (k < A_XTRA) S.xtra[k] = e << 16 | j;
-    return k < A_XTRA;
 }
 
-// Components of the tile's own hits, their features, and each hit's cluster.
-// ToTs and positions (pos[e], from `origin`) of the entries are staged; the
-// caller's barrier is behind them and the links.
-template <class Own>
-__device__ __forceinline__ void arrival_clusters(const Work &w, const Seg &g, uint32_t t, ArrivalShared &S,
-                                                 const Cells &C, uint32_t n_e, Own own, const uint16_t *pos,
+// Components of the staged hits, the clusters of the tile's own, their
+// features, each own hit's cluster, and the pairs with earlier tiles (earlier
+// hits in a cluster of this tile).  ToTs and positions (pos[e], from `origin`)
+// of the entries are staged; the caller's barrier is behind them and the links.
+// false: more clusters than the tile has numbers.
+__device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, uint32_t t, ArrivalShared &S,
+                                                 const Cells &C, uint32_t n_e, const uint16_t *pos,
                                                  uint32_t origin, uint64_t base) {
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t first_c = t * TILE;
     volatile uint16_t *par = S.par;
     // Raster-order parents chain along a track; every hit first jumps to its
     // ancestors a few times (all hits at once, so paths shrink by half and
-    // more each time) before unions and finds walk what is left.  (An earlier
-    // tile's hits are their own parents.)
+    // more each time) before unions and finds walk what is left.
 #pragma unroll 1
     for (int r = 0; r < A_JUMPS; ++r) {
         uint32_t p[A_PER];
 #pragma unroll
-        for (int q = 0; q < A_PER; ++q) p[q] = q * AT + tid < n_e ? par[q * AT + tid] : 0u;
+        for (int q = 0; q < A_PER; ++q)
+            if (q * AT + tid < n_e) p[q] = par[q * AT + tid];
 #pragma unroll
-        for (int q = 0; q < A_PER; ++q) p[q] = q * AT + tid < n_e ? par[p[q]] : 0u;
+        for (int q = 0; q < A_PER; ++q)
+            if (q * AT + tid < n_e) p[q] = par[p[q]];
+#pragma unroll
+        for (int q = 0; q < A_PER; ++q)
+            if (q * AT + tid < n_e) p[q] = par[p[q]];
 #pragma unroll
         for (int q = 0; q < A_PER; ++q)
             if (q * AT + tid < n_e) par[q * AT + tid] = (uint16_t)p[q];
@@ -399,38 +419,37 @@ __device__ __forceinline__ void arrival_clusters(const Work &w, const Seg &g, ui
         }
     }
     __syncthreads();
-    // number the roots, and take every hit to its root's number
-    uint16_t *id = S.id();
-    uint32_t c[A_PER];
-#pragma unroll
-    for (int q = 0; q < A_PER; ++q) {
-        const uint32_t e = q * AT + tid;
-        c[q] = e < n_e ? par[e] : 0xFFFFFFFFu;
-        const bool root = c[q] == e && own(e, S.key[e]);
-        const uint32_t m = __ballot_sync(0xffffffffu, root);
-        if (m) {
-            uint32_t k = 0;
-            if (lane == 0) k = atomicAdd(&S.nroots, (uint32_t)__popc(m));
-            k = __shfl_sync(0xffffffffu, k, 0);
-            if (root) id[e] = (uint16_t)(k + __popc(m & lanes_below()));
-        }
-    }
+    // roots with own hits are the tile's clusters; all are, but for earlier
+    // hits that met none of this tile's
+    uint16_t *id = S.id();   // (the lists are walked)
+    constexpr uint32_t OWNS = 0xFFFEu;
+    for (uint32_t e = tid; e < n_e; e += AT) id[e] = (uint16_t)A_NONE;
     __syncthreads();
+    uint32_t root[A_PER];
 #pragma unroll
     for (int q = 0; q < A_PER; ++q) {
         const uint32_t e = q * AT + tid;
         if (e < n_e) {
-            const uint32_t key = S.key[e], p = par[c[q]];
-            if (!own(e, key)) {
-                c[q] = 0xFFFFFFFFu;
-                continue;
-            }
-            c[q] = id[p == c[q] ? p : arrival_root(par, p)];
-            const uint32_t at = origin + pos[e];
-            w.root_of[at] = first_c + c[q];
-            if (w.rkey) w.rkey[at] = key;
+            root[q] = arrival_root(par, e);
+            if (S.kc[e].y & C_OWN) id[root[q]] = (uint16_t)OWNS;
         }
     }
+    __syncthreads();   // (no path is halved any more)
+#pragma unroll
+    for (int q = 0; q < A_PER; ++q)
+        if (q * AT + tid < n_e) par[q * AT + tid] = (uint16_t)root[q];
+    for (uint32_t e0 = warp * 32; e0 < n_e; e0 += AT) {
+        const uint32_t e = e0 + lane;
+        const bool top = e < n_e && id[e] == OWNS;
+        const uint32_t m = __ballot_sync(0xffffffffu, top);
+        if (m) {
+            uint32_t k = 0;
+            if (lane == 0) k = atomicAdd(&S.nroots, (uint32_t)__popc(m));
+            k = __shfl_sync(0xffffffffu, k, 0);
+            if (top) id[e] = (uint16_t)(k + __popc(m & lanes_below()));
+        }
+    }
+    __syncthreads();
     // Features per cluster, as many clusters at once as the space holds.
     // Shared memory adds 32 bits natively and 64 by compare-and-swap loops:
     // while the tile's whole ToT keeps every sum in bounds (4096 hits of the
@@ -439,16 +458,13 @@ __device__ __forceinline__ void arrival_clusters(const Work &w, const Seg &g, ui
     uint32_t *A = S.sums();
     const uint16_t *tots = S.tot();
     const uint32_t nroots = S.nroots, tsum = S.tsum, magic = C.magic();
-    if (nroots > TILE) {   // more clusters than the tile has numbers (nearly every hit alone, more hits than positions)
-        if (tid == 0) atomicMax(&w.prob->raw_fail, RAW_COVER);
-        return;
-    }
+    if (nroots > TILE) return false;   // (nearly every hit alone, and more hits than positions)
     const bool streaming = g.ss != nullptr;
     const uint32_t reach = max(g.width, g.height);
     const bool slim = tsum < (1u << 19) && (unsigned long long)tsum * reach < (1ull << 32);
     static_assert(A_ENT < (1u << 13), "a size above a 19-bit sum ToT");
     constexpr uint32_t PASS = 2 * A_WORDS / 8;
-    for (uint32_t r0 = 0; r0 < nroots; r0 += PASS) {
+    for (uint32_t r0 = 0; r0 == 0 || r0 < nroots; r0 += PASS) {
         const uint32_t nr = min(nroots - r0, PASS);
         for (uint32_t i = tid; i < nr; i += AT) {
 #pragma unroll
@@ -456,13 +472,25 @@ __device__ __forceinline__ void arrival_clusters(const Work &w, const Seg &g, ui
             A[6 * PASS + i] = A[7 * PASS + i] = 0xFFFFFFFFu;
         }
         __syncthreads();
-#pragma unroll
-        for (int q = 0; q < A_PER; ++q) {
-            const uint32_t i = c[q] - r0;
+#pragma unroll 3
+        for (uint32_t e = tid; e < n_e; e += AT) {
+            const uint2 kc = S.kc[e];
+            const uint32_t c = id[par[e]], i = c - r0, at = origin + pos[e];
+            if (!(kc.y & C_OWN)) {
+                if (c != A_NONE && r0 == 0) {   // an earlier tile's hit in a cluster of this one
+                    const uint32_t x = atomicAdd(&S.ncross, 1u);
+                    if (x < A_PAIRS) w.xlist[(size_t)t * A_PAIRS + x] = make_uint2(first_c + c, at);
+                }
+                continue;
+            }
+            if (r0 == 0) {
+                w.root_of[at] = first_c + c;
+                if (w.rkey) w.rkey[at] = kc.x;
+            }
             if (i < nr) {
-                const uint32_t e = q * AT + tid, tot = tots[e];
+                const uint32_t tot = tots[e];
                 uint32_t x, y;
-                C.pixel(S.code[e], magic, x, y);
+                C.pixel(kc.y, magic, x, y);
                 uint32_t *a = A + i;   // size (and ToT), ToT, x, carry, y, carry, first position, first key
                 if (slim) {
                     atomicAdd(a, (1u << 19) + tot);
@@ -476,7 +504,7 @@ __device__ __forceinline__ void arrival_clusters(const Work &w, const Seg &g, ui
                     if (atomicAdd(a + 4 * PASS, vy) > ~vy) atomicAdd(a + 5 * PASS, 1u);
                 }
                 atomicMin(a + 6 * PASS, (uint32_t)pos[e]);
-                atomicMin(a + 7 * PASS, S.key[e]);
+                atomicMin(a + 7 * PASS, kc.x);
             }
         }
         __syncthreads();
@@ -494,15 +522,18 @@ __device__ __forceinline__ void arrival_clusters(const Work &w, const Seg &g, ui
             __syncthreads();
             for (uint32_t i = tid; i < nr; i += AT) A[7 * PASS + i] = 0;
             __syncthreads();
-#pragma unroll
-            for (int q = 0; q < A_PER; ++q)
-                if (c[q] - r0 < nr) atomicMax(&A[7 * PASS + c[q] - r0], S.key[q * AT + tid]);
+            for (uint32_t e = tid; e < n_e; e += AT) {
+                const uint2 kc = S.kc[e];
+                const uint32_t i = id[par[e]] - r0;
+                if ((kc.y & C_OWN) && i < nr) atomicMax(&A[7 * PASS + i], kc.x);
+            }
             __syncthreads();
             for (uint32_t i = tid; i < nr; i += AT) w.rlast[first_c + r0 + i] = base + A[7 * PASS + i];
         }
         __syncthreads();
     }
     if (tid == 0) w.atile[t].nroots = nroots;
+    return true;
 }
 
 // Cut before tile j of a segment: the median ToA key of 32 hits around its
@@ -551,7 +582,7 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
         }
         if (tid == 0) {
             S.flag = *reinterpret_cast<volatile uint32_t *>(&P.raw_fail);
-            S.nent = S.nown = S.ntail = S.nxtra = S.ncross = S.nlater = S.nroots = S.tsum = 0;
+            S.nent = S.nown = S.ntail = S.nxtra = S.ncross = S.nroots = S.tsum = 0;
         }
         C.clear(S);
         if (warp < 2) {
@@ -584,7 +615,7 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
             bad |= pix ^ r.x;
             kmin = min(kmin, key);
             kmax = max(kmax, key);
-            if ((uint32_t)p >= n_carry) cmin = min(cmin, key);
+            if (n_carry && (uint32_t)p >= n_carry) cmin = min(cmin, key);
             code = C.code(pix);
             return key - lo < span;
         };
@@ -623,9 +654,7 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
                 const int i = h * A_GROUP + q;
                 const uint32_t e = e0 + __popc(mask[q] & lanes_below());
                 if (((staged >> i) & 1u) && e < A_ENT) {
-                    S.key[e] = key[q];
-                    S.code[e] = code[q];
-                    S.par[e] = (uint16_t)e;
+                    S.kc[e] = make_uint2(key[q], code[q] | (key[q] >= cut ? C_OWN : 0u));
                     C.set(S, code[q]);
                     mine[i] |= e << 16;
                 }
@@ -637,7 +666,7 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
         tsum = __reduce_add_sync(0xffffffffu, tsum);
         kmin = __reduce_min_sync(0xffffffffu, kmin);
         kmax = __reduce_max_sync(0xffffffffu, kmax);
-        cmin = __reduce_min_sync(0xffffffffu, cmin);
+        cmin = n_carry ? __reduce_min_sync(0xffffffffu, cmin) : kmin;   // (no carry: every hit is new)
         edge = __reduce_or_sync(0xffffffffu, edge | (bad ? 4u : 0u));
         if (lane == 0) {
             atomicAdd(&S.nown, own_sum & 0xFFFFu);
@@ -676,9 +705,7 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
                     outer |= !side || key >= cut;
                     const uint32_t e = atomicAdd(&S.nent, 1u);
                     if (e < A_ENT && e - e_far < A_FAR) {
-                        S.key[e] = key;
-                        S.code[e] = code;
-                        S.par[e] = (uint16_t)e;
+                        S.kc[e] = make_uint2(key, code | (key >= cut ? C_OWN : 0u));
                         S.far[e - e_far] = (uint16_t)(p - win);
                         C.set(S, code);
                     } else {
@@ -719,27 +746,13 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
             }
         }
         // ---- links -----------------------------------------------------------
-        auto own = [&](uint32_t, uint32_t key) { return key >= cut; };
         // (keys keep 2^27 from both ends of 32 bits and dt is less: the sum wraps for no far pair)
         const uint32_t dt2 = 2u * dt;
-        auto near = [&](uint32_t a, uint32_t b) { return a - b + dt <= dt2; };
-        arrival_links(S, C, n_e, own, near, [&](uint32_t e, bool me, uint32_t o, bool oo, bool &linked) {
-            if (me && oo) {
-                if (join_own(S, e, o, linked)) return;
-            } else if (me == oo) {
-                return;   // two earlier hits: an earlier tile's pair
-            }
-            const uint32_t k = atomicAdd(&S.ncross, 1u);   // (own pairs beyond their list too)
-            if (k < A_CROSS) S.cross[k] = me ? e << 16 | o : o << 16 | e;
-        });
+        arrival_links(S, C, n_e, [&](uint32_t a, uint32_t b) { return a - b + dt <= dt2; },
+                      [&](uint32_t e, uint32_t o, bool &linked) { join_hits(S, e, o, linked); });
         __syncthreads();
         // ---- positions and ToTs of the entries, where the lists were ---------
         uint16_t *pos = S.pos(), *tot = S.tot();
-        const uint32_t nx = S.ncross;
-        if (nx > A_CROSS) {
-            if (tid == 0) atomicMax(&P.raw_fail, RAW_COVER);
-            return;
-        }
 #pragma unroll
         for (int i = 0; i < A_ITEMS; ++i) {
             if ((staged >> i) & 1u) {
@@ -751,14 +764,14 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
             pos[e] = S.far[e - e_far];
             tot[e] = (uint16_t)hit_tot(ld_hit(hits + (win + (int32_t)S.far[e - e_far])));
         }
+        const bool listed = S.nxtra <= A_XTRA;
         __syncthreads();
-        for (uint32_t i = tid; i < nx; i += AT) {   // pairs across tiles, by position
-            const uint32_t x = S.cross[i];
-            w.xlist[(size_t)t * A_PAIRS + i] =
-                make_uint2(off + (uint32_t)(win + pos[x >> 16]), off + (uint32_t)(win + pos[x & 0xFFFFu]));
+        if (!listed || !arrival_clusters(w, g, t, S, C, n_e, pos, off + (uint32_t)win, base) || S.ncross > A_PAIRS) {
+            if (tid == 0) atomicMax(&P.raw_fail, RAW_COVER);
+            return;
         }
-        if (tid == 0) info.nx = nx;
-        arrival_clusters(w, g, t, S, C, n_e, own, pos, off + (uint32_t)win, base);
+        if (tid == 0) info.nx = S.ncross;
+        __syncthreads();   // the counters are reset for the next tile
     }
 }
 
@@ -786,7 +799,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
     bool wide = dt >= A_GUARD;
     const uint32_t new0 = g.n_carry > begin ? g.n_carry - begin : 0;   // first new hit
     uint32_t kmin, kmax, tots[OWN];
-    if (tid == 0) S.nxtra = S.ncross = S.nlater = S.nroots = S.tsum = 0;
+    if (tid == 0) S.nxtra = S.ncross = S.nroots = S.tsum = 0;
     C.clear(S);
     __syncthreads();
     for (int attempt = 0;; ++attempt) {
@@ -811,9 +824,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
             wide |= rel - low > room;
             bad |= pix != v[q].x;
             tots[q] = hit_tot(v[q]);
-            S.key[e] = key;
-            S.code[e] = code;
-            S.par[e] = (uint16_t)e;
+            S.kc[e] = make_uint2(key, code | C_OWN);
             SS.pos[e] = (uint16_t)(begin + e);
             C.set(S, code);
             kmin = min(kmin, key);
@@ -864,16 +875,20 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
     }
 
     // ---- links, with the earlier hits in rounds of A_STEP positions --------
-    auto own = [&](uint32_t e, uint32_t) { return e < n_t; };
     uint32_t h0 = begin;            // every position in [h0, begin) has been looked at
     bool done = begin == 0, redo = false;
     for (bool first = true;; first = false) {
-        if (!first) {               // the earlier hits so far are joined: the next ones beside the own hits
+        if (!first) {               // (redo) the earlier hits so far are joined: the next ones beside the own hits
             __syncthreads();
             C.clear(S);
-            if (tid == 0) S.nlater = 0;
             __syncthreads();
-            for (uint32_t e = tid; e < n_t; e += AT) C.set(S, S.code[e]);
+            for (uint32_t e = tid; e < n_t; e += AT) {
+                const tpc_hit *h = hits + begin + e;
+                const uint4 v = ld_hit(h);
+                const uint32_t code = C.code(clamp_pix(v.x, W, H));
+                S.kc[e] = make_uint2((uint32_t)(hit_toa(v) - base), code | C_OWN);
+                C.set(S, code);
+            }
         }
         uint32_t n_e = n_t;
         for (uint32_t buf = 0; !done;) {
@@ -886,12 +901,11 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
             uint32_t kk[A_HPER], pp[A_HPER], mask[A_HPER], sum = 0;
 #pragma unroll
             for (int u = 0; u < A_HPER; ++u) {
-                const bool in = u * AT + tid < (int)A_STEP;
-                const uint4 v = ld_hit(hits + a + (in ? u * AT + tid : 0));
+                const uint4 v = ld_hit(hits + a + u * AT + tid);
                 const uint64_t rel = hit_toa(v) - base;
                 kk[u] = (uint32_t)rel;
                 pp[u] = C.code(clamp_pix(v.x, W, H));
-                mask[u] = __ballot_sync(0xffffffffu, in && rel >= lo && rel <= hi);
+                mask[u] = __ballot_sync(0xffffffffu, rel >= lo && rel <= hi);
                 sum += __popc(mask[u]);
             }
             if (lane == 0) S.turn[buf][warp] = sum | (mask[0] ? 0x80000000u : 0u);
@@ -900,15 +914,16 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
             buf ^= 1u;   // the next round's barrier separates this one's reads from the round after
             const uint32_t total = __reduce_add_sync(0xffffffffu, c & 0x7FFFFFFFu);
             const bool oldest = __any_sync(0xffffffffu, c >> 31);   // some of the oldest AT positions matter
-            if (n_e + total > A_ENT) break;   // no room beside the staged ones: join those first
+            if (n_e + total > A_ENT) {   // no room beside the staged ones
+                if (!DIRECT) done = redo = true;
+                break;
+            }
             uint32_t e = n_e + __reduce_add_sync(0xffffffffu, lane < warp ? c & 0x7FFFFFFFu : 0u);
 #pragma unroll
             for (int u = 0; u < A_HPER; ++u) {
                 if ((mask[u] >> lane) & 1u) {
                     const uint32_t i = e + __popc(mask[u] & lanes_below());
-                    S.key[i] = kk[u];
-                    S.code[i] = pp[u];
-                    S.par[i] = (uint16_t)i;
+                    S.kc[i] = make_uint2(kk[u], pp[u]);
                     SS.pos[i] = (uint16_t)(a + u * AT + tid);
                     C.set(S, pp[u]);
                 }
@@ -920,40 +935,34 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
             else if (!DIRECT && !oldest) done = true;
             else if (!DIRECT && begin - h0 == A_BACK_ROUNDS * A_STEP) done = redo = true;
         }
-        arrival_links(S, C, n_e, own, [&](uint32_t a, uint32_t b) { return absdiff(a, b) <= dt; },
-                      [&](uint32_t e, bool me, uint32_t o, bool oo, bool &linked) {
-            if (me && oo) {
-                if (!first || (!DIRECT && join_own(S, e, o, linked))) return;
-            } else if (me == oo) {
-                return;   // two earlier hits: an earlier tile's pair
+        auto near = [&](uint32_t a, uint32_t b) { return absdiff(a, b) <= dt; };
+        if (DIRECT) {   // every pair, own or not, is an edge of the graph
+            arrival_links(S, C, n_e, near, [&](uint32_t e, uint32_t o, bool &) {
+                gunion(w.gpar, w.root_of[SS.pos[e]], w.root_of[SS.pos[o]]);
+            });
+        } else {
+            arrival_links(S, C, n_e, near, [&](uint32_t e, uint32_t o, bool &linked) { join_hits(S, e, o, linked); });
+            __syncthreads();
+            redo |= S.nxtra > A_XTRA;
+            uint32_t tsum = 0;
+#pragma unroll
+            for (int q = 0; q < OWN; ++q) {
+                if (q * AT + tid < n_t) S.tot()[q * AT + tid] = (uint16_t)tots[q];
+                tsum += tots[q];
             }
-            const uint32_t a = SS.pos[e], b = SS.pos[o];
-            if (DIRECT) {
-                gunion(w.gpar, w.root_of[a], w.root_of[b]);
-            } else {
-                const uint32_t k = atomicAdd(&S.ncross, 1u);
-                if (k < A_PAIRS) w.xlist[(size_t)t * A_PAIRS + k] = make_uint2(a, b);
-            }
-        });
+            tsum = __reduce_add_sync(0xffffffffu, tsum);
+            if (lane == 0) atomicAdd(&S.tsum, tsum);
+            __syncthreads();
+            arrival_clusters(w, g, t, S, C, n_e, SS.pos, 0u, base);   // (at most TILE clusters)
+        }
         if (done) break;
     }
-    __syncthreads();
     if (DIRECT) return;
     if (tid == 0) {
         info.h0 = h0;
         info.nx = S.ncross;
         info.redo = redo ? 1u : 0u;
     }
-    uint32_t tsum = 0;
-#pragma unroll
-    for (int q = 0; q < OWN; ++q) {
-        if (q * AT + tid < n_t) S.tot()[q * AT + tid] = (uint16_t)tots[q];
-        tsum += tots[q];
-    }
-    tsum = __reduce_add_sync(0xffffffffu, tsum);
-    if (lane == 0) atomicAdd(&S.tsum, tsum);
-    __syncthreads();
-    arrival_clusters(w, g, t, S, C, n_t, own, SS.pos, 0u, base);
 }
 
 __global__ void __launch_bounds__(AT) k_arrival_small(Work w) {
@@ -1020,7 +1029,7 @@ __global__ void __launch_bounds__(AX) k_arrival_cross(Work w, int small, cudaGra
             const uint2 *list = w.xlist + (size_t)t * A_PAIRS;
             for (uint32_t i = tid; i < nx; i += AX) {
                 const uint2 p = list[i];
-                gunion(w.gpar, w.root_of[p.x], w.root_of[p.y]);
+                gunion(w.gpar, p.x, w.root_of[p.y]);
             }
             if (fail) break;   // (lane 0 of warp 0: its other tiles no longer matter)
         }

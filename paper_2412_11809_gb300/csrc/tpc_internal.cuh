@@ -179,7 +179,7 @@ struct Work {
     uint32_t *gpar;            // (parent) per c: union-find over tile clusters (root_of: c per position)
     RootSlot *rslot;           // (slot) per c
     uint64_t *rfirst, *rlast;  // (keys[1] + vals[1], vals[0] + spix) per c: first and last ToA
-    uint2 *xlist;              // (lab_tmp) [tile][A_PAIRS] positions to join across tiles
+    uint2 *xlist;              // (lab_tmp) [tile][A_PAIRS] pairs across tiles: tile cluster, earlier hit's position
     uint32_t *rkey;            // (keys[0]) per position: ToA - the tile's base; may be null
     ATile *atile;              // (hist) per tile
     uint32_t *atmax;           // (tile_base) per tile: largest key
