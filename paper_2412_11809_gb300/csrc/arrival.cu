@@ -1199,14 +1199,17 @@ __device__ void emit_totals(Seg &g, Prob &P, uint32_t n_clusters, uint32_t n_fin
 __global__ void __launch_bounds__(AE) k_arrival_emit(Work w, uint64_t *counts, uint32_t keep) {
     __shared__ uint32_t s_red[AE / 32];
     __shared__ uint16_t s_pos[TILE];
+    __shared__ bool s_last;
     Prob &P = *w.prob;
     if (P.raw_fail) return;
     const uint32_t nt = P.ntiles, cap = P.tile_cap, per = (nt + gridDim.x - 1) / gridDim.x;
     const uint32_t t0 = blockIdx.x * per, t1 = min(t0 + per, nt);
     const uint32_t *cnt = w.tile_cnt;
-    if (blockIdx.x == 0)   // segments without hits
+    if (blockIdx.x == 0) {   // segments without hits
         for (uint32_t s = threadIdx.x; s < P.nsegs; s += AE)
             if (w.seg[s].ntiles == 0) emit_totals(w.seg[s], P, 0, 0);
+        __syncthreads();
+    }
     uint32_t rec = 0, fin = 0, open_total = 0;
     const Seg *cur = nullptr;
     for (uint32_t t = t0; t < t1; ++t) {
@@ -1272,14 +1275,21 @@ __global__ void __launch_bounds__(AE) k_arrival_emit(Work w, uint64_t *counts, u
         }
         rec += n_rec;
         fin += cnt[cap + t];
-        if (t + 1 == g.tile0 + g.ntiles && threadIdx.x == 0) {
-            emit_totals(w.seg[si], P, rec, fin);
-            if (counts) {   // tpc_cluster_static's result words
-                counts[0] = rec;
-                counts[1] = P.err & keep;
-            }
-        }
+        if (t + 1 == g.tile0 + g.ntiles && threadIdx.x == 0) emit_totals(w.seg[si], P, rec, fin);
         __syncthreads();   // s_pos is rewritten for the next tile
+    }
+    // the CTA that ends last sees every total and error bit
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(&P.emitted, 1u) + 1u == gridDim.x;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    for (uint32_t s = threadIdx.x; s < P.nsegs; s += AE) write_info(w.seg[s], P);
+    if (counts && threadIdx.x == 0) {   // tpc_cluster_static's result words
+        counts[0] = *const_cast<volatile uint32_t *>(&w.seg[0].n_clusters);
+        counts[1] = *const_cast<volatile uint32_t *>(&P.err) & keep;
     }
 }
 

@@ -380,11 +380,14 @@ __global__ void __launch_bounds__(TILE_WORDS) k_stream_compact(Work w) {
 
 __global__ void k_stream_end(Work w) {
     const uint32_t nsegs = w.prob->nsegs;
+    for (uint32_t s = threadIdx.x; s < nsegs; s += blockDim.x)
+        if (w.seg[s].ss && w.seg[s].n_open > w.seg[s].carry_cap) atomicOr(&w.prob->err, E_CAP);
+    __syncthreads();
     for (uint32_t s = threadIdx.x; s < nsegs; s += blockDim.x) {
         Seg &g = w.seg[s];
+        write_info(g, *w.prob);
         if (!g.ss) continue;
         StreamState &ss = *g.ss;
-        if (g.n_open > g.carry_cap) atomicOr(&w.prob->err, E_CAP);
         ss.n_carry = g.n_open <= g.carry_cap ? g.n_open : 0;
         ss.seen_max = g.seen_after;
         ss.has_seen = ss.has_seen || g.n != 0;

@@ -52,6 +52,7 @@ __global__ void k_setup(Work w, int nsegs, uint32_t arrival) {
         p.redo_count = 0;
         p.border_count = 0;
         p.merge_count = 0;
+        p.emitted = 0;
         p.raw = arrival;
         p.raw_fail = 0;
         p.err = 0;

@@ -354,14 +354,11 @@ struct tpc_ctx {
     tpc_cluster *res_rec = nullptr;
     size_t out_cap = 0;
 
-    // where the last step's results live: the own workspace after a flush or
-    // push, the context's own result block after a batch (never another
-    // context's memory, which may be freed before this one is read)
-    Seg *res_seg = nullptr;
-    Prob *res_prob = nullptr;
-    Seg *own_res_seg = nullptr;
-    Prob *own_res_prob = nullptr;
+    // the last step's outcome, written by its last kernel into the context's
+    // own pinned memory
+    StepInfo *h_info = nullptr;
     bool has_result = false;
+    bool res_batch = false;        // the step was a batch's: its arrays are the lead's
     bool res_streaming = false;
     uint64_t res_base = 0;
 
@@ -615,6 +612,7 @@ Seg base_seg(const tpc_ctx *c, const Tuning &t) {
     s.height = c->height;
     s.dt = c->dt32;
     s.variant = (uint32_t)c->variant;
+    s.info = c->h_info;
     s.max_disorder = ~0ull;
     s.link_general = link_general(t, c->width, c->height);
     return s;
@@ -749,8 +747,7 @@ int stream_step(tpc_ctx *c, size_t n, bool close_all) {
     c->scur = in;
     c->pushed += n;
     c->carry_ub = close_all ? 0 : positions;
-    c->res_seg = c->ws.w.seg;
-    c->res_prob = c->ws.w.prob;
+    c->res_batch = false;
     c->has_result = true;
     c->res_streaming = true;
     return TPC_OK;
@@ -759,8 +756,8 @@ int stream_step(tpc_ctx *c, size_t n, bool close_all) {
 // tpc_forest of a step on the arrival-order path, whose union-find runs over
 // tile clusters: the (ToA, input) order from the kept keys (a stable radix
 // sort on the host), every hit's parent its cluster's earliest hit.
-int forest_of_arrival(tpc_ctx *c, const Seg &g, uint32_t *parent, uint32_t *input_pos) {
-    const size_t n = g.n, tiles = (n + TILE - 1) / TILE;
+int forest_of_arrival(tpc_ctx *c, size_t n, uint32_t *parent, uint32_t *input_pos) {
+    const size_t tiles = (n + TILE - 1) / TILE;
     const Work &w = c->ws.w;
     try {
         std::vector<uint32_t> cluster(n), key(n), gpar(tiles * TILE), a(n), first(tiles * TILE, 0xFFFFFFFFu);
@@ -795,24 +792,17 @@ int forest_of_arrival(tpc_ctx *c, const Seg &g, uint32_t *parent, uint32_t *inpu
     return TPC_OK;
 }
 
-struct ResultInfo {
-    Seg seg;
-    Prob prob;
-};
-
-int read_result(tpc_ctx *c, ResultInfo &r) {
+int read_result(tpc_ctx *c, StepInfo &r) {
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return TPC_ERR_CUDA;
     if (!c->has_result) {
         std::memset(&r, 0, sizeof(r));
         return TPC_OK;
     }
-    if (cudaMemcpy(&r.seg, c->res_seg, sizeof(Seg), cudaMemcpyDeviceToHost) != cudaSuccess ||
-        cudaMemcpy(&r.prob, c->res_prob, sizeof(Prob), cudaMemcpyDeviceToHost) != cudaSuccess)
-        return TPC_ERR_CUDA;
+    std::memcpy(&r, c->h_info, sizeof(r));
     // the last streaming step's open hits are the exact carry: the next push
     // sizes its arrays from it instead of the running upper bound
-    if (c->res_streaming && c->ss && !r.prob.err && r.seg.n_open <= c->carry_ub) c->carry_ub = r.seg.n_open;
-    return map_err(r.prob.err);
+    if (c->res_streaming && c->ss && !r.err && r.n_open <= c->carry_ub) c->carry_ub = r.n_open;
+    return map_err(r.err);
 }
 
 }  // namespace
@@ -846,8 +836,7 @@ int tpc_create(uint32_t width, uint32_t height, uint64_t dt, int variant, tpc_ct
         ok = cudaEventCreateWithFlags(&c->seg_ev[i], cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->stage_ev, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->done_ev, cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->own_res_seg, sizeof(Seg)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->own_res_prob, sizeof(Prob)) == cudaSuccess;
+    ok = ok && cudaMallocHost(&c->h_info, sizeof(StepInfo)) == cudaSuccess;
     if (!ok) { tpc_destroy(c); return TPC_ERR_CUDA; }
     *out = c;
     return TPC_OK;
@@ -1039,8 +1028,7 @@ static int flush_variant(tpc_ctx *c, Tracer *tr) {
     c->pushed += n;
     c->pending = 0;
     c->zc = nullptr;
-    c->res_seg = c->ws.w.seg;
-    c->res_prob = c->ws.w.prob;
+    c->res_batch = false;
     c->has_result = true;
     c->res_streaming = false;
     return TPC_OK;
@@ -1072,8 +1060,7 @@ static int flush_impl(tpc_ctx *c, Tracer *tr) {
     c->pushed += n;
     c->pending = 0;
     c->zc = nullptr;
-    c->res_seg = c->ws.w.seg;
-    c->res_prob = c->ws.w.prob;
+    c->res_batch = false;
     c->has_result = true;
     c->res_streaming = false;
     return TPC_OK;
@@ -1111,28 +1098,28 @@ int tpc_profile_flush(tpc_ctx *c, const char **names, float *ms, int cap, int *n
 int tpc_sync(tpc_ctx *c) {
     if (!c) return TPC_ERR_ARG;
     std::lock_guard<std::mutex> lk(c->mu);
-    ResultInfo r;
+    StepInfo r;
     return read_result(c, r);
 }
 
 int tpc_counts(tpc_ctx *c, size_t *n_hits, size_t *n_clusters, size_t *n_open) {
     if (!c) return TPC_ERR_ARG;
     std::lock_guard<std::mutex> lk(c->mu);
-    ResultInfo r;
+    StepInfo r;
     int rc = read_result(c, r);
-    if (n_hits) *n_hits = r.seg.n_final;
-    if (n_clusters) *n_clusters = r.seg.n_clusters;
-    if (n_open) *n_open = r.seg.n_open;
+    if (n_hits) *n_hits = r.n_final;
+    if (n_clusters) *n_clusters = r.n_clusters;
+    if (n_open) *n_open = r.n_open;
     return rc;
 }
 
 int tpc_labels(tpc_ctx *c, uint64_t *labels, uint64_t *indices, size_t cap, size_t *n_out, int where) {
     if (!c || !n_out || (where != TPC_HOST && where != TPC_DEVICE)) return TPC_ERR_ARG;
     std::lock_guard<std::mutex> lk(c->mu);
-    ResultInfo r;
+    StepInfo r;
     int rc = read_result(c, r);
     if (rc) return rc;
-    const size_t n = r.seg.n_final;
+    const size_t n = r.n_final;
     *n_out = n;
     if (n > cap) return TPC_ERR_CAP;
     if (n && !labels) return TPC_ERR_ARG;
@@ -1172,10 +1159,10 @@ int tpc_labels_async(tpc_ctx *c, uint64_t *labels, size_t cap, size_t *n_out, in
 int tpc_cluster_features(tpc_ctx *c, tpc_cluster *out, size_t cap, size_t *n_out, int where) {
     if (!c || !n_out || (where != TPC_HOST && where != TPC_DEVICE)) return TPC_ERR_ARG;
     std::lock_guard<std::mutex> lk(c->mu);
-    ResultInfo r;
+    StepInfo r;
     int rc = read_result(c, r);
     if (rc) return rc;
-    const size_t n = r.seg.n_clusters;
+    const size_t n = r.n_clusters;
     *n_out = n;
     if (n > cap) return TPC_ERR_CAP;
     if (n && !out) return TPC_ERR_ARG;
@@ -1236,14 +1223,6 @@ int tpc::batch_step(tpc_ctx **ctxs, int n, bool consume) {
     }
     if (upload_segs(lead, lead->ws.w, segs.data(), n, lead->stream) != cudaSuccess) return TPC_ERR_CUDA;
     if (run_step(lead, lead->ws, n, step_mode(segs.data(), n, positions), lead->stream) != cudaSuccess) return TPC_ERR_CUDA;
-    for (int k = 0; k < n; ++k) {   // each context keeps its own copy of its results
-        tpc_ctx *c = ctxs[perm[k]];
-        if (cudaMemcpyAsync(c->own_res_seg, lead->ws.w.seg + k, sizeof(Seg), cudaMemcpyDeviceToDevice,
-                            lead->stream) != cudaSuccess ||
-            cudaMemcpyAsync(c->own_res_prob, lead->ws.w.prob, sizeof(Prob), cudaMemcpyDeviceToDevice,
-                            lead->stream) != cudaSuccess)
-            return TPC_ERR_CUDA;
-    }
     if (cudaEventRecord(lead->done_ev, lead->stream) != cudaSuccess) return TPC_ERR_CUDA;
     for (int i = 0; i < n; ++i) {
         tpc_ctx *c = ctxs[i];
@@ -1253,8 +1232,7 @@ int tpc::batch_step(tpc_ctx **ctxs, int n, bool consume) {
         c->pushed += c->pending;
         c->pending = 0;
         c->zc = nullptr;
-        c->res_seg = c->own_res_seg;
-        c->res_prob = c->own_res_prob;
+        c->res_batch = true;
         c->has_result = true;
         c->res_streaming = false;
     }
@@ -1275,26 +1253,26 @@ int tpc_forest(tpc_ctx *c, uint32_t *parent, uint32_t *input_pos, size_t cap, si
     if (!c || !n_out) return TPC_ERR_ARG;
     std::lock_guard<std::mutex> lk(c->mu);
     *n_out = 0;
-    ResultInfo r;
+    StepInfo r;
     int rc = read_result(c, r);
     if (rc) return rc;
-    if (!c->has_result || c->res_seg != c->ws.w.seg) return TPC_ERR_STATE;
-    const size_t n = r.seg.n;
+    if (!c->has_result || c->res_batch) return TPC_ERR_STATE;
+    const size_t n = r.n;
     *n_out = n;
     if (n > cap) return TPC_ERR_CAP;
     if (!n) return TPC_OK;
     if (!parent || !input_pos) return TPC_ERR_ARG;
-    if (r.prob.raw && !r.prob.raw_fail) return forest_of_arrival(c, r.seg, parent, input_pos);
+    if (r.arrival) return forest_of_arrival(c, n, parent, input_pos);
     // the sorted order lives in the buffer the step's last sort pass wrote
-    const uint32_t sel = r.prob.npasses & 1u;
-    if (cudaMemcpy(parent, c->ws.w.parent + r.seg.off, n * sizeof(uint32_t), cudaMemcpyDeviceToHost) !=
+    const uint32_t sel = r.npasses & 1u;
+    if (cudaMemcpy(parent, c->ws.w.parent + r.off, n * sizeof(uint32_t), cudaMemcpyDeviceToHost) !=
             cudaSuccess ||
-        cudaMemcpy(input_pos, c->ws.w.vals[sel] + r.seg.off, n * sizeof(uint32_t), cudaMemcpyDeviceToHost) !=
+        cudaMemcpy(input_pos, c->ws.w.vals[sel] + r.off, n * sizeof(uint32_t), cudaMemcpyDeviceToHost) !=
             cudaSuccess)
         return TPC_ERR_CUDA;
     for (size_t i = 0; i < n; ++i) {   // positions and input indices relative to the step
-        parent[i] -= r.seg.off;
-        input_pos[i] -= r.seg.off;
+        parent[i] -= r.off;
+        input_pos[i] -= r.off;
     }
     return TPC_OK;
 }
@@ -1414,11 +1392,7 @@ int tpc_snapshot(tpc_ctx *c, void *buf, size_t cap, size_t *n_out) {
     std::lock_guard<std::mutex> lk(c->mu);
     if (c->max_disorder == ~0ull || !c->ss) return TPC_ERR_STATE;
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return TPC_ERR_CUDA;
-    if (c->has_result) {
-        Prob p;
-        if (cudaMemcpy(&p, c->res_prob, sizeof(Prob), cudaMemcpyDeviceToHost) != cudaSuccess) return TPC_ERR_CUDA;
-        if (p.err) return map_err(p.err);
-    }
+    if (c->has_result && c->h_info->err) return map_err(c->h_info->err);
     StreamState st;
     if (cudaMemcpy(&st, c->ss, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess) return TPC_ERR_CUDA;
     const size_t nc = c->sbuf[0] ? st.n_carry : 0;
@@ -1540,8 +1514,7 @@ void tpc_destroy(tpc_ctx *c) {
     for (int i = 0; i < 2; ++i) { dev_free(c->sbuf[i], c->stream); dev_free(c->sgidx[i], c->stream); }
     dev_free(c->ss, c->stream);
     if (c->stream) cudaStreamSynchronize(c->stream);
-    cudaFree(c->own_res_seg);
-    cudaFree(c->own_res_prob);
+    if (c->h_info) cudaFreeHost(c->h_info);
     if (c->h_flag) cudaFreeHost(c->h_flag);
     if (c->h_seg) cudaFreeHost(c->h_seg);
     if (c->h_stage) cudaFreeHost(c->h_stage);

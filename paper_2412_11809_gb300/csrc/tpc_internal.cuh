@@ -56,6 +56,17 @@ struct StreamState {
 
 enum CloseMode : uint32_t { CLOSE_NONE = 0, CLOSE_ALL = 1, CLOSE_WM = 2 };
 
+// What the host reads of a finished step, per segment: written into pinned
+// host memory by the step's last kernel, so that no copy is queued for it and
+// none waited for.
+struct StepInfo {
+    uint32_t n, off;                          // hits of the step and their first position
+    uint32_t n_final, n_clusters, n_open;
+    uint32_t err;                             // ErrBits of the whole step
+    uint32_t npasses;                         // time-sorted path: its sorted data is in buffer npasses % 2
+    uint32_t arrival;                         // the arrival-order path covered the step
+};
+
 struct Seg {
     // ---- set by the host ----------------------------------------------
     const tpc_hit *hits;       // input hits [0, n); for streaming: set on device
@@ -67,6 +78,7 @@ struct Seg {
     uint64_t *out_labels;      // finalised labels (u64), ordered by global index
     uint64_t *out_index;       // their global indices (streaming only; may be null)
     tpc_cluster *out_rec;      // finalised cluster records ordered by label
+    StepInfo *info;            // pinned host memory; may be null (tpc_cluster_static)
     uint64_t gidx_base;        // global index of the first new hit
     uint64_t max_disorder;     // UINT64_MAX: not streaming (everything closes)
     uint32_t carry_cap;        // streaming: capacity of the carry region
@@ -111,6 +123,7 @@ struct Prob {
     uint32_t redo_count;   // tiles the table-mode link left to the general link kernel
     uint32_t border_count; // tile borders k_border_fast left to k_border_link
     uint32_t merge_count;  // tile borders k_tile_merge left to its whole-window form (listed in redo)
+    uint32_t emitted;      // CTAs of the last kernel that are done
     uint32_t raw;          // the step starts on the arrival-order path
     uint32_t raw_fail;     // ... which could not cover it (RawFail): the time-sorted path takes it
 };
@@ -354,6 +367,25 @@ __device__ __forceinline__ void seg_close(Seg &g, Prob &P) {
     } else {
         g.close_mode = CLOSE_NONE;
     }
+}
+
+// The host's view of segment g, once the step is done (totals that another
+// CTA has just written: read past the L1).
+__device__ __forceinline__ void write_info(const Seg &seg, const Prob &prob) {
+    const volatile Seg &g = seg;
+    const volatile Prob &P = prob;
+    StepInfo *out = g.info;
+    if (!out) return;
+    StepInfo i;
+    i.n = g.n;
+    i.off = g.off;
+    i.n_final = g.n_final;
+    i.n_clusters = g.n_clusters;
+    i.n_open = g.n_open;
+    i.err = P.err;
+    i.npasses = P.npasses;
+    i.arrival = P.raw && !P.raw_fail;
+    *out = i;
 }
 
 // Pixel clamped into the sensor.  The tile sort reports hits outside it
