@@ -240,7 +240,7 @@ struct VarSpace {
             v.k[i] = mem.alloc<uint32_t>(positions, e);
             v.v[i] = mem.alloc<uint32_t>(positions, e);
         }
-        v.changed = mem.alloc<uint32_t>(4, e);
+        v.changed = mem.alloc<uint32_t>(8, e);
         v.prob = mem.alloc<Prob>(1, e);
         if (global) {
             const size_t tiles = positions / TILE + 2;
@@ -268,7 +268,9 @@ struct VarSpace {
         } else {
             v.cpar = mem.alloc<uint32_t>(positions, e);
             v.work = mem.alloc<uint32_t>(1, e);
-            v.big = mem.alloc<uint2>(positions / 512 + 1, e);   // components of more than 512 hits
+            v.big_cap = (uint32_t)(positions / 512 + 1);        // components of more than 512 hits
+            v.big = mem.alloc<uint2>(v.big_cap, e);
+            v.over = mem.alloc<uint2>(v.big_cap, e);
         }
         if (e != cudaSuccess) {
             mem.release();
@@ -373,6 +375,7 @@ struct tpc_ctx {
 
     // launch choices (tpc_set_tuning / tpc_tune_batch); a batch uses its lead's
     Tuning tune{};
+    SideStream side;               // (c): for the long components, made on first use
     tpc_variant_stats vstats{};    // the last (b)/(c) flush (tpc_variant_stats)
     bool vstats_pending = false;   // (c) counters still in h_flag
 
@@ -928,6 +931,17 @@ int tpc_push(tpc_ctx *c, const tpc_hit *hits, size_t n, int where) {
     return TPC_OK;
 }
 
+static cudaError_t ensure_side(tpc_ctx *c) {
+    SideStream &s = c->side;
+    cudaError_t e = cudaSuccess;
+    int low = 0, high = 0;   // its CTAs are placed first: they run longest
+    if (!s.stream) e = cudaDeviceGetStreamPriorityRange(&low, &high);
+    if (e == cudaSuccess && !s.stream) e = cudaStreamCreateWithPriority(&s.stream, cudaStreamNonBlocking, high);
+    if (e == cudaSuccess && !s.fork) e = cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming);
+    if (e == cudaSuccess && !s.join) e = cudaEventCreateWithFlags(&s.join, cudaEventDisableTiming);
+    return e;
+}
+
 // Variants (b) and (c): the (a) forest and its roots first, then the
 // variant's kernels (csrc/variants.cu), then the shared feature / output
 // kernels.
@@ -965,7 +979,7 @@ static int flush_variant(tpc_ctx *c, Tracer *tr) {
     if (c->variant == TPC_STATIC) {
         launch_variant_keys(w, v, 0, L);
         for (int pass = 0; pass < 4; ++pass) launch_radix_pass(wv, pass, L);
-        launch_static_sweep(w, v, L);
+        if (ensure_side(c) != cudaSuccess || launch_static_sweep(w, v, L, c->side) != cudaSuccess) return TPC_ERR_CUDA;
         c->vstats = tpc_variant_stats{};
         if (cudaMemcpyAsync(c->h_flag, v.changed, 3 * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream) !=
             cudaSuccess)
@@ -1521,6 +1535,12 @@ void tpc_destroy(tpc_ctx *c) {
     for (int i = 0; i < SEG_RING; ++i) if (c->seg_ev[i]) cudaEventDestroy(c->seg_ev[i]);
     if (c->stage_ev) cudaEventDestroy(c->stage_ev);
     if (c->done_ev) cudaEventDestroy(c->done_ev);
+    if (c->side.stream) {
+        cudaStreamSynchronize(c->side.stream);
+        cudaStreamDestroy(c->side.stream);
+    }
+    if (c->side.fork) cudaEventDestroy(c->side.fork);
+    if (c->side.join) cudaEventDestroy(c->side.join);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     delete c;
 }

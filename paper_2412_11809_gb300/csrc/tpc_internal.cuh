@@ -215,14 +215,18 @@ struct VarWork {
                                //      entry: (sorted position, id of its group's root, the group's last
                                //      key, its key)
     uint32_t *changed;         // (b): [0] a round merged something, [1] the edge list overflowed;
-                               // (c): [0] windowed components, [1] of those swept again by a CTA,
-                               //      [2] of those swept from global memory
+                               // (c): [0] components of more than 512 hits (listed in big), [1] of
+                               //      those with more than 512 hits within dt, [2] of those longer
+                               //      than 8192 hits, [3] outgrew the window (listed in over), [4]
+                               //      next of big to sweep, [5] listed from big's end, [6] from its start
     unsigned long long *ecount;  // (b): edges pushed to lists 0 and 1 (beyond edge_cap: overflow)
     uint2 *edges[2];           // (b): edges not merged yet (an id of h's group, an id of its neighbour's)
     uint32_t *ekey[2];         // (b): h's key of each edge
     uint32_t edge_cap;         // (b): entries each edge list holds
     uint32_t *work;            // (c): next chunk of the grouped order to sweep
-    uint2 *big;                // (c): (first grouped position, hits) of components for the big window
+    uint2 *big, *over;         // (c): (first grouped position, hits) of long components, and of those
+                               //      their window cannot hold
+    uint32_t big_cap;          // (c): entries each holds
     Prob *prob;                // problem view of the grouping sort
 };
 
@@ -472,7 +476,13 @@ void launch_sorted_roots(const Work &w, const Launch &L);
 void launch_init_roots(const Work &w, const Launch &L);
 void launch_variant_keys(const Work &w, const VarWork &v, int by_pixel, const Launch &L);
 Work variant_view(const Work &w, const VarWork &v);
-void launch_static_sweep(const Work &w, const VarWork &v, const Launch &L);
+// A second stream for work beside a step's own, which waits for it before it
+// goes on (so stream-ordered frees on the step's stream come after both).
+struct SideStream {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+};
+cudaError_t launch_static_sweep(const Work &w, const VarWork &v, const Launch &L, const SideStream &side);
 void launch_pixel_timelines(const Work &w, const VarWork &v, uint32_t npixels, const Launch &L);
 void launch_components(const Work &w, const VarWork &v, const Launch &L);
 void launch_group_last(const VarWork &v, const Launch &L);

@@ -64,22 +64,470 @@ __device__ __forceinline__ uint32_t seq_find(uint32_t *par, uint32_t x) {
     return x;
 }
 
+// Threads and hits staged by the CTA sweep (below) of components that outgrow
+// the warps' windows.
+constexpr int BIG_THREADS = 512;
+constexpr uint32_t BIG_CAP = 8192;
+constexpr int BIG_SMEM = 3 * BIG_CAP * (int)sizeof(uint32_t);
+
 // (c): one warp per component of the root-grouped order (components are
 // contiguous there, in ToA order).  The sweep is sequential over the
-// component's hits, but each step is warp-wide: for hit i the lanes take the
-// earlier hits within dt (32 at a time, newest first), test adjacency and
-// whether the cluster of that hit is still open (its root, the earliest hit,
-// within dt of i), and every open cluster found is joined under the earliest
-// of their roots, together with i.  Whether a cluster is open does not
-// depend on the joins made for i itself (a join only unites open clusters,
-// and the result is open), so the lanes may test their candidates at once.
-// Components of up to SW_CAP hits are staged in shared memory; larger ones
-// run on the grouped arrays in global memory.  Warps take chunks of SW_CHUNK
-// grouped positions from a counter and sweep every component that starts in
-// their chunk.
+// component's hits, but a hit needs few lookups: when a hit lands on a pixel
+// it joins every open cluster with a member there, so of the clusters with a
+// member on a pixel only the one of its latest hit can be open.
+//   up to 32 hits      everything in registers: lane j holds hit j and its
+//                      root; a step tests all earlier hits at once.
+//   up to SW_CAP hits  staged in shared memory with a hash table from pixel
+//                      to its latest hit: nine lanes look up the nine pixels
+//                      of a hit, and three hits are taken per step; the
+//                      second and third count only if they touch neither the
+//                      pixels nor the clusters of those before (else they
+//                      are taken again).
+//   longer             (listed by k_static_long) two warps: one looks up the
+//                      neighbours of 32 hits ahead, which no join changes,
+//                      the other joins; a sliding window of the last hits.
+// A lone warp's chain over the longest component sets the time of the step (its
+// instructions follow one another at four to five cycles each), so what can
+// be taken off that chain is: 8 M hits at 2.5 Ghits/s, longest component 6,544
+// hits, from every earlier hit within dt tested 32 at a time (9.9 ms, and 1.9
+// for components outgrowing a window of 512) to the table (2.4 ms) to the two
+// warps (2.0 ms, of which the sweep of the others beside it takes 0.9).
 constexpr int SW_WARPS = 8;
 constexpr uint32_t SW_CAP = 512;
+constexpr uint32_t SW_TAB = 1024;
 constexpr uint32_t SW_CHUNK = 32;
+constexpr uint32_t LW_CAP = 1024;        // hits in the rings of a long component's sweep
+constexpr uint32_t LW_WIN = LW_CAP - 64; // ... in the window (the looking warp is 32 to 64 ahead)
+constexpr uint32_t LW_TAB = 4096;
+constexpr uint32_t LW_REBUILD = 1024;    // hits between two rebuilds of the window's table
+constexpr uint32_t LW_FIRST = 2048;      // components this long are started first
+constexpr int LW_CTAS = 3;               // per SM: room beside them for the other components' sweep
+constexpr uint32_t HASH_AGE = 4095;      // table entry: pixel id << 12 | index mod 4096
+constexpr uint32_t HASH_EMPTY = 0xFFFFFFFFu;
+constexpr uint32_t NO_ROOT = 0xFFFFFFFFu;
+static_assert(MAX_PIXELS <= 1u << 20, "pixel ids take 20 bits");
+// entries of a window's table: hits since its rebuild and those put back then, so lookups always end
+static_assert(LW_REBUILD + 32 + LW_CAP < LW_TAB && LW_REBUILD + 32 + LW_CAP < HASH_AGE && 2 * SW_CAP <= SW_TAB,
+              "free entries, unambiguous indices");
+
+struct HashSweep {
+    uint32_t key[SW_CAP];
+    uint32_t tab[SW_TAB];
+    uint16_t up[SW_CAP];   // distance to the parent, 0 at a root
+};
+
+// Sweep of component [q0, q0 + n), n <= SW_CAP, of the grouped order.
+__device__ void sweep_hashed(HashSweep &S, const uint32_t *skey, const uint32_t *spix, const uint32_t *gv,
+                             uint32_t *parent, uint32_t q0, uint32_t n, uint32_t dt, uint32_t W, uint32_t H, int lane) {
+    const uint32_t bits = 32 - __clz((int)(2 * n - 1));   // table: at least twice the hits
+    const uint32_t tsize = 1u << bits, tmask = tsize - 1u, shift = 32u - bits;
+    for (uint32_t i = lane; i < tsize / 4; i += 32)
+        reinterpret_cast<uint4 *>(S.tab)[i] = make_uint4(HASH_EMPTY, HASH_EMPTY, HASH_EMPTY, HASH_EMPTY);
+    const int g = lane / 9, d = lane - 9 * g;      // hit of the step and its neighbour pixel (lanes 27..31 idle)
+    const int dx = d % 3 - 1, dy = d / 3 - 1;
+    auto root_of = [&](uint32_t x) -> uint32_t {
+        volatile uint16_t *up = S.up;
+        for (uint32_t k = up[x]; k; k = up[x]) x -= k;
+        return x;
+    };
+    // the next 32 hits are on their way while 32 are swept
+    uint32_t k = 0, p = 0, k1 = 0, p1 = 0;
+    if ((uint32_t)lane < n) {
+        const uint32_t se = gv[q0 + lane];
+        k1 = skey[se];
+        p1 = spix[se];
+    }
+    uint32_t se2 = 32u + lane < n ? gv[q0 + 32 + lane] : 0u;
+    for (uint32_t base = 0; base < n; base += 32) {
+        const uint32_t e = base + lane, cnt = n - base < 32u ? n - base : 32u;
+        k = k1;
+        p = p1;
+        if (e + 32 < n) {
+            k1 = skey[se2];
+            p1 = spix[se2];
+        }
+        if (e + 64 < n) se2 = gv[q0 + e + 64];
+        if (e < n) {
+            S.key[e] = k;
+            S.up[e] = 0;
+        }
+        __syncwarp();
+        for (uint32_t c = 0; c < cnt;) {
+            const uint32_t at = c + (g < 3 ? g : 0), i = base + at;
+            const bool act = g < 3 && at < cnt;
+            const uint32_t ki = __shfl_sync(0xffffffffu, k, at & 31), pi = __shfl_sync(0xffffffffu, p, at & 31);
+            const uint32_t pa = __shfl_sync(0xffffffffu, p, c & 31), pb = __shfl_sync(0xffffffffu, p, (c + 1) & 31),
+                           pc = __shfl_sync(0xffffffffu, p, (c + 2) & 31);
+            const int x = (int)(pi & 0xFFFFu) + dx, y = (int)(pi >> 16) + dy;
+            const bool in = act && x >= 0 && x < (int)W && y >= 0 && y < (int)H;
+            const uint32_t pid = (uint32_t)y * W + (uint32_t)x;
+            uint32_t slot = pid * 0x9E3779B1u >> shift, r = NO_ROOT;
+            if (in) {
+                uint32_t seen = S.tab[slot];
+                while (seen != HASH_EMPTY && seen >> 12 != pid) {
+                    slot = (slot + 1) & tmask;
+                    seen = S.tab[slot];
+                }
+                if (seen != HASH_EMPTY) {
+                    const uint32_t j = i - ((i - seen) & HASH_AGE);   // the pixel's latest hit
+                    if (ki - S.key[j] <= dt) {
+                        const uint32_t rj = root_of(j);
+                        if (ki - S.key[rj] <= dt) {   // its cluster is open
+                            r = rj;
+                            S.up[j] = (uint16_t)(j - rj);   // (each pixel's latest hit is another)
+                        }
+                    }
+                }
+            }
+            // hits 1 and 2 of the step must not touch what 0 and 1 change: pixels
+            // nearby, a cluster, the same free table entry
+            const uint32_t m0 = __reduce_min_sync(0xffffffffu, g == 0 ? r : NO_ROOT);   // the earliest root of
+            const uint32_t m1 = __reduce_min_sync(0xffffffffu, g == 1 ? r : NO_ROOT);   // each hit's open clusters
+            const uint32_t m2 = __reduce_min_sync(0xffffffffu, g == 2 ? r : NO_ROOT);
+            const uint32_t same = __match_any_sync(0xffffffffu, r);
+            const uint32_t clash = __ballot_sync(0xffffffffu, r != NO_ROOT && (same & ((1u << (9 * (g < 3 ? g : 0))) - 1u)));
+            const uint32_t s0 = __shfl_sync(0xffffffffu, slot, 4), s1 = __shfl_sync(0xffffffffu, slot, 13),
+                           s2 = __shfl_sync(0xffffffffu, slot, 22);
+            uint32_t take = 1;
+            if (c + 1 < cnt && !adjacent_v(pa, pb) && !(clash & (0x1FFu << 9)) && s0 != s1) {
+                take = 2;
+                if (c + 2 < cnt && !adjacent_v(pa, pc) && !adjacent_v(pb, pc) && !(clash & (0x1FFu << 18)) && s0 != s2 &&
+                    s1 != s2)
+                    take = 3;
+            }
+            const uint32_t m = g == 0 ? m0 : g == 1 ? m1 : m2;
+            __syncwarp();
+            if (act && (uint32_t)g < take) {
+                if (r != NO_ROOT && r != m) S.up[r] = (uint16_t)(r - m);
+                if (d == 4) {
+                    if (m != NO_ROOT) S.up[i] = (uint16_t)(i - m);
+                    S.tab[slot] = pid << 12 | (i & HASH_AGE);
+                }
+            }
+            __syncwarp();
+            c += take;
+        }
+    }
+    for (uint32_t j = lane; j < n; j += 32) parent[gv[q0 + j]] = gv[q0 + root_of(j)];
+}
+
+// A long component: warp 1 runs a chunk of 32 hits ahead of warp 0 and lists
+// each hit's neighbours, the latest hit within dt on each of its nine pixels:
+// from the table (lane = hit), then from the earlier ones of the 32.  Warp 0
+// joins, up to three hits at a time.  The rings hold the last LW_CAP hits: a
+// (c) cluster spans at most dt, so while every hit within dt of the hit being
+// swept is in the window, a hit that leaves it belongs to a cluster closed for
+// every later hit: its root is final and goes to global memory (cpar), where
+// finds that reach it read it.
+struct LongSweep {
+    uint32_t tab[LW_TAB];
+    uint32_t key[LW_CAP], place[LW_CAP], pid[LW_CAP];   // by index mod LW_CAP; sorted position, pixel id
+    uint16_t up[LW_CAP];       // distance to the parent, 0 at a root (at most the hits within dt, so at most the window)
+    uint16_t back[2][32 * 9];  // of a chunk's hits: distance to the latest hit within dt per pixel, 0: none
+    uint32_t next1[2], next2[2];   // hits beside the hit one, two before
+    uint32_t fail, crowded, job;
+};
+
+// Chunk at `base` (lane = hit).
+__device__ __forceinline__ void long_look(LongSweep &S, uint32_t base, uint32_t n, uint32_t se, uint32_t k, uint32_t p,
+                                          uint32_t dt, uint32_t W, uint32_t H, uint32_t &built, int lane) {
+    constexpr uint32_t tmask = LW_TAB - 1u, shift = 32u - 12u;
+    static_assert(LW_TAB == 1u << 12, "table size");
+    const uint32_t e = base + lane;
+    const int x = (int)(p & 0xFFFFu), y = (int)(p >> 16);
+    const uint32_t pid = (uint32_t)y * W + (uint32_t)x;
+    uint16_t *back = S.back[(base >> 5) & 1u];
+    // an entry of a pixel: an empty slot, or the pixel's own with an earlier hit
+    auto put = [&](uint32_t id, uint32_t i, uint32_t now) {
+        uint32_t slot = id * 0x9E3779B1u >> shift, seen = S.tab[slot];
+        while (true) {
+            if (seen != HASH_EMPTY && seen >> 12 != id) {
+                slot = (slot + 1) & tmask;
+                seen = S.tab[slot];
+                continue;
+            }
+            if (seen != HASH_EMPTY && ((now - seen) & HASH_AGE) <= ((now - i) & HASH_AGE)) return;
+            const uint32_t was = atomicCAS(&S.tab[slot], seen, id << 12 | (i & HASH_AGE));
+            if (was == seen) return;
+            seen = was;
+        }
+    };
+    if (base == 0 || base - built >= LW_REBUILD) {   // only hits within dt are still of use
+        const uint32_t k0 = __shfl_sync(0xffffffffu, k, 0);
+        for (uint32_t i = lane; i < LW_TAB / 4; i += 32)
+            reinterpret_cast<uint4 *>(S.tab)[i] = make_uint4(HASH_EMPTY, HASH_EMPTY, HASH_EMPTY, HASH_EMPTY);
+        __syncwarp();
+        for (uint32_t i = (base > LW_WIN ? base - LW_WIN : 0u) + lane; i < base; i += 32)
+            if (k0 - S.key[i % LW_CAP] <= dt) put(S.pid[i % LW_CAP], i, base);
+        built = base;
+    }
+    if (e < n) {
+        S.key[e % LW_CAP] = k;
+        S.place[e % LW_CAP] = se;
+        S.pid[e % LW_CAP] = pid;
+        S.up[e % LW_CAP] = 0;
+    }
+    __syncwarp();
+    uint32_t slot[9], seen[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const int nx = x + q % 3 - 1, ny = y + q / 3 - 1;
+        const bool in = e < n && nx >= 0 && nx < (int)W && ny >= 0 && ny < (int)H;
+        slot[q] = ((uint32_t)ny * W + (uint32_t)nx) * 0x9E3779B1u >> shift;
+        seen[q] = in ? S.tab[slot[q]] : HASH_EMPTY;
+    }
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        const uint32_t want = (uint32_t)(y + q / 3 - 1) * W + (uint32_t)(x + q % 3 - 1);
+        while (seen[q] != HASH_EMPTY && seen[q] >> 12 != want) {
+            slot[q] = (slot[q] + 1) & tmask;
+            seen[q] = S.tab[slot[q]];
+        }
+        uint32_t a = 0;
+        if (seen[q] != HASH_EMPTY) {
+            a = (e - seen[q]) & HASH_AGE;
+            if (a >= LW_WIN || k - S.key[(e - a) % LW_CAP] > dt) a = 0;   // (what has left the window is older than dt)
+        }
+        back[lane * 9 + q] = (uint16_t)a;
+    }
+    __syncwarp();
+    const uint32_t cnt = n - base < 32u ? n - base : 32u;
+    for (uint32_t j = 0; j + 1 < cnt; ++j) {
+        const uint32_t pj = __shfl_sync(0xffffffffu, p, j), kj = __shfl_sync(0xffffffffu, k, j);
+        const int ax = (int)(pj & 0xFFFFu) - x + 1, ay = (int)(pj >> 16) - y + 1;
+        if ((uint32_t)lane > j && (unsigned)ax < 3u && (unsigned)ay < 3u && k - kj <= dt)
+            back[lane * 9 + ay * 3 + ax] = (uint16_t)(lane - j);
+    }
+    const uint32_t u1 = __shfl_up_sync(0xffffffffu, p, 1), u2 = __shfl_up_sync(0xffffffffu, p, 2);
+    const uint32_t next1 = __ballot_sync(0xffffffffu, adjacent_v(u1, p)), next2 = __ballot_sync(0xffffffffu, adjacent_v(u2, p));
+    if (lane == 0) {
+        S.next1[(base >> 5) & 1u] = next1;
+        S.next2[(base >> 5) & 1u] = next2;
+    }
+    if (e < n) put(pid, e, base + 32);
+    __syncwarp();
+}
+
+__device__ __forceinline__ void long_join(LongSweep &S, uint32_t base, uint32_t n, const uint32_t *gv, uint32_t *parent,
+                                          uint32_t *cpar, uint32_t q0, uint32_t dt, uint32_t &lo, bool &crowded, int lane) {
+    const int g = lane / 9, d = lane - 9 * g;      // hit of the step and its neighbour pixel (lanes 27..31 idle)
+    const uint32_t cnt = n - base < 32u ? n - base : 32u;
+    // root of x, or an index before the window (whose cluster is closed)
+    auto root_of = [&](uint32_t x) -> uint32_t {
+        volatile uint16_t *up = S.up;
+        while (x >= lo) {
+            const uint32_t k = up[x % LW_CAP];
+            if (!k) break;
+            x -= k;
+        }
+        return x;
+    };
+    const uint32_t k0 = S.key[base % LW_CAP];
+    if (base >= SW_CAP && __any_sync(0xffffffffu, k0 - S.key[(base - SW_CAP + lane) % LW_CAP] <= dt)) crowded = true;
+    if (base >= LW_WIN) {   // the 32 oldest leave
+        const uint32_t j = base - LW_WIN + lane;
+        if (__any_sync(0xffffffffu, k0 - S.key[j % LW_CAP] <= dt)) {   // the window is too small
+            if (lane == 0) S.fail = 1u;
+            return;
+        }
+        uint32_t r = root_of(j);
+        const uint32_t to = r < lo ? (r = *reinterpret_cast<volatile uint32_t *>(&cpar[r]), gv[q0 + r]) : S.place[r % LW_CAP];
+        __syncwarp();
+        cpar[j] = r;
+        parent[S.place[j % LW_CAP]] = to;
+        __syncwarp();
+        lo = base - LW_WIN + 32;
+    }
+    const uint16_t *back = S.back[(base >> 5) & 1u];
+    const uint32_t next1 = S.next1[(base >> 5) & 1u], next2 = S.next2[(base >> 5) & 1u] | next1;
+    const uint32_t below = (1u << (9 * (g < 3 ? g : 0))) - 1u;
+    for (uint32_t c = 0; c < cnt;) {
+        const uint32_t at = c + g, i = base + at;
+        uint32_t r = NO_ROOT;
+        const bool act = g < 3 && at < cnt;
+        const uint32_t b = act ? back[at * 9 + d] : 0u;
+        if (b) {
+            const uint32_t rj = root_of(i - b);
+            if (rj >= lo && S.key[i % LW_CAP] - S.key[rj % LW_CAP] <= dt) r = rj;   // its cluster is open
+        }
+        // hits 1 and 2 of the step must not touch what 0 and 1 change:
+        // pixels nearby, a cluster
+        const uint32_t m0 = __reduce_min_sync(0xffffffffu, g == 0 ? r : NO_ROOT);   // the earliest root of
+        const uint32_t m1 = __reduce_min_sync(0xffffffffu, g == 1 ? r : NO_ROOT);   // each hit's open clusters
+        const uint32_t m2 = __reduce_min_sync(0xffffffffu, g == 2 ? r : NO_ROOT);
+        const uint32_t same = __match_any_sync(0xffffffffu, r);
+        const uint32_t clash = __ballot_sync(0xffffffffu, r != NO_ROOT && (same & below));
+        uint32_t take = 1;
+        if (c + 1 < cnt && !((next1 >> (c + 1)) & 1u) && !(clash & (0x1FFu << 9))) {
+            take = 2;
+            if (c + 2 < cnt && !((next2 >> (c + 2)) & 1u) && !(clash & (0x1FFu << 18))) take = 3;
+        }
+        const uint32_t m = g == 0 ? m0 : g == 1 ? m1 : m2;
+        if (act && (uint32_t)g < take) {
+            if (r != NO_ROOT && r != m) S.up[r % LW_CAP] = (uint16_t)(r - m);
+            if (d == 4 && m != NO_ROOT) S.up[i % LW_CAP] = (uint16_t)(i - m);
+        }
+        __syncwarp();
+        c += take;
+    }
+}
+
+// Up to 32 hits: lane j holds hit j (key, pixel) and its root.
+__device__ __forceinline__ void sweep_registers(const uint32_t *skey, const uint32_t *spix, const uint32_t *gv,
+                                                uint32_t *parent, uint32_t q0, uint32_t n, uint32_t dt, int lane) {
+    uint32_t se = 0, k = 0, p = 0, root = lane;
+    if ((uint32_t)lane < n) {
+        se = gv[q0 + lane];
+        k = skey[se];
+        p = spix[se];
+    }
+    for (uint32_t i = 1; i < n; ++i) {
+        const uint32_t ki = __shfl_sync(0xffffffffu, k, i), pi = __shfl_sync(0xffffffffu, p, i);
+        const uint32_t kr = __shfl_sync(0xffffffffu, k, root);
+        const bool joins = (uint32_t)lane < i && adjacent_v(pi, p) && ki - kr <= dt;   // open: so is the hit itself within dt
+        const uint32_t open = __reduce_or_sync(0xffffffffu, joins ? 1u << root : 0u);   // the roots joined
+        if (open && ((open >> root) & 1u || (uint32_t)lane == i)) root = __ffs(open) - 1;
+    }
+    const uint32_t sr = __shfl_sync(0xffffffffu, se, root);
+    if ((uint32_t)lane < n) parent[se] = sr;
+}
+
+// Lists the components of more than SW_CAP hits: a component starts at q and
+// reaches beyond q + SW_CAP; its end by doubling steps, then halving ones.
+__global__ void __launch_bounds__(256) k_static_long(Work w, VarWork v) {
+    const uint32_t sel = v.prob->npasses & 1u;
+    const uint32_t *gk = pick(v.k, sel);
+    const Seg &g = w.seg[0];
+    const uint32_t first = g.off, last = g.off + g.n;
+    for (uint32_t q = first + blockIdx.x * blockDim.x + threadIdx.x; q < last; q += gridDim.x * blockDim.x) {
+        const uint32_t key = gk[q];
+        if ((q != first && gk[q - 1] == key) || last - q <= SW_CAP || gk[q + SW_CAP] != key) continue;
+        uint32_t in = q + SW_CAP, step = SW_CAP;   // gk[in] == key
+        while (last - in > step && gk[in + step] == key) { in += step; step *= 2; }
+        uint32_t out = last - in > step ? in + step : last;
+        while (out - in > 1) {
+            const uint32_t mid = in + (out - in) / 2;
+            if (gk[mid] == key) in = mid; else out = mid;
+        }
+        const uint32_t n = in + 1 - q;
+        atomicAdd(&v.changed[0], 1u);
+        // the list holds all of them (each has > SW_CAP hits), the longest from its end
+        if (n >= LW_FIRST) v.big[v.big_cap - 1 - atomicAdd(&v.changed[5], 1u)] = make_uint2(q, n);
+        else v.big[atomicAdd(&v.changed[6], 1u)] = make_uint2(q, n);
+    }
+}
+
+__global__ void __launch_bounds__(SW_WARPS * 32) k_static_sweep(Work w, VarWork v) {
+    extern __shared__ __align__(16) unsigned char sweep_raw[];
+    const uint32_t *skey = pick(w.keys, sorted_sel(*w.prob));
+    const uint32_t sel = v.prob->npasses & 1u;
+    const uint32_t *gk = pick(v.k, sel), *gv = pick(v.v, sel);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    HashSweep &S = reinterpret_cast<HashSweep *>(sweep_raw)[warp];
+    const Seg &g = w.seg[0];
+    const uint32_t first = g.off, last = g.off + g.n, dt = g.dt, W = g.width, H = g.height;
+    const uint32_t nchunks = (g.n + SW_CHUNK - 1) / SW_CHUNK;
+    while (true) {
+        uint32_t c = 0;
+        if (lane == 0) c = atomicAdd(v.work, 1u);
+        c = __shfl_sync(0xffffffffu, c, 0);
+        if (c >= nchunks) break;
+        const uint32_t q = first + c * SW_CHUNK + lane;
+        uint32_t starts = __ballot_sync(0xffffffffu, q < last && (q == first || gk[q] != gk[q - 1]));
+        while (starts) {
+            const uint32_t q0 = first + c * SW_CHUNK + (__ffs(starts) - 1);
+            starts &= starts - 1;
+            // the component's end: the first grouped position with another root
+            const uint32_t key0 = gk[q0];
+            uint32_t n = 0;
+            for (uint32_t p0 = q0 + 1;; p0 += 32) {
+                const uint32_t p = p0 + lane;
+                const uint32_t stop = __ballot_sync(0xffffffffu, p >= last || gk[p] != key0);
+                if (stop) { n = p0 + (__ffs(stop) - 1) - q0; break; }
+                if (p0 - q0 > SW_CAP) break;   // listed by k_static_long (n = 0)
+            }
+            if (n == 1) {
+                if (lane == 0) w.parent[gv[q0]] = gv[q0];
+            } else if (n && n <= 32) {
+                sweep_registers(skey, w.spix, gv, w.parent, q0, n, dt, lane);
+            } else if (n && n <= SW_CAP) {
+                sweep_hashed(S, skey, w.spix, gv, w.parent, q0, n, dt, W, H, lane);
+            }
+            __syncwarp();   // the staging is rewritten for the next component
+        }
+    }
+}
+
+__global__ void __launch_bounds__(64) k_static_sweep_long(Work w, VarWork v) {
+    extern __shared__ __align__(16) unsigned char sweep_raw[];
+    LongSweep &S = *reinterpret_cast<LongSweep *>(sweep_raw);
+    const uint32_t *skey = pick(w.keys, sorted_sel(*w.prob));
+    const uint32_t *gv = pick(v.v, v.prob->npasses & 1u);
+    const int lane = threadIdx.x & 31;
+    const bool looks = threadIdx.x >= 32;
+    const Seg &g = w.seg[0];
+    const uint32_t nfirst = v.changed[5], nlong = v.changed[0], dt = g.dt, W = g.width, H = g.height;
+    while (true) {
+        if (threadIdx.x == 0) {
+            S.job = atomicAdd(&v.changed[4], 1u);
+            S.fail = S.crowded = 0;
+        }
+        __syncthreads();
+        const uint32_t job = S.job;
+        if (job >= nlong) break;
+        // the longest ones first: a chain started late would end alone
+        const uint2 comp = job < nfirst ? v.big[v.big_cap - 1 - job] : v.big[job - nfirst];
+        const uint32_t q0 = comp.x, n = comp.y;
+        uint32_t *cpar = v.cpar + q0;
+        uint32_t lo = 0, built = 0, se1 = 0, k1 = 0, p1 = 0, se2 = 0;
+        bool crowded = false;
+        if (looks) {
+            se1 = gv[q0 + lane];   // (n > SW_CAP)
+            k1 = skey[se1];
+            p1 = w.spix[se1];
+            se2 = gv[q0 + 32 + lane];
+        }
+        for (uint32_t base = 0; base < n + 32; base += 32) {
+            if (looks) {
+                if (base < n) {
+                    const uint32_t e = base + lane, se = se1, k = k1, p = p1;
+                    se1 = se2;   // the next hits are on their way meanwhile
+                    if (e + 32 < n) {
+                        k1 = skey[se1];
+                        p1 = w.spix[se1];
+                    }
+                    if (e + 64 < n) se2 = gv[q0 + e + 64];
+                    long_look(S, base, n, se, k, p, dt, W, H, built, lane);
+                }
+            } else if (base) {
+                long_join(S, base - 32, n, gv, w.parent, cpar, q0, dt, lo, crowded, lane);
+            }
+            __syncthreads();
+            if (S.fail) break;
+        }
+        if (!looks) {
+            if (lane == 0) {
+                if (crowded) {   // diagnostics
+                    atomicAdd(&v.changed[1], 1u);
+                    if (n > BIG_CAP) atomicAdd(&v.changed[2], 1u);
+                }
+                if (S.fail) v.over[atomicAdd(&v.changed[3], 1u)] = comp;
+            }
+            if (!S.fail) {
+                for (uint32_t j = lo + lane; j < n; j += 32) {   // the hits still in the window
+                    uint32_t r = j;
+                    while (r >= lo) {
+                        const uint32_t k = S.up[r % LW_CAP];
+                        if (!k) break;
+                        r -= k;
+                    }
+                    w.parent[S.place[j % LW_CAP]] = r < lo ? gv[q0 + cpar[r]] : S.place[r % LW_CAP];
+                }
+            }
+        }
+        __syncthreads();   // the rings are rewritten for the next component
+    }
+}
 
 template <bool STAGED>
 struct SweepView {
@@ -102,199 +550,12 @@ struct SweepView {
     }
 };
 
-template <bool STAGED>
-__device__ void sweep_component(const SweepView<STAGED> &V, uint32_t n, uint32_t dt, int lane) {
-    for (uint32_t i = lane; i < n; i += 32) V.sc[i] = i;
-    __syncwarp();
-    for (uint32_t i = 1; i < n; ++i) {
-        const uint32_t ki = V.key(i), pi = V.pix(i);
-        uint32_t root = 0xFFFFFFFFu;   // the earliest open root joined so far
-        for (uint32_t base = 0; base < i; base += 32) {
-            const bool valid = base + lane < i;
-            const uint32_t j = valid ? i - 1 - base - lane : 0;
-            const bool in = valid && ki - V.key(j) <= dt;
-            if (!__any_sync(0xffffffffu, in)) break;   // keys only fall further back
-            uint32_t r = 0xFFFFFFFFu;
-            if (in && adjacent_v(pi, V.pix(j))) {
-                const uint32_t rj = V.find(j);
-                if (ki - V.key(rj) <= dt) r = rj;   // that cluster is still open
-            }
-            const uint32_t m = __reduce_min_sync(0xffffffffu, r);
-            __syncwarp();
-            if (m != 0xFFFFFFFFu) {
-                const uint32_t target = m < root ? m : root;
-                if (r != 0xFFFFFFFFu && r != target) V.sc[r] = target;
-                if (lane == 0 && root != 0xFFFFFFFFu && root != target) V.sc[root] = target;
-                root = target;
-            }
-            __syncwarp();
-        }
-        if (lane == 0 && root != 0xFFFFFFFFu) V.sc[i] = root;
-        __syncwarp();
-    }
-}
-
-// Components of more than SW_CAP hits: the same sweep over a sliding window
-// of the component's last SW_CAP hits in shared memory (slot = index mod
-// SW_CAP).  A (c) cluster spans at most dt, so while every hit within dt of
-// the hit being swept is still in the window, a hit that leaves it belongs
-// to a cluster that is closed for every later hit: its root is final.  On
-// leaving, its root goes to global memory (cpar, by component index, and
-// the parent array); finds that reach a hit that has left read it there.  A
-// batch of 32 hits enters every 32 steps, pushing the 32 oldest out; if one
-// of those is within dt of the first newcomer, the window is too small
-// (returns false): the component is listed for k_static_sweep_big, which
-// sweeps it again with a whole CTA, staged in shared memory up to BIG_CAP
-// hits, from global memory beyond.
-template <uint32_t CAP>
-struct WindowView {
-    uint32_t *wk, *wp, *wc;    // window: key, pixel, parent (component index)
-    uint32_t *cpar;            // global: final root of each hit that left
-    uint32_t lo;               // first component index still in the window
-    __device__ uint32_t key(uint32_t i) const { return wk[i % CAP]; }
-    __device__ uint32_t pix(uint32_t i) const { return wp[i % CAP]; }
-    __device__ uint32_t find(uint32_t x) const {
-        volatile uint32_t *c = wc;
-        while (true) {
-            if (x < lo) return *reinterpret_cast<volatile uint32_t *>(&cpar[x]);
-            const uint32_t p = c[x % CAP];
-            if (p == x) return x;
-            if (p < lo) return *reinterpret_cast<volatile uint32_t *>(&cpar[p]);
-            const uint32_t gp = c[p % CAP];
-            if (gp == p) return p;
-            c[x % CAP] = gp;
-            x = gp;
-        }
-    }
-};
-
-template <uint32_t CAP>
-__device__ bool sweep_windowed(WindowView<CAP> V, const uint32_t *skey, const uint32_t *spix, const uint32_t *gv,
-                               uint32_t *parent, uint32_t q0, uint32_t n, uint32_t dt, int lane) {
-    for (uint32_t i = 0; i < n; ++i) {
-        if ((i & 31u) == 0) {   // hits [i, i + 32) enter, [i - CAP, i - CAP + 32) leave
-            const uint32_t ki = skey[gv[q0 + i]];
-            if (i >= CAP) {
-                const uint32_t j = i - CAP + lane;   // < i <= n - 1
-                if (__any_sync(0xffffffffu, ki - V.key(j) <= dt)) return false;
-                const uint32_t r = V.find(j);
-                __syncwarp();
-                V.cpar[j] = r;
-                parent[gv[q0 + j]] = gv[q0 + r];
-                __syncwarp();
-                V.lo = i - CAP + 32;
-            }
-            const uint32_t e = i + lane;
-            if (e < n) {
-                const uint32_t se = gv[q0 + e];
-                V.wk[e % CAP] = skey[se];
-                V.wp[e % CAP] = spix[se];
-                V.wc[e % CAP] = e;
-            }
-            __syncwarp();
-        }
-        if (i == 0) continue;
-        const uint32_t ki = V.key(i), pi = V.pix(i);
-        uint32_t root = 0xFFFFFFFFu;   // the earliest open root joined so far
-        for (uint32_t base = 0; base < i; base += 32) {
-            const bool valid = base + lane < i && i - 1 - base - lane >= V.lo;
-            const uint32_t j = valid ? i - 1 - base - lane : i;
-            const bool in = valid && ki - V.key(j) <= dt;
-            if (!__any_sync(0xffffffffu, in)) break;   // keys only fall further back
-            uint32_t r = 0xFFFFFFFFu;
-            if (in && adjacent_v(pi, V.pix(j))) {
-                const uint32_t rj = V.find(j);
-                if (rj >= V.lo && ki - V.key(rj) <= dt) r = rj;   // that cluster is still open
-            }
-            const uint32_t m = __reduce_min_sync(0xffffffffu, r);
-            __syncwarp();
-            if (m != 0xFFFFFFFFu) {
-                const uint32_t target = m < root ? m : root;
-                if (r != 0xFFFFFFFFu && r != target) V.wc[r % CAP] = target;
-                if (lane == 0 && root != 0xFFFFFFFFu && root != target) V.wc[root % CAP] = target;
-                root = target;
-            }
-            __syncwarp();
-        }
-        if (lane == 0 && root != 0xFFFFFFFFu) V.wc[i % CAP] = root;
-        __syncwarp();
-    }
-    // the hits still in the window
-    const uint32_t first = V.lo;
-    for (uint32_t j = first + lane; j < n; j += 32) {
-        const uint32_t r = V.find(j);
-        parent[gv[q0 + j]] = gv[q0 + r];
-    }
-    return true;
-}
-
-__global__ void __launch_bounds__(SW_WARPS * 32) k_static_sweep(Work w, VarWork v) {
-    __shared__ uint32_t s_k[SW_WARPS][SW_CAP], s_p[SW_WARPS][SW_CAP], s_c[SW_WARPS][SW_CAP];
-    const uint32_t *skey = pick(w.keys, sorted_sel(*w.prob));
-    const uint32_t sel = v.prob->npasses & 1u;
-    const uint32_t *gk = pick(v.k, sel), *gv = pick(v.v, sel);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const Seg &g = w.seg[0];
-    const uint32_t first = g.off, last = g.off + g.n, dt = g.dt;
-    const uint32_t nchunks = (g.n + SW_CHUNK - 1) / SW_CHUNK;
-    while (true) {
-        uint32_t c = 0;
-        if (lane == 0) c = atomicAdd(v.work, 1u);
-        c = __shfl_sync(0xffffffffu, c, 0);
-        if (c >= nchunks) break;
-        const uint32_t q = first + c * SW_CHUNK + lane;
-        uint32_t starts = __ballot_sync(0xffffffffu, q < last && (q == first || gk[q] != gk[q - 1]));
-        while (starts) {
-            const uint32_t q0 = first + c * SW_CHUNK + (__ffs(starts) - 1);
-            starts &= starts - 1;
-            // the component's end: the first grouped position with another root
-            const uint32_t key0 = gk[q0];
-            uint32_t n = 0;
-            for (uint32_t p0 = q0 + 1;; p0 += 32) {
-                const uint32_t p = p0 + lane;
-                const uint32_t stop = __ballot_sync(0xffffffffu, p >= last || gk[p] != key0);
-                if (stop) { n = p0 + (__ffs(stop) - 1) - q0; break; }
-            }
-            if (n == 1) {
-                if (lane == 0) w.parent[gv[q0]] = gv[q0];
-                continue;
-            }
-            if (n <= SW_CAP) {
-                for (uint32_t i = lane; i < n; i += 32) {
-                    const uint32_t si = gv[q0 + i];
-                    s_k[warp][i] = skey[si];
-                    s_p[warp][i] = w.spix[si];
-                }
-                __syncwarp();
-                const SweepView<true> V{s_k[warp], s_p[warp], s_c[warp], skey, w.spix, gv, q0};
-                sweep_component(V, n, dt, lane);
-                for (uint32_t i = lane; i < n; i += 32) w.parent[gv[q0 + i]] = gv[q0 + V.find(i)];
-            } else {
-                const WindowView<SW_CAP> WV{s_k[warp], s_p[warp], s_c[warp], v.cpar + q0, 0};
-                if (lane == 0) atomicAdd(&v.changed[0], 1u);   // diagnostics: windowed components
-                if (!sweep_windowed(WV, skey, w.spix, gv, w.parent, q0, n, dt, lane)) {
-                    if (lane == 0) {   // more than the window within dt: the big window's list
-                        const uint32_t k = atomicAdd(&v.changed[1], 1u);
-                        v.big[k] = make_uint2(q0, n);   // k < positions / SW_CAP: each has > SW_CAP hits
-                    }
-                    __syncwarp();
-                }
-            }
-            __syncwarp();   // the staging is rewritten for the next component
-        }
-    }
-}
-
 // (c): components whose hits within dt outgrew the warp's window.  One CTA
 // per component, the component staged whole in dynamic shared memory (up to
 // BIG_CAP hits; from global memory beyond): the same sweep, with each
 // step's candidates (the earlier hits within dt) spread over the CTA's
 // threads instead of one warp's lanes, the earliest open root found by a
 // shared-memory minimum.
-constexpr int BIG_THREADS = 512;
-constexpr uint32_t BIG_CAP = 8192;
-constexpr int BIG_SMEM = 3 * BIG_CAP * (int)sizeof(uint32_t);
-
 template <bool STAGED>
 __device__ void sweep_block(const SweepView<STAGED> &V, uint32_t n, uint32_t dt, uint32_t *s_min) {
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) V.sc[i] = i;
@@ -337,9 +598,9 @@ __global__ void __launch_bounds__(BIG_THREADS) k_static_sweep_big(Work w, VarWor
     __shared__ uint32_t s_min[2];
     const uint32_t *skey = pick(w.keys, sorted_sel(*w.prob));
     const uint32_t *gv = pick(v.v, v.prob->npasses & 1u);
-    const uint32_t dt = w.seg[0].dt, nbig = v.changed[1];
+    const uint32_t dt = w.seg[0].dt, nbig = v.changed[3];
     for (uint32_t k = blockIdx.x; k < nbig; k += gridDim.x) {
-        const uint2 job = v.big[k];
+        const uint2 job = v.over[k];
         const uint32_t q0 = job.x, n = job.y;
         if (n <= BIG_CAP) {
             uint32_t *sk = big_raw, *sp = big_raw + BIG_CAP, *sc = big_raw + 2 * BIG_CAP;
@@ -353,7 +614,6 @@ __global__ void __launch_bounds__(BIG_THREADS) k_static_sweep_big(Work w, VarWor
             sweep_block(V, n, dt, s_min);
             for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) w.parent[gv[q0 + i]] = gv[q0 + V.find(i)];
         } else {
-            if (threadIdx.x == 0) atomicAdd(&v.changed[2], 1u);   // diagnostics: swept from global memory
             const SweepView<false> V{nullptr, nullptr, v.cpar + q0, skey, w.spix, gv, q0};
             sweep_block(V, n, dt, s_min);
             for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) w.parent[gv[q0 + i]] = gv[q0 + V.find(i)];
@@ -362,8 +622,21 @@ __global__ void __launch_bounds__(BIG_THREADS) k_static_sweep_big(Work w, VarWor
     }
 }
 
+constexpr int SW_SMEM = SW_WARPS * (int)sizeof(HashSweep);
+constexpr int LW_SMEM = (int)sizeof(LongSweep);
+
 cudaError_t init_variants_attributes() {
-    return cudaFuncSetAttribute(k_static_sweep_big, cudaFuncAttributeMaxDynamicSharedMemorySize, BIG_SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_static_sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, SW_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_static_sweep_long, cudaFuncAttributeMaxDynamicSharedMemorySize, LW_SMEM);
+    // the two sweeps run side by side on the SMs: one split of L1 and shared memory for both
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_static_sweep, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_static_sweep_long, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared);
+    return e == cudaSuccess
+               ? cudaFuncSetAttribute(k_static_sweep_big, cudaFuncAttributeMaxDynamicSharedMemorySize, BIG_SMEM) : e;
 }
 
 // (b): pixel histogram and its exclusive scan (single segment).
@@ -836,13 +1109,25 @@ Work variant_view(const Work &w, const VarWork &v) {
     return wv;
 }
 
-void launch_static_sweep(const Work &w, const VarWork &v, const Launch &L) {
+// The long components take as long as the sweep of all others (8 M hits of the
+// 2.5 Ghits/s stream: 2.0 and 0.9 ms), which runs beside them on `side`.
+cudaError_t launch_static_sweep(const Work &w, const VarWork &v, const Launch &L, const SideStream &side) {
     cudaMemsetAsync(v.work, 0, sizeof(uint32_t), L.stream);
-    cudaMemsetAsync(v.changed, 0, 3 * sizeof(uint32_t), L.stream);
-    k_static_sweep<<<L.fit(k_static_sweep, SW_WARPS * 32, 0), SW_WARPS * 32, 0, L.stream>>>(w, v);
+    cudaMemsetAsync(v.changed, 0, 7 * sizeof(uint32_t), L.stream);
+    k_static_long<<<L.fit(k_static_long, 256, 0), 256, 0, L.stream>>>(w, v);
+    L.mark("k_static_long");
+    cudaError_t e = cudaEventRecord(side.fork, L.stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(side.stream, side.fork, 0);
+    if (e != cudaSuccess) return e;
+    const int fit = L.fit(k_static_sweep_long, 64, LW_SMEM), few = (L.sms > 0 ? L.sms : 1) * LW_CTAS;
+    k_static_sweep_long<<<fit < few ? fit : few, 64, LW_SMEM, side.stream>>>(w, v);
+    k_static_sweep_big<<<L.fit(k_static_sweep_big, BIG_THREADS, BIG_SMEM), BIG_THREADS, BIG_SMEM, side.stream>>>(w, v);
+    e = cudaEventRecord(side.join, side.stream);
+    k_static_sweep<<<L.fit(k_static_sweep, SW_WARPS * 32, SW_SMEM), SW_WARPS * 32, SW_SMEM, L.stream>>>(w, v);
     L.mark("k_static_sweep");
-    k_static_sweep_big<<<L.fit(k_static_sweep_big, BIG_THREADS, BIG_SMEM), BIG_THREADS, BIG_SMEM, L.stream>>>(w, v);
-    L.mark("k_static_sweep_big");
+    const cudaError_t e2 = cudaStreamWaitEvent(L.stream, side.join, 0);   // (the step goes on after both)
+    L.mark("k_static_sweep_long");
+    return e == cudaSuccess ? e2 : e;
 }
 
 void launch_pixel_timelines(const Work &w, const VarWork &v, uint32_t npixels, const Launch &L) {
