@@ -22,9 +22,11 @@
 //                    carry of open hits and the stream state.
 //
 // Small steps (at most SMALL_TILES tiles) work for any order, so that they
-// need no sorted path behind them: k_arrival_small owns hits by position and
-// looks back over earlier positions, and k_arrival_redo joins the tiles that
-// did not look far enough with every earlier tile.
+// need no sorted path behind them: tiles own hits by position and look back
+// over earlier positions, and tiles that did not look far enough are joined
+// with every earlier tile.  All of it is one launch (k_arrival_step), a
+// cluster of one CTA per tile.  As seven launches a call with 1,000 hits took
+// 53 us (41 of them on the host) and one with 65,536 hits 96; now 28 and 65.
 //
 // Owning by time keeps events whole: arrival disorder spreads an event's hits
 // over a thousand positions, and tiles of positions would cut a quarter of
@@ -35,6 +37,8 @@
 // Tile clusters are numbered c = tile * TILE + (index among the tile's
 // clusters), so that everything kept per cluster (32-byte RootSlot, first and
 // last ToA, union-find parent) is dense and a hit's cluster is one 32-bit c.
+#include <cooperative_groups.h>
+
 #include "tpc_internal.cuh"
 
 namespace tpc {
@@ -965,26 +969,14 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
     }
 }
 
-__global__ void __launch_bounds__(AT) k_arrival_small(Work w) {
-    extern __shared__ __align__(16) unsigned char a_raw[];
-    SmallShared &S = *reinterpret_cast<SmallShared *>(a_raw);
-    const uint32_t nt = w.prob->ntiles;
-    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
-        __syncthreads();   // the arrays are free for the next tile
-        small_tile<false>(w, t, S);
-    }
-}
-
-// Tiles that did not look far enough back, or listed more pairs than their
-// list holds.
-__global__ void __launch_bounds__(AT) k_arrival_redo(Work w) {
-    extern __shared__ __align__(16) unsigned char a_raw[];
-    SmallShared &S = *reinterpret_cast<SmallShared *>(a_raw);
-    const uint32_t nt = w.prob->ntiles;
-    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
-        if (!w.atile[t].redo) continue;
-        __syncthreads();
-        small_tile<true>(w, t, S);
+// Joins the listed pairs of a tile.
+template <int NT>
+__device__ __forceinline__ void join_pairs(const Work &w, uint32_t t) {
+    const uint32_t nx = min(w.atile[t].nx, (uint32_t)A_PAIRS);
+    const uint2 *list = w.xlist + (size_t)t * A_PAIRS;
+    for (uint32_t i = threadIdx.x; i < nx; i += NT) {
+        const uint2 p = list[i];
+        gunion(w.gpar, p.x, w.root_of[p.y]);
     }
 }
 
@@ -993,45 +985,26 @@ __global__ void __launch_bounds__(AT) k_arrival_redo(Work w) {
 // up to all hits; and a tile saw every earlier hit within dt of its interval
 // if it counted as many of them as its predecessor counted own hits that
 // late (which are all there are, if dt reaches no further back than the
-// predecessor's interval).  A small step's tile that looked back to position
-// h0 is complete if every hit before h0 is earlier than its first by more
-// than dt.
+// predecessor's interval).
 constexpr int AX = 256;
 
-__global__ void __launch_bounds__(AX) k_arrival_cross(Work w, int small, cudaGraphConditionalHandle sorted) {
+__global__ void __launch_bounds__(AX) k_arrival_cross(Work w, cudaGraphConditionalHandle sorted) {
     Prob &P = *w.prob;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x;
     bool lost = P.raw_fail != 0;
-    if (!small)
-        for (uint32_t s = tid; s < P.nsegs; s += AX) lost |= w.seg[s].n_owned != w.seg[s].n;
+    for (uint32_t s = tid; s < P.nsegs; s += AX) lost |= w.seg[s].n_owned != w.seg[s].n;
     bool fail = __syncthreads_or(lost);
     if (!fail) {
         const uint32_t nt = P.ntiles;
         for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
-            const ATile &info = w.atile[t];
-            if (warp == 0) {
+            if (tid == 0) {
                 const Seg &g = w.seg[w.tile_seg[t]];
-                if (small) {
-                    const uint32_t hc = info.h0 / A_STEP;   // chunks not looked at
-                    uint64_t m = 0;
-                    for (uint32_t i = lane; i < hc; i += 32) {
-                        const uint64_t c = w.atile[i / ACHUNKS].cmax[i % ACHUNKS];
-                        m = c > m ? c : m;
-                    }
-                    m = warp_max_u64(m);
-                    if (lane == 0 && ((hc && m >= info.lo) || info.nx > A_PAIRS)) w.atile[t].redo = 1u;
-                } else if (lane == 0 && t > g.tile0) {
-                    const ATile &prev = w.atile[t - 1];
-                    fail = info.nhalo != prev.ntail || (t - 1 > g.tile0 && info.cut < prev.cut + g.dt);
+                if (t > g.tile0) {
+                    const ATile &info = w.atile[t], &prev = w.atile[t - 1];
+                    fail |= info.nhalo != prev.ntail || (t - 1 > g.tile0 && info.cut < prev.cut + g.dt);
                 }
             }
-            const uint32_t nx = min(info.nx, (uint32_t)A_PAIRS);
-            const uint2 *list = w.xlist + (size_t)t * A_PAIRS;
-            for (uint32_t i = tid; i < nx; i += AX) {
-                const uint2 p = list[i];
-                gunion(w.gpar, p.x, w.root_of[p.y]);
-            }
-            if (fail) break;   // (lane 0 of warp 0: its other tiles no longer matter)
+            join_pairs<AX>(w, t);
         }
     }
     if (fail && tid == 0) {
@@ -1045,32 +1018,33 @@ __global__ void __launch_bounds__(AX) k_arrival_cross(Work w, int small, cudaGra
 // Each tile cluster adds its features to its cluster's, and points straight
 // at it.  The finds write nothing on their way: a path halved with a parent
 // read before another thread's final store would undo that store.
+template <int NT>
+__device__ __forceinline__ void root_tile(const Work &w, uint32_t t, bool streaming) {
+    const uint32_t nr = w.atile[t].nroots;
+    for (uint32_t i = threadIdx.x; i < nr; i += NT) {
+        const uint32_t c = t * TILE + i;
+        volatile uint32_t *par = w.gpar;
+        uint32_t r = c;
+        for (uint32_t p = par[r]; p != r; p = par[r]) r = p;
+        if (r == c) continue;
+        w.gpar[c] = r;
+        const RootSlot s = w.rslot[c];
+        RootSlot &d = w.rslot[r];
+        atomicAdd(&d.tot, s.tot);
+        atomicAdd(&d.wx, s.wx);
+        atomicAdd(&d.wy, s.wy);
+        atomicAdd(&d.size, s.size);
+        atomicMin(&d.min, s.min);
+        atomicMin(reinterpret_cast<unsigned long long *>(&w.rfirst[r]), (unsigned long long)w.rfirst[c]);
+        if (streaming) atomicMax(reinterpret_cast<unsigned long long *>(&w.rlast[r]), (unsigned long long)w.rlast[c]);
+    }
+}
+
 __global__ void __launch_bounds__(256) k_arrival_roots(Work w) {
     const Prob &P = *w.prob;
     if (P.raw_fail) return;
     const uint32_t nt = P.ntiles;
-    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
-        const uint32_t nr = w.atile[t].nroots;
-        const bool streaming = w.seg[w.tile_seg[t]].ss != nullptr;
-        for (uint32_t i = threadIdx.x; i < nr; i += blockDim.x) {
-            const uint32_t c = t * TILE + i;
-            volatile uint32_t *par = w.gpar;
-            uint32_t r = c;
-            for (uint32_t p = par[r]; p != r; p = par[r]) r = p;
-            if (r == c) continue;
-            w.gpar[c] = r;
-            const RootSlot s = w.rslot[c];
-            RootSlot &d = w.rslot[r];
-            atomicAdd(&d.tot, s.tot);
-            atomicAdd(&d.wx, s.wx);
-            atomicAdd(&d.wy, s.wy);
-            atomicAdd(&d.size, s.size);
-            atomicMin(&d.min, s.min);
-            atomicMin(reinterpret_cast<unsigned long long *>(&w.rfirst[r]), (unsigned long long)w.rfirst[c]);
-            if (streaming)
-                atomicMax(reinterpret_cast<unsigned long long *>(&w.rlast[r]), (unsigned long long)w.rlast[c]);
-        }
-    }
+    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) root_tile<256>(w, t, w.seg[w.tile_seg[t]].ss != nullptr);
 }
 
 // Labels of the hits at a tile's positions.  Their clusters are mostly tile
@@ -1078,73 +1052,75 @@ __global__ void __launch_bounds__(256) k_arrival_roots(Work w) {
 // gathered once into shared memory (if they fit), then looked up per hit.
 constexpr uint32_t AL_CAP = 4096;
 
+template <int NT>
+__device__ __forceinline__ void label_tile(const Work &w, uint32_t t, const Seg &g, uint32_t *s_lab, uint32_t *s_cnt) {
+    const int lane = threadIdx.x & 31;
+    constexpr uint32_t CLOSED = 0x80000000u;   // a segment holds at most 2^31 - 1 hits
+    uint32_t begin, end;
+    tile_range(g, t, begin, end);
+    const uint32_t mode = g.close_mode, off = g.off;
+    const uint64_t mark = g.watermark;
+    auto label_of = [&](uint32_t c) -> uint32_t {
+        const uint32_t r = w.gpar[c];
+        const bool closed = mode == CLOSE_ALL || (mode == CLOSE_WM && w.rlast[r] <= mark);
+        return (w.rslot[r].min - off) | (closed ? CLOSED : 0u);
+    };
+    const uint32_t n0 = t > g.tile0 ? w.atile[t - 1].nroots : 0, n1 = w.atile[t].nroots;
+    const uint32_t n2 = t + 1 < g.tile0 + g.ntiles ? w.atile[t + 1].nroots : 0;
+    const bool table = n0 + n1 + n2 <= AL_CAP;
+    // c in [c0, c0 + n0), [c1, c1 + n1), [c2, c2 + n2): s_lab[c - c0], s_lab[n0 + c - c1], ...
+    const uint32_t c1 = t * TILE, c0 = c1 - TILE, c2 = c1 + TILE;
+    if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
+    if (table)
+        for (uint32_t i = threadIdx.x; i < n0 + n1 + n2; i += NT)
+            s_lab[i] = label_of(i < n0 ? c0 + i : i < n0 + n1 ? c1 + i - n0 : c2 + i - n0 - n1);
+    __syncthreads();
+    const bool direct = g.ss == nullptr;   // one-shot: every hit is final
+    uint32_t c_label = 0, c_closed = 0;
+    constexpr int ITEMS = TILE / NT;
+#pragma unroll 8
+    for (int q = 0; q < ITEMS; ++q) {
+        const uint32_t pos = begin + q * NT + threadIdx.x;
+        bool is_label = false, closed = false;
+        if (pos < end) {
+            const uint32_t c = w.root_of[pos];
+            uint32_t v;
+            if (table && c - c1 < n1) v = s_lab[n0 + c - c1];
+            else if (table && c - c0 < n0) v = s_lab[c - c0];
+            else if (table && c - c2 < n2) v = s_lab[n0 + n1 + c - c2];
+            else v = label_of(c);
+            const uint32_t l = v & ~CLOSED;
+            closed = (v & CLOSED) != 0;
+            is_label = closed && l == pos - off;
+            const uint64_t lab = gidx_of(g, l);
+            if (direct) g.out_labels[pos - off] = lab;
+            else w.lab_tmp[pos] = lab;
+        }
+        const uint32_t bl = __ballot_sync(0xffffffffu, is_label);
+        const uint32_t bc = __ballot_sync(0xffffffffu, closed);
+        if (lane == 0) {
+            w.flag_label[pos >> 5] = bl;
+            w.flag_closed[pos >> 5] = bc;
+            c_label += __popc(bl);
+            c_closed += __popc(bc);
+        }
+    }
+    if (lane == 0) {
+        atomicAdd(&s_cnt[0], c_label);
+        atomicAdd(&s_cnt[1], c_closed);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) w.tile_cnt[threadIdx.x * w.prob->tile_cap + t] = s_cnt[threadIdx.x];
+    __syncthreads();
+}
+
 __global__ void __launch_bounds__(256) k_arrival_labels(Work w) {
     __shared__ uint32_t s_lab[AL_CAP];   // label position in the segment, closed flag
     __shared__ uint32_t s_cnt[2];
     const Prob &P = *w.prob;
     if (P.raw_fail) return;
     const uint32_t nt = P.ntiles;
-    const int lane = threadIdx.x & 31;
-    constexpr uint32_t CLOSED = 0x80000000u;   // a segment holds at most 2^31 - 1 hits
-    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
-        const Seg &g = w.seg[w.tile_seg[t]];
-        uint32_t begin, end;
-        tile_range(g, t, begin, end);
-        const uint32_t mode = g.close_mode, off = g.off;
-        const uint64_t mark = g.watermark;
-        auto label_of = [&](uint32_t c) -> uint32_t {
-            const uint32_t r = w.gpar[c];
-            const bool closed = mode == CLOSE_ALL || (mode == CLOSE_WM && w.rlast[r] <= mark);
-            return (w.rslot[r].min - off) | (closed ? CLOSED : 0u);
-        };
-        const uint32_t n0 = t > g.tile0 ? w.atile[t - 1].nroots : 0, n1 = w.atile[t].nroots;
-        const uint32_t n2 = t + 1 < g.tile0 + g.ntiles ? w.atile[t + 1].nroots : 0;
-        const bool table = n0 + n1 + n2 <= AL_CAP;
-        // c in [c0, c0 + n0), [c1, c1 + n1), [c2, c2 + n2): s_lab[c - c0], s_lab[n0 + c - c1], ...
-        const uint32_t c1 = t * TILE, c0 = c1 - TILE, c2 = c1 + TILE;
-        if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
-        if (table)
-            for (uint32_t i = threadIdx.x; i < n0 + n1 + n2; i += blockDim.x)
-                s_lab[i] = label_of(i < n0 ? c0 + i : i < n0 + n1 ? c1 + i - n0 : c2 + i - n0 - n1);
-        __syncthreads();
-        const bool direct = g.ss == nullptr;   // one-shot: every hit is final
-        uint32_t c_label = 0, c_closed = 0;
-        constexpr int ITEMS = TILE / 256;
-#pragma unroll 8
-        for (int q = 0; q < ITEMS; ++q) {
-            const uint32_t pos = begin + q * 256 + threadIdx.x;
-            bool is_label = false, closed = false;
-            if (pos < end) {
-                const uint32_t c = w.root_of[pos];
-                uint32_t v;
-                if (table && c - c1 < n1) v = s_lab[n0 + c - c1];
-                else if (table && c - c0 < n0) v = s_lab[c - c0];
-                else if (table && c - c2 < n2) v = s_lab[n0 + n1 + c - c2];
-                else v = label_of(c);
-                const uint32_t l = v & ~CLOSED;
-                closed = (v & CLOSED) != 0;
-                is_label = closed && l == pos - off;
-                const uint64_t lab = gidx_of(g, l);
-                if (direct) g.out_labels[pos - off] = lab;
-                else w.lab_tmp[pos] = lab;
-            }
-            const uint32_t bl = __ballot_sync(0xffffffffu, is_label);
-            const uint32_t bc = __ballot_sync(0xffffffffu, closed);
-            if (lane == 0) {
-                w.flag_label[pos >> 5] = bl;
-                w.flag_closed[pos >> 5] = bc;
-                c_label += __popc(bl);
-                c_closed += __popc(bc);
-            }
-        }
-        if (lane == 0) {
-            atomicAdd(&s_cnt[0], c_label);
-            atomicAdd(&s_cnt[1], c_closed);
-        }
-        __syncthreads();
-        if (threadIdx.x < 2) w.tile_cnt[threadIdx.x * P.tile_cap + t] = s_cnt[threadIdx.x];
-        __syncthreads();
-    }
+    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) label_tile<256>(w, t, w.seg[w.tile_seg[t]], s_lab, s_cnt);
 }
 
 // Records in label order (and, streaming, the finalised hits and the carry).
@@ -1196,7 +1172,64 @@ __device__ void emit_totals(Seg &g, Prob &P, uint32_t n_clusters, uint32_t n_fin
     if (g.close_mode == CLOSE_WM) ss.watermark = g.watermark;
 }
 
-__global__ void __launch_bounds__(AE) k_arrival_emit(Work w, uint64_t *counts, uint32_t keep) {
+// One tile's records, from record `rec` of its segment; streaming: its
+// finalised hits from `fin` and its open ones, open_total in the segment.
+template <int NT>
+__device__ __forceinline__ void emit_tile(const Work &w, uint32_t t, const Seg &g, uint32_t begin, uint32_t end,
+                                          uint32_t rec, uint32_t n_rec, uint32_t fin, uint32_t open_total,
+                                          uint32_t *s_red, uint16_t *s_pos) {
+    const uint32_t nwords = (end - begin + 31) >> 5;
+    uint32_t bits = threadIdx.x < nwords ? w.flag_label[(begin >> 5) + threadIdx.x] : 0;
+    uint32_t k = emit_prefix(bits, s_red);
+    while (bits) {
+        const int b = __ffs(bits) - 1;
+        bits &= bits - 1;
+        s_pos[k++] = (uint16_t)((threadIdx.x << 5) + b);
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < n_rec; i += NT) {
+        if (rec + i >= g.out_cap) break;
+        const uint32_t pos = begin + s_pos[i];
+        const uint32_t r = w.gpar[w.root_of[pos]];
+        const RootSlot s = w.rslot[r];
+        tpc_cluster out;
+        out.label = gidx_of(g, pos - g.off);
+        out.size = (int64_t)s.size;
+        out.sum_tot = (int64_t)s.tot;
+        out.first_toa = w.rfirst[r];
+        // fp32 quotient of the exact integer sums: three roundings, each
+        // at most 2^-24 relative (FP64 is a slow pipe on this GPU)
+        const float sw = (float)s.tot;
+        out.cx = (float)s.wx / sw;
+        out.cy = (float)s.wy / sw;
+        g.out_rec[rec + i] = out;
+    }
+    if (g.ss) {
+        const bool fits = open_total <= g.carry_cap;
+        const bool vw = threadIdx.x < nwords;
+        const uint32_t cl = vw ? w.flag_closed[(begin >> 5) + threadIdx.x] : 0;
+        uint32_t closed = fin + emit_prefix(cl, s_red);
+        if (vw) {
+            const uint32_t first = begin + (threadIdx.x << 5), last = min(first + 32, end);
+            for (uint32_t pos = first; pos < last; ++pos) {
+                const uint32_t local = pos - g.off;
+                if ((cl >> (pos - first)) & 1u) {
+                    if (closed < g.out_cap) {
+                        g.out_labels[closed] = w.lab_tmp[pos];
+                        if (g.out_index) g.out_index[closed] = gidx_of(g, local);
+                    }
+                    ++closed;
+                } else if (fits) {
+                    const uint32_t dst = g.carry_cap - open_total + (local - closed);
+                    g.carry_out[dst] = g.hits[local];
+                    g.carry_gidx_out[dst] = gidx_of(g, local);
+                }
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(AE) k_arrival_emit(Work w) {
     __shared__ uint32_t s_red[AE / 32];
     __shared__ uint16_t s_pos[TILE];
     __shared__ bool s_last;
@@ -1223,56 +1256,8 @@ __global__ void __launch_bounds__(AE) k_arrival_emit(Work w, uint64_t *counts, u
             fin = emit_sum(cnt + cap + g.tile0, t - g.tile0, s_red);
             if (g.ss) open_total = g.n - emit_sum(cnt + cap + g.tile0, g.ntiles, s_red);
         }
-        const uint32_t nwords = (end - begin + 31) >> 5;
-        uint32_t bits = threadIdx.x < nwords ? w.flag_label[(begin >> 5) + threadIdx.x] : 0;
-        uint32_t k = emit_prefix(bits, s_red);
-        while (bits) {
-            const int b = __ffs(bits) - 1;
-            bits &= bits - 1;
-            s_pos[k++] = (uint16_t)((threadIdx.x << 5) + b);
-        }
-        __syncthreads();
         const uint32_t n_rec = cnt[t];
-        for (uint32_t i = threadIdx.x; i < n_rec; i += AE) {
-            if (rec + i >= g.out_cap) break;
-            const uint32_t pos = begin + s_pos[i];
-            const uint32_t r = w.gpar[w.root_of[pos]];
-            const RootSlot s = w.rslot[r];
-            tpc_cluster out;
-            out.label = gidx_of(g, pos - g.off);
-            out.size = (int64_t)s.size;
-            out.sum_tot = (int64_t)s.tot;
-            out.first_toa = w.rfirst[r];
-            // fp32 quotient of the exact integer sums: three roundings, each
-            // at most 2^-24 relative (FP64 is a slow pipe on this GPU)
-            const float sw = (float)s.tot;
-            out.cx = (float)s.wx / sw;
-            out.cy = (float)s.wy / sw;
-            g.out_rec[rec + i] = out;
-        }
-        if (g.ss) {
-            const bool fits = open_total <= g.carry_cap;
-            const bool vw = threadIdx.x < nwords;
-            const uint32_t cl = vw ? w.flag_closed[(begin >> 5) + threadIdx.x] : 0;
-            uint32_t closed = fin + emit_prefix(cl, s_red);
-            if (vw) {
-                const uint32_t first = begin + (threadIdx.x << 5), last = min(first + 32, end);
-                for (uint32_t pos = first; pos < last; ++pos) {
-                    const uint32_t local = pos - g.off;
-                    if ((cl >> (pos - first)) & 1u) {
-                        if (closed < g.out_cap) {
-                            g.out_labels[closed] = w.lab_tmp[pos];
-                            if (g.out_index) g.out_index[closed] = gidx_of(g, local);
-                        }
-                        ++closed;
-                    } else if (fits) {
-                        const uint32_t dst = g.carry_cap - open_total + (local - closed);
-                        g.carry_out[dst] = g.hits[local];
-                        g.carry_gidx_out[dst] = gidx_of(g, local);
-                    }
-                }
-            }
-        }
+        emit_tile<AE>(w, t, g, begin, end, rec, n_rec, fin, open_total, s_red, s_pos);
         rec += n_rec;
         fin += cnt[cap + t];
         if (t + 1 == g.tile0 + g.ntiles && threadIdx.x == 0) emit_totals(w.seg[si], P, rec, fin);
@@ -1287,49 +1272,138 @@ __global__ void __launch_bounds__(AE) k_arrival_emit(Work w, uint64_t *counts, u
     __syncthreads();
     if (!s_last) return;
     for (uint32_t s = threadIdx.x; s < P.nsegs; s += AE) write_info(w.seg[s], P);
-    if (counts && threadIdx.x == 0) {   // tpc_cluster_static's result words
-        counts[0] = *const_cast<volatile uint32_t *>(&w.seg[0].n_clusters);
-        counts[1] = *const_cast<volatile uint32_t *>(&P.err) & keep;
+}
+
+// A whole small step in one launch: a cluster of SMALL_TILES CTAs or fewer,
+// CTA t for tile t, with cluster barriers between the stages.  `seg`: the
+// step's segment for callers that queue no copy of it (tpc_cluster_static);
+// otherwise it is in w.seg.
+__global__ void __launch_bounds__(AT, 1) k_arrival_step(Work w, Seg seg, uint32_t given, uint32_t tile_cap, uint64_t *counts,
+                                                     uint32_t keep) {
+    extern __shared__ __align__(16) unsigned char a_raw[];
+    SmallShared &S = *reinterpret_cast<SmallShared *>(a_raw);
+    __shared__ uint32_t s_red[AW];
+    __shared__ uint32_t s_cnt[2];
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const uint32_t t = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    Prob &P = *w.prob;
+    Seg &g = w.seg[0];
+    if (t == 0 && tid == 0) {
+        if (given) {
+            g = seg;
+            P.tile_cap = tile_cap;
+            P.pos_cap = tile_cap * TILE;
+        }
+        uint32_t off = 0, tile = 0;
+        setup_seg(g, off, tile);
+        setup_prob(P, 1, tile, off, 1u);
+    }
+    cluster.sync();
+    const uint32_t nt = *const_cast<volatile uint32_t *>(&P.ntiles);
+    const bool mine = t < nt;
+    if (mine) {
+        if (tid == 0) w.tile_seg[t] = 0;
+        small_tile<false>(w, t, S);
+    }
+    cluster.sync();
+    if (mine) {
+        if (warp == 0) {   // complete if every hit before h0 is earlier than the tile's first by more than dt
+            const ATile &info = w.atile[t];
+            const uint32_t hc = info.h0 / A_STEP;   // chunks not looked at
+            uint64_t m = 0;
+            for (uint32_t i = lane; i < hc; i += 32) {
+                const uint64_t c = w.atile[i / ACHUNKS].cmax[i % ACHUNKS];
+                m = c > m ? c : m;
+            }
+            m = warp_max_u64(m);
+            if (lane == 0 && ((hc && m >= info.lo) || info.nx > A_PAIRS)) w.atile[t].redo = 1u;
+        }
+        join_pairs<AT>(w, t);
+    }
+    if (t == 0 && tid == 0) seg_close(g, P);
+    cluster.sync();
+    bool redo = false;
+    for (uint32_t i = 0; i < nt; ++i) redo |= *const_cast<volatile uint32_t *>(&w.atile[i].redo) != 0;
+    if (redo) {
+        if (mine && *const_cast<volatile uint32_t *>(&w.atile[t].redo)) small_tile<true>(w, t, S);
+        cluster.sync();
+    }
+    if (mine) root_tile<AT>(w, t, g.ss != nullptr);
+    cluster.sync();
+    if (mine) label_tile<AT>(w, t, g, reinterpret_cast<uint32_t *>(a_raw), s_cnt);
+    cluster.sync();
+    const uint32_t *cnt = w.tile_cnt, cap = P.tile_cap;
+    if (mine) {
+        uint32_t rec = 0, fin = 0, all = 0;   // of the tiles before, and (finalised) of all
+        for (uint32_t i = 0; i < nt; ++i) {
+            const uint32_t f = cnt[cap + i];
+            if (i < t) { rec += cnt[i]; fin += f; }
+            all += f;
+        }
+        uint32_t begin, end;
+        tile_range(g, t, begin, end);
+        emit_tile<AT>(w, t, g, begin, end, rec, cnt[t], fin, g.n - all, s_red, reinterpret_cast<uint16_t *>(a_raw));
+        if (t + 1 == nt && tid == 0) emit_totals(g, P, rec + cnt[t], all);
+    } else if (nt == 0 && t == 0 && tid == 0) {
+        emit_totals(g, P, 0, 0);
+    }
+    if (tid == 0 && (nt ? t + 1 == nt : t == 0)) {
+        write_info(g, P);
+        if (counts) {   // tpc_cluster_static's result words
+            counts[0] = g.n_clusters;
+            counts[1] = P.err & keep;
+        }
     }
 }
 
 cudaError_t init_arrival_attributes() {
     cudaError_t e = cudaFuncSetAttribute(k_arrival_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_arrival_small, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMALL_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_arrival_redo, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMALL_SMEM);
+        e = cudaFuncSetAttribute(k_arrival_step, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMALL_SMEM);
+    if (e == cudaSuccess)   // clusters of 16 (a GPC of this GPU has 16 SMs and more)
+        e = cudaFuncSetAttribute(k_arrival_step, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
 }
 
-// A small step has at most SMALL_TILES tiles.
-static int grid_of(int fit, bool small) { return small && fit > (int)SMALL_TILES ? (int)SMALL_TILES : fit; }
-
 // Links and the decision; `sorted` (0: none) is the conditional node that
 // holds the time-sorted path.
-void launch_arrival_link(const Work &w, bool small, cudaGraphConditionalHandle sorted, const Launch &L) {
-    if (small) {
-        k_arrival_small<<<SMALL_TILES, AT, A_SMALL_SMEM, L.stream>>>(w);
-        L.mark("k_arrival_small");
-    } else {
-        k_arrival_tile<<<L.fit(k_arrival_tile, AT, A_SMEM, G_LINK), AT, A_SMEM, L.stream>>>(w);
-        L.mark("k_arrival_tile");
-    }
-    k_arrival_cross<<<grid_of(L.fit(k_arrival_cross, AX, 0, G_LINK), small), AX, 0, L.stream>>>(w, small, sorted);
+void launch_arrival_link(const Work &w, cudaGraphConditionalHandle sorted, const Launch &L) {
+    k_arrival_tile<<<L.fit(k_arrival_tile, AT, A_SMEM, G_LINK), AT, A_SMEM, L.stream>>>(w);
+    L.mark("k_arrival_tile");
+    k_arrival_cross<<<L.fit(k_arrival_cross, AX, 0, G_LINK), AX, 0, L.stream>>>(w, sorted);
     L.mark("k_arrival_cross");
-    if (small) {
-        k_arrival_redo<<<SMALL_TILES, AT, A_SMALL_SMEM, L.stream>>>(w);
-        L.mark("k_arrival_redo");
-    }
 }
 
-void launch_arrival_output(const Work &w, bool small, uint64_t *counts, uint32_t keep, const Launch &L) {
-    k_arrival_roots<<<grid_of(L.fit(k_arrival_roots, 256, 0, G_ACC), small), 256, 0, L.stream>>>(w);
+void launch_arrival_output(const Work &w, const Launch &L) {
+    k_arrival_roots<<<L.fit(k_arrival_roots, 256, 0, G_ACC), 256, 0, L.stream>>>(w);
     L.mark("k_arrival_roots");
-    k_arrival_labels<<<grid_of(L.fit(k_arrival_labels, 256, 0, G_OUT), small), 256, 0, L.stream>>>(w);
+    k_arrival_labels<<<L.fit(k_arrival_labels, 256, 0, G_OUT), 256, 0, L.stream>>>(w);
     L.mark("k_arrival_labels");
-    k_arrival_emit<<<grid_of(L.fit(k_arrival_emit, AE, 0, G_OUT), small), AE, 0, L.stream>>>(w, counts, keep);
+    k_arrival_emit<<<L.fit(k_arrival_emit, AE, 0, G_OUT), AE, 0, L.stream>>>(w);
     L.mark("k_arrival_emit");
+}
+
+// A small step of at most `tiles` tiles; seg: its segment, or null if w.seg
+// holds it already.
+cudaError_t launch_arrival_step(const Work &w, const Seg *seg, uint32_t tiles, uint32_t tile_cap, uint64_t *counts,
+                                uint32_t keep, const Launch &L) {
+    uint32_t ctas = 1;
+    while (ctas < tiles) ctas *= 2;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(AT);
+    cfg.dynamicSmemBytes = A_SMALL_SMEM;
+    cfg.stream = L.stream;
+    cudaLaunchAttribute a{};
+    a.id = cudaLaunchAttributeClusterDimension;
+    a.val.clusterDim.x = ctas;
+    a.val.clusterDim.y = a.val.clusterDim.z = 1;
+    cfg.attrs = &a;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_arrival_step, w, seg ? *seg : Seg{}, seg ? 1u : 0u, tile_cap, counts, keep);
+    L.mark("k_arrival_step");
+    return e;
 }
 
 }  // namespace tpc

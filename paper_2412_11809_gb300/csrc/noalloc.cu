@@ -9,8 +9,8 @@
 // working memory comes from the fixed array below, which every GPU that
 // loads the library holds until the process exits.
 //
-// The kernels are the library's own (those of a small tpc_flush); only the
-// source of their scratch differs.  Every call shares
+// The kernel is the library's own (that of a small tpc_flush); only the
+// source of its scratch differs.  Every call shares
 // the one array and leaves its last contents behind: nothing in it has to
 // start at zero, because each call first rewrites the segment and problem
 // descriptors and every other array is fully written before it is read.
@@ -86,14 +86,6 @@ int na_setup(int dev, unsigned char **base, int *sms) {
     return TPC_OK;
 }
 
-__global__ void k_na_begin(Work w, Seg s, uint32_t tile_cap, uint32_t pos_cap) {
-    w.seg[0] = s;
-    Prob p{};
-    p.tile_cap = tile_cap;
-    p.pos_cap = pos_cap;
-    *w.prob = p;
-}
-
 __global__ void k_na_empty(uint64_t *counts) {
     counts[0] = 0;
     counts[1] = 0;
@@ -153,15 +145,12 @@ extern "C" int tpc_cluster_static(const tpc_hit *hits, size_t n, uint32_t width,
     s.variant = TPC_LOCAL;
 
     const Launch L{sms * 4, st, nullptr, sms};
-    k_na_begin<<<1, 1, 0, st>>>(w, s, NA_TILES, NA_POS);
     // counts[1] keeps the public bits only; with no record buffer
     // (record_cap == 0) the caller asked for labels alone, so more clusters
     // than records is not an error then
     static_assert(E_RANGE == TPC_STATIC_E_RANGE && E_SPAN == TPC_STATIC_E_SPAN && E_CAP == TPC_STATIC_E_CAP,
                   "public error bits");
     const uint32_t keep = TPC_STATIC_E_RANGE | TPC_STATIC_E_SPAN | (record_cap ? TPC_STATIC_E_CAP : 0u);
-    launch_setup(w, 1, L, true);
-    launch_arrival_link(w, true, 0, L);
-    launch_arrival_output(w, true, counts, keep, L);
-    return cudaGetLastError() == cudaSuccess ? TPC_OK : TPC_ERR_CUDA;
+    return launch_arrival_step(w, &s, (uint32_t)((n + TILE - 1) / TILE), NA_TILES, counts, keep, L) == cudaSuccess
+               ? TPC_OK : TPC_ERR_CUDA;
 }

@@ -15,52 +15,11 @@ __global__ void k_setup(Work w, int nsegs, uint32_t arrival) {
         uint32_t off = 0, tile = 0;
         for (int s = 0; s < nsegs; ++s) {
             Seg &g = w.seg[s];
-            if (g.ss) {
-                g.n_carry = g.ss->n_carry;
-                g.hits = g.carry_in + (g.carry_cap - g.n_carry);
-                g.carry_gidx = g.carry_gidx_in + (g.carry_cap - g.n_carry);
-            } else {
-                g.n_carry = 0;
-                g.carry_gidx = nullptr;
-            }
-            g.n = g.n_carry + g.n_new;
-            const uint64_t t0 = g.n ? hit_toa(ld_hit(g.hits)) : 0;
-            g.fast_base = fast_key_base(t0);
-            g.raw_base = t0 > ARRIVAL_BACK ? t0 - ARRIVAL_BACK : 0;
-            g.n_owned = 0;
-            g.off = off;
-            g.tile0 = tile;
-            g.ntiles = (g.n + TILE - 1) / TILE;
-            off += g.ntiles * TILE;
-            tile += g.ntiles;
-            g.toa_min = ~0ull;
-            g.toa_max = 0;
-            g.chunk_min = ~0ull;
-            g.npasses = 0;
-            g.watermark = 0;
-            g.close_mode = CLOSE_NONE;
-            g.seen_after = 0;
-            g.n_final = g.n_clusters = g.n_open = 0;
+            setup_seg(g, off, tile);
             s_tile0[s] = g.tile0;
         }
         s_tile0[nsegs] = tile;
-        Prob &p = *w.prob;
-        p.nsegs = (uint32_t)nsegs;
-        p.npasses = 0;
-        p.fallback = 0;
-        p.lsd_passes = 0;
-        p.redo_count = 0;
-        p.border_count = 0;
-        p.merge_count = 0;
-        p.emitted = 0;
-        p.raw = arrival;
-        p.raw_fail = 0;
-        p.err = 0;
-        p.ntiles = tile;
-        if (tile > p.tile_cap || off > p.pos_cap) {
-            p.err |= E_CAP;
-            p.ntiles = 0;
-        }
+        setup_prob(*w.prob, (uint32_t)nsegs, tile, off, arrival);
     }
     __syncthreads();
     const uint32_t nt = w.prob->ntiles;

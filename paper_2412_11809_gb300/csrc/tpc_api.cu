@@ -480,51 +480,49 @@ void enqueue_sorted(const Work &w, const Launch &L) {
 // in a conditional node that its cross kernel switches on, the time-sorted
 // path for the steps it cannot cover.
 cudaError_t capture_step(const Work &w, int nsegs, StepMode mode, const Launch &L) {
+    if (mode == STEP_SMALL) return launch_arrival_step(w, nullptr, SMALL_TILES, 0, nullptr, 0, L);
     launch_setup(w, nsegs, L, mode != STEP_SORTED);
     if (mode == STEP_SORTED) {
         enqueue_sorted(w, L);
         return cudaGetLastError();
     }
-    const bool small = mode == STEP_SMALL;
     cudaGraphConditionalHandle cond = 0;
     cudaStreamCaptureStatus status;
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamGetCaptureInfo(L.stream, &status, nullptr, &graph, nullptr, nullptr, nullptr);
-    if (e == cudaSuccess && !small) e = cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault);
+    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault);
     if (e != cudaSuccess) return e;
-    launch_arrival_link(w, small, cond, L);
-    if (!small) {
-        const cudaGraphNode_t *deps = nullptr;
-        const cudaGraphEdgeData *edges = nullptr;
-        size_t ndeps = 0;
-        e = cudaStreamGetCaptureInfo(L.stream, &status, nullptr, &graph, &deps, &edges, &ndeps);
-        if (e != cudaSuccess) return e;
-        cudaGraphNodeParams p{};
-        p.type = cudaGraphNodeTypeConditional;
-        p.conditional.handle = cond;
-        p.conditional.type = cudaGraphCondTypeIf;
-        p.conditional.size = 1;
-        cudaGraphNode_t node = nullptr;
-        e = cudaGraphAddNode(&node, graph, deps, edges, ndeps, &p);
-        if (e != cudaSuccess) return e;
-        cudaStream_t body;
-        e = cudaStreamCreateWithFlags(&body, cudaStreamNonBlocking);
-        if (e != cudaSuccess) return e;
-        e = cudaStreamBeginCaptureToGraph(body, p.conditional.phGraph_out[0], nullptr, nullptr, 0,
-                                          cudaStreamCaptureModeThreadLocal);
-        if (e == cudaSuccess) {
-            Launch B = L;
-            B.stream = body;
-            enqueue_sorted(w, B);
-            cudaGraph_t same = nullptr;
-            e = cudaStreamEndCapture(body, &same);
-        }
-        cudaStreamDestroy(body);
-        if (e != cudaSuccess) return e;
-        e = cudaStreamUpdateCaptureDependencies(L.stream, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
-        if (e != cudaSuccess) return e;
+    launch_arrival_link(w, cond, L);
+    const cudaGraphNode_t *deps = nullptr;
+    const cudaGraphEdgeData *edges = nullptr;
+    size_t ndeps = 0;
+    e = cudaStreamGetCaptureInfo(L.stream, &status, nullptr, &graph, &deps, &edges, &ndeps);
+    if (e != cudaSuccess) return e;
+    cudaGraphNodeParams p{};
+    p.type = cudaGraphNodeTypeConditional;
+    p.conditional.handle = cond;
+    p.conditional.type = cudaGraphCondTypeIf;
+    p.conditional.size = 1;
+    cudaGraphNode_t node = nullptr;
+    e = cudaGraphAddNode(&node, graph, deps, edges, ndeps, &p);
+    if (e != cudaSuccess) return e;
+    cudaStream_t body;
+    e = cudaStreamCreateWithFlags(&body, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = cudaStreamBeginCaptureToGraph(body, p.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                      cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        Launch B = L;
+        B.stream = body;
+        enqueue_sorted(w, B);
+        cudaGraph_t same = nullptr;
+        e = cudaStreamEndCapture(body, &same);
     }
-    launch_arrival_output(w, small, nullptr, 0, L);
+    cudaStreamDestroy(body);
+    if (e != cudaSuccess) return e;
+    e = cudaStreamUpdateCaptureDependencies(L.stream, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
+    if (e != cudaSuccess) return e;
+    launch_arrival_output(w, L);
     return cudaGetLastError();
 }
 
@@ -538,16 +536,17 @@ cudaError_t run_step(tpc_ctx *owner, Workspace &ws, int nsegs, StepMode mode, cu
         cudaEventRecord(tr->ev[0], st);
         Launch T = L;
         T.tr = tr;
+        if (mode == STEP_SMALL) return capture_step(ws.w, nsegs, mode, T);   // (one launch)
         launch_setup(ws.w, nsegs, T, mode != STEP_SORTED);
         uint32_t sorted = mode == STEP_SORTED;
         if (!sorted) {
-            launch_arrival_link(ws.w, mode == STEP_SMALL, 0, T);
+            launch_arrival_link(ws.w, 0, T);
             cudaError_t e = cudaMemcpyAsync(&sorted, &ws.w.prob->raw_fail, sizeof(sorted), cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
             if (e != cudaSuccess) return e;
         }
         if (sorted) enqueue_sorted(ws.w, T);
-        else launch_arrival_output(ws.w, mode == STEP_SMALL, nullptr, 0, T);
+        else launch_arrival_output(ws.w, T);
         return cudaGetLastError();
     }
     if (!owner->graph || owner->graph_nsegs != nsegs || owner->graph_mode != mode || owner->graph_gen != ws.gen ||

@@ -344,6 +344,58 @@ __device__ __forceinline__ uint64_t fast_key_base(uint64_t t0) {
     return t0 > (1ull << 31) ? t0 - (1ull << 31) : 0;
 }
 
+// A segment at position `off`, tile `tile` (both moved on), with its per-step
+// state reset.  A streaming one picks up the carry left by the previous step:
+// it sits right-aligned in the carry region of its input buffer, immediately
+// followed by the new chunk.
+__device__ __forceinline__ void setup_seg(Seg &g, uint32_t &off, uint32_t &tile) {
+    if (g.ss) {
+        g.n_carry = g.ss->n_carry;
+        g.hits = g.carry_in + (g.carry_cap - g.n_carry);
+        g.carry_gidx = g.carry_gidx_in + (g.carry_cap - g.n_carry);
+    } else {
+        g.n_carry = 0;
+        g.carry_gidx = nullptr;
+    }
+    g.n = g.n_carry + g.n_new;
+    const uint64_t t0 = g.n ? hit_toa(ld_hit(g.hits)) : 0;
+    g.fast_base = fast_key_base(t0);
+    g.raw_base = t0 > ARRIVAL_BACK ? t0 - ARRIVAL_BACK : 0;
+    g.n_owned = 0;
+    g.off = off;
+    g.tile0 = tile;
+    g.ntiles = (g.n + TILE - 1) / TILE;
+    off += g.ntiles * TILE;
+    tile += g.ntiles;
+    g.toa_min = ~0ull;
+    g.toa_max = 0;
+    g.chunk_min = ~0ull;
+    g.npasses = 0;
+    g.watermark = 0;
+    g.close_mode = CLOSE_NONE;
+    g.seen_after = 0;
+    g.n_final = g.n_clusters = g.n_open = 0;
+}
+
+__device__ __forceinline__ void setup_prob(Prob &p, uint32_t nsegs, uint32_t tiles, uint32_t positions, uint32_t arrival) {
+    p.nsegs = nsegs;
+    p.npasses = 0;
+    p.fallback = 0;
+    p.lsd_passes = 0;
+    p.redo_count = 0;
+    p.border_count = 0;
+    p.merge_count = 0;
+    p.emitted = 0;
+    p.raw = arrival;
+    p.raw_fail = 0;
+    p.err = 0;
+    p.ntiles = tiles;
+    if (tiles > p.tile_cap || positions > p.pos_cap) {
+        p.err |= E_CAP;
+        p.ntiles = 0;
+    }
+}
+
 // Once a segment's ToA extremes are known: its ToA span check and, streaming,
 // the watermark.  A later hit j satisfies toa_j > seen_max - max_disorder (the
 // t-ordered property, Section 3.1), and can join hit i only if
@@ -461,8 +513,10 @@ cudaError_t init_kernel_attributes();   // once per process and device, before c
 cudaError_t init_variants_attributes();
 void launch_setup(const Work &w, int nsegs, const Launch &L, bool arrival = false);
 cudaError_t init_arrival_attributes();
-void launch_arrival_link(const Work &w, bool small, cudaGraphConditionalHandle sorted, const Launch &L);
-void launch_arrival_output(const Work &w, bool small, uint64_t *counts, uint32_t keep, const Launch &L);
+void launch_arrival_link(const Work &w, cudaGraphConditionalHandle sorted, const Launch &L);
+void launch_arrival_output(const Work &w, const Launch &L);
+cudaError_t launch_arrival_step(const Work &w, const Seg *seg, uint32_t tiles, uint32_t tile_cap, uint64_t *counts,
+                                uint32_t keep, const Launch &L);
 void launch_seg_finalize(const Work &w, const Launch &L);
 void launch_make_keys(const Work &w, const Launch &L);
 void launch_sort_fast(const Work &w, const Launch &L);
