@@ -59,7 +59,7 @@ HIT_DTYPE_NP = np.dtype([("x", "<u2"), ("y", "<u2"), ("tot", "<u2"), ("reserved"
 # record bytes are charged per cluster.  Used for the dominant kernel's roofline.
 KERNEL_BYTES_PER_HIT = {
     # arrival order: read the record; write the hit's tile cluster and its key
-    "k_arrival_tile": 16 + 8, "k_arrival_small": 16 + 8,
+    "k_arrival_tile": 16 + 8, "k_arrival_step": 16 + 8,
     # read the tile cluster, write the label
     "k_arrival_labels": 4 + 8,
     # the time-sorted path (steps the arrival-order path cannot cover):

@@ -782,7 +782,7 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
 // ---------------------------------------------------------------------------
 // Small steps: tiles own their positions, whatever the order.
 
-// One tile.  DIRECT (k_arrival_redo): pairs are joined at once in the global
+// One tile.  DIRECT (k_arrival_step): pairs are joined at once in the global
 // forest, every earlier position is looked at, nothing else is written.
 template <bool DIRECT>
 __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShared &SS) {

@@ -42,8 +42,48 @@ constexpr int acc_smem() {
 // shared-memory counter (size << 32 | sum ToT: a span holds at most ACC_SPAN
 // hits of ToT < 2^16, so neither part overflows), and the last key is kept
 // only when a streaming watermark needs it.
-template <int ACC_SPAN>
-__global__ void __launch_bounds__(ACC_THREADS, ACC_SPAN >= 2048 ? 2 : 4) k_accumulate(Work w) {
+//
+// LARGE (variant (b), where one cluster can hold most hits): the sums of the
+// far cluster that a warp last saw more than half its lanes in stay in the
+// warp's own shared-memory slot, and reach the global slot when another takes
+// over or the CTA ends.  Adding them hit group by hit group, all warps queue on
+// one address: 808 us for 8 M hits, 205 with the slot.
+struct WarpSum {
+    uint32_t root;   // NONE: empty
+    uint32_t size, min, max;
+    unsigned long long tot, wx, wy;
+    static constexpr uint32_t NONE = 0xFFFFFFFFu;
+
+    __device__ __forceinline__ void add(uint32_t c, uint32_t t, unsigned long long x, unsigned long long y, uint32_t mn,
+                                        uint32_t mx) {
+        size += c;
+        tot += t;
+        wx += x;
+        wy += y;
+        min = mn < min ? mn : min;
+        max = mx > max ? mx : max;
+    }
+    __device__ __forceinline__ void flush(Slot *slot) const {
+        if (root == NONE || !size) return;
+        Slot &sl = slot[root];
+        atomicAdd(&sl.size, size);
+        atomicAdd(&sl.tot, tot);
+        atomicAdd(&sl.wx, wx);
+        atomicAdd(&sl.wy, wy);
+        atomicMin(&sl.min, min);
+        atomicMax(&sl.maxkey, max);
+    }
+    __device__ __forceinline__ void start(uint32_t r) {
+        root = r;
+        size = 0;
+        tot = wx = wy = 0;
+        min = 0xFFFFFFFFu;
+        max = 0;
+    }
+};
+
+template <int ACC_SPAN, bool LARGE>
+__global__ void __launch_bounds__(ACC_THREADS, ACC_SPAN >= 2048 || LARGE ? 2 : 4) k_accumulate(Work w) {
     constexpr int ACC_ITEMS = ACC_SPAN / ACC_THREADS;
     extern __shared__ __align__(16) unsigned char acc_raw[];
     unsigned long long *a_wx = reinterpret_cast<unsigned long long *>(acc_raw);
@@ -55,6 +95,10 @@ __global__ void __launch_bounds__(ACC_THREADS, ACC_SPAN >= 2048 ? 2 : 4) k_accum
     const uint32_t *skey = pick(w.keys, sorted_sel(P));
     const uint32_t *sidx = pick(w.vals, sorted_sel(P));
     const int lane = threadIdx.x & 31;
+    __shared__ WarpSum s_far[LARGE ? ACC_THREADS / 32 : 1];
+    WarpSum &far = s_far[LARGE ? threadIdx.x >> 5 : 0];
+    if (LARGE && lane == 0) far.start(WarpSum::NONE);
+    if (LARGE) __syncwarp();
     for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
         const Seg &g = w.seg[w.tile_seg[t]];
         uint32_t begin, end;
@@ -106,13 +150,24 @@ __global__ void __launch_bounds__(ACC_THREADS, ACC_SPAN >= 2048 ? 2 : 4) k_accum
                 const uint32_t r = rr[q], pix = px[q], tot = tt[q];
                 const uint32_t peers = __match_any_sync(vmask, r);
                 const uint32_t cnt = __popc(peers);
+                uint32_t far_root = WarpSum::NONE;
+                if (LARGE) {
+                    __syncwarp(vmask);   // the sums of the items before
+                    if (r < b && cnt > 16u && lane == __ffs(peers) - 1 && far.root != r) {   // (one lane at most)
+                        far.flush(w.slot);
+                        far.start(r);
+                    }
+                    __syncwarp(vmask);
+                    far_root = far.root;
+                    __syncwarp(vmask);
+                }
                 uint32_t sum_tot = tot, mn = ps[q], mx = kk[q];
                 unsigned long long wx = (unsigned long long)tot * (pix & 0xFFFFu);
                 unsigned long long wy = (unsigned long long)tot * (pix >> 16);
                 // combine this cluster's hits of the warp when there are
                 // enough of them to contend; smaller groups add their hits
                 // one by one (a group reduction runs once per distinct group)
-                const bool agg = cnt >= 3u;
+                const bool agg = cnt >= 3u || (LARGE && r == far_root);
                 uint32_t c = 1;
                 if (agg) {
                     const uint32_t wx32 = tot * (pix & 0xFFFFu), wy32 = tot * (pix >> 16);
@@ -133,6 +188,8 @@ __global__ void __launch_bounds__(ACC_THREADS, ACC_SPAN >= 2048 ? 2 : 4) k_accum
                     atomicAdd(&a_wy[k], wy);
                     atomicMin(&a_min[k], mn);
                     if (want_max) atomicMax(&a_max[k], mx);
+                } else if (LARGE && r == far_root) {   // (one lane: the group's first)
+                    far.add(c, sum_tot, wx, wy, mn, mx);
                 } else {
                     Slot &sl = w.slot[r];
                     atomicAdd(&sl.size, c);
@@ -165,6 +222,23 @@ __global__ void __launch_bounds__(ACC_THREADS, ACC_SPAN >= 2048 ? 2 : 4) k_accum
             // touches slot k until after that barrier
         }
     }
+    if (!LARGE) return;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int q = 1; q < ACC_THREADS / 32; ++q) {   // mostly one cluster in all warps
+        const WarpSum &o = s_far[LARGE ? q : 0];
+        if (o.root == far.root) {
+            far.size += o.size;
+            far.tot += o.tot;
+            far.wx += o.wx;
+            far.wy += o.wy;
+            far.min = min(far.min, o.min);
+            far.max = max(far.max, o.max);
+        } else {
+            o.flush(w.slot);
+        }
+    }
+    far.flush(w.slot);
 }
 
 __device__ __forceinline__ bool cluster_closed(const Seg &g, uint32_t maxkey) {
@@ -395,24 +469,30 @@ __global__ void k_stream_end(Work w) {
     }
 }
 
+template <int SPAN, bool LARGE>
+static cudaError_t accumulate_attributes() {
+    return cudaFuncSetAttribute(k_accumulate<SPAN, LARGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, acc_smem<SPAN>());
+}
+
 cudaError_t init_features_attributes() {
-    cudaError_t e = cudaFuncSetAttribute(k_accumulate<512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         acc_smem<512>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_accumulate<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, acc_smem<1024>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_accumulate<2048>, cudaFuncAttributeMaxDynamicSharedMemorySize, acc_smem<2048>());
+    cudaError_t e = accumulate_attributes<512, false>();
+    if (e == cudaSuccess) e = accumulate_attributes<1024, false>();
+    if (e == cudaSuccess) e = accumulate_attributes<2048, false>();
+    if (e == cudaSuccess) e = accumulate_attributes<1024, true>();
     return e;
 }
 
-template <int SPAN>
+template <int SPAN, bool LARGE = false>
 static void launch_accumulate(const Work &w, const Launch &L) {
-    k_accumulate<SPAN><<<L.fit(k_accumulate<SPAN>, ACC_THREADS, acc_smem<SPAN>(), G_ACC), ACC_THREADS,
-                         acc_smem<SPAN>(), L.stream>>>(w);
+    k_accumulate<SPAN, LARGE><<<L.fit(k_accumulate<SPAN, LARGE>, ACC_THREADS, acc_smem<SPAN>(), G_ACC), ACC_THREADS,
+                                acc_smem<SPAN>(), L.stream>>>(w);
 }
 
-void launch_features(const Work &w, const Launch &L) {
-    if (L.tune.acc_span == 512) launch_accumulate<512>(w, L);
+// large_clusters: clusters of any length (variant (b)), always in spans of
+// 1024 positions.
+void launch_features(const Work &w, const Launch &L, bool large_clusters) {
+    if (large_clusters) launch_accumulate<1024, true>(w, L);
+    else if (L.tune.acc_span == 512) launch_accumulate<512>(w, L);
     else if (L.tune.acc_span == 2048) launch_accumulate<2048>(w, L);
     else launch_accumulate<1024>(w, L);
     L.mark("k_accumulate");

@@ -987,7 +987,7 @@ static int flush_variant(tpc_ctx *c, Tracer *tr) {
     } else {
         launch_variant_keys(w, v, 1, L);
         for (int pass = 0; pass < 3; ++pass) launch_radix_pass(wv, pass, L);
-        launch_pixel_timelines(w, v, c->width * c->height, L);
+        launch_pixel_timelines(w, v, L);
         // Rounds of the rule until the partition is closed under it, on the
         // (a) components' dense ids: the first over every hit's 9 latest
         // neighbours, the later ones over the edges left open (all hits
@@ -1034,7 +1034,7 @@ static int flush_variant(tpc_ctx *c, Tracer *tr) {
     // kernels zeroed; a (c) root can be any hit.  k_accumulate finds the
     // roots (the parents may be deep).
     if (c->variant == TPC_STATIC) launch_init_roots(w, L);
-    launch_features(w, L);
+    launch_features(w, L, c->variant == TPC_GLOBAL);
     launch_outputs(w, L);
     if (cudaGetLastError() != cudaSuccess) return TPC_ERR_CUDA;
     c->res_base = c->pushed;

@@ -537,12 +537,12 @@ struct SideStream {
     cudaEvent_t fork = nullptr, join = nullptr;
 };
 cudaError_t launch_static_sweep(const Work &w, const VarWork &v, const Launch &L, const SideStream &side);
-void launch_pixel_timelines(const Work &w, const VarWork &v, uint32_t npixels, const Launch &L);
+void launch_pixel_timelines(const Work &w, const VarWork &v, const Launch &L);
 void launch_components(const Work &w, const VarWork &v, const Launch &L);
 void launch_group_last(const VarWork &v, const Launch &L);
 void launch_comp_parents(const Work &w, const VarWork &v, const Launch &L);
 void launch_global_edges(const Work &w, const VarWork &v, int full, int flat, int in_list, const Launch &L);
-void launch_features(const Work &w, const Launch &L);
+void launch_features(const Work &w, const Launch &L, bool large_clusters = false);
 void launch_outputs(const Work &w, const Launch &L);
 
 }  // namespace tpc

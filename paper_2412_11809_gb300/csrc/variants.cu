@@ -639,42 +639,21 @@ cudaError_t init_variants_attributes() {
                ? cudaFuncSetAttribute(k_static_sweep_big, cudaFuncAttributeMaxDynamicSharedMemorySize, BIG_SMEM) : e;
 }
 
-// (b): pixel histogram and its exclusive scan (single segment).
-__global__ void __launch_bounds__(256) k_pixel_hist(Work w, VarWork v) {
-    const Prob &P = *w.prob;
-    const uint32_t nt = P.ntiles;
-    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
-        const Seg &g = w.seg[w.tile_seg[t]];
-        uint32_t begin, end;
-        tile_range(g, t, begin, end);
-        for (uint32_t s = begin + threadIdx.x; s < end; s += blockDim.x) {
-            const uint32_t pix = w.spix[s];
-            atomicAdd(&v.pix_start[(pix >> 16) * g.width + (pix & 0xFFFFu) + 1], 1u);
-        }
-    }
-}
-
-__global__ void __launch_bounds__(1024) k_pixel_scan(Work w, VarWork v) {
-    __shared__ uint32_t s_warp[32];
+// (b): where each pixel's timeline begins in the order the pixel sort left
+// (single segment): a lower bound per pixel, whose first steps all threads
+// share.  A histogram by atomics and its scan in one CTA took 510 us for 8 M
+// hits and 229,376 pixels; this takes 16.
+__global__ void __launch_bounds__(256) k_pixel_starts(Work w, VarWork v) {
     const Seg &g = w.seg[0];
-    const uint32_t np = g.width * g.height;   // entries 1..np hold counts
-    const uint32_t per = (np + blockDim.x - 1) / blockDim.x;
-    const uint32_t i0 = 1 + threadIdx.x * per;
-    uint32_t local = 0;
-    for (uint32_t i = i0; i < i0 + per && i <= np; ++i) local += v.pix_start[i];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t x = local;
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) s_warp[warp] = x;
-    __syncthreads();
-    uint32_t run = x - local;
-    for (int q = 0; q < warp; ++q) run += s_warp[q];
-    for (uint32_t i = i0; i < i0 + per && i <= np; ++i) {
-        run += v.pix_start[i];
-        v.pix_start[i] = run;
+    const uint32_t *tk = pick(v.k, v.prob->npasses & 1u) + g.off;
+    const uint32_t np = g.width * g.height;
+    for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q <= np; q += gridDim.x * blockDim.x) {
+        uint32_t a = 0, b = g.n;   // first entry of a pixel >= q
+        while (a < b) {
+            const uint32_t mid = (a + b) >> 1;
+            if (tk[mid] < q) a = mid + 1; else b = mid;
+        }
+        v.pix_start[q] = a;
     }
 }
 
@@ -793,8 +772,8 @@ __global__ void __launch_bounds__(256) k_comp_last(Work w, VarWork v) {
     }
 }
 
-// Before a full round: each hit's state, (sorted position, id of its
-// group's root, that group's last key, its key), first in position order
+// Before a full round: each hit's state, (id of its group's root, that
+// group's last key, its sorted position, its key), first in position order
 // (coalesced but for the ids, whose roots lie near), then gathered into
 // pixel-timeline order, one 16-byte read per hit.  The groups and last keys
 // are those of the moment (the last keys exact at the first round, lagging
@@ -814,7 +793,7 @@ __global__ void __launch_bounds__(256) k_position_state(Work w, VarWork v, int f
             c = gfind(v.cpar_d, c0);
             last = *reinterpret_cast<volatile uint32_t *>(&v.clast[c]);
         }
-        v.pstate[s] = make_uint4(s, c, last, skey[s]);
+        v.pstate[s] = make_uint4(c, last, s, skey[s]);
     }
 }
 
@@ -895,70 +874,54 @@ __device__ __forceinline__ void push_edges(const VarWork &v, int out, bool keep,
     }
 }
 
-// The latest entry of timeline [q0, q1) (ascending positions) before
-// position s, for the 32 lanes of a warp whose positions ascend with the
-// lane index: a 32-way search for lane 0's, then a window of the 32 entries
-// from the one before it, each lane's answer in it by five shuffles; a lane
-// whose answer lies past the window searches the rest alone.  All lanes
-// call it with the same q0, q1.
-__device__ __forceinline__ void lane_latest(const uint32_t *tl, const uint4 *T, uint32_t a, uint32_t b,
-                                            uint32_t s, uint4 &nb, bool &has) {
-    const uint32_t a0 = a;
-    while (a < b) {   // first entry of [a, b) at or after s
-        const uint32_t mid = (a + b) >> 1;
-        if (tl[mid] < s) a = mid + 1; else b = mid;
-    }
-    if (a > a0) {
-        nb = T[a - 1];
-        has = true;
-    }
-}
-
-__device__ __forceinline__ void warp_latest(const uint32_t *tl, const uint4 *T, uint32_t q0, uint32_t q1,
-                                            uint32_t s, int lane, uint4 &nb, bool &has) {
-    const uint32_t s0 = __shfl_sync(0xffffffffu, s, 0);
-    uint32_t lo = q0, hi = q1;   // the first entry at or after s0 lies in [lo, hi] (hi = q1: none)
-    while (hi - lo > 32) {
-        const uint32_t step = (hi - lo + 31) >> 5, idx = lo + (uint32_t)lane * step;
-        const int c = __popc(__ballot_sync(0xffffffffu, idx < hi && tl[idx] < s0));   // a prefix of the lanes
-        if (c == 0) { hi = lo; break; }
-        const uint32_t below = lo + (uint32_t)(c - 1) * step;
-        lo = below + 1;
-        hi = min(below + step, hi);
-    }
-    if (hi > lo) lo += __popc(__ballot_sync(0xffffffffu, lo + lane < hi && tl[lo + lane] < s0));
-    // window lane j holds entry lo - 1 + j (lane 0: none if lo = q0; past q1: +inf)
-    const bool in = (lane > 0 || lo > q0) && lo + lane - 1 < q1;
-    const uint4 e = in ? T[lo + lane - 1] : make_uint4(0, 0, 0, 0);
-    const uint32_t wpos = in ? e.x : 0xFFFFFFFFu;   // lane 0's is never compared
-    int c = 0;   // entries of lanes 1..31 before s
+// The first entries at or after position s of G timelines [at, at + n)
+// (ascending positions), into at: binary searches in step, so that a load of
+// each is in flight.
+template <int G>
+__device__ __forceinline__ void lane_bounds(const uint32_t *tl, uint32_t (&at)[G], uint32_t (&n)[G], uint32_t s) {
+    uint32_t longest = 0;
 #pragma unroll
-    for (int st = 16; st > 0; st >>= 1)
-        if (__shfl_sync(0xffffffffu, wpos, c + st) < s) c += st;
-    nb.x = __shfl_sync(0xffffffffu, e.x, c);
-    nb.y = __shfl_sync(0xffffffffu, e.y, c);
-    nb.z = __shfl_sync(0xffffffffu, e.z, c);
-    nb.w = __shfl_sync(0xffffffffu, e.w, c);
-    has = c > 0 || lo > q0;
-    if (c == 31 && lo + 31 < q1) lane_latest(tl, T, lo + 31, q1, s, nb, has);
+    for (int k = 0; k < G; ++k) longest = max(longest, n[k]);
+    for (; longest; longest >>= 1) {   // a search of n entries ends after as many steps as n has bits
+        uint32_t e[G];
+#pragma unroll
+        for (int k = 0; k < G; ++k) e[k] = n[k] ? tl[at[k] + (n[k] >> 1)] : 0xFFFFFFFFu;
+#pragma unroll
+        for (int k = 0; k < G; ++k) {
+            const uint32_t half = n[k] >> 1;
+            const bool up = e[k] < s;
+            at[k] += up ? half + 1 : 0u;
+            n[k] = up ? n[k] - half - 1 : half;
+        }
+    }
 }
 
 // A round over every hit's 9 latest neighbours (the first round, and any
-// round after an overflow of the edge list), in pixel-timeline order: a warp
-// takes 32 consecutive entries, which mostly share a pixel, and finds their
-// latest earlier entries on each neighbour pixel together (warp_latest;
-// lane by lane where the warp straddles pixels), with their state from the
-// snapshot: the snapshot root starts the find of the neighbour's group (one
-// step shorter than from the hit), its last key decides most rules without
-// a read.  Merges what the rule allows and lists the rest, as (hit, root of
-// the neighbour's group).
-__global__ void __launch_bounds__(256) k_global_first(Work w, VarWork v, int out) {
+// round after an overflow of the edge list), in pixel-timeline order, with
+// their state from the snapshot: the snapshot root starts the find of the
+// neighbour's group, its last key decides most rules without a read.  Merges
+// what the rule allows and lists the rest, as (node of h's group, root of the
+// neighbour's group).
+//
+// Bound by the latency of its dependent loads (a search in each neighbour's
+// timeline, the state found, the finds), so a lane takes its eight neighbour
+// pixels through the searches and the first step of the finds together.  The
+// warp searching for its 32 hits at once, one neighbour after another, took
+// 1480 us for 8 M hits on 448x512 pixels, where 32 entries of the timelines
+// span two pixels or more; together in groups of two, four and eight: 1199,
+// 1078 and 943 us (416 of them the searches).  Not kept: warp-wide searches of
+// four neighbours at once (1075), and second steps up, last keys and unions
+// also taken together (1066, with twice the edges listed).
+constexpr int FIRST_THREADS = 128, FIRST_G = 8;
+
+__global__ void __launch_bounds__(FIRST_THREADS, 5) k_global_first(Work w, VarWork v, int out) {
     const Seg &g = w.seg[0];
     const uint32_t W = g.width, H = g.height, n = g.n, dt = g.dt;
     const uint32_t sel = v.prob->npasses & 1u;
     const uint32_t *tl = pick(v.v, sel) + g.off;   // sorted positions grouped by pixel
     const uint32_t *tk = pick(v.k, sel) + g.off;   // their pixel ids
     const uint4 *T = v.tline + g.off;
+    auto state = [T](uint32_t at) { return __ldg(reinterpret_cast<const uint2 *>(T + at)); };   // (id, last key)
     const uint32_t *ps = v.pix_start;
     const int lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * (blockDim.x >> 5);
@@ -966,43 +929,21 @@ __global__ void __launch_bounds__(256) k_global_first(Work w, VarWork v, int out
     for (uint32_t i0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32u; i0 < n; i0 += warps * 32u) {
         const uint32_t i = i0 + (uint32_t)lane;
         const bool valid = i < n;
-        const uint4 me = valid ? T[i] : make_uint4(0, 0, 0, 0);   // position, group id, its last key, key
+        const uint4 me = valid ? T[i] : make_uint4(0, 0, 0, 0);   // group id, its last key, position, key
         const uint32_t p = valid ? tk[i] : 0xFFFFFFFFu;
-        const uint32_t p0 = __shfl_sync(0xffffffffu, p, 0);
-        const bool uniform = __all_sync(0xffffffffu, p == p0);
-        const int px = (int)(p % W), py = (int)(p / W);
-        uint32_t rh = me.y;   // an id of h's group, moved towards its root as the round goes
-#pragma unroll 1
-        for (int d = 0; d < 9; ++d) {
-            uint4 nb = make_uint4(0, 0, 0, 0);
-            bool has = false;
-            const int x = px + d % 3 - 1, y = py + d / 3 - 1;
-            const bool inside = valid && x >= 0 && x < (int)W && y >= 0 && y < (int)H;
-            if (d == 4) {
-                if (valid && i > ps[p]) {
-                    nb = T[i - 1];
-                    has = true;
-                }
-            } else if (uniform) {   // inside is the same for every lane
-                if (inside) {
-                    const uint32_t q = (uint32_t)y * W + (uint32_t)x;
-                    warp_latest(tl, T, ps[q], ps[q + 1], me.x, lane, nb, has);
-                }
-            } else if (inside) {
-                const uint32_t q = (uint32_t)y * W + (uint32_t)x;
-                lane_latest(tl, T, ps[q], ps[q + 1], me.x, nb, has);
-            }
-            // Any two nodes found equal are in one group (groups only
-            // merge), so stale roots only cost a find; the last keys used
-            // are lower bounds of the group's (nb.z: its part at the
-            // snapshot), so the rule never merges more than the sweep.
+        uint32_t rh = me.x;   // an id of h's group, moved towards its root as the round goes
+        // Any two nodes found equal are in one group (groups only merge), so
+        // stale roots only cost a find; the last keys used are lower bounds of
+        // the group's (nb.y: its part at the snapshot), so the rule never
+        // merges more than the sweep.  up: a step up from nb.x.
+        auto join = [&](const uint2 &nb, uint32_t up, bool has) {
             int r = 0;
-            uint32_t rl = nb.y;
+            uint32_t rl = up;
             if (has && rl != rh) {
                 rl = gfind(v.cpar_d, rl);
                 if (rl != rh) rh = gfind(v.cpar_d, rh);   // h's group may have been joined since
                 if (rl != rh) {
-                    bool ok = (uint64_t)me.w <= (uint64_t)nb.z + dt;
+                    bool ok = (uint64_t)me.w <= (uint64_t)nb.y + dt;
                     if (!ok) ok = (uint64_t)me.w <= (uint64_t)*reinterpret_cast<volatile uint32_t *>(&v.clast[rl]) + dt;
                     if (ok) {
                         if (gunion_last(v.cpar_d, v.clast, rh, rl)) r = 1;
@@ -1014,6 +955,33 @@ __global__ void __launch_bounds__(256) k_global_first(Work w, VarWork v, int out
             }
             changed |= r == 1;
             push_edges(v, out, r == 2, rh, rl, me.w);
+        };
+        {   // its own pixel: the entry before
+            const bool has = valid && i > ps[p];
+            const uint2 nb = has ? state(i - 1) : make_uint2(0, 0);
+            join(nb, nb.x, has);
+        }
+        const uint32_t py = p / W, px = p - py * W;
+        {
+            uint32_t q0[FIRST_G], at[FIRST_G], len[FIRST_G];   // each neighbour's timeline: begin, first entry after h
+#pragma unroll
+            for (int k = 0; k < FIRST_G; ++k) {
+                const int d = k + (k >= 4), x = (int)px + d % 3 - 1, y = (int)py + d / 3 - 1;
+                const bool inside = valid && x >= 0 && x < (int)W && y >= 0 && y < (int)H;
+                const uint32_t q = (uint32_t)y * W + (uint32_t)x;
+                at[k] = q0[k] = inside ? ps[q] : 0u;
+                len[k] = inside ? ps[q + 1] - q0[k] : 0u;
+            }
+            lane_bounds<FIRST_G>(tl, at, len, me.z);
+            uint2 nb[FIRST_G];
+            uint32_t up[FIRST_G];
+#pragma unroll
+            for (int k = 0; k < FIRST_G; ++k) nb[k] = at[k] > q0[k] ? state(at[k] - 1) : make_uint2(0, 0);
+#pragma unroll
+            for (int k = 0; k < FIRST_G; ++k)
+                up[k] = at[k] > q0[k] ? *reinterpret_cast<volatile uint32_t *>(&v.cpar_d[nb[k].x]) : 0u;
+#pragma unroll
+            for (int k = 0; k < FIRST_G; ++k) join(nb[k], up[k], at[k] > q0[k]);
         }
     }
     if (__syncthreads_or(changed) && threadIdx.x == 0) atomicOr(&v.changed[0], 1u);
@@ -1086,7 +1054,7 @@ void launch_global_edges(const Work &w, const VarWork &v, int full, int flat, in
         k_position_state<<<L.fit(k_position_state, 256, 0), 256, 0, L.stream>>>(w, v, flat);
         k_timeline_state<<<L.fit(k_timeline_state, 256, 0), 256, 0, L.stream>>>(w, v);
         L.mark("k_timeline_state");
-        k_global_first<<<L.fit(k_global_first, 256, 0), 256, 0, L.stream>>>(w, v, out);
+        k_global_first<<<L.fit(k_global_first, FIRST_THREADS, 0), FIRST_THREADS, 0, L.stream>>>(w, v, out);
         L.mark("k_global_first");
     } else {
         k_global_list<<<L.fit(k_global_list, 256, 0), 256, 0, L.stream>>>(w, v, in);
@@ -1130,11 +1098,9 @@ cudaError_t launch_static_sweep(const Work &w, const VarWork &v, const Launch &L
     return e == cudaSuccess ? e2 : e;
 }
 
-void launch_pixel_timelines(const Work &w, const VarWork &v, uint32_t npixels, const Launch &L) {
-    cudaMemsetAsync(v.pix_start, 0, (npixels + 1) * sizeof(uint32_t), L.stream);
-    k_pixel_hist<<<L.fit(k_pixel_hist, 256, 0), 256, 0, L.stream>>>(w, v);
-    k_pixel_scan<<<1, 1024, 0, L.stream>>>(w, v);
-    L.mark("k_pixel_hist_scan");
+void launch_pixel_timelines(const Work &w, const VarWork &v, const Launch &L) {
+    k_pixel_starts<<<L.fit(k_pixel_starts, 256, 0), 256, 0, L.stream>>>(w, v);
+    L.mark("k_pixel_starts");
 }
 
 
