@@ -51,7 +51,9 @@ __global__ void __launch_bounds__(256) k_var_keys(Work w, VarWork v, int by_pixe
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *v.prob = P;
-        v.prob->npasses = by_pixel ? 3 : 4;   // pixel ids < 2^20; roots < 2^32
+        // as many digits as the largest pixel id (< 2^20) or root has
+        const uint32_t top = (by_pixel ? w.seg[0].width * w.seg[0].height : w.seg[0].off + w.seg[0].n) - 1u;
+        v.prob->npasses = top ? (32 - __clz(top) + RADIX_BITS - 1) / RADIX_BITS : 0;
     }
 }
 
