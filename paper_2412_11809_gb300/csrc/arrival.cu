@@ -26,7 +26,8 @@
 // over earlier positions, and tiles that did not look far enough are joined
 // with every earlier tile.  All of it is one launch (k_arrival_step), a
 // cluster of one CTA per tile.  As seven launches a call with 1,000 hits took
-// 53 us (41 of them on the host) and one with 65,536 hits 96; now 28 and 65.
+// 53 us (41 of them on the host) and one with 65,536 hits 96; now 26 and 58 (64
+// with 512 threads per CTA, which left an SM's issue slots idle).
 //
 // Owning by time keeps events whole: arrival disorder spreads an event's hits
 // over a thousand positions, and tiles of positions would cut a quarter of
@@ -39,30 +40,30 @@
 // last ToA, union-find parent) is dense and a hit's cluster is one 32-bit c.
 #include <cooperative_groups.h>
 
+#include <cstddef>
+
 #include "tpc_internal.cuh"
 
 namespace tpc {
 
-constexpr int AT = 512;                          // threads of the tile kernels (64 registers, two CTAs per SM)
-constexpr int AW = AT / 32;
+constexpr int AT = 512;                          // threads of k_arrival_tile (64 registers, two CTAs per SM)
+constexpr int ST = 1024;                         // ... and where a CTA has an SM to itself
+constexpr int AW = 32;                           // warps, at most
 constexpr uint32_t A_MARGIN = 1024;              // positions around the tile read at once
-constexpr int A_ITEMS = (TILE + 2 * A_MARGIN) / AT;   // records per thread
-constexpr int A_GROUP = 2;                       // ... looked at while the next ones are in flight
+constexpr int A_GROUP = 2;                       // records per thread looked at while the next ones are in flight
+constexpr int A_GROUPS = (TILE + 2 * A_MARGIN) / (512 * A_GROUP);   // ... of 512 threads, at most
 constexpr uint32_t A_STEP = TILE / ACHUNKS;      // positions per further round
-constexpr int A_HPER = (A_STEP + AT - 1) / AT;
 constexpr uint32_t A_ENT = 5632;                 // hits staged: a tile's own and the earlier ones
-constexpr int A_PER = A_ENT / AT;
 constexpr uint32_t A_WORDS = 2304;               // 256 rows of nine 30-pixel words
 constexpr uint32_t A_XTRA = 2048;                // unions beyond each hit's first
 constexpr uint32_t A_LATER = 2048;               // hits beside cells of several hits
 constexpr uint32_t A_FAR = 1024;                 // hits found beyond the margins
-constexpr int A_JUMPS = 2;                       // path-shortening passes over the tile's forest
+constexpr int A_JUMPS = 1;                       // path-shortening passes over the tile's forest
 constexpr int A_ROUNDS = 4;                      // further rounds on each side
 constexpr int A_BACK_ROUNDS = 16;                // rounds back of a small step's tiles
 constexpr uint32_t A_NONE = 0x7FFFu;             // no hit
 constexpr uint32_t A_MULTI = 0x8000u;            // head flag: the cell holds several hits
 static_assert(A_WORDS <= 4096, "word indices take 12 bits");
-static_assert(A_ITEMS * AT == TILE + 2 * (int)A_MARGIN && A_PER * AT == (int)A_ENT && A_ITEMS % A_GROUP == 0, "whole rounds");
 
 // A cell is a pixel column x of a row (y mod R).  Occupied cells are found by
 // a bitmap (30 pixels per word, the outer two bits repeating the neighbour
@@ -82,17 +83,20 @@ struct ArrivalShared {
     uint16_t later[A_LATER];     // hits beside cells of several hits
     uint16_t far[A_FAR];         // hits beyond the margins: position - window start
     uint32_t red[4][AW];
+    uint16_t first[AW][A_GROUPS];    // first entry of each warp's records of a group
     uint32_t cnt[2][AW], turn[2][AW];
     unsigned long long m64[2][AW];
     uint32_t cut[2];
     uint32_t nent, nown, ntail, nxtra, ncross, nlater, nroots, tsum, flag;
     // After the links, in the place of what is no longer needed:
-    __device__ uint16_t *tot() { return head; }                                   // [A_ENT] ToT per entry
-    __device__ uint16_t *pos() { return next; }                                   // [A_ENT] position per entry
-    __device__ uint16_t *id() { return reinterpret_cast<uint16_t *>(xtra); }      // [A_ENT] cluster of each tile root
+    __device__ uint32_t *where() { return reinterpret_cast<uint32_t *>(head); }   // [A_ENT] position << 16 | ToT per entry
+    __device__ uint2 *tops() { return reinterpret_cast<uint2 *>(later); }         // [A_TOPS] roots of the tile's clusters
     __device__ uint32_t *sums() { return reinterpret_cast<uint32_t *>(word); }    // [2 * A_WORDS] feature sums
 };
-static_assert(A_XTRA * 4 + A_LATER * 2 >= A_ENT * 2, "cluster indices fit the lists");
+constexpr uint32_t A_TOPS = A_ENT / 32;   // words of a bitmap over the entries
+static_assert(A_LATER * 2 >= A_TOPS * sizeof(uint2) && A_ENT % 32 == 0, "the bitmap fits the list");
+static_assert(offsetof(ArrivalShared, next) == offsetof(ArrivalShared, head) + A_ENT * 2 && offsetof(ArrivalShared, head) % 4 == 0 &&
+                  offsetof(ArrivalShared, later) % 8 == 0, "words over the heads and the lists");
 
 // Code of a hit: word << 5 | bit of its cell, (y / R) << 17, and whether it is
 // the tile's own (otherwise an earlier tile's).
@@ -151,8 +155,9 @@ struct Cells {
     }
     // word / nw = umulhi(word, magic) for words < 2^12, nw > 1 (nw = 1 apart: the factor would be 2^32)
     __device__ __forceinline__ uint32_t magic() const { return 0xFFFFFFFFu / nw + 1u; }
+    template <int NT>
     __device__ __forceinline__ void clear(ArrivalShared &S) const {
-        for (uint32_t i = threadIdx.x; i < (nwords + 1) / 2; i += AT)
+        for (uint32_t i = threadIdx.x; i < (nwords + 1) / 2; i += NT)
             reinterpret_cast<uint4 *>(S.word)[i] = make_uint4(0, 0, 0, 0);
     }
 };
@@ -186,7 +191,7 @@ __device__ __forceinline__ bool arrival_hook(uint16_t *par, uint32_t a, uint32_t
 // order (row above, left), on one pixel by the earlier hit.
 // near(a, b): two keys within dt; join(e, j, linked): takes a pair; linked: e
 // has been joined before.  ALIAS: rows share cells.
-template <bool ALIAS, class Near, class Join>
+template <int NT, bool ALIAS, class Near, class Join>
 __device__ __forceinline__ void arrival_pairs(ArrivalShared &S, const Cells &C, uint32_t n_e, Near near, Join join) {
     const int tid = threadIdx.x;
     // Heads of the cells left, above left, above and above right (A_NONE: none)
@@ -247,7 +252,7 @@ __device__ __forceinline__ void arrival_pairs(ArrivalShared &S, const Cells &C, 
         }
     };
 #pragma unroll 1
-    for (uint32_t e = tid; e < n_e; e += AT) {
+    for (uint32_t e = tid; e < n_e; e += NT) {
         const uint2 me = S.kc[e];
         const uint32_t code = me.y & C_CELL, key = me.x;
         uint32_t hd[4], up;
@@ -296,17 +301,17 @@ __device__ __forceinline__ void arrival_pairs(ArrivalShared &S, const Cells &C, 
     __syncthreads();
     const uint32_t listed = S.nlater;
     if (listed <= A_LATER)
-        for (uint32_t i = tid; i < listed; i += AT) crowded(S.later[i]);
+        for (uint32_t i = tid; i < listed; i += NT) crowded(S.later[i]);
     else   // (more than the list holds: all of them, those without such cells have nothing to do)
-        for (uint32_t e = tid; e < n_e; e += AT) crowded(e);
+        for (uint32_t e = tid; e < n_e; e += NT) crowded(e);
 }
 
-template <class Near, class Join>
+template <int NT, class Near, class Join>
 __device__ __forceinline__ void arrival_links(ArrivalShared &S, const Cells &C, uint32_t n_e, Near near, Join join) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __syncthreads();                // bits and entries are in place
     {   // repeat the border pixels in the neighbour words, and count the cells before each word
-        constexpr uint32_t PER = (A_WORDS + AT - 1) / AT;
+        constexpr uint32_t PER = (A_WORDS + NT - 1) / NT;
         const uint32_t i0 = tid * PER;
         uint32_t bits[PER], sum = 0;
         const uint32_t before = i0 && i0 < C.nwords ? S.word[i0 - 1].x : 0u;
@@ -323,7 +328,7 @@ __device__ __forceinline__ void arrival_links(ArrivalShared &S, const Cells &C, 
         if (lane == 31) S.cnt[0][warp] = x;
         if (tid == 0) S.nlater = 0;
         __syncthreads();
-        uint32_t run = x - sum + __reduce_add_sync(0xffffffffu, lane < warp ? S.cnt[0][min(lane, AW - 1)] : 0u);
+        uint32_t run = x - sum + __reduce_add_sync(0xffffffffu, lane < warp ? S.cnt[0][min(lane, (NT / 32) - 1)] : 0u);
 #pragma unroll
         for (uint32_t i = 0; i < PER; ++i) {
             const uint32_t l = i ? bits[i - 1] : before, r = i + 1 < PER ? bits[i + 1] : after;
@@ -333,10 +338,11 @@ __device__ __forceinline__ void arrival_links(ArrivalShared &S, const Cells &C, 
         }
     }
     __syncthreads();
+    constexpr int A_PER = (A_ENT + NT - 1) / NT;
     uint32_t slots[A_PER];
 #pragma unroll
     for (int q = 0; q < A_PER; ++q) {   // any hit of a cell becomes its head
-        const uint32_t e = q * AT + tid;
+        const uint32_t e = q * NT + tid;
         slots[q] = 0;
         if (e < n_e) {
             const uint32_t code = S.kc[e].y;
@@ -350,7 +356,7 @@ __device__ __forceinline__ void arrival_links(ArrivalShared &S, const Cells &C, 
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < A_PER; ++q) {   // the others hang behind it
-        const uint32_t e = q * AT + tid;
+        const uint32_t e = q * NT + tid;
         if (e >= n_e) continue;
         const uint32_t s = slots[q], h = S.head[s] & A_NONE;
         if (h == e) continue;
@@ -366,7 +372,7 @@ __device__ __forceinline__ void arrival_links(ArrivalShared &S, const Cells &C, 
         S.head[s] = (uint16_t)(h | A_MULTI);
     }
     __syncthreads();
-    if (C.alias) arrival_pairs<true>(S, C, n_e, near, join); else arrival_pairs<false>(S, C, n_e, near, join);
+    if (C.alias) arrival_pairs<NT, true>(S, C, n_e, near, join); else arrival_pairs<NT, false>(S, C, n_e, near, join);
 }
 
 // A pair: the hit's first makes the other its parent (always raster-earlier,
@@ -383,15 +389,19 @@ __device__ __forceinline__ void join_hits(ArrivalShared &S, uint32_t e, uint32_t
 
 // Components of the staged hits, the clusters of the tile's own, their
 // features, each own hit's cluster, and the pairs with earlier tiles (earlier
-// hits in a cluster of this tile).  ToTs and positions (pos[e], from `origin`)
-// of the entries are staged; the caller's barrier is behind them and the links.
+// hits in a cluster of this tile).  where()[e] (position from `origin`, ToT) of
+// the entries is staged; the caller's barrier is behind it and the links.
 // false: more clusters than the tile has numbers.
+template <int NT>
 __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, uint32_t t, ArrivalShared &S,
-                                                 const Cells &C, uint32_t n_e, const uint16_t *pos,
-                                                 uint32_t origin, uint64_t base) {
+                                                 const Cells &C, uint32_t n_e, uint32_t origin, uint64_t base) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int A_PER = (A_ENT + NT - 1) / NT;
     const uint32_t first_c = t * TILE;
     volatile uint16_t *par = S.par;
+    uint2 *tops = S.tops();
+    static_assert(A_TOPS <= (uint32_t)NT && A_TOPS <= 6 * 32, "a thread per word, six words per lane");
+    if (tid < (int)A_TOPS) tops[tid] = make_uint2(0, 0);
     // Raster-order parents chain along a track; every hit first jumps to its
     // ancestors a few times (all hits at once, so paths shrink by half and
     // more each time) before unions and finds walk what is left.
@@ -400,19 +410,19 @@ __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, ui
         uint32_t p[A_PER];
 #pragma unroll
         for (int q = 0; q < A_PER; ++q)
-            if (q * AT + tid < n_e) p[q] = par[q * AT + tid];
+            if (q * NT + tid < n_e) p[q] = par[q * NT + tid];
 #pragma unroll
         for (int q = 0; q < A_PER; ++q)
-            if (q * AT + tid < n_e) p[q] = par[p[q]];
+            if (q * NT + tid < n_e) p[q] = par[p[q]];
 #pragma unroll
         for (int q = 0; q < A_PER; ++q)
-            if (q * AT + tid < n_e) p[q] = par[p[q]];
+            if (q * NT + tid < n_e) p[q] = par[p[q]];
 #pragma unroll
         for (int q = 0; q < A_PER; ++q)
-            if (q * AT + tid < n_e) par[q * AT + tid] = (uint16_t)p[q];
+            if (q * NT + tid < n_e) par[q * NT + tid] = (uint16_t)p[q];
     }
     __syncthreads();
-    for (uint32_t i = tid; i < min(S.nxtra, A_XTRA); i += AT) {
+    for (uint32_t i = tid; i < min(S.nxtra, A_XTRA); i += NT) {
         uint32_t a = S.xtra[i] >> 16, b = S.xtra[i] & 0xFFFFu;
         while (true) {   // hook the larger root under the smaller
             a = arrival_root(S.par, a);
@@ -423,44 +433,71 @@ __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, ui
         }
     }
     __syncthreads();
-    // roots with own hits are the tile's clusters; all are, but for earlier
-    // hits that met none of this tile's
-    uint16_t *id = S.id();   // (the lists are walked)
-    constexpr uint32_t OWNS = 0xFFFEu;
-    for (uint32_t e = tid; e < n_e; e += AT) id[e] = (uint16_t)A_NONE;
-    __syncthreads();
-    uint32_t root[A_PER];
+    // Roots of all a thread's hits in step, their loads in flight together, each
+    // step stored for the hits behind it (hit after hit, and marks, numbers and
+    // parents in arrays: 2480 us for 64 Mi hits, in step 2364; without the
+    // stores 3401, chains of a track's hits being long).
+    // Roots with own hits are the tile's clusters (all are, but for earlier
+    // hits that met none of this tile's): marked in a bitmap, numbered by rank.
+    uint32_t top[A_PER];   // root of entry q * NT + tid
+#pragma unroll
+    for (int q = 0; q < A_PER; ++q) top[q] = q * NT + tid < n_e ? par[q * NT + tid] : 0u;
+    for (bool more = true; more;) {
+        more = false;
+#pragma unroll
+        for (int q = 0; q < A_PER; ++q) {
+            if (q * NT + tid >= n_e) continue;
+            const uint32_t p = par[top[q]];
+            if (p != top[q]) {
+                more = true;
+                top[q] = p;
+                par[q * NT + tid] = (uint16_t)p;
+            }
+        }
+    }
 #pragma unroll
     for (int q = 0; q < A_PER; ++q) {
-        const uint32_t e = q * AT + tid;
-        if (e < n_e) {
-            root[q] = arrival_root(par, e);
-            if (S.kc[e].y & C_OWN) id[root[q]] = (uint16_t)OWNS;
-        }
+        const uint32_t e = q * NT + tid;
+        if (e < n_e && S.kc[e].y & C_OWN) atomicOr(&tops[top[q] >> 5].x, 1u << (top[q] & 31u));
     }
-    __syncthreads();   // (no path is halved any more)
+    __syncthreads();
+    if (warp == 0) {
+        uint32_t c[6], sum = 0;
 #pragma unroll
-    for (int q = 0; q < A_PER; ++q)
-        if (q * AT + tid < n_e) par[q * AT + tid] = (uint16_t)root[q];
-    for (uint32_t e0 = warp * 32; e0 < n_e; e0 += AT) {
-        const uint32_t e = e0 + lane;
-        const bool top = e < n_e && id[e] == OWNS;
-        const uint32_t m = __ballot_sync(0xffffffffu, top);
-        if (m) {
-            uint32_t k = 0;
-            if (lane == 0) k = atomicAdd(&S.nroots, (uint32_t)__popc(m));
-            k = __shfl_sync(0xffffffffu, k, 0);
-            if (top) id[e] = (uint16_t)(k + __popc(m & lanes_below()));
+        for (uint32_t k = 0; k < 6; ++k) {
+            c[k] = lane * 6 + k < A_TOPS ? __popc(tops[lane * 6 + k].x) : 0u;
+            sum += c[k];
+        }
+        uint32_t run = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, run, o);
+            if (lane >= o) run += y;
+        }
+        if (lane == 31) S.nroots = run;
+        run -= sum;
+#pragma unroll
+        for (uint32_t k = 0; k < 6; ++k) {
+            if (lane * 6 + k < A_TOPS) tops[lane * 6 + k].y = run;
+            run += c[k];
         }
     }
     __syncthreads();
+    uint32_t mine[(A_PER + 1) / 2];   // cluster (A_NONE: none) of entry q * NT + tid, two to a register
+#pragma unroll
+    for (int q = 0; q < A_PER; ++q) {
+        const uint2 v = tops[top[q] >> 5];
+        const uint32_t bit = 1u << (top[q] & 31u);
+        const uint32_t c = v.x & bit ? v.y + __popc(v.x & (bit - 1u)) : A_NONE;
+        mine[q >> 1] = q & 1 ? mine[q >> 1] | c << 16 : c;
+    }
+    auto cluster = [&](int q) { return q & 1 ? mine[q >> 1] >> 16 : mine[q >> 1] & 0xFFFFu; };
     // Features per cluster, as many clusters at once as the space holds.
     // Shared memory adds 32 bits natively and 64 by compare-and-swap loops:
     // while the tile's whole ToT keeps every sum in bounds (4096 hits of the
     // usual ToTs do, 40 times over) size and ToT share a word and the moments
     // take one each; otherwise the moments carry into a second word.
     uint32_t *A = S.sums();
-    const uint16_t *tots = S.tot();
+    const uint32_t *where = S.where();
     const uint32_t nroots = S.nroots, tsum = S.tsum, magic = C.magic();
     if (nroots > TILE) return false;   // (nearly every hit alone, and more hits than positions)
     const bool streaming = g.ss != nullptr;
@@ -470,16 +507,18 @@ __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, ui
     constexpr uint32_t PASS = 2 * A_WORDS / 8;
     for (uint32_t r0 = 0; r0 == 0 || r0 < nroots; r0 += PASS) {
         const uint32_t nr = min(nroots - r0, PASS);
-        for (uint32_t i = tid; i < nr; i += AT) {
+        for (uint32_t i = tid; i < nr; i += NT) {
 #pragma unroll
             for (int k = 0; k < 6; ++k) A[k * PASS + i] = 0;
             A[6 * PASS + i] = A[7 * PASS + i] = 0xFFFFFFFFu;
         }
         __syncthreads();
-#pragma unroll 3
-        for (uint32_t e = tid; e < n_e; e += AT) {
+#pragma unroll
+        for (int q = 0; q < A_PER; ++q) {
+            const uint32_t e = q * NT + tid;
+            if (e >= n_e) break;
             const uint2 kc = S.kc[e];
-            const uint32_t c = id[par[e]], i = c - r0, at = origin + pos[e];
+            const uint32_t c = cluster(q), i = c - r0, pt = where[e], at = origin + (pt >> 16);
             if (!(kc.y & C_OWN)) {
                 if (c != A_NONE && r0 == 0) {   // an earlier tile's hit in a cluster of this one
                     const uint32_t x = atomicAdd(&S.ncross, 1u);
@@ -492,7 +531,7 @@ __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, ui
                 if (w.rkey) w.rkey[at] = kc.x;
             }
             if (i < nr) {
-                const uint32_t tot = tots[e];
+                const uint32_t tot = pt & 0xFFFFu;
                 uint32_t x, y;
                 C.pixel(kc.y, magic, x, y);
                 uint32_t *a = A + i;   // size (and ToT), ToT, x, carry, y, carry, first position, first key
@@ -507,12 +546,12 @@ __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, ui
                     if (atomicAdd(a + 2 * PASS, vx) > ~vx) atomicAdd(a + 3 * PASS, 1u);
                     if (atomicAdd(a + 4 * PASS, vy) > ~vy) atomicAdd(a + 5 * PASS, 1u);
                 }
-                atomicMin(a + 6 * PASS, (uint32_t)pos[e]);
+                atomicMin(a + 6 * PASS, pt >> 16);
                 atomicMin(a + 7 * PASS, kc.x);
             }
         }
         __syncthreads();
-        for (uint32_t i = tid; i < nr; i += AT) {
+        for (uint32_t i = tid; i < nr; i += NT) {
             const uint4 a = make_uint4(A[i], A[PASS + i], A[2 * PASS + i], A[3 * PASS + i]);
             const uint4 b = make_uint4(A[4 * PASS + i], A[5 * PASS + i], A[6 * PASS + i], A[7 * PASS + i]);
             const uint32_t cc = first_c + r0 + i;
@@ -524,15 +563,17 @@ __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, ui
         }
         if (streaming) {   // last ToAs, in the place of the first ones
             __syncthreads();
-            for (uint32_t i = tid; i < nr; i += AT) A[7 * PASS + i] = 0;
+            for (uint32_t i = tid; i < nr; i += NT) A[7 * PASS + i] = 0;
             __syncthreads();
-            for (uint32_t e = tid; e < n_e; e += AT) {
+#pragma unroll
+            for (int q = 0; q < A_PER; ++q) {
+                const uint32_t e = q * NT + tid, i = cluster(q) - r0;
+                if (e >= n_e) break;
                 const uint2 kc = S.kc[e];
-                const uint32_t i = id[par[e]] - r0;
                 if ((kc.y & C_OWN) && i < nr) atomicMax(&A[7 * PASS + i], kc.x);
             }
             __syncthreads();
-            for (uint32_t i = tid; i < nr; i += AT) w.rlast[first_c + r0 + i] = base + A[7 * PASS + i];
+            for (uint32_t i = tid; i < nr; i += NT) w.rlast[first_c + r0 + i] = base + A[7 * PASS + i];
         }
         __syncthreads();
     }
@@ -557,7 +598,17 @@ __device__ __forceinline__ uint32_t arrival_cut(const Seg &g, uint32_t j, uint64
     return __shfl_sync(0xffffffffu, key, __ffs(__ballot_sync(0xffffffffu, rank == 16u)) - 1);
 }
 
-__global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
+// Bound by issue and shared-memory latency, not by bytes: 64 Mi hits (256x256)
+// take 2260 us at 16 B read and 4 B written each.  Of a tile's time the records
+// take 22 percent, cell numbers and heads 9, the walk over neighbour cells 17,
+// crowded cells 8, positions and ToTs 7, the forest and its roots 24, features
+// 10.  Two CTAs of 512 threads at 64 registers; one of 1024 takes 2906 (its
+// barriers leave nothing to run), 768 threads at 40 registers spill (2936).  Entry
+// numbers are counted again for the positions instead of kept: 2324 -> 2260.
+template <int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
+    constexpr int A_ITEMS = (TILE + 2 * A_MARGIN) / NT;   // records per thread
+    static_assert(A_ITEMS * NT == TILE + 2 * (int)A_MARGIN && A_ITEMS % A_GROUP == 0, "whole rounds");
     extern __shared__ __align__(16) unsigned char a_raw[];
     ArrivalShared &S = *reinterpret_cast<ArrivalShared *>(a_raw);
     Prob &P = *w.prob;
@@ -581,14 +632,14 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
         uint4 v[A_GROUP];
 #pragma unroll
         for (int q = 0; q < A_GROUP; ++q) {
-            const int32_t p = p0 + q * AT;
+            const int32_t p = p0 + q * NT;
             if ((uint32_t)p < n) v[q] = ld_hit(hits + p);
         }
         if (tid == 0) {
             S.flag = *reinterpret_cast<volatile uint32_t *>(&P.raw_fail);
             S.nent = S.nown = S.ntail = S.nxtra = S.ncross = S.nroots = S.tsum = 0;
         }
-        C.clear(S);
+        C.clear<NT>(S);
         if (warp < 2) {
             const uint32_t k = arrival_cut(g, j + warp, base, lane);
             if (lane == 0) S.cut[warp] = k;
@@ -607,7 +658,7 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
         const uint32_t tail = last ? 0xFFFFFFFFu : cut1 > dt ? cut1 - dt : 0u;   // own hits the next tile must see
         const uint32_t guard = base ? ARRIVAL_DT : 0u;
         uint32_t high = 0, bad = 0, kmin = 0xFFFFFFFFu, kmax = 0, cmin = 0xFFFFFFFFu;
-        uint32_t mine[A_ITEMS], staged = 0, own_sum = 0, tsum = 0, edge = 0;   // own_sum: own | tail << 16
+        uint32_t tots[A_ITEMS / 2], staged = 0, own_sum = 0, tsum = 0, edge = 0;   // own_sum: own | tail << 16
         // one record: its key and code; whether it is staged
         auto look = [&](const uint4 &r, int32_t p, uint32_t &key, uint32_t &code) -> bool {
             key = 0;
@@ -629,15 +680,15 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
 #pragma unroll
             for (int q = 0; q < A_GROUP; ++q) {
                 const int i = h * A_GROUP + q;
-                const bool kept = look(v[q], p0 + i * AT, key[q], code[q]);
+                const bool kept = look(v[q], p0 + i * NT, key[q], code[q]);
                 mask[q] = __ballot_sync(0xffffffffu, kept);
                 sum += __popc(mask[q]);
-                mine[i] = hit_tot(v[q]);
+                tots[i >> 1] = i & 1 ? tots[i >> 1] | hit_tot(v[q]) << 16 : hit_tot(v[q]);
                 if (kept) {
                     staged |= 1u << i;
                     if (key[q] >= cut) {
                         own_sum += key[q] >= tail && !last ? 0x10001u : 1u;
-                        tsum += mine[i];
+                        tsum += hit_tot(v[q]);
                         if (i == A_ITEMS - 1) edge |= 2u;
                     }
                     if (i == 0) edge |= 1u;
@@ -646,12 +697,13 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
             if (h + 1 < A_ITEMS / A_GROUP) {
 #pragma unroll
                 for (int q = 0; q < A_GROUP; ++q) {
-                    const int32_t p = p0 + ((h + 1) * A_GROUP + q) * AT;
+                    const int32_t p = p0 + ((h + 1) * A_GROUP + q) * NT;
                     if ((uint32_t)p < n) v[q] = ld_hit(hits + p);
                 }
             }
             uint32_t e0 = 0;
             if (lane == 0) e0 = atomicAdd(&S.nent, sum);
+            if (lane == 0) S.first[warp][h] = (uint16_t)e0;   // (more than 2^16: not covered)
             e0 = __shfl_sync(0xffffffffu, e0, 0);
 #pragma unroll
             for (int q = 0; q < A_GROUP; ++q) {
@@ -660,7 +712,6 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
                 if (((staged >> i) & 1u) && e < A_ENT) {
                     S.kc[e] = make_uint2(key[q], code[q] | (key[q] >= cut ? C_OWN : 0u));
                     C.set(S, code[q]);
-                    mine[i] |= e << 16;
                 }
                 e0 += __popc(mask[q]);
             }
@@ -686,7 +737,7 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
             if (tid == 0) atomicMax(&P.raw_fail, RAW_COVER);
             return;
         }
-        edge = __reduce_or_sync(0xffffffffu, S.red[3][min(lane, AW - 1)]);
+        edge = __reduce_or_sync(0xffffffffu, S.red[3][min(lane, (NT / 32) - 1)]);
         // ---- hits beyond the margins: rounds while the outermost hits
         // read still held some of the tile --------------------------
         const uint32_t e_far = min(S.nent, A_ENT);
@@ -700,7 +751,7 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
             for (int r = 0; more && r < A_ROUNDS && (side ? a < (int32_t)n : a + (int32_t)A_STEP > 0); ++r) {
                 bool outer = false;
 #pragma unroll 1
-                for (uint32_t u = tid; u < A_STEP; u += AT) {
+                for (uint32_t u = tid; u < A_STEP; u += NT) {
                     const int32_t p = a + (int32_t)u;
                     uint32_t key, code;
                     uint4 x = make_uint4(0, 0, 0, 0);
@@ -732,9 +783,9 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
         }
         ATile &info = w.atile[t];
         if (warp == 0) {
-            kmin = __reduce_min_sync(0xffffffffu, S.red[0][min(lane, AW - 1)]);
-            kmax = __reduce_max_sync(0xffffffffu, S.red[1][min(lane, AW - 1)]);
-            cmin = __reduce_min_sync(0xffffffffu, S.red[2][min(lane, AW - 1)]);
+            kmin = __reduce_min_sync(0xffffffffu, S.red[0][min(lane, (NT / 32) - 1)]);
+            kmax = __reduce_max_sync(0xffffffffu, S.red[1][min(lane, (NT / 32) - 1)]);
+            cmin = __reduce_min_sync(0xffffffffu, S.red[2][min(lane, (NT / 32) - 1)]);
             if (lane == 0) {
                 Seg &gw = w.seg[si];
                 atomicMin(reinterpret_cast<unsigned long long *>(&gw.toa_min), (unsigned long long)(base + kmin));
@@ -752,25 +803,28 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
         // ---- links -----------------------------------------------------------
         // (keys keep 2^27 from both ends of 32 bits and dt is less: the sum wraps for no far pair)
         const uint32_t dt2 = 2u * dt;
-        arrival_links(S, C, n_e, [&](uint32_t a, uint32_t b) { return a - b + dt <= dt2; },
+        arrival_links<NT>(S, C, n_e, [&](uint32_t a, uint32_t b) { return a - b + dt <= dt2; },
                       [&](uint32_t e, uint32_t o, bool &linked) { join_hits(S, e, o, linked); });
         __syncthreads();
         // ---- positions and ToTs of the entries, where the lists were ---------
-        uint16_t *pos = S.pos(), *tot = S.tot();
+        uint32_t *where = S.where();
 #pragma unroll
-        for (int i = 0; i < A_ITEMS; ++i) {
-            if ((staged >> i) & 1u) {
-                pos[mine[i] >> 16] = (uint16_t)(p0 + i * AT - win);
-                tot[mine[i] >> 16] = (uint16_t)mine[i];
+        for (int h = 0; h < A_ITEMS / A_GROUP; ++h) {   // (the entries as they were counted above)
+            uint32_t e0 = S.first[warp][h];
+#pragma unroll
+            for (int i = h * A_GROUP; i < (h + 1) * A_GROUP; ++i) {
+                const uint32_t kept = __ballot_sync(0xffffffffu, (staged >> i) & 1u);
+                if ((staged >> i) & 1u)
+                    where[e0 + __popc(kept & lanes_below())] =
+                        (uint32_t)(p0 + i * NT - win) << 16 | (tots[i >> 1] >> (i & 1) * 16 & 0xFFFFu);
+                e0 += __popc(kept);
             }
         }
-        for (uint32_t e = e_far + tid; e < n_e; e += AT) {
-            pos[e] = S.far[e - e_far];
-            tot[e] = (uint16_t)hit_tot(ld_hit(hits + (win + (int32_t)S.far[e - e_far])));
-        }
+        for (uint32_t e = e_far + tid; e < n_e; e += NT)
+            where[e] = (uint32_t)S.far[e - e_far] << 16 | hit_tot(ld_hit(hits + (win + (int32_t)S.far[e - e_far])));
         const bool listed = S.nxtra <= A_XTRA;
         __syncthreads();
-        if (!listed || !arrival_clusters(w, g, t, S, C, n_e, pos, off + (uint32_t)win, base) || S.ncross > A_PAIRS) {
+        if (!listed || !arrival_clusters<NT>(w, g, t, S, C, n_e, off + (uint32_t)win, base) || S.ncross > A_PAIRS) {
             if (tid == 0) atomicMax(&P.raw_fail, RAW_COVER);
             return;
         }
@@ -784,7 +838,7 @@ __global__ void __launch_bounds__(AT, 2) k_arrival_tile(Work w) {
 
 // One tile.  DIRECT (k_arrival_step): pairs are joined at once in the global
 // forest, every earlier position is looked at, nothing else is written.
-template <bool DIRECT>
+template <int NT, bool DIRECT>
 __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShared &SS) {
     ArrivalShared &S = SS.s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -795,7 +849,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
     const tpc_hit *hits = g.hits;
     const Cells C(W, H);
     ATile &info = w.atile[t];
-    constexpr int OWN = (TILE + AT - 1) / AT;
+    constexpr int OWN = (TILE + NT - 1) / NT, A_HPER = (A_STEP + NT - 1) / NT;
 
     // ---- the tile's own hits ---------------------------------------------
     uint64_t base = g.raw_base;
@@ -804,7 +858,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
     const uint32_t new0 = g.n_carry > begin ? g.n_carry - begin : 0;   // first new hit
     uint32_t kmin, kmax, tots[OWN];
     if (tid == 0) S.nxtra = S.ncross = S.nroots = S.tsum = 0;
-    C.clear(S);
+    C.clear<NT>(S);
     __syncthreads();
     for (int attempt = 0;; ++attempt) {
         bool bad = false;
@@ -815,10 +869,10 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
         uint4 v[OWN];
 #pragma unroll
         for (int q = 0; q < OWN; ++q)
-            if (q * AT + tid < n_t) v[q] = ld_hit(hits + begin + q * AT + tid);
+            if (q * NT + tid < n_t) v[q] = ld_hit(hits + begin + q * NT + tid);
 #pragma unroll
         for (int q = 0; q < OWN; ++q) {
-            const uint32_t e = q * AT + tid;
+            const uint32_t e = q * NT + tid;
             tots[q] = 0;
             const uint32_t top = __reduce_max_sync(0xffffffffu, e < n_t ? (uint32_t)(hit_toa(v[q]) - base) : 0u);
             if (lane == 0 && e < n_t) atomicMax(&S.cnt[1][e / A_STEP], top);   // (a warp's hits share a chunk)
@@ -842,7 +896,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
         // keys relative to the segment's smallest ToA (which hold its ToAs
         // unless they span 2^32 ticks: an error)
         uint64_t m = ~0ull, mx = 0;
-        for (uint32_t i = tid; i < g.n; i += AT) {
+        for (uint32_t i = tid; i < g.n; i += NT) {
             const uint64_t a = hit_toa(ld_hit(hits + i));
             m = a < m ? a : m;
             mx = a > mx ? a : mx;
@@ -851,7 +905,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
         mx = warp_max_u64(mx);
         if (lane == 0) { S.m64[0][warp] = m; S.m64[1][warp] = mx; }
         __syncthreads();
-        for (int q = 0; q < AW; ++q) {
+        for (int q = 0; q < (NT / 32); ++q) {
             m = S.m64[0][q] < m ? S.m64[0][q] : m;
             mx = S.m64[1][q] > mx ? S.m64[1][q] : mx;
         }
@@ -859,13 +913,13 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
         base = m;
     }
     {
-        kmin = __reduce_min_sync(0xffffffffu, S.red[0][min(lane, AW - 1)]);
+        kmin = __reduce_min_sync(0xffffffffu, S.red[0][min(lane, (NT / 32) - 1)]);
         kmax = __reduce_max_sync(0xffffffffu, S.cnt[1][min(lane, (int)ACHUNKS - 1)]);
     }
     const uint32_t lo = kmin > dt ? kmin - dt : 0u;       // earlier hits below it join nothing here
     const uint64_t hi = (uint64_t)kmax + dt;
     if (!DIRECT && warp == 0) {
-        const uint32_t cmin = __reduce_min_sync(0xffffffffu, S.red[1][min(lane, AW - 1)]);
+        const uint32_t cmin = __reduce_min_sync(0xffffffffu, S.red[1][min(lane, (NT / 32) - 1)]);
         if (lane < (int)ACHUNKS) info.cmax[lane] = base + S.cnt[1][lane];
         if (lane == 0) {
             Seg &gw = w.seg[0];
@@ -884,9 +938,9 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
     for (bool first = true;; first = false) {
         if (!first) {               // (redo) the earlier hits so far are joined: the next ones beside the own hits
             __syncthreads();
-            C.clear(S);
+            C.clear<NT>(S);
             __syncthreads();
-            for (uint32_t e = tid; e < n_t; e += AT) {
+            for (uint32_t e = tid; e < n_t; e += NT) {
                 const tpc_hit *h = hits + begin + e;
                 const uint4 v = ld_hit(h);
                 const uint32_t code = C.code(clamp_pix(v.x, W, H));
@@ -905,7 +959,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
             uint32_t kk[A_HPER], pp[A_HPER], mask[A_HPER], sum = 0;
 #pragma unroll
             for (int u = 0; u < A_HPER; ++u) {
-                const uint4 v = ld_hit(hits + a + u * AT + tid);
+                const uint4 v = ld_hit(hits + a + u * NT + tid);
                 const uint64_t rel = hit_toa(v) - base;
                 kk[u] = (uint32_t)rel;
                 pp[u] = C.code(clamp_pix(v.x, W, H));
@@ -914,10 +968,10 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
             }
             if (lane == 0) S.turn[buf][warp] = sum | (mask[0] ? 0x80000000u : 0u);
             __syncthreads();
-            const uint32_t c = lane < AW ? S.turn[buf][lane] : 0u;
+            const uint32_t c = lane < (NT / 32) ? S.turn[buf][lane] : 0u;
             buf ^= 1u;   // the next round's barrier separates this one's reads from the round after
             const uint32_t total = __reduce_add_sync(0xffffffffu, c & 0x7FFFFFFFu);
-            const bool oldest = __any_sync(0xffffffffu, c >> 31);   // some of the oldest AT positions matter
+            const bool oldest = __any_sync(0xffffffffu, c >> 31);   // some of the oldest NT positions matter
             if (n_e + total > A_ENT) {   // no room beside the staged ones
                 if (!DIRECT) done = redo = true;
                 break;
@@ -928,7 +982,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
                 if ((mask[u] >> lane) & 1u) {
                     const uint32_t i = e + __popc(mask[u] & lanes_below());
                     S.kc[i] = make_uint2(kk[u], pp[u]);
-                    SS.pos[i] = (uint16_t)(a + u * AT + tid);
+                    SS.pos[i] = (uint16_t)(a + u * NT + tid);
                     C.set(S, pp[u]);
                 }
                 e += __popc(mask[u]);
@@ -941,23 +995,25 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
         }
         auto near = [&](uint32_t a, uint32_t b) { return absdiff(a, b) <= dt; };
         if (DIRECT) {   // every pair, own or not, is an edge of the graph
-            arrival_links(S, C, n_e, near, [&](uint32_t e, uint32_t o, bool &) {
+            arrival_links<NT>(S, C, n_e, near, [&](uint32_t e, uint32_t o, bool &) {
                 gunion(w.gpar, w.root_of[SS.pos[e]], w.root_of[SS.pos[o]]);
             });
         } else {
-            arrival_links(S, C, n_e, near, [&](uint32_t e, uint32_t o, bool &linked) { join_hits(S, e, o, linked); });
+            arrival_links<NT>(S, C, n_e, near, [&](uint32_t e, uint32_t o, bool &linked) { join_hits(S, e, o, linked); });
             __syncthreads();
             redo |= S.nxtra > A_XTRA;
             uint32_t tsum = 0;
 #pragma unroll
             for (int q = 0; q < OWN; ++q) {
-                if (q * AT + tid < n_t) S.tot()[q * AT + tid] = (uint16_t)tots[q];
+                const uint32_t e = q * NT + tid;
+                if (e < n_t) S.where()[e] = (uint32_t)SS.pos[e] << 16 | tots[q];
                 tsum += tots[q];
             }
+            for (uint32_t e = n_t + tid; e < n_e; e += NT) S.where()[e] = (uint32_t)SS.pos[e] << 16;
             tsum = __reduce_add_sync(0xffffffffu, tsum);
             if (lane == 0) atomicAdd(&S.tsum, tsum);
             __syncthreads();
-            arrival_clusters(w, g, t, S, C, n_e, SS.pos, 0u, base);   // (at most TILE clusters)
+            arrival_clusters<NT>(w, g, t, S, C, n_e, 0u, base);   // (at most TILE clusters)
         }
         if (done) break;
     }
@@ -1278,11 +1334,11 @@ __global__ void __launch_bounds__(AE) k_arrival_emit(Work w) {
 // CTA t for tile t, with cluster barriers between the stages.  `seg`: the
 // step's segment for callers that queue no copy of it (tpc_cluster_static);
 // otherwise it is in w.seg.
-__global__ void __launch_bounds__(AT, 1) k_arrival_step(Work w, Seg seg, uint32_t given, uint32_t tile_cap, uint64_t *counts,
+__global__ void __launch_bounds__(ST, 1) k_arrival_step(Work w, Seg seg, uint32_t given, uint32_t tile_cap, uint64_t *counts,
                                                      uint32_t keep) {
     extern __shared__ __align__(16) unsigned char a_raw[];
     SmallShared &S = *reinterpret_cast<SmallShared *>(a_raw);
-    __shared__ uint32_t s_red[AW];
+    __shared__ uint32_t s_red[ST / 32];
     __shared__ uint32_t s_cnt[2];
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const uint32_t t = blockIdx.x;
@@ -1304,7 +1360,7 @@ __global__ void __launch_bounds__(AT, 1) k_arrival_step(Work w, Seg seg, uint32_
     const bool mine = t < nt;
     if (mine) {
         if (tid == 0) w.tile_seg[t] = 0;
-        small_tile<false>(w, t, S);
+        small_tile<ST, false>(w, t, S);
     }
     cluster.sync();
     if (mine) {
@@ -1319,19 +1375,19 @@ __global__ void __launch_bounds__(AT, 1) k_arrival_step(Work w, Seg seg, uint32_
             m = warp_max_u64(m);
             if (lane == 0 && ((hc && m >= info.lo) || info.nx > A_PAIRS)) w.atile[t].redo = 1u;
         }
-        join_pairs<AT>(w, t);
+        join_pairs<ST>(w, t);
     }
     if (t == 0 && tid == 0) seg_close(g, P);
     cluster.sync();
     bool redo = false;
     for (uint32_t i = 0; i < nt; ++i) redo |= *const_cast<volatile uint32_t *>(&w.atile[i].redo) != 0;
     if (redo) {
-        if (mine && *const_cast<volatile uint32_t *>(&w.atile[t].redo)) small_tile<true>(w, t, S);
+        if (mine && *const_cast<volatile uint32_t *>(&w.atile[t].redo)) small_tile<ST, true>(w, t, S);
         cluster.sync();
     }
-    if (mine) root_tile<AT>(w, t, g.ss != nullptr);
+    if (mine) root_tile<ST>(w, t, g.ss != nullptr);
     cluster.sync();
-    if (mine) label_tile<AT>(w, t, g, reinterpret_cast<uint32_t *>(a_raw), s_cnt);
+    if (mine) label_tile<ST>(w, t, g, reinterpret_cast<uint32_t *>(a_raw), s_cnt);
     cluster.sync();
     const uint32_t *cnt = w.tile_cnt, cap = P.tile_cap;
     if (mine) {
@@ -1343,7 +1399,7 @@ __global__ void __launch_bounds__(AT, 1) k_arrival_step(Work w, Seg seg, uint32_
         }
         uint32_t begin, end;
         tile_range(g, t, begin, end);
-        emit_tile<AT>(w, t, g, begin, end, rec, cnt[t], fin, g.n - all, s_red, reinterpret_cast<uint16_t *>(a_raw));
+        emit_tile<ST>(w, t, g, begin, end, rec, cnt[t], fin, g.n - all, s_red, reinterpret_cast<uint16_t *>(a_raw));
         if (t + 1 == nt && tid == 0) emit_totals(g, P, rec + cnt[t], all);
     } else if (nt == 0 && t == 0 && tid == 0) {
         emit_totals(g, P, 0, 0);
@@ -1358,7 +1414,7 @@ __global__ void __launch_bounds__(AT, 1) k_arrival_step(Work w, Seg seg, uint32_
 }
 
 cudaError_t init_arrival_attributes() {
-    cudaError_t e = cudaFuncSetAttribute(k_arrival_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_arrival_tile<AT>, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMEM);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_arrival_step, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMALL_SMEM);
     if (e == cudaSuccess)   // clusters of 16 (a GPC of this GPU has 16 SMs and more)
@@ -1369,7 +1425,7 @@ cudaError_t init_arrival_attributes() {
 // Links and the decision; `sorted` (0: none) is the conditional node that
 // holds the time-sorted path.
 void launch_arrival_link(const Work &w, cudaGraphConditionalHandle sorted, const Launch &L) {
-    k_arrival_tile<<<L.fit(k_arrival_tile, AT, A_SMEM, G_LINK), AT, A_SMEM, L.stream>>>(w);
+    k_arrival_tile<AT><<<L.fit(k_arrival_tile<AT>, AT, A_SMEM, G_LINK), AT, A_SMEM, L.stream>>>(w);
     L.mark("k_arrival_tile");
     k_arrival_cross<<<L.fit(k_arrival_cross, AX, 0, G_LINK), AX, 0, L.stream>>>(w, sorted);
     L.mark("k_arrival_cross");
@@ -1392,7 +1448,7 @@ cudaError_t launch_arrival_step(const Work &w, const Seg *seg, uint32_t tiles, u
     while (ctas < tiles) ctas *= 2;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(ctas);
-    cfg.blockDim = dim3(AT);
+    cfg.blockDim = dim3(ST);
     cfg.dynamicSmemBytes = A_SMALL_SMEM;
     cfg.stream = L.stream;
     cudaLaunchAttribute a{};
