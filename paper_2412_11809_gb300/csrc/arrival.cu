@@ -1025,14 +1025,18 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
     }
 }
 
-// Joins the listed pairs of a tile.
+// Joins the listed pairs of a tile, `first` of NT threads.  Many pairs join the
+// same two clusters: of a warp's pairs that do, one thread joins them.
 template <int NT>
-__device__ __forceinline__ void join_pairs(const Work &w, uint32_t t) {
+__device__ __forceinline__ void join_pairs(const Work &w, uint32_t t, uint32_t first) {
     const uint32_t nx = min(w.atile[t].nx, (uint32_t)A_PAIRS);
     const uint2 *list = w.xlist + (size_t)t * A_PAIRS;
-    for (uint32_t i = threadIdx.x; i < nx; i += NT) {
+    volatile uint32_t *par = w.gpar;
+    for (uint32_t i = first; i < nx; i += NT) {
         const uint2 p = list[i];
-        gunion(w.gpar, p.x, w.root_of[p.y]);
+        const uint32_t a = par[p.x], b = par[w.root_of[p.y]];
+        const uint32_t same = __match_any_sync(__activemask(), (unsigned long long)a << 32 | b);
+        if (a != b && __ffs(same) - 1 == (int)(threadIdx.x & 31)) gunion(w.gpar, a, b);
     }
 }
 
@@ -1041,7 +1045,10 @@ __device__ __forceinline__ void join_pairs(const Work &w, uint32_t t) {
 // up to all hits; and a tile saw every earlier hit within dt of its interval
 // if it counted as many of them as its predecessor counted own hits that
 // late (which are all there are, if dt reaches no further back than the
-// predecessor's interval).
+// predecessor's interval).  A warp per tile: the few pairs of a tile of time
+// (six of 64 Mi hits) are one chain of dependent reads, and with a CTA per tile
+// too few of them were under way (96 us, 39 with a warp and one join per
+// distinct pair of clusters).
 constexpr int AX = 256;
 
 __global__ void __launch_bounds__(AX) k_arrival_cross(Work w, cudaGraphConditionalHandle sorted) {
@@ -1052,18 +1059,16 @@ __global__ void __launch_bounds__(AX) k_arrival_cross(Work w, cudaGraphCondition
     bool fail = __syncthreads_or(lost);
     if (!fail) {
         const uint32_t nt = P.ntiles;
-        for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
-            if (tid == 0) {
-                const Seg &g = w.seg[w.tile_seg[t]];
-                if (t > g.tile0) {
-                    const ATile &info = w.atile[t], &prev = w.atile[t - 1];
-                    fail |= info.nhalo != prev.ntail || (t - 1 > g.tile0 && info.cut < prev.cut + g.dt);
-                }
+        for (uint32_t t = (blockIdx.x * AX + tid) / 32; t < nt; t += gridDim.x * (AX / 32)) {
+            const Seg &g = w.seg[w.tile_seg[t]];
+            if (t > g.tile0) {   // (every lane)
+                const ATile &info = w.atile[t], &prev = w.atile[t - 1];
+                fail |= info.nhalo != prev.ntail || (t - 1 > g.tile0 && info.cut < prev.cut + g.dt);
             }
-            join_pairs<AX>(w, t);
+            join_pairs<32>(w, t, tid & 31);
         }
     }
-    if (fail && tid == 0) {
+    if (fail && (tid & 31) == 0) {
         atomicMax(&P.raw_fail, RAW_COVER);
         if (sorted) cudaGraphSetConditional(sorted, 1u);
     }
@@ -1106,6 +1111,9 @@ __global__ void __launch_bounds__(256) k_arrival_roots(Work w) {
 // Labels of the hits at a tile's positions.  Their clusters are mostly tile
 // clusters of this time tile and the two beside it: those tiles' labels are
 // gathered once into shared memory (if they fit), then looked up per hit.
+// Bound by DRAM and the two dependent reads behind a table entry; the hits'
+// clusters are read beside those (64 Mi hits: 311 us after them, 247 so, for
+// 256 MB read, 512 MB written and the clusters' slots).
 constexpr uint32_t AL_CAP = 4096;
 
 template <int NT>
@@ -1124,6 +1132,13 @@ __device__ __forceinline__ void label_tile(const Work &w, uint32_t t, const Seg 
     const uint32_t n0 = t > g.tile0 ? w.atile[t - 1].nroots : 0, n1 = w.atile[t].nroots;
     const uint32_t n2 = t + 1 < g.tile0 + g.ntiles ? w.atile[t + 1].nroots : 0;
     const bool table = n0 + n1 + n2 <= AL_CAP;
+    constexpr int ITEMS = TILE / NT;
+    uint32_t cc[ITEMS];   // the hits' clusters, on their way while the table is filled
+#pragma unroll
+    for (int q = 0; q < ITEMS; ++q) {
+        const uint32_t pos = begin + q * NT + threadIdx.x;
+        cc[q] = pos < end ? w.root_of[pos] : 0u;
+    }
     // c in [c0, c0 + n0), [c1, c1 + n1), [c2, c2 + n2): s_lab[c - c0], s_lab[n0 + c - c1], ...
     const uint32_t c1 = t * TILE, c0 = c1 - TILE, c2 = c1 + TILE;
     if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
@@ -1133,13 +1148,12 @@ __device__ __forceinline__ void label_tile(const Work &w, uint32_t t, const Seg 
     __syncthreads();
     const bool direct = g.ss == nullptr;   // one-shot: every hit is final
     uint32_t c_label = 0, c_closed = 0;
-    constexpr int ITEMS = TILE / NT;
-#pragma unroll 8
+#pragma unroll
     for (int q = 0; q < ITEMS; ++q) {
         const uint32_t pos = begin + q * NT + threadIdx.x;
         bool is_label = false, closed = false;
         if (pos < end) {
-            const uint32_t c = w.root_of[pos];
+            const uint32_t c = cc[q];
             uint32_t v;
             if (table && c - c1 < n1) v = s_lab[n0 + c - c1];
             else if (table && c - c0 < n0) v = s_lab[c - c0];
@@ -1182,11 +1196,14 @@ __global__ void __launch_bounds__(256) k_arrival_labels(Work w) {
 // Records in label order (and, streaming, the finalised hits and the carry).
 // CTAs take contiguous tiles and sum the counts of their segment's earlier
 // tiles themselves: a sum over 16384 counts costs less than a launch and the
-// one-CTA scan it replaces.
-constexpr int AE = 256;
+// one-CTA scan it replaces.  Bound by the chain from a flag word to its
+// record: small CTAs, so that more tiles are under way (64 Mi hits: 125 us with
+// 256 threads, 110 with 128).
+constexpr int AE = 128;
 
 __device__ uint32_t emit_sum(const uint32_t *cnt, uint32_t n, uint32_t *s_red) {
     uint32_t m = 0;
+#pragma unroll 8
     for (uint32_t i = threadIdx.x; i < n; i += AE) m += cnt[i];
     m = __reduce_add_sync(0xffffffffu, m);
     __syncthreads();
@@ -1261,25 +1278,29 @@ __device__ __forceinline__ void emit_tile(const Work &w, uint32_t t, const Seg &
         g.out_rec[rec + i] = out;
     }
     if (g.ss) {
+        // a warp takes the 32 positions of a word together
         const bool fits = open_total <= g.carry_cap;
-        const bool vw = threadIdx.x < nwords;
-        const uint32_t cl = vw ? w.flag_closed[(begin >> 5) + threadIdx.x] : 0;
-        uint32_t closed = fin + emit_prefix(cl, s_red);
-        if (vw) {
-            const uint32_t first = begin + (threadIdx.x << 5), last = min(first + 32, end);
-            for (uint32_t pos = first; pos < last; ++pos) {
-                const uint32_t local = pos - g.off;
-                if ((cl >> (pos - first)) & 1u) {
-                    if (closed < g.out_cap) {
-                        g.out_labels[closed] = w.lab_tmp[pos];
-                        if (g.out_index) g.out_index[closed] = gidx_of(g, local);
-                    }
-                    ++closed;
-                } else if (fits) {
-                    const uint32_t dst = g.carry_cap - open_total + (local - closed);
-                    g.carry_out[dst] = g.hits[local];
-                    g.carry_gidx_out[dst] = gidx_of(g, local);
+        const uint32_t cl = threadIdx.x < nwords ? w.flag_closed[(begin >> 5) + threadIdx.x] : 0;
+        const uint32_t before = emit_prefix(cl, s_red);
+        __syncthreads();   // the records have read s_pos
+        if (threadIdx.x < nwords) s_pos[threadIdx.x] = (uint16_t)before;
+        __syncthreads();
+        const int lane = threadIdx.x & 31;
+#pragma unroll 4
+        for (uint32_t k = threadIdx.x >> 5; k < nwords; k += NT / 32) {
+            const uint32_t pos = begin + 32 * k + lane, local = pos - g.off;
+            const uint32_t bits = w.flag_closed[(begin >> 5) + k];
+            const uint32_t closed = fin + s_pos[k] + __popc(bits & lanes_below());   // before this position
+            if (pos >= end) continue;
+            if ((bits >> lane) & 1u) {
+                if (closed < g.out_cap) {
+                    g.out_labels[closed] = w.lab_tmp[pos];
+                    if (g.out_index) g.out_index[closed] = gidx_of(g, local);
                 }
+            } else if (fits) {
+                const uint32_t dst = g.carry_cap - open_total + (local - closed);
+                g.carry_out[dst] = g.hits[local];
+                g.carry_gidx_out[dst] = gidx_of(g, local);
             }
         }
     }
@@ -1375,7 +1396,7 @@ __global__ void __launch_bounds__(ST, 1) k_arrival_step(Work w, Seg seg, uint32_
             m = warp_max_u64(m);
             if (lane == 0 && ((hc && m >= info.lo) || info.nx > A_PAIRS)) w.atile[t].redo = 1u;
         }
-        join_pairs<ST>(w, t);
+        join_pairs<ST>(w, t, tid);
     }
     if (t == 0 && tid == 0) seg_close(g, P);
     cluster.sync();
