@@ -87,13 +87,16 @@ constexpr int BIG_SMEM = 3 * BIG_CAP * (int)sizeof(uint32_t);
 //                      are taken again).
 //   longer             (listed by k_static_long) two warps: one looks up the
 //                      neighbours of 32 hits ahead, which no join changes,
-//                      the other joins; a sliding window of the last hits.
+//                      the other joins; a sliding window of the last hits,
+//                      which the first writes out behind them.
 // A lone warp's chain over the longest component sets the time of the step (its
 // instructions follow one another at four to five cycles each), so what can
 // be taken off that chain is: 8 M hits at 2.5 Ghits/s, longest component 6,544
 // hits, from every earlier hit within dt tested 32 at a time (9.9 ms, and 1.9
 // for components outgrowing a window of 512) to the table (2.4 ms) to the two
-// warps (2.0 ms, of which the sweep of the others beside it takes 0.9).
+// warps (1.4 ms; 1.2 with what leaves the window written by the looking one and
+// the next step's lookups read a step ahead).  It runs beside the sweep of the
+// others (0.9 ms alone): 1.3 ms for both.
 constexpr int SW_WARPS = 8;
 constexpr uint32_t SW_CAP = 512;
 constexpr uint32_t SW_TAB = 1024;
@@ -227,7 +230,7 @@ struct LongSweep {
     uint16_t up[LW_CAP];       // distance to the parent, 0 at a root (at most the hits within dt, so at most the window)
     uint16_t back[2][32 * 9];  // of a chunk's hits: distance to the latest hit within dt per pixel, 0: none
     uint32_t next1[2], next2[2];   // hits beside the hit one, two before
-    uint32_t fail, crowded, job;
+    uint32_t job;
 };
 
 // Chunk at `base` (lane = hit).
@@ -310,47 +313,62 @@ __device__ __forceinline__ void long_look(LongSweep &S, uint32_t base, uint32_t 
     __syncwarp();
 }
 
-__device__ __forceinline__ void long_join(LongSweep &S, uint32_t base, uint32_t n, const uint32_t *gv, uint32_t *parent,
-                                          uint32_t *cpar, uint32_t q0, uint32_t dt, uint32_t &lo, bool &crowded, int lane) {
-    const int g = lane / 9, d = lane - 9 * g;      // hit of the step and its neighbour pixel (lanes 27..31 idle)
-    const uint32_t cnt = n - base < 32u ? n - base : 32u;
-    // root of x, or an index before the window (whose cluster is closed)
-    auto root_of = [&](uint32_t x) -> uint32_t {
-        volatile uint16_t *up = S.up;
-        while (x >= lo) {
-            const uint32_t k = up[x % LW_CAP];
-            if (!k) break;
-            x -= k;
-        }
-        return x;
-    };
+// Root of x in the window, or an index before it (whose cluster is closed).
+__device__ __forceinline__ uint32_t long_root(LongSweep &S, uint32_t x, uint32_t lo) {
+    volatile uint16_t *up = S.up;
+    uint32_t k = x >= lo ? up[x % LW_CAP] : 0u;
+    while (k) {
+        x -= k;
+        k = x >= lo ? up[x % LW_CAP] : 0u;
+    }
+    return x;
+}
+
+// Before the chunk at `base` is joined the 32 oldest hits leave the window.
+// They and so their roots are older than dt: no join changes them any more,
+// and the looking warp can write their parents while the other goes on.
+// false: the window is too small.
+__device__ __forceinline__ bool long_leave(LongSweep &S, uint32_t base, const uint32_t *gv, uint32_t *parent, uint32_t *cpar,
+                                           uint32_t q0, uint32_t dt, bool &crowded, int lane) {
     const uint32_t k0 = S.key[base % LW_CAP];
     if (base >= SW_CAP && __any_sync(0xffffffffu, k0 - S.key[(base - SW_CAP + lane) % LW_CAP] <= dt)) crowded = true;
-    if (base >= LW_WIN) {   // the 32 oldest leave
-        const uint32_t j = base - LW_WIN + lane;
-        if (__any_sync(0xffffffffu, k0 - S.key[j % LW_CAP] <= dt)) {   // the window is too small
-            if (lane == 0) S.fail = 1u;
-            return;
-        }
-        uint32_t r = root_of(j);
-        const uint32_t to = r < lo ? (r = *reinterpret_cast<volatile uint32_t *>(&cpar[r]), gv[q0 + r]) : S.place[r % LW_CAP];
-        __syncwarp();
-        cpar[j] = r;
-        parent[S.place[j % LW_CAP]] = to;
-        __syncwarp();
-        lo = base - LW_WIN + 32;
-    }
-    const uint16_t *back = S.back[(base >> 5) & 1u];
-    const uint32_t next1 = S.next1[(base >> 5) & 1u], next2 = S.next2[(base >> 5) & 1u] | next1;
-    const uint32_t below = (1u << (9 * (g < 3 ? g : 0))) - 1u;
+    if (base < LW_WIN) return true;
+    const uint32_t j = base - LW_WIN + lane, lo = base - LW_WIN;
+    if (__any_sync(0xffffffffu, k0 - S.key[j % LW_CAP] <= dt)) return false;
+    uint32_t r = long_root(S, j, lo);
+    const uint32_t to = r < lo ? (r = *reinterpret_cast<volatile uint32_t *>(&cpar[r]), gv[q0 + r]) : S.place[r % LW_CAP];
+    __syncwarp();
+    cpar[j] = r;
+    parent[S.place[j % LW_CAP]] = to;
+    __syncwarp();
+    return true;
+}
+
+// First hit of the window while the chunk at `base` is joined.
+__device__ __forceinline__ uint32_t long_first(uint32_t base) { return base >= LW_WIN ? base - LW_WIN + 32 : 0u; }
+
+// Joins the hits of the chunk at `base`; lo: the first hit of the window.
+__device__ __forceinline__ void long_join(LongSweep &S, uint32_t base, uint32_t n, uint32_t dt, uint32_t lo, int lane) {
+    // lanes 0..26: hit g of the step and its neighbour pixel d; 27..29: hit g itself
+    const int g = lane < 27 ? lane / 9 : lane - 27;
+    const bool looks = lane < 27;
+    const uint32_t cnt = n - base < 32u ? n - base : 32u;
+    const uint16_t *back = S.back[(base >> 5) & 1u] + lane;   // (hit * 9 + d = (hit - g) * 9 + lane)
+    // hits that must wait for the one before them, the two before them (or do not exist)
+    const uint32_t none = cnt < 32u ? 0xFFFFFFFFu << cnt : 0u;
+    const uint32_t next1 = S.next1[(base >> 5) & 1u] | none, next2 = S.next2[(base >> 5) & 1u] | next1;
+    const uint32_t below = (1u << (9 * (looks ? g : 0))) - 1u;
+    auto ahead = [&](uint32_t c) -> uint32_t { return looks && c + g < cnt ? back[c * 9] : 0u; };
+    uint32_t b = ahead(0);
     for (uint32_t c = 0; c < cnt;) {
+        const uint32_t b1 = ahead(c + 1), b2 = ahead(c + 2), b3 = ahead(c + 3);   // the next step's, whatever this one takes
         const uint32_t at = c + g, i = base + at;
+        const bool wait1 = c + 1 >= 32u || ((next1 >> (c + 1)) & 1u), wait2 = c + 2 >= 32u || ((next2 >> (c + 2)) & 1u);
         uint32_t r = NO_ROOT;
-        const bool act = g < 3 && at < cnt;
-        const uint32_t b = act ? back[at * 9 + d] : 0u;
+        const uint32_t ki = S.key[i % LW_CAP];
         if (b) {
-            const uint32_t rj = root_of(i - b);
-            if (rj >= lo && S.key[i % LW_CAP] - S.key[rj % LW_CAP] <= dt) r = rj;   // its cluster is open
+            const uint32_t rj = long_root(S, i - b, lo);
+            if (rj >= lo && ki - S.key[rj % LW_CAP] <= dt) r = rj;   // its cluster is open
         }
         // hits 1 and 2 of the step must not touch what 0 and 1 change:
         // pixels nearby, a cluster
@@ -359,18 +377,14 @@ __device__ __forceinline__ void long_join(LongSweep &S, uint32_t base, uint32_t 
         const uint32_t m2 = __reduce_min_sync(0xffffffffu, g == 2 ? r : NO_ROOT);
         const uint32_t same = __match_any_sync(0xffffffffu, r);
         const uint32_t clash = __ballot_sync(0xffffffffu, r != NO_ROOT && (same & below));
-        uint32_t take = 1;
-        if (c + 1 < cnt && !((next1 >> (c + 1)) & 1u) && !(clash & (0x1FFu << 9))) {
-            take = 2;
-            if (c + 2 < cnt && !((next2 >> (c + 2)) & 1u) && !(clash & (0x1FFu << 18))) take = 3;
-        }
+        const bool two = !wait1 && !(clash & (0x1FFu << 9)), three = two && !wait2 && !(clash & (0x1FFu << 18));
         const uint32_t m = g == 0 ? m0 : g == 1 ? m1 : m2;
-        if (act && (uint32_t)g < take) {
-            if (r != NO_ROOT && r != m) S.up[r % LW_CAP] = (uint16_t)(r - m);
-            if (d == 4 && m != NO_ROOT) S.up[i % LW_CAP] = (uint16_t)(i - m);
-        }
+        const uint32_t x = looks ? r : i;   // a cluster joined, or the hit
+        if (m != NO_ROOT && x != NO_ROOT && x != m && (g == 0 || (g == 1 && two) || (g == 2 && three)))
+            S.up[x % LW_CAP] = (uint16_t)(x - m);
         __syncwarp();
-        c += take;
+        b = three ? b3 : two ? b2 : b1;
+        c += three ? 3 : two ? 2 : 1;
     }
 }
 
@@ -470,10 +484,7 @@ __global__ void __launch_bounds__(64) k_static_sweep_long(Work w, VarWork v) {
     const Seg &g = w.seg[0];
     const uint32_t nfirst = v.changed[5], nlong = v.changed[0], dt = g.dt, W = g.width, H = g.height;
     while (true) {
-        if (threadIdx.x == 0) {
-            S.job = atomicAdd(&v.changed[4], 1u);
-            S.fail = S.crowded = 0;
-        }
+        if (threadIdx.x == 0) S.job = atomicAdd(&v.changed[4], 1u);
         __syncthreads();
         const uint32_t job = S.job;
         if (job >= nlong) break;
@@ -481,8 +492,8 @@ __global__ void __launch_bounds__(64) k_static_sweep_long(Work w, VarWork v) {
         const uint2 comp = job < nfirst ? v.big[v.big_cap - 1 - job] : v.big[job - nfirst];
         const uint32_t q0 = comp.x, n = comp.y;
         uint32_t *cpar = v.cpar + q0;
-        uint32_t lo = 0, built = 0, se1 = 0, k1 = 0, p1 = 0, se2 = 0;
-        bool crowded = false;
+        uint32_t built = 0, se1 = 0, k1 = 0, p1 = 0, se2 = 0;
+        bool crowded = false, kept = true;
         if (looks) {
             se1 = gv[q0 + lane];   // (n > SW_CAP)
             k1 = skey[se1];
@@ -499,32 +510,30 @@ __global__ void __launch_bounds__(64) k_static_sweep_long(Work w, VarWork v) {
                         p1 = w.spix[se1];
                     }
                     if (e + 64 < n) se2 = gv[q0 + e + 64];
+                    if (base) kept = long_leave(S, base - 32, gv, w.parent, cpar, q0, dt, crowded, lane);
                     long_look(S, base, n, se, k, p, dt, W, H, built, lane);
+                } else {
+                    kept = long_leave(S, base - 32, gv, w.parent, cpar, q0, dt, crowded, lane);
                 }
             } else if (base) {
-                long_join(S, base - 32, n, gv, w.parent, cpar, q0, dt, lo, crowded, lane);
+                long_join(S, base - 32, n, dt, long_first(base - 32), lane);
             }
-            __syncthreads();
-            if (S.fail) break;
+            kept = __syncthreads_and(kept);
+            if (!kept) break;
         }
-        if (!looks) {
+        if (looks) {
             if (lane == 0) {
                 if (crowded) {   // diagnostics
                     atomicAdd(&v.changed[1], 1u);
                     if (n > BIG_CAP) atomicAdd(&v.changed[2], 1u);
                 }
-                if (S.fail) v.over[atomicAdd(&v.changed[3], 1u)] = comp;
+                if (!kept) v.over[atomicAdd(&v.changed[3], 1u)] = comp;
             }
-            if (!S.fail) {
-                for (uint32_t j = lo + lane; j < n; j += 32) {   // the hits still in the window
-                    uint32_t r = j;
-                    while (r >= lo) {
-                        const uint32_t k = S.up[r % LW_CAP];
-                        if (!k) break;
-                        r -= k;
-                    }
-                    w.parent[S.place[j % LW_CAP]] = r < lo ? gv[q0 + cpar[r]] : S.place[r % LW_CAP];
-                }
+        } else if (kept) {
+            const uint32_t lo = long_first((n - 1) / 32 * 32);
+            for (uint32_t j = lo + lane; j < n; j += 32) {   // the hits still in the window
+                const uint32_t r = long_root(S, j, lo);
+                w.parent[S.place[j % LW_CAP]] = r < lo ? gv[q0 + *reinterpret_cast<volatile uint32_t *>(&cpar[r])] : S.place[r % LW_CAP];
             }
         }
         __syncthreads();   // the rings are rewritten for the next component
@@ -1079,8 +1088,12 @@ Work variant_view(const Work &w, const VarWork &v) {
     return wv;
 }
 
-// The long components take as long as the sweep of all others (8 M hits of the
-// 2.5 Ghits/s stream: 2.0 and 0.9 ms), which runs beside them on `side`.
+// The sweep of the long components, a few chains, and that of all others,
+// which fills the SMs, run side by side.  The long ones follow on the step's own
+// stream, so that they are on the SMs before the others, which wait for an
+// event; the other way around they started when the others ended (8 M hits of
+// the 2.5 Ghits/s stream: 2.1 ms for both, 1.5 this way, 1.3 with the shorter
+// chain).
 cudaError_t launch_static_sweep(const Work &w, const VarWork &v, const Launch &L, const SideStream &side) {
     cudaMemsetAsync(v.work, 0, sizeof(uint32_t), L.stream);
     cudaMemsetAsync(v.changed, 0, 7 * sizeof(uint32_t), L.stream);
@@ -1090,13 +1103,13 @@ cudaError_t launch_static_sweep(const Work &w, const VarWork &v, const Launch &L
     if (e == cudaSuccess) e = cudaStreamWaitEvent(side.stream, side.fork, 0);
     if (e != cudaSuccess) return e;
     const int fit = L.fit(k_static_sweep_long, 64, LW_SMEM), few = (L.sms > 0 ? L.sms : 1) * LW_CTAS;
-    k_static_sweep_long<<<fit < few ? fit : few, 64, LW_SMEM, side.stream>>>(w, v);
-    k_static_sweep_big<<<L.fit(k_static_sweep_big, BIG_THREADS, BIG_SMEM), BIG_THREADS, BIG_SMEM, side.stream>>>(w, v);
+    k_static_sweep_long<<<fit < few ? fit : few, 64, LW_SMEM, L.stream>>>(w, v);
+    k_static_sweep<<<L.fit(k_static_sweep, SW_WARPS * 32, SW_SMEM), SW_WARPS * 32, SW_SMEM, side.stream>>>(w, v);
     e = cudaEventRecord(side.join, side.stream);
-    k_static_sweep<<<L.fit(k_static_sweep, SW_WARPS * 32, SW_SMEM), SW_WARPS * 32, SW_SMEM, L.stream>>>(w, v);
-    L.mark("k_static_sweep");
-    const cudaError_t e2 = cudaStreamWaitEvent(L.stream, side.join, 0);   // (the step goes on after both)
+    k_static_sweep_big<<<L.fit(k_static_sweep_big, BIG_THREADS, BIG_SMEM), BIG_THREADS, BIG_SMEM, L.stream>>>(w, v);
     L.mark("k_static_sweep_long");
+    const cudaError_t e2 = cudaStreamWaitEvent(L.stream, side.join, 0);   // (the step goes on after both)
+    L.mark("k_static_sweep");
     return e == cudaSuccess ? e2 : e;
 }
 
@@ -1104,6 +1117,5 @@ void launch_pixel_timelines(const Work &w, const VarWork &v, const Launch &L) {
     k_pixel_starts<<<L.fit(k_pixel_starts, 256, 0), 256, 0, L.stream>>>(w, v);
     L.mark("k_pixel_starts");
 }
-
 
 }  // namespace tpc
