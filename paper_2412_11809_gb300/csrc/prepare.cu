@@ -37,9 +37,9 @@ __global__ void k_setup(Work w, int nsegs, uint32_t arrival) {
 // count, the ToA span check, the choice of sort (the tile sort's keys are
 // relative to fast_key_base; if a ToA lies outside 2^32 ticks of that base,
 // or the check found the tiles out of order, every segment takes the
-// general sort with keys relative to its minimum ToA) and the streaming
-// watermark (seg_close).
-__global__ void k_seg_finalize(Work w) {
+// general sort with keys relative to its minimum ToA; `general`, if not 0, is
+// the graph condition it runs under) and the streaming watermark (seg_close).
+__global__ void k_seg_finalize(Work w, cudaGraphConditionalHandle general) {
     __shared__ uint32_t s_fallback;
     const uint32_t nsegs = w.prob->nsegs;
     if (threadIdx.x == 0) s_fallback = w.prob->fallback;
@@ -69,6 +69,7 @@ __global__ void k_seg_finalize(Work w) {
     if (threadIdx.x == 0 && fallback) {
         w.prob->fallback = 1u;
         w.prob->npasses = w.prob->lsd_passes;
+        if (general) cudaGraphSetConditional(general, 1u);
     }
 }
 
@@ -138,8 +139,8 @@ void launch_setup(const Work &w, int nsegs, const Launch &L, bool arrival) {
     k_setup<<<1, 1024, 0, L.stream>>>(w, nsegs, arrival);
     L.mark("k_setup");
 }
-void launch_seg_finalize(const Work &w, const Launch &L) {
-    k_seg_finalize<<<1, 256, 0, L.stream>>>(w);
+void launch_seg_finalize(const Work &w, const Launch &L, cudaGraphConditionalHandle general) {
+    k_seg_finalize<<<1, 256, 0, L.stream>>>(w, general);
     L.mark("k_seg_finalize");
 }
 void launch_make_keys(const Work &w, const Launch &L) {

@@ -231,16 +231,18 @@ struct VarSpace {
     VarWork v{};
     DevMem mem;
     size_t pos_cap = 0, pixels = 0;
+    uint64_t gen = 0;   // bumped by every (re)allocation, as the workspace's
     cudaError_t ensure(size_t positions, size_t npixels, bool global) {
         if (v.k[0] && positions <= pos_cap && npixels <= pixels) return cudaSuccess;
         mem.release();
+        ++gen;
         v = VarWork{};
         cudaError_t e = cudaSuccess;
         for (int i = 0; i < 2; ++i) {
             v.k[i] = mem.alloc<uint32_t>(positions, e);
             v.v[i] = mem.alloc<uint32_t>(positions, e);
         }
-        v.changed = mem.alloc<uint32_t>(8, e);
+        v.changed = mem.alloc<uint32_t>(ROUNDS_STATUS + ROUNDS_WORDS, e);
         v.prob = mem.alloc<Prob>(1, e);
         if (global) {
             const size_t tiles = positions / TILE + 2;
@@ -255,7 +257,7 @@ struct VarSpace {
             v.clast = mem.alloc<uint32_t>(positions, e);
             v.pstate = mem.alloc<uint4>(positions, e);
             v.tline = mem.alloc<uint4>(positions, e);
-            v.ecount = mem.alloc<unsigned long long>(2, e);
+            v.ecount = mem.alloc<unsigned long long>(3, e);
             // open edges: 2 per position per list (the first round of the
             // 2.5 Ghits/s Timepix4 stream leaves 0.64 per hit open, later
             // rounds fewer); a round that finds more marks the overflow and
@@ -310,7 +312,7 @@ __global__ void k_iota_u64(uint64_t *out, uint64_t base, size_t n) {
 // time-sorted path behind it, in arrival order alone (small steps), or
 // time-sorted from the start (launch choices that name a sorted link kernel,
 // time windows the arrival-order keys cannot hold).
-enum StepMode { STEP_ARRIVAL, STEP_SMALL, STEP_SORTED };
+enum StepMode { STEP_ARRIVAL, STEP_SMALL, STEP_SORTED, STEP_VARIANT };   // (STEP_VARIANT: (b), (c))
 
 struct tpc_ctx {
     int device = 0;
@@ -343,7 +345,7 @@ struct tpc_ctx {
 
     Workspace ws;
     VarSpace vs;                   // variants (b), (c)
-    uint32_t *h_flag = nullptr;    // pinned: (b) round result ([0..1]) and list size ([2..3]); (c) counters
+    uint32_t *h_flag = nullptr;    // pinned: (b) end of the rounds; (c) counters
     DevMem outmem;                 // output buffers
     uint64_t *d_labels = nullptr, *d_index = nullptr;
     tpc_cluster *d_rec = nullptr;
@@ -384,6 +386,7 @@ struct tpc_ctx {
     int graph_nsegs = 0;
     StepMode graph_mode{};         // the path the graph starts on
     uint64_t graph_gen = 0;        // workspace generation the graph was captured on
+    uint64_t graph_vgen = 0;       // ... and of the (b)/(c) arrays
     int graph_grid = 0;
     Tuning graph_tune{};           // launch choices the graph was captured with
 
@@ -464,16 +467,64 @@ cudaError_t upload_segs(tpc_ctx *c, const Work &w, const Seg *segs, int nsegs, c
     return cudaEventRecord(c->seg_ev[slot], st);
 }
 
+// What orders the hits if the tile sort did not (the kernels return at once if it did).
+void enqueue_general_sort(const Work &w, const Launch &L) {
+    launch_make_keys(w, L);
+    for (int pass = 0; pass < 4; ++pass) launch_radix_pass(w, pass, L);
+    launch_gather(w, L);
+}
+
 // The time-sorted path, after the set-up.
 void enqueue_sorted(const Work &w, const Launch &L) {
     launch_sort_fast(w, L);
     launch_seg_finalize(w, L);
-    launch_make_keys(w, L);
-    for (int pass = 0; pass < 4; ++pass) launch_radix_pass(w, pass, L);
-    launch_gather(w, L);
+    enqueue_general_sort(w, L);
     launch_link(w, L);
     launch_features(w, L);
     launch_outputs(w, L);
+}
+
+// A condition of the graph that L.stream is capturing, off unless a kernel sets
+// it, and a node on that stream that runs what body(Launch) queues if it is set.
+cudaError_t new_condition(const Launch &L, cudaGraphConditionalHandle &cond) {
+    cudaStreamCaptureStatus status;
+    cudaGraph_t graph = nullptr;
+    const cudaError_t e = cudaStreamGetCaptureInfo(L.stream, &status, nullptr, &graph, nullptr, nullptr, nullptr);
+    return e == cudaSuccess ? cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault) : e;
+}
+
+template <class Body>
+cudaError_t capture_if(const Launch &L, cudaGraphConditionalHandle cond, Body body) {
+    cudaStreamCaptureStatus status;
+    cudaGraph_t graph = nullptr;
+    const cudaGraphNode_t *deps = nullptr;
+    const cudaGraphEdgeData *edges = nullptr;
+    size_t ndeps = 0;
+    cudaError_t e = cudaStreamGetCaptureInfo(L.stream, &status, nullptr, &graph, &deps, &edges, &ndeps);
+    if (e != cudaSuccess) return e;
+    cudaGraphNodeParams p{};
+    p.type = cudaGraphNodeTypeConditional;
+    p.conditional.handle = cond;
+    p.conditional.type = cudaGraphCondTypeIf;
+    p.conditional.size = 1;
+    cudaGraphNode_t node = nullptr;
+    e = cudaGraphAddNode(&node, graph, deps, edges, ndeps, &p);
+    if (e != cudaSuccess) return e;
+    cudaStream_t st;
+    e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = cudaStreamBeginCaptureToGraph(st, p.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                      cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        Launch B = L;
+        B.stream = st;
+        body(B);
+        cudaGraph_t same = nullptr;
+        e = cudaStreamEndCapture(st, &same);
+    }
+    cudaStreamDestroy(st);
+    if (e != cudaSuccess) return e;
+    return cudaStreamUpdateCaptureDependencies(L.stream, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
 }
 
 // A whole step on the capturing stream L.stream: the arrival-order path and,
@@ -487,43 +538,58 @@ cudaError_t capture_step(const Work &w, int nsegs, StepMode mode, const Launch &
         return cudaGetLastError();
     }
     cudaGraphConditionalHandle cond = 0;
-    cudaStreamCaptureStatus status;
-    cudaGraph_t graph = nullptr;
-    cudaError_t e = cudaStreamGetCaptureInfo(L.stream, &status, nullptr, &graph, nullptr, nullptr, nullptr);
-    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault);
+    cudaError_t e = new_condition(L, cond);
     if (e != cudaSuccess) return e;
     launch_arrival_link(w, cond, L);
-    const cudaGraphNode_t *deps = nullptr;
-    const cudaGraphEdgeData *edges = nullptr;
-    size_t ndeps = 0;
-    e = cudaStreamGetCaptureInfo(L.stream, &status, nullptr, &graph, &deps, &edges, &ndeps);
-    if (e != cudaSuccess) return e;
-    cudaGraphNodeParams p{};
-    p.type = cudaGraphNodeTypeConditional;
-    p.conditional.handle = cond;
-    p.conditional.type = cudaGraphCondTypeIf;
-    p.conditional.size = 1;
-    cudaGraphNode_t node = nullptr;
-    e = cudaGraphAddNode(&node, graph, deps, edges, ndeps, &p);
-    if (e != cudaSuccess) return e;
-    cudaStream_t body;
-    e = cudaStreamCreateWithFlags(&body, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return e;
-    e = cudaStreamBeginCaptureToGraph(body, p.conditional.phGraph_out[0], nullptr, nullptr, 0,
-                                      cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        Launch B = L;
-        B.stream = body;
-        enqueue_sorted(w, B);
-        cudaGraph_t same = nullptr;
-        e = cudaStreamEndCapture(body, &same);
-    }
-    cudaStreamDestroy(body);
-    if (e != cudaSuccess) return e;
-    e = cudaStreamUpdateCaptureDependencies(L.stream, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
+    e = capture_if(L, cond, [&](const Launch &B) { enqueue_sorted(w, B); });
     if (e != cudaSuccess) return e;
     launch_arrival_output(w, L);
     return cudaGetLastError();
+}
+
+// The context's graph holds the step that enqueue(Launch) queues, captured
+// now if the one it has is of another step or on older arrays.
+template <class Enqueue>
+cudaError_t ensure_graph(tpc_ctx *owner, const Workspace &ws, int nsegs, StepMode mode, const Launch &L, Enqueue enqueue) {
+    if (owner->graph && owner->graph_nsegs == nsegs && owner->graph_mode == mode && owner->graph_gen == ws.gen &&
+        owner->graph_vgen == owner->vs.gen && owner->graph_grid == L.grid &&
+        std::memcmp(&owner->graph_tune, &owner->tune, sizeof(Tuning)) == 0)
+        return cudaSuccess;
+    if (owner->graph) {
+        cudaGraphExecDestroy(owner->graph);
+        owner->graph = nullptr;
+    }
+    cudaStream_t cap_st;
+    // (kernels take the priority of the stream they are captured on: above that
+    // of the side stream's)
+    int low = 0, high = 0;
+    cudaError_t e = cudaDeviceGetStreamPriorityRange(&low, &high);
+    if (e == cudaSuccess)
+        e = cudaStreamCreateWithPriority(&cap_st, cudaStreamNonBlocking, mode == STEP_VARIANT && high < low ? low - 1 : low);
+    if (e != cudaSuccess) return e;
+    cudaGraph_t g = nullptr;
+    e = cudaStreamBeginCapture(cap_st, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        Launch C = L;
+        C.stream = cap_st;
+        e = enqueue(C);
+        const cudaError_t end = cudaStreamEndCapture(cap_st, &g);
+        if (e == cudaSuccess) e = end;
+    }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&owner->graph, g, 0);
+    if (g) cudaGraphDestroy(g);
+    cudaStreamDestroy(cap_st);
+    if (e != cudaSuccess) {
+        owner->graph = nullptr;
+        return e;
+    }
+    owner->graph_nsegs = nsegs;
+    owner->graph_mode = mode;
+    owner->graph_gen = ws.gen;
+    owner->graph_vgen = owner->vs.gen;
+    owner->graph_grid = L.grid;
+    owner->graph_tune = owner->tune;
+    return cudaSuccess;
 }
 
 // One step of a context: its kernel sequence, from a CUDA graph captured on
@@ -549,37 +615,9 @@ cudaError_t run_step(tpc_ctx *owner, Workspace &ws, int nsegs, StepMode mode, cu
         else launch_arrival_output(ws.w, T);
         return cudaGetLastError();
     }
-    if (!owner->graph || owner->graph_nsegs != nsegs || owner->graph_mode != mode || owner->graph_gen != ws.gen ||
-        owner->graph_grid != L.grid || std::memcmp(&owner->graph_tune, &owner->tune, sizeof(Tuning)) != 0) {
-        if (owner->graph) {
-            cudaGraphExecDestroy(owner->graph);
-            owner->graph = nullptr;
-        }
-        cudaStream_t cap_st;
-        cudaError_t e = cudaStreamCreateWithFlags(&cap_st, cudaStreamNonBlocking);
-        if (e != cudaSuccess) return e;
-        cudaGraph_t g = nullptr;
-        e = cudaStreamBeginCapture(cap_st, cudaStreamCaptureModeThreadLocal);
-        if (e == cudaSuccess) {
-            Launch C = L;
-            C.stream = cap_st;
-            e = capture_step(ws.w, nsegs, mode, C);
-            const cudaError_t end = cudaStreamEndCapture(cap_st, &g);
-            if (e == cudaSuccess) e = end;
-        }
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&owner->graph, g, 0);
-        if (g) cudaGraphDestroy(g);
-        cudaStreamDestroy(cap_st);
-        if (e != cudaSuccess) {
-            owner->graph = nullptr;
-            return e;
-        }
-        owner->graph_nsegs = nsegs;
-        owner->graph_mode = mode;
-        owner->graph_gen = ws.gen;
-        owner->graph_grid = L.grid;
-        owner->graph_tune = owner->tune;
-    }
+    const cudaError_t e = ensure_graph(owner, ws, nsegs, mode, L,
+                                       [&](const Launch &C) { return capture_step(ws.w, nsegs, mode, C); });
+    if (e != cudaSuccess) return e;
     return cudaGraphLaunch(owner->graph, st);
 }
 
@@ -933,18 +971,66 @@ int tpc_push(tpc_ctx *c, const tpc_hit *hits, size_t n, int where) {
 static cudaError_t ensure_side(tpc_ctx *c) {
     SideStream &s = c->side;
     cudaError_t e = cudaSuccess;
-    int low = 0, high = 0;   // its CTAs are placed first: they run longest
-    if (!s.stream) e = cudaDeviceGetStreamPriorityRange(&low, &high);
-    if (e == cudaSuccess && !s.stream) e = cudaStreamCreateWithPriority(&s.stream, cudaStreamNonBlocking, high);
+    if (!s.stream) e = cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking);
     if (e == cudaSuccess && !s.fork) e = cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming);
     if (e == cudaSuccess && !s.join) e = cudaEventCreateWithFlags(&s.join, cudaEventDisableTiming);
     return e;
 }
 
-// Variants (b) and (c): the (a) forest and its roots first, then the
-// variant's kernels (csrc/variants.cu), then the shared feature / output
-// kernels.
-// Launched without a graph; (b) waits for the host between rounds.
+static cudaError_t read_rounds(tpc_ctx *c, cudaStream_t st) {
+    return cudaMemcpyAsync(c->h_flag, c->vs.v.changed + ROUNDS_STATUS, ROUNDS_WORDS * sizeof(uint32_t),
+                           cudaMemcpyDeviceToHost, st);
+}
+
+// A step of variant (b) or (c), once its segment is on the device: the (a)
+// forest and its roots first, then the variant's kernels (csrc/variants.cu),
+// then the shared feature / output kernels.
+static cudaError_t enqueue_variant(tpc_ctx *c, const Launch &L) {
+    const Work &w = c->ws.w;
+    const VarWork &v = c->vs.v;
+    const Work wv = variant_view(w, v);
+    const bool global = c->variant == TPC_GLOBAL;
+    cudaError_t e = cudaSuccess;
+    cudaGraphConditionalHandle cond = 0;
+    if (!L.tr && (e = new_condition(L, cond)) != cudaSuccess) return e;
+    launch_setup(w, 1, L);
+    launch_sort_fast(w, L);
+    launch_seg_finalize(w, L, cond);
+    if (L.tr) enqueue_general_sort(w, L);
+    else if ((e = capture_if(L, cond, [&](const Launch &B) { enqueue_general_sort(w, B); })) != cudaSuccess) return e;
+    launch_tile_border(w, L);
+    launch_sorted_roots(w, L);
+    launch_variant_keys(w, v, global, L);
+    for (int pass = 0; pass < (global ? 3 : 4); ++pass) launch_radix_pass(wv, pass, L);
+    if (global) {
+        // Rounds of the rule until the partition is closed under it, on the
+        // (a) components' dense ids: the first over every hit's 9 latest
+        // neighbours, the later ones over the edges left open; the groups'
+        // last keys are exact at the start (each group one component).
+        launch_pixel_timelines(w, v, L);
+        launch_components(w, v, L);
+        e = launch_global_rounds(w, v, true, true, L);   // (k_sorted_roots' roots hold)
+        launch_comp_parents(w, v, L);
+        if (e == cudaSuccess) e = read_rounds(c, L.stream);
+    } else {
+        e = launch_static_sweep(w, v, L, c->side);
+        launch_init_roots(w, L);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(c->h_flag, v.changed, 3 * sizeof(uint32_t), cudaMemcpyDeviceToHost, L.stream);
+    }
+    // (b) only merges, so its roots are (a) roots, whose slots the tile
+    // kernels zeroed; a (c) root can be any hit.  k_accumulate finds the
+    // roots (the parents may be deep).
+    launch_features(w, L, global);
+    launch_outputs(w, L);
+    return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
+// Variants (b) and (c): one graph, as the steps of (a).  (b) waits for it: if
+// a list of open edges overflowed, every hit's neighbours are looked at again
+// and the features summed anew.  As some fifty launches, with the host looking
+// at (b)'s flags after each round, a call with 10,000 hits took 1120 us ((b)) and
+// 1210 ((c)), mostly between kernels; 430 and 510 so.
 static int flush_variant(tpc_ctx *c, Tracer *tr) {
     const size_t n = c->pending;
     c->has_result = false;   // the workspace may move: the last result is gone
@@ -955,87 +1041,48 @@ static int flush_variant(tpc_ctx *c, Tracer *tr) {
     if (!c->bound_labels && ensure_out(c, n) != cudaSuccess) return TPC_ERR_NOMEM;
     if (!c->h_flag && host_alloc(&c->fail_alloc, (void **)&c->h_flag, 8 * sizeof(uint32_t)) != cudaSuccess)
         return TPC_ERR_NOMEM;
+    if (c->variant == TPC_STATIC && ensure_side(c) != cudaSuccess) return TPC_ERR_CUDA;
     Seg s = base_seg(c);
     s.hits = c->zc ? c->zc : c->in;
     set_outputs(c, s);
     s.gidx_base = c->pushed;
     s.n_new = (uint32_t)n;
     if (upload_segs(c, c->ws.w, &s, 1, c->stream) != cudaSuccess) return TPC_ERR_CUDA;
-    const Work &w = c->ws.w;
-    const VarWork &v = c->vs.v;
     Launch L{grid_of(c), c->stream, tr, c->sms, c->ctas_per_sm};
     L.tune = c->tune;
-    if (tr) cudaEventRecord(tr->ev[0], c->stream);
-    launch_setup(w, 1, L);
-    launch_sort_fast(w, L);
-    launch_seg_finalize(w, L);
-    launch_make_keys(w, L);
-    for (int pass = 0; pass < 4; ++pass) launch_radix_pass(w, pass, L);
-    launch_gather(w, L);
-    launch_tile_border(w, L);
-    launch_sorted_roots(w, L);
-    const Work wv = variant_view(w, v);
-    if (c->variant == TPC_STATIC) {
-        launch_variant_keys(w, v, 0, L);
-        for (int pass = 0; pass < 4; ++pass) launch_radix_pass(wv, pass, L);
-        if (ensure_side(c) != cudaSuccess || launch_static_sweep(w, v, L, c->side) != cudaSuccess) return TPC_ERR_CUDA;
-        c->vstats = tpc_variant_stats{};
-        if (cudaMemcpyAsync(c->h_flag, v.changed, 3 * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream) !=
-            cudaSuccess)
-            return TPC_ERR_CUDA;
-        c->vstats_pending = true;   // read at tpc_variant_stats, after the stream
-    } else {
-        launch_variant_keys(w, v, 1, L);
-        for (int pass = 0; pass < 3; ++pass) launch_radix_pass(wv, pass, L);
-        launch_pixel_timelines(w, v, L);
-        // Rounds of the rule until the partition is closed under it, on the
-        // (a) components' dense ids: the first over every hit's 9 latest
-        // neighbours, the later ones over the edges left open (all hits
-        // again after an overflow of the list); the groups' last keys are
-        // exact at the start (each group one component) and kept at the
-        // roots by the unions (never above the exact value), and recomputed
-        // exactly when a round merges nothing: the end is a round without
-        // merges on exact values.
-        launch_components(w, v, L);
-        bool full = true, exact = true;
-        int in = 0;
-        c->vstats = tpc_variant_stats{};
-        c->vstats_pending = false;
-        for (int round = 0;; ++round) {
-            if (round > 4096) return TPC_ERR_TIMEOUT;
-            launch_global_edges(w, v, full, round == 0, in, L);   // round 0: k_sorted_roots' roots hold
-            ++c->vstats.rounds;
-            if (full) ++c->vstats.full_rounds;
-            if (cudaMemcpyAsync(c->h_flag, v.changed, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream) !=
-                    cudaSuccess ||
-                (round == 0 && cudaMemcpyAsync(c->h_flag + 2, v.ecount, sizeof(unsigned long long),
-                                               cudaMemcpyDeviceToHost, c->stream) != cudaSuccess) ||
-                cudaStreamSynchronize(c->stream) != cudaSuccess)
-                return TPC_ERR_CUDA;
-            if (round == 0) {
-                const unsigned long long listed = *reinterpret_cast<unsigned long long *>(c->h_flag + 2);
-                c->vstats.first_open_edges = (uint32_t)std::min<unsigned long long>(listed, v.edge_cap);
-            }
-            const bool merged = c->h_flag[0] != 0, overflow = c->h_flag[1] != 0;
-            in = full ? 0 : 1 - in;   // the list just written
-            full = overflow;
-            if (merged) {
-                exact = false;
-                continue;
-            }
-            if (exact) break;
-            launch_group_last(v, L);
-            ++c->vstats.exact_checks;
-            exact = true;
-        }
-        launch_comp_parents(w, v, L);
+    if (tr) {
+        cudaEventRecord(tr->ev[0], c->stream);
+        if (enqueue_variant(c, L) != cudaSuccess) return TPC_ERR_CUDA;
+    } else if (ensure_graph(c, c->ws, 1, STEP_VARIANT, L, [c](const Launch &C) { return enqueue_variant(c, C); }) !=
+                   cudaSuccess ||
+               cudaGraphLaunch(c->graph, c->stream) != cudaSuccess) {
+        return TPC_ERR_CUDA;
     }
-    // (b) only merges, so its roots are (a) roots, whose slots the tile
-    // kernels zeroed; a (c) root can be any hit.  k_accumulate finds the
-    // roots (the parents may be deep).
-    if (c->variant == TPC_STATIC) launch_init_roots(w, L);
-    launch_features(w, L, c->variant == TPC_GLOBAL);
-    launch_outputs(w, L);
+    c->vstats = tpc_variant_stats{};
+    c->vstats_pending = c->variant == TPC_STATIC;   // read at tpc_variant_stats, after the stream
+    if (c->variant == TPC_GLOBAL) {
+        bool again = false;
+        while (true) {
+            if (cudaStreamSynchronize(c->stream) != cudaSuccess) return TPC_ERR_CUDA;
+            const uint32_t *f = c->h_flag;   // (rounds, exact recomputations, overflow, exact, edges left open, too many)
+            if (!again) c->vstats.first_open_edges = f[4];
+            c->vstats.rounds += 1 + f[0];
+            ++c->vstats.full_rounds;
+            c->vstats.exact_checks += f[1];
+            if (f[5] || c->vstats.rounds > 4096) return TPC_ERR_TIMEOUT;
+            if (!f[2]) break;
+            again = true;
+            if (launch_global_rounds(c->ws.w, c->vs.v, false, f[3] != 0, L) != cudaSuccess ||
+                read_rounds(c, c->stream) != cudaSuccess)
+                return TPC_ERR_CUDA;
+        }
+        if (again) {
+            launch_comp_parents(c->ws.w, c->vs.v, L);
+            launch_init_roots(c->ws.w, L);
+            launch_features(c->ws.w, L, true);
+            launch_outputs(c->ws.w, L);
+        }
+    }
     if (cudaGetLastError() != cudaSuccess) return TPC_ERR_CUDA;
     c->res_base = c->pushed;
     c->pushed += n;

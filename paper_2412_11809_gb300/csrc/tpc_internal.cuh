@@ -201,6 +201,8 @@ static_assert(sizeof(ATile) <= RADIX * sizeof(uint32_t) && A_PAIRS * sizeof(uint
               sizeof(RootSlot) <= sizeof(Slot), "arrival-order arrays fit the sorted path's");
 
 // Extra arrays of the (b)/(c) variants (single-segment steps only).
+constexpr uint32_t ROUNDS_STATUS = 8, ROUNDS_WORDS = 6;
+
 struct VarWork {
     uint32_t *k[2], *v[2];     // grouping radix sort: keys / sorted positions
     uint32_t *cpar;            // (c): forest over the root-grouped order
@@ -212,14 +214,17 @@ struct VarWork {
     uint32_t *cpar_d;          // (b): forest over dense ids (a group's root: its smallest id)
     uint32_t *clast0, *clast;  // (b): per dense id: its component's last key; at a group's root, the group's
     uint4 *pstate, *tline;     // (b): before a full round, per sorted position and per pixel-timeline
-                               //      entry: (sorted position, id of its group's root, the group's last
-                               //      key, its key)
-    uint32_t *changed;         // (b): [0] a round merged something, [1] the edge list overflowed;
+                               //      entry: (id of its group's root, the group's last key, its sorted
+                               //      position, its key)
+    uint32_t *changed;         // (b): [0] a round merged something, [1] its edge list overflowed, twice
+                               //      more for the rounds after; from [ROUNDS_STATUS] on the end of the
+                               //      rounds: their number, exact recomputations, overflow, whether
+                               //      the last keys are exact, edges open after the full round, too many
                                // (c): [0] components of more than 512 hits (listed in big), [1] of
                                //      those with more than 512 hits within dt, [2] of those longer
                                //      than 8192 hits, [3] outgrew the window (listed in over), [4]
                                //      next of big to sweep, [5] listed from big's end, [6] from its start
-    unsigned long long *ecount;  // (b): edges pushed to lists 0 and 1 (beyond edge_cap: overflow)
+    unsigned long long *ecount;  // (b): edges listed by a round (beyond edge_cap: overflow), three in turn
     uint2 *edges[2];           // (b): edges not merged yet (an id of h's group, an id of its neighbour's)
     uint32_t *ekey[2];         // (b): h's key of each edge
     uint32_t edge_cap;         // (b): entries each edge list holds
@@ -517,7 +522,7 @@ void launch_arrival_link(const Work &w, cudaGraphConditionalHandle sorted, const
 void launch_arrival_output(const Work &w, const Launch &L);
 cudaError_t launch_arrival_step(const Work &w, const Seg *seg, uint32_t tiles, uint32_t tile_cap, uint64_t *counts,
                                 uint32_t keep, const Launch &L);
-void launch_seg_finalize(const Work &w, const Launch &L);
+void launch_seg_finalize(const Work &w, const Launch &L, cudaGraphConditionalHandle general = 0);
 void launch_make_keys(const Work &w, const Launch &L);
 void launch_sort_fast(const Work &w, const Launch &L);
 cudaError_t init_sortfast_attributes();
@@ -539,9 +544,8 @@ struct SideStream {
 cudaError_t launch_static_sweep(const Work &w, const VarWork &v, const Launch &L, const SideStream &side);
 void launch_pixel_timelines(const Work &w, const VarWork &v, const Launch &L);
 void launch_components(const Work &w, const VarWork &v, const Launch &L);
-void launch_group_last(const VarWork &v, const Launch &L);
 void launch_comp_parents(const Work &w, const VarWork &v, const Launch &L);
-void launch_global_edges(const Work &w, const VarWork &v, int full, int flat, int in_list, const Launch &L);
+cudaError_t launch_global_rounds(const Work &w, const VarWork &v, bool flat, bool exact, const Launch &L);
 void launch_features(const Work &w, const Launch &L, bool large_clusters = false);
 void launch_outputs(const Work &w, const Launch &L);
 

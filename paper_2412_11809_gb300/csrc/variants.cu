@@ -24,6 +24,8 @@
 // after a round without merges on exact values.  The rounds join (a)
 // components, each by a dense id; per-pixel timelines come from a stable
 // radix sort of the hits by pixel.
+#include <cooperative_groups.h>
+
 #include "tpc_internal.cuh"
 
 namespace tpc {
@@ -816,22 +818,6 @@ __global__ void __launch_bounds__(256) k_timeline_state(Work w, VarWork v) {
         T[j] = v.pstate[tl[j]];
 }
 
-// Exact last keys of the groups (when a round merged nothing): reset at
-// the roots, then each id's own last key raised into its root's.
-__global__ void __launch_bounds__(256) k_group_last_reset(VarWork v) {
-    const uint32_t n = *v.ncomp;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x)
-        if (v.cpar_d[c] == c) v.clast[c] = 0;
-}
-
-__global__ void __launch_bounds__(256) k_group_last(VarWork v) {
-    const uint32_t n = *v.ncomp;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
-        const uint32_t f = gfind(v.cpar_d, c), k = v.clast0[c];
-        if (*reinterpret_cast<volatile uint32_t *>(&v.clast[f]) < k) atomicMax(&v.clast[f], k);
-    }
-}
-
 // The result on the hits' forest: each component's root hooked under its
 // group's root (an earlier position: ids follow the roots' order).
 __global__ void __launch_bounds__(256) k_comp_parents(Work w, VarWork v) {
@@ -864,15 +850,15 @@ __device__ __forceinline__ bool gunion_last(uint32_t *parent, uint32_t *glast, u
 // Append the warp's open edges (a node of h's group, a node of its
 // neighbour's group, h's key) to list `out` (one atomic per warp); on
 // overflow the list is marked and the next round takes every hit again.
-__device__ __forceinline__ void push_edges(const VarWork &v, int out, bool keep, uint32_t a, uint32_t b,
-                                           uint32_t key) {
+__device__ __forceinline__ void push_edges(const VarWork &v, int out, unsigned long long *listed, uint32_t *flags, bool keep,
+                                           uint32_t a, uint32_t b, uint32_t key) {
     uint2 *list = pick(v.edges, out);
     uint32_t *keys = pick(v.ekey, out);
     const uint32_t m = __ballot_sync(0xffffffffu, keep);
     if (!m) return;
     const int lane = threadIdx.x & 31;
     unsigned long long base = 0;   // 64 bits: a full round can push more than 2^32 edges
-    if (lane == __ffs(m) - 1) base = atomicAdd(&v.ecount[out], (unsigned long long)__popc(m));
+    if (lane == __ffs(m) - 1) base = atomicAdd(listed, (unsigned long long)__popc(m));
     base = __shfl_sync(0xffffffffu, base, __ffs(m) - 1);
     const unsigned long long slot = base + __popc(m & ((1u << lane) - 1u));
     if (keep) {
@@ -880,7 +866,7 @@ __device__ __forceinline__ void push_edges(const VarWork &v, int out, bool keep,
             list[slot] = make_uint2(a, b);
             keys[slot] = key;
         } else {
-            v.changed[1] = 1u;
+            flags[1] = 1u;
         }
     }
 }
@@ -925,7 +911,7 @@ __device__ __forceinline__ void lane_bounds(const uint32_t *tl, uint32_t (&at)[G
 // also taken together (1066, with twice the edges listed).
 constexpr int FIRST_THREADS = 128, FIRST_G = 8;
 
-__global__ void __launch_bounds__(FIRST_THREADS, 5) k_global_first(Work w, VarWork v, int out) {
+__global__ void __launch_bounds__(FIRST_THREADS, 5) k_global_first(Work w, VarWork v) {
     const Seg &g = w.seg[0];
     const uint32_t W = g.width, H = g.height, n = g.n, dt = g.dt;
     const uint32_t sel = v.prob->npasses & 1u;
@@ -965,7 +951,7 @@ __global__ void __launch_bounds__(FIRST_THREADS, 5) k_global_first(Work w, VarWo
                 }
             }
             changed |= r == 1;
-            push_edges(v, out, r == 2, rh, rl, me.w);
+            push_edges(v, 0, v.ecount, v.changed, r == 2, rh, rl, me.w);
         };
         {   // its own pixel: the entry before
             const bool has = valid && i > ps[p];
@@ -998,14 +984,13 @@ __global__ void __launch_bounds__(FIRST_THREADS, 5) k_global_first(Work w, VarWo
     if (__syncthreads_or(changed) && threadIdx.x == 0) atomicOr(&v.changed[0], 1u);
 }
 
-// A round over the open edges of list `in` only: both ends' first steps
-// up the forest at once.
-__global__ void __launch_bounds__(256) k_global_list(Work w, VarWork v, int in) {
+// A round over the `count` open edges of list `in`, those left open listed in
+// the other: both ends' first steps up the forest at once.
+__device__ __forceinline__ void list_round(const VarWork &v, int in, unsigned long long count, uint32_t dt, uint32_t *flags,
+                                           unsigned long long *listed) {
     const uint2 *list = pick(v.edges, in);
     const uint32_t *keys = pick(v.ekey, in);
-    const uint32_t dt = w.seg[0].dt;
-    const unsigned long long n = v.ecount[in];
-    const uint32_t cnt = n < v.edge_cap ? (uint32_t)n : v.edge_cap;
+    const uint32_t cnt = count < v.edge_cap ? (uint32_t)count : v.edge_cap;
     bool changed = false;
     const uint32_t stride = gridDim.x * blockDim.x;
     for (uint32_t e0 = blockIdx.x * blockDim.x; e0 < cnt; e0 += stride) {
@@ -1013,11 +998,11 @@ __global__ void __launch_bounds__(256) k_global_list(Work w, VarWork v, int in) 
         const bool valid = e < cnt;
         uint2 ed = make_uint2(0, 0);
         uint32_t ks = 0, ux = 0, uy = 0;
-        if (valid) {
-            ed = list[e];
-            ks = keys[e];
-            ux = v.cpar_d[ed.x];
-            uy = v.cpar_d[ed.y];
+        if (valid) {   // (written by other SMs in the rounds before: not from L1)
+            ed = __ldcg(list + e);
+            ks = __ldcg(keys + e);
+            ux = __ldcg(v.cpar_d + ed.x);
+            uy = __ldcg(v.cpar_d + ed.y);
         }
         int r = 0;
         uint32_t rh = ed.x, rl = ed.y;
@@ -1031,9 +1016,71 @@ __global__ void __launch_bounds__(256) k_global_list(Work w, VarWork v, int in) 
             }
         }
         changed |= r == 1;
-        push_edges(v, 1 - in, r == 2, rh, rl, ks);
+        push_edges(v, 1 - in, listed, flags, r == 2, rh, rl, ks);
     }
-    if (__syncthreads_or(changed) && threadIdx.x == 0) atomicOr(&v.changed[0], 1u);
+    if (__syncthreads_or(changed) && threadIdx.x == 0) atomicOr(flags, 1u);
+}
+
+// The rounds over the open edges after a full round (cooperative: a barrier of
+// the grid between rounds), until the partition is closed under the rule: the
+// last one merged nothing on exact last keys.  When a round merges nothing on
+// keys that may lag, the groups' last keys are made exact: reset at the roots,
+// then each id's own raised into its root's.  Ends early if a list overflowed
+// (the host starts another full round).  Flags and counts of a round rotate
+// through three slots, so that one is cleared while one is read and one written.
+// One launch for all of them: launch by launch, the host looking at the flags
+// after each, six rounds of 8 M hits took some 25 us each beside their work.
+constexpr uint32_t MAX_ROUNDS = 4096;
+
+__global__ void __launch_bounds__(256) k_global_rounds(Work w, VarWork v, uint32_t exact) {
+    cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+    const uint32_t dt = w.seg[0].dt, n = *v.ncomp, stride = gridDim.x * blockDim.x;
+    const uint32_t first = blockIdx.x * blockDim.x + threadIdx.x;
+    volatile uint32_t *flags = v.changed;
+    volatile unsigned long long *counts = v.ecount;
+    uint32_t rounds = 0, checks = 0, slot = 0, over = 0;
+    int in = 0;
+    const unsigned long long open = counts[0];
+    while (true) {   // (every thread takes the same way)
+        over = flags[2 * slot + 1];
+        if (flags[2 * slot]) {
+            exact = 0;
+        } else if (exact) {
+            over = 0;
+            break;
+        } else {
+            for (uint32_t c = first; c < n; c += stride)
+                if (__ldcg(v.cpar_d + c) == c) v.clast[c] = 0;
+            grid.sync();
+            for (uint32_t c = first; c < n; c += stride) {
+                const uint32_t f = gfind(v.cpar_d, c), k = v.clast0[c];
+                if (*reinterpret_cast<volatile uint32_t *>(&v.clast[f]) < k) atomicMax(&v.clast[f], k);
+            }
+            grid.sync();
+            exact = 1;
+            ++checks;
+        }
+        if (over || rounds == MAX_ROUNDS) break;
+        const uint32_t next = slot == 2 ? 0 : slot + 1, after = next == 2 ? 0 : next + 1;
+        if (first == 0) {
+            flags[2 * after] = flags[2 * after + 1] = 0;
+            counts[after] = 0;
+        }
+        list_round(v, in, counts[slot], dt, v.changed + 2 * next, v.ecount + next);
+        ++rounds;
+        in = 1 - in;
+        slot = next;
+        grid.sync();
+    }
+    if (first == 0) {
+        uint32_t *status = v.changed + ROUNDS_STATUS;
+        status[0] = rounds;
+        status[1] = checks;
+        status[2] = over;
+        status[3] = exact;
+        status[4] = open < v.edge_cap ? (uint32_t)open : v.edge_cap;
+        status[5] = rounds == MAX_ROUNDS;
+    }
 }
 
 void launch_components(const Work &w, const VarWork &v, const Launch &L) {
@@ -1044,33 +1091,34 @@ void launch_components(const Work &w, const VarWork &v, const Launch &L) {
     L.mark("k_components");
 }
 
-void launch_group_last(const VarWork &v, const Launch &L) {
-    k_group_last_reset<<<L.fit(k_group_last_reset, 256, 0), 256, 0, L.stream>>>(v);
-    k_group_last<<<L.fit(k_group_last, 256, 0), 256, 0, L.stream>>>(v);
-    L.mark("k_group_last");
-}
-
 void launch_comp_parents(const Work &w, const VarWork &v, const Launch &L) {
     k_comp_parents<<<L.fit(k_comp_parents, 256, 0), 256, 0, L.stream>>>(w, v);
     L.mark("k_comp_parents");
 }
 
-// One round: list `1 - in` (or, if full, every hit) into list `in`'s
-// partner.  full: out = list 0 after reading every hit.
-void launch_global_edges(const Work &w, const VarWork &v, int full, int flat, int in, const Launch &L) {
-    const int out = full ? 0 : 1 - in;
-    cudaMemsetAsync(v.changed, 0, 2 * sizeof(uint32_t), L.stream);
-    cudaMemsetAsync(v.ecount + out, 0, sizeof(unsigned long long), L.stream);
-    if (full) {
-        k_position_state<<<L.fit(k_position_state, 256, 0), 256, 0, L.stream>>>(w, v, flat);
-        k_timeline_state<<<L.fit(k_timeline_state, 256, 0), 256, 0, L.stream>>>(w, v);
-        L.mark("k_timeline_state");
-        k_global_first<<<L.fit(k_global_first, FIRST_THREADS, 0), FIRST_THREADS, 0, L.stream>>>(w, v, out);
-        L.mark("k_global_first");
-    } else {
-        k_global_list<<<L.fit(k_global_list, 256, 0), 256, 0, L.stream>>>(w, v, in);
-        L.mark("k_global_list");
-    }
+// A full round into list 0 and the rounds over the edges it leaves open.  flat:
+// the first one, where each group is one component; exact: the last keys are
+// exact (they are then).
+cudaError_t launch_global_rounds(const Work &w, const VarWork &v, bool flat, bool exact, const Launch &L) {
+    cudaMemsetAsync(v.changed, 0, 6 * sizeof(uint32_t), L.stream);
+    cudaMemsetAsync(v.ecount, 0, 3 * sizeof(unsigned long long), L.stream);
+    k_position_state<<<L.fit(k_position_state, 256, 0), 256, 0, L.stream>>>(w, v, flat);
+    k_timeline_state<<<L.fit(k_timeline_state, 256, 0), 256, 0, L.stream>>>(w, v);
+    L.mark("k_timeline_state");
+    k_global_first<<<L.fit(k_global_first, FIRST_THREADS, 0), FIRST_THREADS, 0, L.stream>>>(w, v);
+    L.mark("k_global_first");
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(L.fit(k_global_rounds, 256, 0));
+    cfg.blockDim = dim3(256);
+    cfg.stream = L.stream;
+    cudaLaunchAttribute a{};
+    a.id = cudaLaunchAttributeCooperative;
+    a.val.cooperative = 1;
+    cfg.attrs = &a;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_global_rounds, w, v, exact ? 1u : 0u);
+    L.mark("k_global_rounds");
+    return e;
 }
 
 void launch_variant_keys(const Work &w, const VarWork &v, int by_pixel, const Launch &L) {
