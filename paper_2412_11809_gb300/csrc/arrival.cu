@@ -15,7 +15,9 @@
 //   k_arrival_cross  joins tile clusters over the listed pairs, closes the
 //                    segments (watermark), and proves that every hit found its
 //                    tile and every tile the hits before it; if not, the step
-//                    takes the time-sorted path (link.cu).
+//                    takes the time-sorted path (link.cu), at once or, if tiles
+//                    only held too many hits, after both kernels have run again
+//                    for those, in parts.
 //   k_arrival_roots  adds each tile cluster's features to its cluster's.
 //   k_arrival_labels labels, closed flags and label flags per hit.
 //   k_arrival_emit   records in label order; streaming: finalised hits, the
@@ -49,9 +51,9 @@ namespace tpc {
 constexpr int AT = 512;                          // threads of k_arrival_tile (64 registers, two CTAs per SM)
 constexpr int ST = 1024;                         // ... and where a CTA has an SM to itself
 constexpr int AW = 32;                           // warps, at most
-constexpr uint32_t A_MARGIN = 1024;              // positions around the tile read at once
+constexpr uint32_t A_MARGIN = 1024, A_WIDE = 2048;   // positions around the tile read at once; for tiles taken in parts
 constexpr int A_GROUP = 2;                       // records per thread looked at while the next ones are in flight
-constexpr int A_GROUPS = (TILE + 2 * A_MARGIN) / (512 * A_GROUP);   // ... of 512 threads, at most
+constexpr int A_GROUPS = (TILE + 2 * A_WIDE) / (512 * A_GROUP);   // ... of 512 threads, at most
 constexpr uint32_t A_STEP = TILE / ACHUNKS;      // positions per further round
 constexpr uint32_t A_ENT = 5632;                 // hits staged: a tile's own and the earlier ones
 constexpr uint32_t A_WORDS = 2304;               // 256 rows of nine 30-pixel words
@@ -88,6 +90,8 @@ struct ArrivalShared {
     unsigned long long m64[2][AW];
     uint32_t cut[2];
     uint32_t nent, nown, ntail, nxtra, ncross, nlater, nroots, tsum, flag;
+    uint32_t kept_tail;              // ntail of the parts that are done
+    uint32_t from, to, numbered;     // the part of the tile's interval at hand; clusters of the parts before
     // After the links, in the place of what is no longer needed:
     __device__ uint32_t *where() { return reinterpret_cast<uint32_t *>(head); }   // [A_ENT] position << 16 | ToT per entry
     __device__ uint2 *tops() { return reinterpret_cast<uint2 *>(later); }         // [A_TOPS] roots of the tile's clusters
@@ -397,7 +401,7 @@ __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, ui
                                                  const Cells &C, uint32_t n_e, uint32_t origin, uint64_t base) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int A_PER = (A_ENT + NT - 1) / NT;
-    const uint32_t first_c = t * TILE;
+    const uint32_t first_c = t * TILE + S.numbered;
     volatile uint16_t *par = S.par;
     uint2 *tops = S.tops();
     static_assert(A_TOPS <= (uint32_t)NT && A_TOPS <= 6 * 32, "a thread per word, six words per lane");
@@ -499,7 +503,7 @@ __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, ui
     uint32_t *A = S.sums();
     const uint32_t *where = S.where();
     const uint32_t nroots = S.nroots, tsum = S.tsum, magic = C.magic();
-    if (nroots > TILE) return false;   // (nearly every hit alone, and more hits than positions)
+    if (nroots + S.numbered > TILE) return false;   // (nearly every hit alone, and more hits than positions)
     const bool streaming = g.ss != nullptr;
     const uint32_t reach = max(g.width, g.height);
     const bool slim = tsum < (1u << 19) && (unsigned long long)tsum * reach < (1ull << 32);
@@ -577,7 +581,7 @@ __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, ui
         }
         __syncthreads();
     }
-    if (tid == 0) w.atile[t].nroots = nroots;
+    if (tid == 0) w.atile[t].nroots = S.numbered += nroots;
     return true;
 }
 
@@ -605,19 +609,30 @@ __device__ __forceinline__ uint32_t arrival_cut(const Seg &g, uint32_t j, uint64
 // 10.  Two CTAs of 512 threads at 64 registers; one of 1024 takes 2906 (its
 // barriers leave nothing to run), 768 threads at 40 registers spill (2936).  Entry
 // numbers are counted again for the positions instead of kept: 2324 -> 2260.
-template <int NT>
+//
+// PARTS: the tiles that did not fit (listed by the kernel without it), their
+// intervals taken in halves (and those again, while they are half of dt or
+// longer), each one seeing the dt before it.  Every part reads as far as the
+// whole tile asks for, so what is proved of the first part's earlier hits holds
+// for the others': they are among those, or the tile's own.  8 M hits on 448x512
+// at 2.5 Ghits/s, dt 384, where no tile fits: 1100 us, 1300 time-sorted.  A
+// kernel of its own: with the parts in the loop, their state spilled (2456 us
+// for 64 Mi hits).
+template <int NT, bool PARTS>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
-    constexpr int A_ITEMS = (TILE + 2 * A_MARGIN) / NT;   // records per thread
-    static_assert(A_ITEMS * NT == TILE + 2 * (int)A_MARGIN && A_ITEMS % A_GROUP == 0, "whole rounds");
+    constexpr uint32_t MARGIN = PARTS ? A_WIDE : A_MARGIN;
+    constexpr int A_ITEMS = (TILE + 2 * MARGIN) / NT;   // records per thread
+    static_assert(A_ITEMS * NT == TILE + 2 * (int)MARGIN && A_ITEMS % A_GROUP == 0 && A_ITEMS <= 32, "whole rounds");
     extern __shared__ __align__(16) unsigned char a_raw[];
     ArrivalShared &S = *reinterpret_cast<ArrivalShared *>(a_raw);
     Prob &P = *w.prob;
-    const uint32_t nt = P.ntiles, nsegs = P.nsegs;
+    const uint32_t nt = PARTS ? (P.raw_fail == RAW_PARTS ? P.parts_count : 0u) : P.ntiles, nsegs = P.nsegs;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) {
+    for (uint32_t u = blockIdx.x; u < nt; u += gridDim.x) {
+        const uint32_t t = PARTS ? w.redo[u] : u;
         const uint32_t si = nsegs == 1 ? 0u : w.tile_seg[t];
         const Seg &g = w.seg[si];
-        if (t + gridDim.x < nt) {   // the next tile's records on their way to L2
+        if (!PARTS && t + gridDim.x < nt) {   // the next tile's records on their way to L2
             const uint32_t t1 = t + gridDim.x;
             const Seg &g1 = nsegs == 1 ? g : w.seg[w.tile_seg[t1]];
             const uint32_t p = (t1 - g1.tile0) * TILE + tid * (128u / sizeof(tpc_hit));
@@ -627,8 +642,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
         const uint64_t base = g.raw_base;
         const tpc_hit *hits = g.hits;
         const Cells C(W, H);
+        bool first = true;
+        while (true) {   // (once without PARTS)
         // ---- records around the tile --------------------------------------
-        const int32_t p0 = (int32_t)(j * TILE) - (int32_t)A_MARGIN + tid;   // position (in the segment) of record 0
+        const int32_t p0 = (int32_t)(j * TILE) - (int32_t)MARGIN + tid;   // position (in the segment) of record 0
         uint4 v[A_GROUP];
 #pragma unroll
         for (int q = 0; q < A_GROUP; ++q) {
@@ -636,26 +653,33 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
             if ((uint32_t)p < n) v[q] = ld_hit(hits + p);
         }
         if (tid == 0) {
-            S.flag = *reinterpret_cast<volatile uint32_t *>(&P.raw_fail);
-            S.nent = S.nown = S.ntail = S.nxtra = S.ncross = S.nroots = S.tsum = 0;
+            S.flag = *reinterpret_cast<volatile uint32_t *>(&P.raw_fail) > RAW_PARTS;
+            S.nent = S.nown = S.nxtra = S.nroots = S.tsum = 0;
+            if (first) S.ntail = S.kept_tail = S.ncross = S.numbered = 0;
         }
         C.clear<NT>(S);
-        if (warp < 2) {
+        if (first && warp < 2) {
             const uint32_t k = arrival_cut(g, j + warp, base, lane);
             if (lane == 0) S.cut[warp] = k;
+            if (PARTS && lane == 0) (warp ? S.to : S.from) = k;
         }
         const uint32_t n_carry = g.n_carry, limit = (W - 1u) | (H - 1u) << 16;
         __syncthreads();
         const bool last = j + 1 == g.ntiles;
-        const uint32_t cut = S.cut[0], cut1 = S.cut[1];   // own keys: cut <= key < cut1
+        if (PARTS && first) {   // halves from the start
+            if (tid == 0 && j && j + 1 < g.ntiles && S.to > S.from && S.to - S.from >= max(dt, 2u)) S.to = S.from + (S.to - S.from) / 2;
+            __syncthreads();
+        }
+        const uint32_t cut = PARTS ? S.from : S.cut[0], cut1 = PARTS ? S.to : S.cut[1];   // own keys: cut <= key < cut1
         if (S.flag) return;           // the time-sorted path takes the step
-        if (cut1 < cut) {             // no time order to speak of
+        if (S.cut[1] < S.cut[0]) {    // no time order to speak of
             if (tid == 0) P.raw_fail = RAW_UNORDERED;
             return;
         }
         const uint32_t lo = cut > dt ? cut - dt : 0u;             // earlier hits below it join nothing here
         const uint32_t span = cut1 - lo;                          // kept keys: key - lo < span
-        const uint32_t tail = last ? 0xFFFFFFFFu : cut1 > dt ? cut1 - dt : 0u;   // own hits the next tile must see
+        const uint32_t whole = S.cut[0] > dt ? S.cut[0] - dt : 0u, reach = S.cut[1] - whole;   // (PARTS) of all parts
+        const uint32_t tail = last ? 0xFFFFFFFFu : S.cut[1] > dt ? S.cut[1] - dt : 0u;   // own hits the next tile must see
         const uint32_t guard = base ? ARRIVAL_DT : 0u;
         uint32_t high = 0, bad = 0, kmin = 0xFFFFFFFFu, kmax = 0, cmin = 0xFFFFFFFFu;
         uint32_t tots[A_ITEMS / 2], staged = 0, own_sum = 0, tsum = 0, edge = 0;   // own_sum: own | tail << 16
@@ -691,8 +715,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
                         tsum += hit_tot(v[q]);
                         if (i == A_ITEMS - 1) edge |= 2u;
                     }
-                    if (i == 0) edge |= 1u;
+                    if (!PARTS && i == 0) edge |= 1u;
                 }
+                if (PARTS && i == 0 && (uint32_t)(p0 + i * NT) < n && key[q] - whole < reach) edge |= 1u;
             }
             if (h + 1 < A_ITEMS / A_GROUP) {
 #pragma unroll
@@ -716,7 +741,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
                 e0 += __popc(mask[q]);
             }
         }
-        const bool given_up = tid == 0 && *reinterpret_cast<volatile uint32_t *>(&P.raw_fail) != 0;
+        const bool given_up = tid == 0 && *reinterpret_cast<volatile uint32_t *>(&P.raw_fail) > RAW_PARTS;
         own_sum = __reduce_add_sync(0xffffffffu, own_sum);
         tsum = __reduce_add_sync(0xffffffffu, tsum);
         kmin = __reduce_min_sync(0xffffffffu, kmin);
@@ -742,11 +767,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
         // read still held some of the tile --------------------------
         const uint32_t e_far = min(S.nent, A_ENT);
         if (edge & 3u) __syncthreads();   // read by all before a round adds to it
-        const int32_t win = (int32_t)(j * TILE) - (int32_t)(A_MARGIN + A_ROUNDS * A_STEP);   // origin of positions
+        const int32_t win = (int32_t)(j * TILE) - (int32_t)(MARGIN + A_ROUNDS * A_STEP);   // origin of positions
 #pragma unroll 1
         for (int side = 0; side < 2; ++side) {
             bool more = (edge >> side) & 1u;
-            int32_t a = side ? (int32_t)((j + 1) * TILE + A_MARGIN) : (int32_t)(j * TILE) - (int32_t)(A_MARGIN + A_STEP);
+            int32_t a = side ? (int32_t)((j + 1) * TILE + MARGIN) : (int32_t)(j * TILE) - (int32_t)(MARGIN + A_STEP);
 #pragma unroll 1
             for (int r = 0; more && r < A_ROUNDS && (side ? a < (int32_t)n : a + (int32_t)A_STEP > 0); ++r) {
                 bool outer = false;
@@ -756,8 +781,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
                     uint32_t key, code;
                     uint4 x = make_uint4(0, 0, 0, 0);
                     if ((uint32_t)p < n) x = ld_hit(hits + p);
-                    if (!look(x, p, key, code)) continue;
-                    outer |= !side || key >= cut;
+                    const bool kept = look(x, p, key, code);
+                    if (PARTS && !side) outer |= (uint32_t)p < n && key - whole < reach;
+                    if (!kept) continue;
+                    outer |= side ? key >= cut : !PARTS;
                     const uint32_t e = atomicAdd(&S.nent, 1u);
                     if (e < A_ENT && e - e_far < A_FAR) {
                         S.kc[e] = make_uint2(key, code | (key >= cut ? C_OWN : 0u));
@@ -778,8 +805,32 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
         }
         const uint32_t n_e = S.nent;
         if (n_e > A_ENT || S.flag) {
-            if (tid == 0) atomicMax(&P.raw_fail, RAW_COVER);
-            return;
+            if (!PARTS) {   // left to the kernel with PARTS
+                if (tid == 0) {
+                    w.redo[atomicAdd(&P.parts_count, 1u)] = t;
+                    atomicMax(&P.raw_fail, RAW_PARTS);
+                }
+                __syncthreads();   // the counters are reset for the next tile
+                break;
+            }
+            bool lost = false;
+            __syncthreads();   // (S.nent is read by all)
+            if (tid == 0) {   // the first half of it
+                uint32_t lowest = 0xFFFFFFFFu, highest = 0;
+                for (int q = 0; q < NT / 32; ++q) {
+                    lowest = min(lowest, S.red[0][q]);
+                    highest = max(highest, S.red[1][q]);
+                }
+                const uint32_t begin = max(cut, lowest), end = min(cut1, highest + 1u);
+                const uint32_t half = end > begin ? (end - begin) / 2 : 0u;
+                S.to = begin + half;
+                S.ntail = S.kept_tail;
+                lost = n_e <= A_ENT || 2 * half < dt || !half;   // too many far hits; parts too short
+                if (lost) atomicMax(&P.raw_fail, RAW_COVER);
+            }
+            if (__syncthreads_or(lost)) return;
+            first = false;
+            continue;
         }
         ATile &info = w.atile[t];
         if (warp == 0) {
@@ -794,10 +845,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
                     atomicMin(reinterpret_cast<unsigned long long *>(&gw.chunk_min), (unsigned long long)(base + cmin));
                 atomicAdd(&gw.n_owned, S.nown);
                 if (edge & 4u) atomicOr(&P.err, E_RANGE);
-                info.base = base;
-                info.cut = cut;
-                info.nhalo = n_e - S.nown;
+                if (!PARTS || cut == S.cut[0]) {
+                    info.base = base;
+                    info.cut = cut;
+                    info.nhalo = n_e - S.nown;
+                }
                 info.ntail = S.ntail;
+                if (PARTS) S.kept_tail = S.ntail;
             }
         }
         // ---- links -----------------------------------------------------------
@@ -828,8 +882,18 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
             if (tid == 0) atomicMax(&P.raw_fail, RAW_COVER);
             return;
         }
-        if (tid == 0) info.nx = S.ncross;
-        __syncthreads();   // the counters are reset for the next tile
+        if (tid == 0) {
+            info.nx = S.ncross;
+            if (PARTS) {
+                S.from = cut1;
+                S.to = S.cut[1];
+            }
+        }
+        const bool all = !PARTS || cut1 == S.cut[1];
+        __syncthreads();   // the counters are reset for the next part, or tile
+        if (all) break;
+        first = false;
+        }
     }
 }
 
@@ -857,7 +921,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
     bool wide = dt >= A_GUARD;
     const uint32_t new0 = g.n_carry > begin ? g.n_carry - begin : 0;   // first new hit
     uint32_t kmin, kmax, tots[OWN];
-    if (tid == 0) S.nxtra = S.ncross = S.nroots = S.tsum = 0;
+    if (tid == 0) S.nxtra = S.ncross = S.nroots = S.tsum = S.numbered = 0;
     C.clear<NT>(S);
     __syncthreads();
     for (int attempt = 0;; ++attempt) {
@@ -1051,10 +1115,11 @@ __device__ __forceinline__ void join_pairs(const Work &w, uint32_t t, uint32_t f
 // distinct pair of clusters).
 constexpr int AX = 256;
 
-__global__ void __launch_bounds__(AX) k_arrival_cross(Work w, cudaGraphConditionalHandle sorted) {
+__global__ void __launch_bounds__(AX) k_arrival_cross(Work w, cudaGraphConditionalHandle otherwise, bool parts) {
     Prob &P = *w.prob;
     const int tid = threadIdx.x;
-    bool lost = P.raw_fail != 0;
+    const uint32_t failed = *reinterpret_cast<volatile uint32_t *>(&P.raw_fail);
+    bool lost = parts ? failed > RAW_PARTS : failed != 0;
     for (uint32_t s = tid; s < P.nsegs; s += AX) lost |= w.seg[s].n_owned != w.seg[s].n;
     bool fail = __syncthreads_or(lost);
     if (!fail) {
@@ -1069,10 +1134,10 @@ __global__ void __launch_bounds__(AX) k_arrival_cross(Work w, cudaGraphCondition
         }
     }
     if (fail && (tid & 31) == 0) {
-        atomicMax(&P.raw_fail, RAW_COVER);
-        if (sorted) cudaGraphSetConditional(sorted, 1u);
+        if (parts || failed != RAW_PARTS) atomicMax(&P.raw_fail, RAW_COVER);
+        if (otherwise) cudaGraphSetConditional(otherwise, !parts && failed == RAW_PARTS ? 0u : 1u);
     }
-    if (blockIdx.x == 0)
+    if (blockIdx.x == 0 && (parts || failed != RAW_PARTS))
         for (uint32_t s = tid; s < P.nsegs; s += AX) seg_close(w.seg[s], P);
 }
 
@@ -1103,7 +1168,7 @@ __device__ __forceinline__ void root_tile(const Work &w, uint32_t t, bool stream
 
 __global__ void __launch_bounds__(256) k_arrival_roots(Work w) {
     const Prob &P = *w.prob;
-    if (P.raw_fail) return;
+    if (P.raw_fail > RAW_PARTS) return;
     const uint32_t nt = P.ntiles;
     for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) root_tile<256>(w, t, w.seg[w.tile_seg[t]].ss != nullptr);
 }
@@ -1188,7 +1253,7 @@ __global__ void __launch_bounds__(256) k_arrival_labels(Work w) {
     __shared__ uint32_t s_lab[AL_CAP];   // label position in the segment, closed flag
     __shared__ uint32_t s_cnt[2];
     const Prob &P = *w.prob;
-    if (P.raw_fail) return;
+    if (P.raw_fail > RAW_PARTS) return;
     const uint32_t nt = P.ntiles;
     for (uint32_t t = blockIdx.x; t < nt; t += gridDim.x) label_tile<256>(w, t, w.seg[w.tile_seg[t]], s_lab, s_cnt);
 }
@@ -1311,7 +1376,7 @@ __global__ void __launch_bounds__(AE) k_arrival_emit(Work w) {
     __shared__ uint16_t s_pos[TILE];
     __shared__ bool s_last;
     Prob &P = *w.prob;
-    if (P.raw_fail) return;
+    if (P.raw_fail > RAW_PARTS) return;
     const uint32_t nt = P.ntiles, cap = P.tile_cap, per = (nt + gridDim.x - 1) / gridDim.x;
     const uint32_t t0 = blockIdx.x * per, t1 = min(t0 + per, nt);
     const uint32_t *cnt = w.tile_cnt;
@@ -1435,7 +1500,9 @@ __global__ void __launch_bounds__(ST, 1) k_arrival_step(Work w, Seg seg, uint32_
 }
 
 cudaError_t init_arrival_attributes() {
-    cudaError_t e = cudaFuncSetAttribute(k_arrival_tile<AT>, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_arrival_tile<AT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_arrival_tile<AT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMEM);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_arrival_step, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMALL_SMEM);
     if (e == cudaSuccess)   // clusters of 16 (a GPC of this GPU has 16 SMs and more)
@@ -1443,12 +1510,15 @@ cudaError_t init_arrival_attributes() {
     return e;
 }
 
-// Links and the decision; `sorted` (0: none) is the conditional node that
-// holds the time-sorted path.
-void launch_arrival_link(const Work &w, cudaGraphConditionalHandle sorted, const Launch &L) {
-    k_arrival_tile<AT><<<L.fit(k_arrival_tile<AT>, AT, A_SMEM, G_LINK), AT, A_SMEM, L.stream>>>(w);
-    L.mark("k_arrival_tile");
-    k_arrival_cross<<<L.fit(k_arrival_cross, AX, 0, G_LINK), AX, 0, L.stream>>>(w, sorted);
+// Links and the decision; `otherwise` (0: none) is the condition of what follows
+// if they do not cover the step: 0 the same with parts, 1 the time-sorted path.
+// parts: the tiles that did not fit.
+void launch_arrival_link(const Work &w, cudaGraphConditionalHandle otherwise, bool parts, const Launch &L) {
+    const int grid = L.fit(k_arrival_tile<AT, false>, AT, A_SMEM, G_LINK);
+    if (parts) k_arrival_tile<AT, true><<<grid, AT, A_SMEM, L.stream>>>(w);
+    else k_arrival_tile<AT, false><<<grid, AT, A_SMEM, L.stream>>>(w);
+    L.mark(parts ? "k_arrival_tile_parts" : "k_arrival_tile");
+    k_arrival_cross<<<L.fit(k_arrival_cross, AX, 0, G_LINK), AX, 0, L.stream>>>(w, otherwise, parts);
     L.mark("k_arrival_cross");
 }
 

@@ -484,17 +484,18 @@ void enqueue_sorted(const Work &w, const Launch &L) {
     launch_outputs(w, L);
 }
 
-// A condition of the graph that L.stream is capturing, off unless a kernel sets
-// it, and a node on that stream that runs what body(Launch) queues if it is set.
-cudaError_t new_condition(const Launch &L, cudaGraphConditionalHandle &cond) {
+// A condition of the graph that L.stream is capturing, `otherwise` unless a
+// kernel sets it, and a node on that stream that runs what body(Launch, value)
+// queues: value 1 if it is not 0, or, of several bodies, the one it numbers.
+cudaError_t new_condition(const Launch &L, cudaGraphConditionalHandle &cond, unsigned otherwise = 0) {
     cudaStreamCaptureStatus status;
     cudaGraph_t graph = nullptr;
     const cudaError_t e = cudaStreamGetCaptureInfo(L.stream, &status, nullptr, &graph, nullptr, nullptr, nullptr);
-    return e == cudaSuccess ? cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault) : e;
+    return e == cudaSuccess ? cudaGraphConditionalHandleCreate(&cond, graph, otherwise, cudaGraphCondAssignDefault) : e;
 }
 
 template <class Body>
-cudaError_t capture_if(const Launch &L, cudaGraphConditionalHandle cond, Body body) {
+cudaError_t capture_if(const Launch &L, cudaGraphConditionalHandle cond, int bodies, Body body) {
     cudaStreamCaptureStatus status;
     cudaGraph_t graph = nullptr;
     const cudaGraphNode_t *deps = nullptr;
@@ -505,24 +506,26 @@ cudaError_t capture_if(const Launch &L, cudaGraphConditionalHandle cond, Body bo
     cudaGraphNodeParams p{};
     p.type = cudaGraphNodeTypeConditional;
     p.conditional.handle = cond;
-    p.conditional.type = cudaGraphCondTypeIf;
-    p.conditional.size = 1;
+    p.conditional.type = bodies > 1 ? cudaGraphCondTypeSwitch : cudaGraphCondTypeIf;
+    p.conditional.size = bodies;
     cudaGraphNode_t node = nullptr;
     e = cudaGraphAddNode(&node, graph, deps, edges, ndeps, &p);
-    if (e != cudaSuccess) return e;
-    cudaStream_t st;
-    e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return e;
-    e = cudaStreamBeginCaptureToGraph(st, p.conditional.phGraph_out[0], nullptr, nullptr, 0,
-                                      cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        Launch B = L;
-        B.stream = st;
-        body(B);
-        cudaGraph_t same = nullptr;
-        e = cudaStreamEndCapture(st, &same);
+    for (int i = 0; e == cudaSuccess && i < bodies; ++i) {
+        cudaStream_t st;
+        e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+        if (e != cudaSuccess) return e;
+        e = cudaStreamBeginCaptureToGraph(st, p.conditional.phGraph_out[i], nullptr, nullptr, 0,
+                                          cudaStreamCaptureModeThreadLocal);
+        if (e == cudaSuccess) {
+            Launch B = L;
+            B.stream = st;
+            e = body(B, bodies > 1 ? i : 1);
+            cudaGraph_t same = nullptr;
+            const cudaError_t end = cudaStreamEndCapture(st, &same);
+            if (e == cudaSuccess) e = end;
+        }
+        cudaStreamDestroy(st);
     }
-    cudaStreamDestroy(st);
     if (e != cudaSuccess) return e;
     return cudaStreamUpdateCaptureDependencies(L.stream, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
 }
@@ -537,11 +540,24 @@ cudaError_t capture_step(const Work &w, int nsegs, StepMode mode, const Launch &
         enqueue_sorted(w, L);
         return cudaGetLastError();
     }
+    // k_arrival_cross decides: 0 some tiles in parts (then time-sorted if that
+    // fails), 1 time-sorted, 2 all is done
+    auto sorted = [&w](const Launch &B, int) {
+        enqueue_sorted(w, B);
+        return cudaGetLastError();
+    };
     cudaGraphConditionalHandle cond = 0;
-    cudaError_t e = new_condition(L, cond);
+    cudaError_t e = new_condition(L, cond, 2);
     if (e != cudaSuccess) return e;
-    launch_arrival_link(w, cond, L);
-    e = capture_if(L, cond, [&](const Launch &B) { enqueue_sorted(w, B); });
+    launch_arrival_link(w, cond, false, L);
+    e = capture_if(L, cond, 2, [&](const Launch &B, int way) {
+        if (way == 1) return sorted(B, 1);
+        cudaGraphConditionalHandle failed = 0;
+        const cudaError_t c = new_condition(B, failed);
+        if (c != cudaSuccess) return c;
+        launch_arrival_link(w, failed, true, B);
+        return capture_if(B, failed, 1, sorted);
+    });
     if (e != cudaSuccess) return e;
     launch_arrival_output(w, L);
     return cudaGetLastError();
@@ -606,10 +622,14 @@ cudaError_t run_step(tpc_ctx *owner, Workspace &ws, int nsegs, StepMode mode, cu
         launch_setup(ws.w, nsegs, T, mode != STEP_SORTED);
         uint32_t sorted = mode == STEP_SORTED;
         if (!sorted) {
-            launch_arrival_link(ws.w, 0, T);
-            cudaError_t e = cudaMemcpyAsync(&sorted, &ws.w.prob->raw_fail, sizeof(sorted), cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            if (e != cudaSuccess) return e;
+            for (int parts = 0; parts < 2; ++parts) {
+                launch_arrival_link(ws.w, 0, parts, T);
+                cudaError_t e = cudaMemcpyAsync(&sorted, &ws.w.prob->raw_fail, sizeof(sorted), cudaMemcpyDeviceToHost, st);
+                if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+                if (e != cudaSuccess) return e;
+                if (sorted != RAW_PARTS) break;
+            }
+            sorted = sorted > RAW_PARTS;
         }
         if (sorted) enqueue_sorted(ws.w, T);
         else launch_arrival_output(ws.w, T);
@@ -997,7 +1017,11 @@ static cudaError_t enqueue_variant(tpc_ctx *c, const Launch &L) {
     launch_sort_fast(w, L);
     launch_seg_finalize(w, L, cond);
     if (L.tr) enqueue_general_sort(w, L);
-    else if ((e = capture_if(L, cond, [&](const Launch &B) { enqueue_general_sort(w, B); })) != cudaSuccess) return e;
+    else if ((e = capture_if(L, cond, 1, [&w](const Launch &B, int) {
+                 enqueue_general_sort(w, B);
+                 return cudaGetLastError();
+             })) != cudaSuccess)
+        return e;
     launch_tile_border(w, L);
     launch_sorted_roots(w, L);
     launch_variant_keys(w, v, global, L);

@@ -126,11 +126,13 @@ struct Prob {
     uint32_t emitted;      // CTAs of the last kernel that are done
     uint32_t raw;          // the step starts on the arrival-order path
     uint32_t raw_fail;     // ... which could not cover it (RawFail): the time-sorted path takes it
+    uint32_t parts_count;  // tiles of the arrival-order path to be taken in parts (listed in redo)
 };
 
 enum RawFail : uint32_t {
-    RAW_COVER = 1u,        // a tile's hits did not fit, lay too far around it or too far in time
-    RAW_UNORDERED = 2u,    // tiles out of order in time: the general sort
+    RAW_PARTS = 1u,        // some tiles' hits did not fit at once: taken in parts (no failure yet)
+    RAW_COVER = 2u,        // a tile's hits did not fit, lay too far around it or too far in time
+    RAW_UNORDERED = 3u,    // tiles out of order in time: the general sort
 };
 
 // One tile of the arrival-order path.
@@ -393,6 +395,7 @@ __device__ __forceinline__ void setup_prob(Prob &p, uint32_t nsegs, uint32_t til
     p.emitted = 0;
     p.raw = arrival;
     p.raw_fail = 0;
+    p.parts_count = 0;
     p.err = 0;
     p.ntiles = tiles;
     if (tiles > p.tile_cap || positions > p.pos_cap) {
@@ -445,7 +448,7 @@ __device__ __forceinline__ void write_info(const Seg &seg, const Prob &prob) {
     i.n_open = g.n_open;
     i.err = P.err;
     i.npasses = P.npasses;
-    i.arrival = P.raw && !P.raw_fail;
+    i.arrival = P.raw && P.raw_fail <= RAW_PARTS;
     *out = i;
 }
 
@@ -518,7 +521,7 @@ cudaError_t init_kernel_attributes();   // once per process and device, before c
 cudaError_t init_variants_attributes();
 void launch_setup(const Work &w, int nsegs, const Launch &L, bool arrival = false);
 cudaError_t init_arrival_attributes();
-void launch_arrival_link(const Work &w, cudaGraphConditionalHandle sorted, const Launch &L);
+void launch_arrival_link(const Work &w, cudaGraphConditionalHandle otherwise, bool parts, const Launch &L);
 void launch_arrival_output(const Work &w, const Launch &L);
 cudaError_t launch_arrival_step(const Work &w, const Seg *seg, uint32_t tiles, uint32_t tile_cap, uint64_t *counts,
                                 uint32_t keep, const Launch &L);
