@@ -25,8 +25,9 @@
 //
 // Small steps (at most SMALL_TILES tiles) work for any order, so that they
 // need no sorted path behind them: tiles own hits by position and look back
-// over earlier positions, and tiles that did not look far enough are joined
-// with every earlier tile.  All of it is one launch (k_arrival_step), a
+// over earlier positions; if some did not look far enough, tiles own intervals
+// of time instead and look at every position; and if those hold too many hits
+// the tiles of positions are joined with every earlier one.  All of it is one launch (k_arrival_step), a
 // cluster of one CTA per tile.  As seven launches a call with 1,000 hits took
 // 53 us (41 of them on the host) and one with 65,536 hits 96; now 26 and 58 (64
 // with 512 threads per CTA, which left an SM's issue slots idle).
@@ -1089,6 +1090,90 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
     }
 }
 
+// Tile t of a small step whose hits are in no order: those of an interval of
+// ToAs, wherever they lie, and the hits of the dt before it.  The cuts are
+// quantiles of one sampled hit per thread, the same in both tiles that need one,
+// found by bisection with a barrier's count.  Nothing is left to prove: every
+// position is looked at.  false: more hits, pairs or clusters than a tile holds.
+// (A call with 54,685 hits in 14 tiles: 1150 us with every tile beside every
+// earlier one, 225 so.)
+template <int NT>
+__device__ __forceinline__ bool time_tile(const Work &w, uint32_t t, SmallShared &SS) {
+    ArrivalShared &S = SS.s;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const Seg &g = w.seg[0];
+    const uint32_t n = g.n, nt = g.ntiles, dt = g.dt, W = g.width, H = g.height;
+    const tpc_hit *hits = g.hits;
+    const uint64_t base = *reinterpret_cast<const volatile uint64_t *>(&g.toa_min);   // (of all tiles by now)
+    const Cells C(W, H);
+    if (tid == 0) S.nent = S.nxtra = S.ncross = S.nroots = S.tsum = S.numbered = 0;
+    C.clear<NT>(S);
+    const uint32_t sample = (uint32_t)(hit_toa(ld_hit(hits + (uint64_t)tid * n / NT)) - base);
+    uint32_t cut[2];
+#pragma unroll 1
+    for (uint32_t k = 0; k < 2; ++k) {
+        const int below = (int)((t + k) * NT / nt);   // samples below the cut
+        uint32_t lo = 0, hi = 0xFFFFFFFFu;
+        while (t + k && lo < hi) {   // the smallest key with more samples up to it
+            const uint32_t mid = lo + (hi - lo) / 2;
+            if (__syncthreads_count(sample <= mid) > below) hi = mid; else lo = mid + 1;
+        }
+        cut[k] = lo;
+    }
+    __syncthreads();
+    const bool last = t + 1 == nt;
+    const uint32_t from = cut[0], lo = from > dt ? from - dt : 0u;
+    uint32_t tsum = 0;
+    constexpr int U = 4;
+#pragma unroll 1
+    for (uint32_t p0 = 0; p0 < n; p0 += U * NT) {
+        uint4 v[U];
+        uint32_t mask[U], sum = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (p0 + u * NT + tid < n) v[u] = ld_hit(hits + p0 + u * NT + tid);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t key = (uint32_t)(hit_toa(v[u]) - base);
+            mask[u] = __ballot_sync(0xffffffffu, p0 + u * NT + tid < n && key >= lo && (last || key < cut[1]));
+            sum += __popc(mask[u]);
+        }
+        if (!sum) continue;
+        uint32_t e0 = 0;
+        if (lane == 0) e0 = atomicAdd(&S.nent, sum);
+        e0 = __shfl_sync(0xffffffffu, e0, 0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t e = e0 + __popc(mask[u] & lanes_below());
+            if (((mask[u] >> lane) & 1u) && e < A_ENT) {
+                const uint32_t key = (uint32_t)(hit_toa(v[u]) - base), code = C.code(clamp_pix(v[u].x, W, H));
+                S.kc[e] = make_uint2(key, code | (key >= from ? C_OWN : 0u));
+                SS.pos[e] = (uint16_t)(p0 + u * NT + tid);
+                C.set(S, code);
+                if (key >= from) tsum += hit_tot(v[u]);
+            }
+            e0 += __popc(mask[u]);
+        }
+    }
+    tsum = __reduce_add_sync(0xffffffffu, tsum);
+    if (lane == 0) atomicAdd(&S.tsum, tsum);
+    __syncthreads();
+    const uint32_t n_e = S.nent;
+    if (n_e > A_ENT) return false;
+    arrival_links<NT>(S, C, n_e, [&](uint32_t a, uint32_t b) { return absdiff(a, b) <= dt; },
+                      [&](uint32_t e, uint32_t o, bool &linked) { join_hits(S, e, o, linked); });
+    __syncthreads();
+    if (S.nxtra > A_XTRA) return false;
+    for (uint32_t e = tid; e < n_e; e += NT) S.where()[e] = (uint32_t)SS.pos[e] << 16 | hit_tot(ld_hit(hits + SS.pos[e]));
+    __syncthreads();
+    if (!arrival_clusters<NT>(w, g, t, S, C, n_e, 0u, base) || S.ncross > A_PAIRS) return false;
+    if (tid == 0) {
+        w.atile[t].nx = S.ncross;
+        w.atile[t].base = base;
+    }
+    return true;
+}
+
 // Joins the listed pairs of a tile, `first` of NT threads.  Many pairs join the
 // same two clusters: of a warp's pairs that do, one thread joins them.
 template <int NT>
@@ -1416,6 +1501,55 @@ __global__ void __launch_bounds__(AE) k_arrival_emit(Work w) {
     for (uint32_t s = threadIdx.x; s < P.nsegs; s += AE) write_info(w.seg[s], P);
 }
 
+// Whether the tile looked far enough: every hit before h0 is earlier than its
+// first by more than dt (first warp).
+__device__ __forceinline__ void small_check(const Work &w, uint32_t t) {
+    if (threadIdx.x >= 32) return;
+    const uint32_t lane = threadIdx.x;
+    const ATile &info = w.atile[t];
+    const uint32_t hc = info.h0 / A_STEP;   // chunks not looked at
+    uint64_t m = 0;
+    for (uint32_t i = lane; i < hc; i += 32) {
+        const uint64_t c = w.atile[i / ACHUNKS].cmax[i % ACHUNKS];
+        m = c > m ? c : m;
+    }
+    m = warp_max_u64(m);
+    if (lane == 0 && ((hc && m >= info.lo) || info.nx > A_PAIRS)) w.atile[t].redo = 1u;
+}
+
+// Tiles that are not done (between two barriers of the cluster).
+__device__ __forceinline__ bool tiles_left(const Work &w, uint32_t nt) {
+    bool any = false;
+    for (uint32_t i = 0; i < nt; ++i) any |= *const_cast<volatile uint32_t *>(&w.atile[i].redo) != 0;
+    return any;
+}
+
+// Links of a small step that tiles of positions did not cover (out of line: its
+// registers are not the usual path's).
+__device__ __noinline__ void any_order(const Work &w, uint32_t t, uint32_t nt, SmallShared &S) {
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const bool mine = t < nt;
+    cluster.sync();   // (the flags are read)
+    if (mine) {
+        const bool done = time_tile<ST>(w, t, S);
+        if (threadIdx.x == 0) w.atile[t].redo = done ? 0u : 1u;
+    }
+    cluster.sync();
+    const bool lost = tiles_left(w, nt);
+    if (mine && !lost) join_pairs<ST>(w, t, threadIdx.x);
+    cluster.sync();
+    if (!lost) return;
+    if (mine) small_tile<ST, false>(w, t, S);   // the tiles of positions again
+    cluster.sync();
+    if (mine) {
+        small_check(w, t);
+        join_pairs<ST>(w, t, threadIdx.x);
+    }
+    cluster.sync();
+    if (mine && *const_cast<volatile uint32_t *>(&w.atile[t].redo)) small_tile<ST, true>(w, t, S);
+    cluster.sync();
+}
+
 // A whole small step in one launch: a cluster of SMALL_TILES CTAs or fewer,
 // CTA t for tile t, with cluster barriers between the stages.  `seg`: the
 // step's segment for callers that queue no copy of it (tpc_cluster_static);
@@ -1428,7 +1562,7 @@ __global__ void __launch_bounds__(ST, 1) k_arrival_step(Work w, Seg seg, uint32_
     __shared__ uint32_t s_cnt[2];
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const uint32_t t = blockIdx.x;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x;
     Prob &P = *w.prob;
     Seg &g = w.seg[0];
     if (t == 0 && tid == 0) {
@@ -1444,33 +1578,16 @@ __global__ void __launch_bounds__(ST, 1) k_arrival_step(Work w, Seg seg, uint32_
     cluster.sync();
     const uint32_t nt = *const_cast<volatile uint32_t *>(&P.ntiles);
     const bool mine = t < nt;
-    if (mine) {
-        if (tid == 0) w.tile_seg[t] = 0;
-        small_tile<ST, false>(w, t, S);
-    }
+    if (mine && tid == 0) w.tile_seg[t] = 0;
+    if (mine) small_tile<ST, false>(w, t, S);
     cluster.sync();
     if (mine) {
-        if (warp == 0) {   // complete if every hit before h0 is earlier than the tile's first by more than dt
-            const ATile &info = w.atile[t];
-            const uint32_t hc = info.h0 / A_STEP;   // chunks not looked at
-            uint64_t m = 0;
-            for (uint32_t i = lane; i < hc; i += 32) {
-                const uint64_t c = w.atile[i / ACHUNKS].cmax[i % ACHUNKS];
-                m = c > m ? c : m;
-            }
-            m = warp_max_u64(m);
-            if (lane == 0 && ((hc && m >= info.lo) || info.nx > A_PAIRS)) w.atile[t].redo = 1u;
-        }
+        small_check(w, t);
         join_pairs<ST>(w, t, tid);
     }
     if (t == 0 && tid == 0) seg_close(g, P);
     cluster.sync();
-    bool redo = false;
-    for (uint32_t i = 0; i < nt; ++i) redo |= *const_cast<volatile uint32_t *>(&w.atile[i].redo) != 0;
-    if (redo) {
-        if (mine && *const_cast<volatile uint32_t *>(&w.atile[t].redo)) small_tile<ST, true>(w, t, S);
-        cluster.sync();
-    }
+    if (tiles_left(w, nt)) any_order(w, t, nt, S);
     if (mine) root_tile<ST>(w, t, g.ss != nullptr);
     cluster.sync();
     if (mine) label_tile<ST>(w, t, g, reinterpret_cast<uint32_t *>(a_raw), s_cnt);
