@@ -195,14 +195,16 @@ int tpc_batch_flush(tpc_ctx **ctxs, int n);
    least 10,000 hits per thread, Section 4.1); here the work per CTA is a
    tile of 4096 hits and these choices set how the launches fill the GPU. */
 typedef struct tpc_tuning {
-    uint8_t ctas_sort;    /* CTAs per SM of the tile sort and merge, 0 = as many as fit */
+    uint8_t ctas_sort;    /* CTAs per SM of the tile sort and merge, 0 = as many as fit
+                             (time-sorted path) */
     uint8_t ctas_link;    /* CTAs per SM of the link kernels, 0 = as many as fit */
     uint8_t ctas_acc;     /* CTAs per SM of the feature kernel, 0 = as many as fit */
     uint8_t ctas_out;     /* CTAs per SM of the label and record kernels, 0 = as many as fit */
     uint16_t acc_span;    /* positions per pass of the feature kernel: 512, 1024 or 2048
-                             (0 = 1024, the default) */
+                             (0 = 1024, the default; time-sorted path) */
     uint8_t general_link; /* bit 0: sensors the shared-memory pixel table covers at once,
-                             bit 1: sensors it covers in bands, take the general link kernel */
+                             bit 1: sensors it covers in bands, take the time-sorted path
+                             with the general link kernel */
     uint8_t order;        /* batches: 0 = contexts in the given order, 1 = most hits first */
 } tpc_tuning;             /* 8 bytes; all zero = the defaults */
 
@@ -275,9 +277,9 @@ int tpc_forest(tpc_ctx *ctx, uint32_t *parent, uint32_t *input_pos, size_t cap, 
    every hit (the first, and any after the list of open edges overflowed),
    exact recomputations of the groups' last ToA, and the edges the first
    round left open (capped at the list's size); (c) components longer than
-   a warp's shared-memory staging (512 hits), swept by one warp through a
+   a warp's shared-memory staging (512 hits), swept by two warps through a
    sliding window; of those, the ones with more than 512 hits within dt, and
-   of those the ones over 8192 hits.  (A window holds 2048 hits; components
+   of those the ones over 8192 hits.  (A window holds 960 hits; components
    with more within dt are swept again by a whole CTA, from shared memory up
    to 8192 hits, from global memory beyond.)  Waits for the context's work. */
 typedef struct tpc_variant_stats {

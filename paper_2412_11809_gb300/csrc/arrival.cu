@@ -60,7 +60,7 @@ constexpr uint32_t A_ENT = 5632;                 // hits staged: a tile's own an
 constexpr uint32_t A_WORDS = 2304;               // 256 rows of nine 30-pixel words
 constexpr uint32_t A_XTRA = 2048;                // unions beyond each hit's first
 constexpr uint32_t A_LATER = 2048;               // hits beside cells of several hits
-constexpr uint32_t A_FAR = 1024;                 // hits found beyond the margins
+constexpr uint32_t A_FAR = 1920;                 // hits found beyond the margins (all that two CTAs per SM leave room for)
 constexpr int A_JUMPS = 1;                       // path-shortening passes over the tile's forest
 constexpr int A_ROUNDS = 4;                      // further rounds on each side
 constexpr int A_BACK_ROUNDS = 16;                // rounds back of a small step's tiles
@@ -75,7 +75,7 @@ static_assert(A_WORDS <= 4096, "word indices take 12 bits");
 // the word, so a cell's slot is word.y + the set bits below it and the cells
 // of a row's neighbourhood have consecutive slots.  head[slot] is a hit of
 // the cell; further hits (a pixel hit more than once, or rows that share a
-// cell on sensors taller than R) hang on next[].  110 KB: two CTAs per SM.
+// cell on sensors taller than R) hang on next[].  113 KB: two CTAs per SM.
 struct ArrivalShared {
     uint2 word[A_WORDS];         // bits; cells before the word (minus the repeated low bit)
     uint16_t head[A_ENT];
@@ -396,10 +396,12 @@ __device__ __forceinline__ void join_hits(ArrivalShared &S, uint32_t e, uint32_t
 // features, each own hit's cluster, and the pairs with earlier tiles (earlier
 // hits in a cluster of this tile).  where()[e] (position from `origin`, ToT) of
 // the entries is staged; the caller's barrier is behind it and the links.
-// false: more clusters than the tile has numbers.
+// Earlier hits with keys from `within` on are of parts of this tile before: their
+// clusters are joined at once.  false: more clusters than the tile has numbers.
 template <int NT>
 __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, uint32_t t, ArrivalShared &S,
-                                                 const Cells &C, uint32_t n_e, uint32_t origin, uint64_t base) {
+                                                 const Cells &C, uint32_t n_e, uint32_t origin, uint64_t base,
+                                                 uint32_t within = 0xFFFFFFFFu) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int A_PER = (A_ENT + NT - 1) / NT;
     const uint32_t first_c = t * TILE + S.numbered;
@@ -525,7 +527,7 @@ __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, ui
             const uint2 kc = S.kc[e];
             const uint32_t c = cluster(q), i = c - r0, pt = where[e], at = origin + (pt >> 16);
             if (!(kc.y & C_OWN)) {
-                if (c != A_NONE && r0 == 0) {   // an earlier tile's hit in a cluster of this one
+                if (c != A_NONE && r0 == 0 && kc.x < within) {   // an earlier tile's hit in a cluster of this one
                     const uint32_t x = atomicAdd(&S.ncross, 1u);
                     if (x < A_PAIRS) w.xlist[(size_t)t * A_PAIRS + x] = make_uint2(first_c + c, at);
                 }
@@ -582,6 +584,15 @@ __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, ui
         }
         __syncthreads();
     }
+    if (within != 0xFFFFFFFFu) {
+#pragma unroll
+        for (int q = 0; q < A_PER; ++q) {
+            const uint32_t e = q * NT + tid, c = cluster(q);
+            if (e >= n_e) break;
+            const uint2 kc = S.kc[e];
+            if (!(kc.y & C_OWN) && c != A_NONE && kc.x >= within) gunion(w.gpar, first_c + c, w.root_of[origin + (where[e] >> 16)]);
+        }
+    }
     if (tid == 0) w.atile[t].nroots = S.numbered += nroots;
     return true;
 }
@@ -612,11 +623,11 @@ __device__ __forceinline__ uint32_t arrival_cut(const Seg &g, uint32_t j, uint64
 // numbers are counted again for the positions instead of kept: 2324 -> 2260.
 //
 // PARTS: the tiles that did not fit (listed by the kernel without it), their
-// intervals taken in halves (and those again, while they are half of dt or
+// intervals taken in halves (and those again, while they are a quarter of dt or
 // longer), each one seeing the dt before it.  Every part reads as far as the
 // whole tile asks for, so what is proved of the first part's earlier hits holds
 // for the others': they are among those, or the tile's own.  8 M hits on 448x512
-// at 2.5 Ghits/s, dt 384, where no tile fits: 1100 us, 1300 time-sorted.  A
+// at 2.5 Ghits/s, dt 384, where no tile fits: 1110 us, 1300 time-sorted.  A
 // kernel of its own: with the parts in the loop, their state spilled (2456 us
 // for 64 Mi hits).
 template <int NT, bool PARTS>
@@ -826,7 +837,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
                 const uint32_t half = end > begin ? (end - begin) / 2 : 0u;
                 S.to = begin + half;
                 S.ntail = S.kept_tail;
-                lost = n_e <= A_ENT || 2 * half < dt || !half;   // too many far hits; parts too short
+                lost = n_e <= A_ENT || 4 * (uint64_t)half < dt || !half;   // too many far hits; parts too short
                 if (lost) atomicMax(&P.raw_fail, RAW_COVER);
             }
             if (__syncthreads_or(lost)) return;
@@ -879,7 +890,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
             where[e] = (uint32_t)S.far[e - e_far] << 16 | hit_tot(ld_hit(hits + (win + (int32_t)S.far[e - e_far])));
         const bool listed = S.nxtra <= A_XTRA;
         __syncthreads();
-        if (!listed || !arrival_clusters<NT>(w, g, t, S, C, n_e, off + (uint32_t)win, base) || S.ncross > A_PAIRS) {
+        if (!listed || !arrival_clusters<NT>(w, g, t, S, C, n_e, off + (uint32_t)win, base, PARTS && cut != S.cut[0] ? S.cut[0] : 0xFFFFFFFFu) || S.ncross > A_PAIRS) {
             if (tid == 0) atomicMax(&P.raw_fail, RAW_COVER);
             return;
         }
