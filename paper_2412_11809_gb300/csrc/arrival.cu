@@ -624,12 +624,16 @@ __device__ __forceinline__ uint32_t arrival_cut(const Seg &g, uint32_t j, uint64
 //
 // PARTS: the tiles that did not fit (listed by the kernel without it), their
 // intervals taken in halves (and those again, while they are a quarter of dt or
-// longer), each one seeing the dt before it.  Every part reads as far as the
-// whole tile asks for, so what is proved of the first part's earlier hits holds
-// for the others': they are among those, or the tile's own.  8 M hits on 448x512
-// at 2.5 Ghits/s, dt 384, where no tile fits: 1110 us, 1300 time-sorted.  A
-// kernel of its own: with the parts in the loop, their state spilled (2456 us
-// for 64 Mi hits).
+// longer), each one seeing the dt before it.  On both sides every part reads on
+// while the outermost positions hold hits of the whole tile, its earlier ones
+// among them, whether they are the part's or not: so all parts read the same
+// positions, what is proved of the first part's earlier hits holds for the
+// others' (they are among those, or the tile's own), and an own hit that a part
+// meets was numbered by an earlier part.  (A part that reads on to the right for
+// its own hits only misses one that arrived late and belongs to an earlier part,
+// or meets one that no part numbered.)  8 M hits on 448x512 at 2.5 Ghits/s, dt
+// 384, where no tile fits: 1110 us, 1300 time-sorted.  A kernel of its own: with
+// the parts in the loop, their state spilled (2456 us for 64 Mi hits).
 template <int NT, bool PARTS>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
     constexpr uint32_t MARGIN = PARTS ? A_WIDE : A_MARGIN;
@@ -725,11 +729,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
                     if (key[q] >= cut) {
                         own_sum += key[q] >= tail && !last ? 0x10001u : 1u;
                         tsum += hit_tot(v[q]);
-                        if (i == A_ITEMS - 1) edge |= 2u;
+                        if (!PARTS && i == A_ITEMS - 1) edge |= 2u;
                     }
                     if (!PARTS && i == 0) edge |= 1u;
                 }
-                if (PARTS && i == 0 && (uint32_t)(p0 + i * NT) < n && key[q] - whole < reach) edge |= 1u;
+                if (PARTS && (i == 0 || i == A_ITEMS - 1) && (uint32_t)(p0 + i * NT) < n && key[q] - whole < reach)
+                    edge |= i ? 2u : 1u;
             }
             if (h + 1 < A_ITEMS / A_GROUP) {
 #pragma unroll
@@ -794,9 +799,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
                     uint4 x = make_uint4(0, 0, 0, 0);
                     if ((uint32_t)p < n) x = ld_hit(hits + p);
                     const bool kept = look(x, p, key, code);
-                    if (PARTS && !side) outer |= (uint32_t)p < n && key - whole < reach;
+                    if (PARTS) outer |= (uint32_t)p < n && key - whole < reach;
                     if (!kept) continue;
-                    outer |= side ? key >= cut : !PARTS;
+                    if (!PARTS) outer |= !side || key >= cut;
                     const uint32_t e = atomicAdd(&S.nent, 1u);
                     if (e < A_ENT && e - e_far < A_FAR) {
                         S.kc[e] = make_uint2(key, code | (key >= cut ? C_OWN : 0u));
