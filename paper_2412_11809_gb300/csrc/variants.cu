@@ -106,13 +106,16 @@ constexpr uint32_t SW_CHUNK = 32;
 constexpr uint32_t LW_CAP = 1024;        // hits in the rings of a long component's sweep
 constexpr uint32_t LW_WIN = LW_CAP - 64; // ... in the window (the looking warp is 32 to 64 ahead)
 constexpr uint32_t LW_TAB = 4096;
-constexpr uint32_t LW_REBUILD = 1024;    // hits between two rebuilds of the window's table
+constexpr uint32_t LW_REBUILD = 960;     // hits between two rebuilds of the window's table
 constexpr uint32_t LW_FIRST = 2048;      // components this long are started first
 constexpr int LW_CTAS = 3;               // per SM: room beside them for the other components' sweep
-constexpr uint32_t HASH_AGE = 4095;      // table entry: pixel id << 12 | index mod 4096
+// Table entry: pixel id << 11 | index mod 2048.  Bit 31 is set in none, so no
+// entry is the empty one (with 12 bits of index the last pixel of a sensor of
+// 2^20 pixels had one that was).
+constexpr uint32_t HASH_BITS = 11, HASH_AGE = (1u << HASH_BITS) - 1u;
 constexpr uint32_t HASH_EMPTY = 0xFFFFFFFFu;
 constexpr uint32_t NO_ROOT = 0xFFFFFFFFu;
-static_assert(MAX_PIXELS <= 1u << 20, "pixel ids take 20 bits");
+static_assert(MAX_PIXELS <= 1u << (31 - HASH_BITS), "pixel ids leave the top bit clear");
 // entries of a window's table: hits since its rebuild and those put back then, so lookups always end
 static_assert(LW_REBUILD + 32 + LW_CAP < LW_TAB && LW_REBUILD + 32 + LW_CAP < HASH_AGE && 2 * SW_CAP <= SW_TAB,
               "free entries, unambiguous indices");
@@ -171,7 +174,7 @@ __device__ void sweep_hashed(HashSweep &S, const uint32_t *skey, const uint32_t 
             uint32_t slot = pid * 0x9E3779B1u >> shift, r = NO_ROOT;
             if (in) {
                 uint32_t seen = S.tab[slot];
-                while (seen != HASH_EMPTY && seen >> 12 != pid) {
+                while (seen != HASH_EMPTY && seen >> HASH_BITS != pid) {
                     slot = (slot + 1) & tmask;
                     seen = S.tab[slot];
                 }
@@ -208,7 +211,7 @@ __device__ void sweep_hashed(HashSweep &S, const uint32_t *skey, const uint32_t 
                 if (r != NO_ROOT && r != m) S.up[r] = (uint16_t)(r - m);
                 if (d == 4) {
                     if (m != NO_ROOT) S.up[i] = (uint16_t)(i - m);
-                    S.tab[slot] = pid << 12 | (i & HASH_AGE);
+                    S.tab[slot] = pid << HASH_BITS | (i & HASH_AGE);
                 }
             }
             __syncwarp();
@@ -248,13 +251,13 @@ __device__ __forceinline__ void long_look(LongSweep &S, uint32_t base, uint32_t 
     auto put = [&](uint32_t id, uint32_t i, uint32_t now) {
         uint32_t slot = id * 0x9E3779B1u >> shift, seen = S.tab[slot];
         while (true) {
-            if (seen != HASH_EMPTY && seen >> 12 != id) {
+            if (seen != HASH_EMPTY && seen >> HASH_BITS != id) {
                 slot = (slot + 1) & tmask;
                 seen = S.tab[slot];
                 continue;
             }
             if (seen != HASH_EMPTY && ((now - seen) & HASH_AGE) <= ((now - i) & HASH_AGE)) return;
-            const uint32_t was = atomicCAS(&S.tab[slot], seen, id << 12 | (i & HASH_AGE));
+            const uint32_t was = atomicCAS(&S.tab[slot], seen, id << HASH_BITS | (i & HASH_AGE));
             if (was == seen) return;
             seen = was;
         }
@@ -286,7 +289,7 @@ __device__ __forceinline__ void long_look(LongSweep &S, uint32_t base, uint32_t 
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
         const uint32_t want = (uint32_t)(y + q / 3 - 1) * W + (uint32_t)(x + q % 3 - 1);
-        while (seen[q] != HASH_EMPTY && seen[q] >> 12 != want) {
+        while (seen[q] != HASH_EMPTY && seen[q] >> HASH_BITS != want) {
             slot[q] = (slot[q] + 1) & tmask;
             seen[q] = S.tab[slot[q]];
         }
