@@ -822,6 +822,21 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
         }
         const uint32_t n_e = S.nent;
         if (n_e > A_ENT || S.flag) {
+            // own hits as far out as the last rounds on both sides: disorder that
+            // sorting by tiles cannot mend either
+            int out[2];
+            for (int side = 0; side < 2; ++side) {
+                bool own = false;
+                for (uint32_t u = tid; u < A_STEP; u += NT) {
+                    const int32_t p = side ? (int32_t)((j + 1) * TILE + MARGIN + (A_ROUNDS - 1) * A_STEP + u) : win + (int32_t)u;
+                    if ((uint32_t)p < n) own |= (uint32_t)(hit_toa(ld_hit(hits + p)) - base) - S.cut[0] < S.cut[1] - S.cut[0];
+                }
+                out[side] = __syncthreads_count(own);
+            }
+            if (min(out[0], out[1]) >= 32) {
+                if (tid == 0) atomicMax(&P.raw_fail, RAW_UNORDERED);
+                return;
+            }
             if (!PARTS) {   // left to the kernel with PARTS
                 if (tid == 0) {
                     w.redo[atomicAdd(&P.parts_count, 1u)] = t;
@@ -1217,13 +1232,17 @@ __device__ __forceinline__ void join_pairs(const Work &w, uint32_t t, uint32_t f
 constexpr int AX = 256;
 
 __global__ void __launch_bounds__(AX) k_arrival_cross(Work w, cudaGraphConditionalHandle otherwise, bool parts) {
+    __shared__ uint32_t s_failed;
     Prob &P = *w.prob;
     const int tid = threadIdx.x;
-    const uint32_t failed = *reinterpret_cast<volatile uint32_t *>(&P.raw_fail);
-    bool lost = parts ? failed > RAW_PARTS : failed != 0;
-    for (uint32_t s = tid; s < P.nsegs; s += AX) lost |= w.seg[s].n_owned != w.seg[s].n;
-    bool fail = __syncthreads_or(lost);
-    if (!fail) {
+    bool stray = false;
+    for (uint32_t s = tid; s < P.nsegs; s += AX) stray |= w.seg[s].n_owned != w.seg[s].n;
+    if (tid == 0) s_failed = *reinterpret_cast<volatile uint32_t *>(&P.raw_fail);
+    stray = __syncthreads_or(stray);
+    const uint32_t failed = s_failed;
+    const bool lost = stray || (parts ? failed > RAW_PARTS : failed != 0);
+    bool fail = false;
+    if (!lost) {
         const uint32_t nt = P.ntiles;
         for (uint32_t t = (blockIdx.x * AX + tid) / 32; t < nt; t += gridDim.x * (AX / 32)) {
             const Seg &g = w.seg[w.tile_seg[t]];
@@ -1234,9 +1253,12 @@ __global__ void __launch_bounds__(AX) k_arrival_cross(Work w, cudaGraphCondition
             join_pairs<32>(w, t, tid & 31);
         }
     }
-    if (fail && (tid & 31) == 0) {
-        if (parts || failed != RAW_PARTS) atomicMax(&P.raw_fail, RAW_COVER);
-        if (otherwise) cudaGraphSetConditional(otherwise, !parts && failed == RAW_PARTS ? 0u : 1u);
+    // (one thread where all agree: a thousand of them took 10 us.  Hits beyond
+    // the positions read are beyond the sorted path's merge too.)
+    if (lost ? blockIdx.x == 0 && tid == 0 : fail && (tid & 31) == 0) {
+        const bool again = !parts && failed == RAW_PARTS;
+        if (!again) atomicMax(&P.raw_fail, stray && failed <= RAW_PARTS ? RAW_UNORDERED : RAW_COVER);
+        if (otherwise) cudaGraphSetConditional(otherwise, again ? 0u : 1u);
     }
     if (blockIdx.x == 0 && (parts || failed != RAW_PARTS))
         for (uint32_t s = tid; s < P.nsegs; s += AX) seg_close(w.seg[s], P);
@@ -1589,7 +1611,7 @@ __global__ void __launch_bounds__(ST, 1) k_arrival_step(Work w, Seg seg, uint32_
         }
         uint32_t off = 0, tile = 0;
         setup_seg(g, off, tile);
-        setup_prob(P, 1, tile, off, 1u);
+        setup_prob(P, 1, tile, off, RAW_SMALL);
     }
     cluster.sync();
     const uint32_t nt = *const_cast<volatile uint32_t *>(&P.ntiles);

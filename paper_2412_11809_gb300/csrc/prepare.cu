@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(256) k_gather(Work w) {
 }
 
 void launch_setup(const Work &w, int nsegs, const Launch &L, bool arrival) {
-    k_setup<<<1, 1024, 0, L.stream>>>(w, nsegs, arrival);
+    k_setup<<<1, 1024, 0, L.stream>>>(w, nsegs, arrival ? RAW_TRY : RAW_NONE);
     L.mark("k_setup");
 }
 void launch_seg_finalize(const Work &w, const Launch &L, cudaGraphConditionalHandle general) {

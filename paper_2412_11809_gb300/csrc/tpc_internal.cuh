@@ -124,10 +124,21 @@ struct Prob {
     uint32_t border_count; // tile borders k_border_fast left to k_border_link
     uint32_t merge_count;  // tile borders k_tile_merge left to its whole-window form (listed in redo)
     uint32_t emitted;      // CTAs of the last kernel that are done
-    uint32_t raw;          // the step starts on the arrival-order path
-    uint32_t raw_fail;     // ... which could not cover it (RawFail): the time-sorted path takes it
+    uint32_t raw;          // RawStart
+    uint32_t raw_fail;     // the arrival-order path could not cover the step (RawFail): the time-sorted path takes it
     uint32_t parts_count;  // tiles of the arrival-order path to be taken in parts (listed in redo)
+    // kept from step to step (setup_prob):
+    uint32_t hold;         // steps to come that go straight to the time-sorted path
+    uint32_t backoff;      // how many the last failure in a row asked for
+    uint32_t held, hold_as;   // this step is one of them; the RawFail they start with
 };
+
+enum RawStart : uint32_t {
+    RAW_NONE = 0u,         // time-sorted
+    RAW_TRY = 1u,          // on the arrival-order path, the time-sorted one behind it
+    RAW_SMALL = 2u,        // a small step
+};
+constexpr uint32_t HOLD_MOST = 63;
 
 enum RawFail : uint32_t {
     RAW_PARTS = 1u,        // some tiles' hits did not fit at once: taken in parts (no failure yet)
@@ -384,7 +395,13 @@ __device__ __forceinline__ void setup_seg(Seg &g, uint32_t &off, uint32_t &tile)
     g.n_final = g.n_clusters = g.n_open = 0;
 }
 
+// The step's state.  A stream that one step of a context could not be taken on
+// the arrival-order path for (disordered too far, too many hits within dt)
+// mostly goes on like that, and finding out again took 6 to 40 percent of each
+// step: after such a step the next 1, 3, 7, ... 63 start on the time-sorted
+// path, until one tried in between is covered.
 __device__ __forceinline__ void setup_prob(Prob &p, uint32_t nsegs, uint32_t tiles, uint32_t positions, uint32_t arrival) {
+    const uint32_t fail = p.raw_fail;
     p.nsegs = nsegs;
     p.npasses = 0;
     p.fallback = 0;
@@ -393,8 +410,21 @@ __device__ __forceinline__ void setup_prob(Prob &p, uint32_t nsegs, uint32_t til
     p.border_count = 0;
     p.merge_count = 0;
     p.emitted = 0;
+    const bool tried = p.raw == RAW_TRY && !p.held, lost = fail > RAW_PARTS;
     p.raw = arrival;
     p.raw_fail = 0;
+    p.held = 0;
+    if (arrival == RAW_TRY) {
+        if (tried) {
+            p.hold = p.backoff = lost ? min(2u * p.backoff + 1u, HOLD_MOST) : 0u;
+            p.hold_as = fail;
+        }
+        if (p.hold) {
+            --p.hold;
+            p.held = 1;
+            p.raw_fail = p.hold_as;
+        }
+    }
     p.parts_count = 0;
     p.err = 0;
     p.ntiles = tiles;
