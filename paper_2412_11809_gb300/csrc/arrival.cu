@@ -23,14 +23,13 @@
 //   k_arrival_emit   records in label order; streaming: finalised hits, the
 //                    carry of open hits and the stream state.
 //
-// Small steps (at most SMALL_TILES tiles) work for any order, so that they
-// need no sorted path behind them: tiles own hits by position and look back
-// over earlier positions; if some did not look far enough, tiles own intervals
-// of time instead and look at every position; and if those hold too many hits
-// the tiles of positions are joined with every earlier one.  All of it is one launch (k_arrival_step), a
-// cluster of one CTA per tile.  As seven launches a call with 1,000 hits took
-// 53 us (41 of them on the host) and one with 65,536 hits 96; now 26 and 58 (64
-// with 512 threads per CTA, which left an SM's issue slots idle).
+// Small steps (at most SMALL_TILES tiles) need no sorted path behind them: tiles
+// own hits by position and look back over earlier positions, and a step that
+// some tile is not done with (no order, too many hits within dt or on one pixel)
+// is sorted and joined hit by hit (any_order).  All of it is one launch
+// (k_arrival_step), a cluster of one CTA per tile.  As seven launches a call with
+// 1,000 hits took 53 us (41 of them on the host) and one with 65,536 hits 96; now
+// 26 and 58 (64 with 512 threads per CTA, which left an SM's issue slots idle).
 //
 // Owning by time keeps events whole: arrival disorder spreads an event's hits
 // over a thousand positions, and tiles of positions would cut a quarter of
@@ -61,6 +60,13 @@ constexpr uint32_t A_WORDS = 2304;               // 256 rows of nine 30-pixel wo
 constexpr uint32_t A_XTRA = 2048;                // unions beyond each hit's first
 constexpr uint32_t A_LATER = 2048;               // hits beside cells of several hits
 constexpr uint32_t A_FAR = 1920;                 // hits found beyond the margins (all that two CTAs per SM leave room for)
+// A small step's tile is given up (S.flag) once a thread has walked over this
+// many hits of crowded cells, or tried this often to hang a hit behind a cell's
+// first: with hundreds of hits on a pixel both take the square of their number.
+// (Not in k_arrival_tile: the counters cost it 1 percent.)
+constexpr uint32_t A_WALK = 1024, A_TRIES = 256;
+template <int NT>
+constexpr bool GIVES_UP = NT == ST;
 constexpr int A_JUMPS = 1;                       // path-shortening passes over the tile's forest
 constexpr int A_ROUNDS = 4;                      // further rounds on each side
 constexpr int A_BACK_ROUNDS = 16;                // rounds back of a small step's tiles
@@ -107,11 +113,20 @@ static_assert(offsetof(ArrivalShared, next) == offsetof(ArrivalShared, head) + A
 // the tile's own (otherwise an earlier tile's).
 constexpr uint32_t C_OWN = 1u << 31, C_CELL = C_OWN - 1u;
 
-// Small steps stage every entry's position too.
+// Small steps stage every entry's position too, and have room for more unions.
+constexpr uint32_t A_SMALL_XTRA = 8192;
 struct SmallShared {
     ArrivalShared s;
     uint16_t pos[A_ENT];
+    uint32_t xtra[A_SMALL_XTRA];
 };
+template <int NT>
+constexpr uint32_t XTRA = NT == ST ? A_SMALL_XTRA : A_XTRA;
+template <int NT>
+__device__ __forceinline__ uint32_t *xtra_list(ArrivalShared &S) {
+    if constexpr (NT == ST) return reinterpret_cast<SmallShared &>(S).xtra;   // (its first member)
+    else return S.xtra;
+}
 constexpr int A_SMEM = (int)sizeof(ArrivalShared), A_SMALL_SMEM = (int)sizeof(SmallShared);
 static_assert((unsigned long long)A_ENT * 0xFFFFu < (1ull << 32), "a tile's sum ToT fits 32 bits");
 
@@ -225,6 +240,8 @@ __device__ __forceinline__ void arrival_pairs(ArrivalShared &S, const Cells &C, 
     // Cells of several hits: on a neighbour pixel the latest hit at or before
     // this one and the earliest after it (the others within dt are joined to
     // those along their pixel), on the own pixel the next one.
+    auto give_up = [](uint32_t count, uint32_t most) { return GIVES_UP<NT> && count > most; };
+    uint32_t walked = 0;
     auto crowded = [&](uint32_t e) {
         const uint2 me = S.kc[e];
         const uint32_t code = me.y & C_CELL, key = me.x;
@@ -251,7 +268,7 @@ __device__ __forceinline__ void arrival_pairs(ArrivalShared &S, const Cells &C, 
                     }
                 }
                 j = S.next[j];
-            } while (j != A_NONE);
+            } while (j != A_NONE && !give_up(++walked, A_WALK));
             if (i != 4 && jlo != A_NONE && near(key, klo)) join(e, jlo, linked);
             if (jhi != A_NONE && near(khi, key)) join(e, jhi, linked);
         }
@@ -306,9 +323,10 @@ __device__ __forceinline__ void arrival_pairs(ArrivalShared &S, const Cells &C, 
     __syncthreads();
     const uint32_t listed = S.nlater;
     if (listed <= A_LATER)
-        for (uint32_t i = tid; i < listed; i += NT) crowded(S.later[i]);
+        for (uint32_t i = tid; i < listed && !give_up(walked, A_WALK); i += NT) crowded(S.later[i]);
     else   // (more than the list holds: all of them, those without such cells have nothing to do)
-        for (uint32_t e = tid; e < n_e; e += NT) crowded(e);
+        for (uint32_t e = tid; e < n_e && !give_up(walked, A_WALK); e += NT) crowded(e);
+    if (give_up(walked, A_WALK)) S.flag = 1u;
 }
 
 template <int NT, class Near, class Join>
@@ -359,6 +377,8 @@ __device__ __forceinline__ void arrival_links(ArrivalShared &S, const Cells &C, 
         }
     }
     __syncthreads();
+    auto give_up = [](uint32_t count, uint32_t most) { return GIVES_UP<NT> && count > most; };
+    uint32_t tries = 0;
 #pragma unroll
     for (int q = 0; q < A_PER; ++q) {   // the others hang behind it
         const uint32_t e = q * NT + tid;
@@ -373,15 +393,21 @@ __device__ __forceinline__ void arrival_links(ArrivalShared &S, const Cells &C, 
             const uint32_t seen = atomicCAS(half, old, (old & ~(0xFFFFu << shift)) | e << shift);
             if (seen == old) break;
             old = seen;
+            if (give_up(++tries, A_TRIES)) {   // (hundreds of hits on one pixel)
+                S.flag = 1u;
+                break;
+            }
         }
         S.head[s] = (uint16_t)(h | A_MULTI);
     }
     __syncthreads();
+    if (GIVES_UP<NT> && S.flag) return;   // (by all: no thread writes it before the barrier in arrival_pairs)
     if (C.alias) arrival_pairs<NT, true>(S, C, n_e, near, join); else arrival_pairs<NT, false>(S, C, n_e, near, join);
 }
 
 // A pair: the hit's first makes the other its parent (always raster-earlier,
 // or the next hit of its pixel, so parents form no cycle), others are listed.
+template <int NT>
 __device__ __forceinline__ void join_hits(ArrivalShared &S, uint32_t e, uint32_t j, bool &linked) {
     if (!linked) {
         S.par[e] = (uint16_t)j;
@@ -389,7 +415,7 @@ __device__ __forceinline__ void join_hits(ArrivalShared &S, uint32_t e, uint32_t
         return;
     }
     const uint32_t k = atomicAdd(&S.nxtra, 1u);
-    if (k < A_XTRA) S.xtra[k] = e << 16 | j;
+    if (k < XTRA<NT>) xtra_list<NT>(S)[k] = e << 16 | j;
 }
 
 // Components of the staged hits, the clusters of the tile's own, their
@@ -429,8 +455,9 @@ __device__ __forceinline__ bool arrival_clusters(const Work &w, const Seg &g, ui
             if (q * NT + tid < n_e) par[q * NT + tid] = (uint16_t)p[q];
     }
     __syncthreads();
-    for (uint32_t i = tid; i < min(S.nxtra, A_XTRA); i += NT) {
-        uint32_t a = S.xtra[i] >> 16, b = S.xtra[i] & 0xFFFFu;
+    const uint32_t *xtra = xtra_list<NT>(S);
+    for (uint32_t i = tid; i < min(S.nxtra, XTRA<NT>); i += NT) {
+        uint32_t a = xtra[i] >> 16, b = xtra[i] & 0xFFFFu;
         while (true) {   // hook the larger root under the smaller
             a = arrival_root(S.par, a);
             b = arrival_root(S.par, b);
@@ -890,7 +917,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
         // (keys keep 2^27 from both ends of 32 bits and dt is less: the sum wraps for no far pair)
         const uint32_t dt2 = 2u * dt;
         arrival_links<NT>(S, C, n_e, [&](uint32_t a, uint32_t b) { return a - b + dt <= dt2; },
-                      [&](uint32_t e, uint32_t o, bool &linked) { join_hits(S, e, o, linked); });
+                      [&](uint32_t e, uint32_t o, bool &linked) { join_hits<NT>(S, e, o, linked); });
         __syncthreads();
         // ---- positions and ToTs of the entries, where the lists were ---------
         uint32_t *where = S.where();
@@ -932,10 +959,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_arrival_tile(Work w) {
 // ---------------------------------------------------------------------------
 // Small steps: tiles own their positions, whatever the order.
 
-// One tile.  DIRECT (k_arrival_step): pairs are joined at once in the global
-// forest, every earlier position is looked at, nothing else is written.
-template <int NT, bool DIRECT>
-__device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShared &SS) {
+// One tile; false: left to any_order (more hits within dt, pairs or hits of
+// single pixels than it holds, or earlier hits too far back).
+template <int NT>
+__device__ __forceinline__ bool small_tile(const Work &w, uint32_t t, SmallShared &SS) {
     ArrivalShared &S = SS.s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const Seg &g = w.seg[0];   // (a small step has one segment)
@@ -953,7 +980,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
     bool wide = dt >= A_GUARD;
     const uint32_t new0 = g.n_carry > begin ? g.n_carry - begin : 0;   // first new hit
     uint32_t kmin, kmax, tots[OWN];
-    if (tid == 0) S.nxtra = S.ncross = S.nroots = S.tsum = S.numbered = 0;
+    if (tid == 0) S.nxtra = S.ncross = S.nroots = S.tsum = S.numbered = S.flag = 0;
     C.clear<NT>(S);
     __syncthreads();
     for (int attempt = 0;; ++attempt) {
@@ -984,7 +1011,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
             kmin = min(kmin, key);
             if (e >= new0) cmin = min(cmin, key);
         }
-        if (!DIRECT && __any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&w.prob->err, E_RANGE);
+        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&w.prob->err, E_RANGE);
         kmin = __reduce_min_sync(0xffffffffu, kmin);
         cmin = __reduce_min_sync(0xffffffffu, cmin);
         if (lane == 0) { S.red[0][warp] = kmin; S.red[1][warp] = cmin; }
@@ -1005,7 +1032,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
             m = S.m64[0][q] < m ? S.m64[0][q] : m;
             mx = S.m64[1][q] > mx ? S.m64[1][q] : mx;
         }
-        if (!DIRECT && tid == 0 && (mx - m) >> 32) atomicOr(&w.prob->err, E_SPAN);
+        if (tid == 0 && (mx - m) >> 32) atomicOr(&w.prob->err, E_SPAN);
         base = m;
     }
     {
@@ -1014,7 +1041,7 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
     }
     const uint32_t lo = kmin > dt ? kmin - dt : 0u;       // earlier hits below it join nothing here
     const uint64_t hi = (uint64_t)kmax + dt;
-    if (!DIRECT && warp == 0) {
+    if (warp == 0) {
         const uint32_t cmin = __reduce_min_sync(0xffffffffu, S.red[1][min(lane, (NT / 32) - 1)]);
         if (lane < (int)ACHUNKS) info.cmax[lane] = base + S.cnt[1][lane];
         if (lane == 0) {
@@ -1030,177 +1057,62 @@ __device__ __forceinline__ void small_tile(const Work &w, uint32_t t, SmallShare
 
     // ---- links, with the earlier hits in rounds of A_STEP positions --------
     uint32_t h0 = begin;            // every position in [h0, begin) has been looked at
-    bool done = begin == 0, redo = false;
-    for (bool first = true;; first = false) {
-        if (!first) {               // (redo) the earlier hits so far are joined: the next ones beside the own hits
-            __syncthreads();
-            C.clear<NT>(S);
-            __syncthreads();
-            for (uint32_t e = tid; e < n_t; e += NT) {
-                const tpc_hit *h = hits + begin + e;
-                const uint4 v = ld_hit(h);
-                const uint32_t code = C.code(clamp_pix(v.x, W, H));
-                S.kc[e] = make_uint2((uint32_t)(hit_toa(v) - base), code | C_OWN);
-                C.set(S, code);
-            }
-        }
-        uint32_t n_e = n_t;
-        for (uint32_t buf = 0; !done;) {
-            const uint32_t a = h0 - A_STEP;
-            if (DIRECT && w.atile[a / TILE].cmax[(a % TILE) / A_STEP] < base + lo) {
-                h0 = a;
-                done = h0 == 0;
-                continue;
-            }
-            uint32_t kk[A_HPER], pp[A_HPER], mask[A_HPER], sum = 0;
+    uint32_t n_e = n_t;
+    bool done = begin == 0;
+    for (uint32_t buf = 0; !done;) {
+        const uint32_t a = h0 - A_STEP;
+        uint32_t kk[A_HPER], pp[A_HPER], mask[A_HPER], sum = 0;
 #pragma unroll
-            for (int u = 0; u < A_HPER; ++u) {
-                const uint4 v = ld_hit(hits + a + u * NT + tid);
-                const uint64_t rel = hit_toa(v) - base;
-                kk[u] = (uint32_t)rel;
-                pp[u] = C.code(clamp_pix(v.x, W, H));
-                mask[u] = __ballot_sync(0xffffffffu, rel >= lo && rel <= hi);
-                sum += __popc(mask[u]);
-            }
-            if (lane == 0) S.turn[buf][warp] = sum | (mask[0] ? 0x80000000u : 0u);
-            __syncthreads();
-            const uint32_t c = lane < (NT / 32) ? S.turn[buf][lane] : 0u;
-            buf ^= 1u;   // the next round's barrier separates this one's reads from the round after
-            const uint32_t total = __reduce_add_sync(0xffffffffu, c & 0x7FFFFFFFu);
-            const bool oldest = __any_sync(0xffffffffu, c >> 31);   // some of the oldest NT positions matter
-            if (n_e + total > A_ENT) {   // no room beside the staged ones
-                if (!DIRECT) done = redo = true;
-                break;
-            }
-            uint32_t e = n_e + __reduce_add_sync(0xffffffffu, lane < warp ? c & 0x7FFFFFFFu : 0u);
-#pragma unroll
-            for (int u = 0; u < A_HPER; ++u) {
-                if ((mask[u] >> lane) & 1u) {
-                    const uint32_t i = e + __popc(mask[u] & lanes_below());
-                    S.kc[i] = make_uint2(kk[u], pp[u]);
-                    SS.pos[i] = (uint16_t)(a + u * NT + tid);
-                    C.set(S, pp[u]);
-                }
-                e += __popc(mask[u]);
-            }
-            n_e += total;
-            h0 = a;
-            if (h0 == 0) done = true;
-            else if (!DIRECT && !oldest) done = true;
-            else if (!DIRECT && begin - h0 == A_BACK_ROUNDS * A_STEP) done = redo = true;
-        }
-        auto near = [&](uint32_t a, uint32_t b) { return absdiff(a, b) <= dt; };
-        if (DIRECT) {   // every pair, own or not, is an edge of the graph
-            arrival_links<NT>(S, C, n_e, near, [&](uint32_t e, uint32_t o, bool &) {
-                gunion(w.gpar, w.root_of[SS.pos[e]], w.root_of[SS.pos[o]]);
-            });
-        } else {
-            arrival_links<NT>(S, C, n_e, near, [&](uint32_t e, uint32_t o, bool &linked) { join_hits(S, e, o, linked); });
-            __syncthreads();
-            redo |= S.nxtra > A_XTRA;
-            uint32_t tsum = 0;
-#pragma unroll
-            for (int q = 0; q < OWN; ++q) {
-                const uint32_t e = q * NT + tid;
-                if (e < n_t) S.where()[e] = (uint32_t)SS.pos[e] << 16 | tots[q];
-                tsum += tots[q];
-            }
-            for (uint32_t e = n_t + tid; e < n_e; e += NT) S.where()[e] = (uint32_t)SS.pos[e] << 16;
-            tsum = __reduce_add_sync(0xffffffffu, tsum);
-            if (lane == 0) atomicAdd(&S.tsum, tsum);
-            __syncthreads();
-            arrival_clusters<NT>(w, g, t, S, C, n_e, 0u, base);   // (at most TILE clusters)
-        }
-        if (done) break;
-    }
-    if (DIRECT) return;
-    if (tid == 0) {
-        info.h0 = h0;
-        info.nx = S.ncross;
-        info.redo = redo ? 1u : 0u;
-    }
-}
-
-// Tile t of a small step whose hits are in no order: those of an interval of
-// ToAs, wherever they lie, and the hits of the dt before it.  The cuts are
-// quantiles of one sampled hit per thread, the same in both tiles that need one,
-// found by bisection with a barrier's count.  Nothing is left to prove: every
-// position is looked at.  false: more hits, pairs or clusters than a tile holds.
-// (A call with 54,685 hits in 14 tiles: 1150 us with every tile beside every
-// earlier one, 225 so.)
-template <int NT>
-__device__ __forceinline__ bool time_tile(const Work &w, uint32_t t, SmallShared &SS) {
-    ArrivalShared &S = SS.s;
-    const int tid = threadIdx.x, lane = tid & 31;
-    const Seg &g = w.seg[0];
-    const uint32_t n = g.n, nt = g.ntiles, dt = g.dt, W = g.width, H = g.height;
-    const tpc_hit *hits = g.hits;
-    const uint64_t base = *reinterpret_cast<const volatile uint64_t *>(&g.toa_min);   // (of all tiles by now)
-    const Cells C(W, H);
-    if (tid == 0) S.nent = S.nxtra = S.ncross = S.nroots = S.tsum = S.numbered = 0;
-    C.clear<NT>(S);
-    const uint32_t sample = (uint32_t)(hit_toa(ld_hit(hits + (uint64_t)tid * n / NT)) - base);
-    uint32_t cut[2];
-#pragma unroll 1
-    for (uint32_t k = 0; k < 2; ++k) {
-        const int below = (int)((t + k) * NT / nt);   // samples below the cut
-        uint32_t lo = 0, hi = 0xFFFFFFFFu;
-        while (t + k && lo < hi) {   // the smallest key with more samples up to it
-            const uint32_t mid = lo + (hi - lo) / 2;
-            if (__syncthreads_count(sample <= mid) > below) hi = mid; else lo = mid + 1;
-        }
-        cut[k] = lo;
-    }
-    __syncthreads();
-    const bool last = t + 1 == nt;
-    const uint32_t from = cut[0], lo = from > dt ? from - dt : 0u;
-    uint32_t tsum = 0;
-    constexpr int U = 4;
-#pragma unroll 1
-    for (uint32_t p0 = 0; p0 < n; p0 += U * NT) {
-        uint4 v[U];
-        uint32_t mask[U], sum = 0;
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (p0 + u * NT + tid < n) v[u] = ld_hit(hits + p0 + u * NT + tid);
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t key = (uint32_t)(hit_toa(v[u]) - base);
-            mask[u] = __ballot_sync(0xffffffffu, p0 + u * NT + tid < n && key >= lo && (last || key < cut[1]));
+        for (int u = 0; u < A_HPER; ++u) {
+            const uint4 v = ld_hit(hits + a + u * NT + tid);
+            const uint64_t rel = hit_toa(v) - base;
+            kk[u] = (uint32_t)rel;
+            pp[u] = C.code(clamp_pix(v.x, W, H));
+            mask[u] = __ballot_sync(0xffffffffu, rel >= lo && rel <= hi);
             sum += __popc(mask[u]);
         }
-        if (!sum) continue;
-        uint32_t e0 = 0;
-        if (lane == 0) e0 = atomicAdd(&S.nent, sum);
-        e0 = __shfl_sync(0xffffffffu, e0, 0);
+        if (lane == 0) S.turn[buf][warp] = sum | (mask[0] ? 0x80000000u : 0u);
+        __syncthreads();
+        const uint32_t c = lane < (NT / 32) ? S.turn[buf][lane] : 0u;
+        buf ^= 1u;   // the next round's barrier separates this one's reads from the round after
+        const uint32_t total = __reduce_add_sync(0xffffffffu, c & 0x7FFFFFFFu);
+        const bool oldest = __any_sync(0xffffffffu, c >> 31);   // some of the oldest NT positions matter
+        if (n_e + total > A_ENT) return false;   // no room beside the staged ones
+        uint32_t e = n_e + __reduce_add_sync(0xffffffffu, lane < warp ? c & 0x7FFFFFFFu : 0u);
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t e = e0 + __popc(mask[u] & lanes_below());
-            if (((mask[u] >> lane) & 1u) && e < A_ENT) {
-                const uint32_t key = (uint32_t)(hit_toa(v[u]) - base), code = C.code(clamp_pix(v[u].x, W, H));
-                S.kc[e] = make_uint2(key, code | (key >= from ? C_OWN : 0u));
-                SS.pos[e] = (uint16_t)(p0 + u * NT + tid);
-                C.set(S, code);
-                if (key >= from) tsum += hit_tot(v[u]);
+        for (int u = 0; u < A_HPER; ++u) {
+            if ((mask[u] >> lane) & 1u) {
+                const uint32_t i = e + __popc(mask[u] & lanes_below());
+                S.kc[i] = make_uint2(kk[u], pp[u]);
+                SS.pos[i] = (uint16_t)(a + u * NT + tid);
+                C.set(S, pp[u]);
             }
-            e0 += __popc(mask[u]);
+            e += __popc(mask[u]);
         }
+        n_e += total;
+        h0 = a;
+        done = h0 == 0 || !oldest;
+        if (!done && begin - h0 == A_BACK_ROUNDS * A_STEP) return false;
     }
+    arrival_links<NT>(S, C, n_e, [&](uint32_t a, uint32_t b) { return absdiff(a, b) <= dt; },
+                      [&](uint32_t e, uint32_t o, bool &linked) { join_hits<NT>(S, e, o, linked); });
+    __syncthreads();
+    if (S.nxtra > XTRA<NT> || S.flag) return false;
+    uint32_t tsum = 0;
+#pragma unroll
+    for (int q = 0; q < OWN; ++q) {
+        const uint32_t e = q * NT + tid;
+        if (e < n_t) S.where()[e] = (uint32_t)SS.pos[e] << 16 | tots[q];
+        tsum += tots[q];
+    }
+    for (uint32_t e = n_t + tid; e < n_e; e += NT) S.where()[e] = (uint32_t)SS.pos[e] << 16;
     tsum = __reduce_add_sync(0xffffffffu, tsum);
     if (lane == 0) atomicAdd(&S.tsum, tsum);
     __syncthreads();
-    const uint32_t n_e = S.nent;
-    if (n_e > A_ENT) return false;
-    arrival_links<NT>(S, C, n_e, [&](uint32_t a, uint32_t b) { return absdiff(a, b) <= dt; },
-                      [&](uint32_t e, uint32_t o, bool &linked) { join_hits(S, e, o, linked); });
-    __syncthreads();
-    if (S.nxtra > A_XTRA) return false;
-    for (uint32_t e = tid; e < n_e; e += NT) S.where()[e] = (uint32_t)SS.pos[e] << 16 | hit_tot(ld_hit(hits + SS.pos[e]));
-    __syncthreads();
-    if (!arrival_clusters<NT>(w, g, t, S, C, n_e, 0u, base) || S.ncross > A_PAIRS) return false;
+    arrival_clusters<NT>(w, g, t, S, C, n_e, 0u, base);   // (at most TILE clusters)
     if (tid == 0) {
-        w.atile[t].nx = S.ncross;
-        w.atile[t].base = base;
+        info.h0 = h0;
+        info.nx = S.ncross;
     }
     return true;
 }
@@ -1539,20 +1451,20 @@ __global__ void __launch_bounds__(AE) k_arrival_emit(Work w) {
     for (uint32_t s = threadIdx.x; s < P.nsegs; s += AE) write_info(w.seg[s], P);
 }
 
-// Whether the tile looked far enough: every hit before h0 is earlier than its
-// first by more than dt (first warp).
-__device__ __forceinline__ void small_check(const Work &w, uint32_t t) {
+// Whether the tile is done: every hit before h0 is earlier than its first by
+// more than dt (first warp).
+__device__ __forceinline__ void small_check(const Work &w, uint32_t t, bool linked) {
     if (threadIdx.x >= 32) return;
     const uint32_t lane = threadIdx.x;
     const ATile &info = w.atile[t];
-    const uint32_t hc = info.h0 / A_STEP;   // chunks not looked at
+    const uint32_t hc = linked ? info.h0 / A_STEP : 0u;   // chunks not looked at
     uint64_t m = 0;
     for (uint32_t i = lane; i < hc; i += 32) {
         const uint64_t c = w.atile[i / ACHUNKS].cmax[i % ACHUNKS];
         m = c > m ? c : m;
     }
     m = warp_max_u64(m);
-    if (lane == 0 && ((hc && m >= info.lo) || info.nx > A_PAIRS)) w.atile[t].redo = 1u;
+    if (lane == 0) w.atile[t].redo = !linked || (hc && m >= info.lo) || info.nx > A_PAIRS;
 }
 
 // Tiles that are not done (between two barriers of the cluster).
@@ -1562,29 +1474,309 @@ __device__ __forceinline__ bool tiles_left(const Work &w, uint32_t nt) {
     return any;
 }
 
-// Links of a small step that tiles of positions did not cover (out of line: its
-// registers are not the usual path's).
-__device__ __noinline__ void any_order(const Work &w, uint32_t t, uint32_t nt, SmallShared &S) {
+constexpr int SORT_BITS = 10;
+constexpr uint32_t DIGITS = 1u << SORT_BITS;
+static_assert(DIGITS == (uint32_t)ST && DIGITS / 32 == 32, "a thread per digit, a lane per warp's sum");
+static_assert(DIGITS * sizeof(uint32_t) <= A_PAIRS * sizeof(uint2), "a tile's counts fit its list of pairs");
+
+struct SortShared {
+    union {
+        struct {
+            uint16_t cnt[ST / 32][DIGITS];   // hits of each digit per warp, then those of the warps before
+            uint32_t base[DIGITS];           // first place of this tile's hits of each digit
+            uint32_t sum[32];
+        };
+        uint2 near[2 * TILE];                // after the sort: key and pixel of this tile's hits and of the tile before
+    };
+};
+static_assert(sizeof(SortShared) <= sizeof(SmallShared), "in the place of a tile");
+
+// One stable pass over SORT_BITS bits of the sort that the cluster's CTAs do
+// together, each placing the entries of its tile.  hist: [tile][DIGITS].
+__device__ __forceinline__ void sort_pass(const uint4 *src, uint4 *dst, uint32_t *hist, uint32_t t, uint32_t nt, uint32_t n,
+                                          bool pixel, uint32_t shift, SortShared &S) {
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, first = t * TILE + warp * (TILE / (ST / 32)) + lane;
+    constexpr int PER = TILE / ST;
     const bool mine = t < nt;
-    cluster.sync();   // (the flags are read)
-    if (mine) {
-        const bool done = time_tile<ST>(w, t, S);
-        if (threadIdx.x == 0) w.atile[t].redo = done ? 0u : 1u;
+    uint4 e[PER];
+    uint32_t rank[PER];
+#pragma unroll
+    for (int r = 0; r < PER; ++r)
+        if (mine && first + 32 * r < n) e[r] = src[first + 32 * r];
+    for (uint32_t i = tid; i < sizeof(S.cnt) / sizeof(uint4); i += ST) reinterpret_cast<uint4 *>(S.cnt)[i] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+        const bool valid = mine && first + 32 * r < n;
+        const uint32_t d = valid ? ((pixel ? e[r].y : e[r].x) >> shift) & (DIGITS - 1) : DIGITS;
+        const uint32_t same = __match_any_sync(0xffffffffu, d);
+        if (valid) rank[r] = S.cnt[warp][d] + __popc(same & lanes_below());
+        __syncwarp();
+        if (valid && !(same & lanes_below())) S.cnt[warp][d] += (uint16_t)__popc(same);
+        __syncwarp();
+    }
+    __syncthreads();
+    uint32_t run = 0;
+#pragma unroll
+    for (int q = 0; q < ST / 32; ++q) {
+        const uint32_t c = S.cnt[q][tid];
+        S.cnt[q][tid] = (uint16_t)run;
+        run += c;
+    }
+    if (mine) hist[t * DIGITS + tid] = run;
+    cluster.sync();
+    uint32_t before = 0, all = 0;   // hits of this thread's digit in the tiles before, in all
+#pragma unroll
+    for (uint32_t q = 0; q < SMALL_TILES; ++q) {
+        const uint32_t h = q < nt ? hist[q * DIGITS + tid] : 0u;
+        before += q < t ? h : 0u;
+        all += h;
+    }
+    uint32_t x = all;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= (uint32_t)o) x += y;
+    }
+    if (lane == 31) S.sum[warp] = x;
+    __syncthreads();
+    S.base[tid] = before + x - all + __reduce_add_sync(0xffffffffu, lane < warp ? S.sum[lane] : 0u);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+        if (!mine || first + 32 * r >= n) continue;
+        const uint32_t d = ((pixel ? e[r].y : e[r].x) >> shift) & (DIGITS - 1);
+        dst[S.base[d] + S.cnt[warp][d] + rank[r]] = e[r];
     }
     cluster.sync();
-    const bool lost = tiles_left(w, nt);
-    if (mine && !lost) join_pairs<ST>(w, t, threadIdx.x);
-    cluster.sync();
-    if (!lost) return;
-    if (mine) small_tile<ST, false>(w, t, S);   // the tiles of positions again
-    cluster.sync();
-    if (mine) {
-        small_check(w, t);
-        join_pairs<ST>(w, t, threadIdx.x);
+}
+
+// A small step whose tiles of positions are not all done: hits in no order,
+// too many of them within dt or on one pixel.  The cluster sorts the step by
+// pixel and time (in the place of the feature sums).  A hit is joined to the one
+// before it on its pixel and, on its four neighbour pixels before it in raster
+// order, to the latest at or before it and the earliest after it (the others
+// within dt are joined to those along their pixel): the first of these becomes
+// its parent, those that are within dt of another one beside them are left out,
+// and the few that remain are joined in the forest over the sorted hits.  Any
+// order, any density, any dt.  Bound by the latency of its stages on 16 SMs:
+// 65,536 shuffled hits 193 us on the GPU, 27 of them the tiles of positions, 45
+// the four passes of the sort, 34 the searches, 28 the features.  (Tiles of ToA
+// intervals that each scanned all hits took 215, and where those held too many
+// hits every tile was joined with every earlier one: 1480 at dt 384 with 4 hits a
+// tick; all pairs joined at once in global memory 700.)  Out of line, so that its
+// registers are not the usual path's.
+__device__ __noinline__ void any_order(const Work &w, uint32_t t, uint32_t nt, SortShared &S) {
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const Seg &g = w.seg[0];
+    const uint32_t tid = threadIdx.x, lane = tid & 31, n = g.n, W = g.width, H = g.height, dt = g.dt;
+    const uint32_t begin = t < nt ? t * TILE : n, end = min(begin + (uint32_t)TILE, n);
+    const uint64_t base = *reinterpret_cast<const volatile uint64_t *>(&g.toa_min);
+    const uint64_t span = *reinterpret_cast<const volatile uint64_t *>(&g.toa_max) - base;
+    const bool streaming = g.ss != nullptr;
+    static_assert(sizeof(RootSlot) == 2 * sizeof(uint4), "the sort's two buffers");
+    uint4 *src = reinterpret_cast<uint4 *>(w.rslot), *dst = src + (size_t)nt * TILE;   // key, pixel, position, ToT
+    uint32_t *hist = reinterpret_cast<uint32_t *>(w.xlist);
+    for (uint32_t i = begin + tid; i < end; i += ST) {
+        const uint4 v = ld_hit(g.hits + i);
+        const uint32_t pix = clamp_pix(v.x, W, H);
+        src[i] = make_uint4((uint32_t)(hit_toa(v) - base), (pix >> 16) * W + (pix & 0xFFFFu), i, hit_tot(v));
     }
     cluster.sync();
-    if (mine && *const_cast<volatile uint32_t *>(&w.atile[t].redo)) small_tile<ST, true>(w, t, S);
+    const uint32_t last_pixel = W * H - 1u;
+    for (int pass = 0; pass < 8; ++pass) {
+        const uint32_t shift = (uint32_t)(pass & 3) * SORT_BITS;
+        if (!(pass < 4 ? span >> shift : last_pixel >> shift)) continue;
+        sort_pass(src, dst, hist, t, nt, n, pass >= 4, shift, S);
+        uint4 *x = src;
+        src = dst;
+        dst = x;
+    }
+    constexpr int PER = TILE / ST;
+    uint32_t more[PER];        // neighbours to be joined later (bits as in `order`)
+    uint32_t at01[PER], at23[PER];   // on each neighbour pixel, the first entry beyond the hit's key (two to a word)
+    // In turn: the hit before (-), then of the pixels left, above left, above,
+    // above right (0 to 3) the latest and the earliest after; neighbours beside one another.
+    constexpr int order[9] = {-1, 2, 2, 0, 0, 1, 1, 3, 3};
+    auto beside = [](int a, int b) { return a < 0 || b < 0 || a == b || a == 2 || b == 2 || (a < 2 && b < 2); };
+    volatile uint32_t *par = w.gpar;   // (over the sorted hits)
+    // The searches mostly end among this tile's hits and those of the tile before.
+    const uint32_t near0 = begin > TILE ? begin - TILE : 0u;
+    for (uint32_t i = near0 + tid; i < end; i += ST) S.near[i - near0] = *reinterpret_cast<const uint2 *>(src + i);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+        const uint32_t i = begin + r * ST + tid;
+        more[r] = at01[r] = at23[r] = 0;
+        if (i >= end) continue;
+        const uint2 me = S.near[i - near0];
+        const uint32_t y = me.y / W, x = me.y - y * W;
+        uint32_t at[4], q[4];
+        bool far = false;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const bool in = k == 0 ? x > 0 : y > 0 && (k == 1 ? x > 0 : k == 2 || x + 1 < W);
+            q[k] = !in ? 0xFFFFFFFFu : k == 0 ? me.y - 1u : me.y - W + (uint32_t)k - 2u;
+        }
+        auto search = [&](uint32_t from, uint32_t to, auto entry) {   // first entry of [from, to) beyond the key, or to
+            uint32_t len[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                at[k] = q[k] == 0xFFFFFFFFu ? 0u : from;
+                len[k] = q[k] == 0xFFFFFFFFu ? 0u : to - from;
+            }
+            for (uint32_t longest = to - from; longest; longest >>= 1) {
+                uint2 o[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) o[k] = len[k] ? entry(at[k] + (len[k] >> 1)) : make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const bool up = len[k] && (o[k].y < q[k] || (o[k].y == q[k] && o[k].x <= me.x));
+                    const uint32_t half = len[k] >> 1;
+                    at[k] += up ? half + 1u : 0u;
+                    len[k] = up ? len[k] - half - 1u : half;
+                }
+            }
+        };
+        search(near0, i, [&](uint32_t a) { return S.near[a - near0]; });
+#pragma unroll
+        for (int k = 0; k < 4; ++k) far |= near0 && at[k] == near0;
+        if (far) search(0u, i, [&](uint32_t a) { return *reinterpret_cast<const uint2 *>(src + a); });
+        uint32_t key[9], found = 0;
+#pragma unroll
+        for (int c = 0; c < 9; ++c) {
+            const int k = order[c];
+            const bool after = c && c % 2 == 0;
+            const uint32_t want = k < 0 ? me.y : q[k < 0 ? 0 : k], u = k < 0 ? i : at[k < 0 ? 0 : k];
+            uint2 o = make_uint2(0, 0xFFFFFFFEu);
+            const uint32_t j = after ? u : u - 1u;
+            if (after || u) o = j >= near0 ? S.near[j - near0] : *reinterpret_cast<const uint2 *>(src + j);
+            key[c] = o.x;
+            if (o.y == want && (after ? o.x - me.x : me.x - o.x) <= dt) found |= 1u << c;
+        }
+        uint32_t parent = i, rest = 0;
+#pragma unroll
+        for (int c = 0; c < 9; ++c) {
+            bool take = (found >> c) & 1u;
+#pragma unroll
+            for (int b = 0; b < c; ++b)
+                if (beside(order[b], order[c])) take = take && !(((found >> b) & 1u) && absdiff(key[b], key[c]) <= dt);
+            if (!take) continue;
+            const int k = order[c];
+            const uint32_t j = k < 0 ? i - 1u : at[k < 0 ? 0 : k] - (c % 2 ? 1u : 0u);
+            if (parent == i) parent = j; else rest |= 1u << c;
+        }
+        par[i] = parent;
+        more[r] = rest;
+        at01[r] = at[0] | at[1] << 16;
+        at23[r] = at[2] | at[3] << 16;
+    }
+    cluster.sync();
+    // parents to roots, all in step (chains along a pixel or a track halve with every hop)
+    uint32_t top[PER];
+#pragma unroll
+    for (int r = 0; r < PER; ++r) top[r] = begin + r * ST + tid < end ? par[begin + r * ST + tid] : 0u;
+    for (bool any = true; any;) {
+        any = false;
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            if (begin + r * ST + tid >= end) continue;
+            const uint32_t p = par[top[r]];
+            if (p == top[r]) continue;
+            any = true;
+            top[r] = p;
+            par[begin + r * ST + tid] = p;
+        }
+    }
+    cluster.sync();
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+        while (more[r]) {
+            const int c = __ffs(more[r]) - 1;
+            more[r] &= more[r] - 1u;
+            const int k = (c + 1) / 2;   // c 1, 2: above; 3, 4: left; 5, 6: above left; 7, 8: above right
+            const uint32_t u = k == 1 ? at23[r] & 0xFFFFu : k == 2 ? at01[r] & 0xFFFFu : k == 3 ? at01[r] >> 16 : at23[r] >> 16;
+            gunion(w.gpar, begin + r * ST + tid, u - (c % 2 ? 1u : 0u));
+        }
+    }
+    uint4 e[PER];
+#pragma unroll
+    for (int r = 0; r < PER; ++r)
+        if (begin + r * ST + tid < end) e[r] = src[begin + r * ST + tid];
+    cluster.sync();
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {   // each hit's own features (only those at the roots are added to and read)
+        const uint32_t i = begin + r * ST + tid;
+        if (i >= end) continue;
+        const uint32_t y = e[r].y / W, x = e[r].y - y * W, tot = e[r].w;
+        uint4 *slot = reinterpret_cast<uint4 *>(w.rslot + i);
+        slot[0] = make_uint4(tot, 0u, tot * x, 0u);
+        slot[1] = make_uint4(tot * y, 0u, 1u, e[r].z);
+        w.rfirst[i] = base + e[r].x;
+        if (streaming) w.rlast[i] = base + e[r].x;
+    }
+    if (t < nt && tid == 0) {
+        w.atile[t].nroots = 0;   // every hit points at its cluster's root
+        w.atile[t].base = base;
+    }
+    cluster.sync();
+    // The others' are added to their roots', a warp's hits of one cluster at once: a
+    // lane sums up those of the lanes behind it in its group, twice as many with each
+    // step (hit by hit 39 us for 65,536 hits, group after group 79).
+#pragma unroll
+    for (int r = 0; r < PER; ++r) top[r] = begin + r * ST + tid < end ? par[begin + r * ST + tid] : 0u;
+    for (bool any = true; any;) {   // (nothing writes them any more)
+        any = false;
+#pragma unroll
+        for (int r = 0; r < PER; ++r) {
+            const uint32_t p = par[top[r]];
+            any |= p != top[r];
+            top[r] = p;
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+        const uint32_t i = begin + r * ST + tid, root = top[r];
+        const bool valid = i < end;
+        const bool adds = valid && root != i;
+        if (valid) {
+            w.root_of[e[r].z] = root;
+            if (w.rkey) w.rkey[e[r].z] = e[r].x;
+        }
+        const uint32_t y = e[r].y / W, x = e[r].y - y * W;
+        uint32_t size = adds ? 1u : 0u, mn = adds ? e[r].z : 0xFFFFFFFFu, k0 = adds ? e[r].x : 0xFFFFFFFFu, k1 = adds ? e[r].x : 0u;
+        uint32_t sum = adds ? e[r].w : 0u;
+        unsigned long long sx = sum * x, sy = sum * y;   // (products below 2^32)
+        const uint32_t same = __match_any_sync(0xffffffffu, adds ? root : 0xFFFFFFFFu), behind = same & ~(lanes_below() | 1u << lane);
+        int next = adds && behind ? __ffs(behind) - 1 : 32;
+        while (__any_sync(0xffffffffu, next < 32)) {
+            const int from = next & 31;
+            const bool has = next < 32;
+            const uint32_t c1 = __shfl_sync(0xffffffffu, size, from), s1 = __shfl_sync(0xffffffffu, sum, from);
+            const unsigned long long x1 = __shfl_sync(0xffffffffu, sx, from), y1 = __shfl_sync(0xffffffffu, sy, from);
+            const uint32_t m1 = __shfl_sync(0xffffffffu, mn, from), a1 = __shfl_sync(0xffffffffu, k0, from),
+                           b1 = __shfl_sync(0xffffffffu, k1, from);
+            const int n1 = __shfl_sync(0xffffffffu, next, from);
+            if (!has) continue;
+            size += c1;
+            sum += s1;
+            sx += x1;
+            sy += y1;
+            mn = min(mn, m1);
+            k0 = min(k0, a1);
+            k1 = max(k1, b1);
+            next = n1;
+        }
+        if (!adds || (same & lanes_below())) continue;
+        RootSlot &d = w.rslot[root];
+        atomicAdd(&d.tot, (unsigned long long)sum);
+        atomicAdd(&d.wx, sx);
+        atomicAdd(&d.wy, sy);
+        atomicAdd(&d.size, size);
+        atomicMin(&d.min, mn);
+        atomicMin(reinterpret_cast<unsigned long long *>(&w.rfirst[root]), (unsigned long long)(base + k0));
+        if (streaming) atomicMax(reinterpret_cast<unsigned long long *>(&w.rlast[root]), (unsigned long long)(base + k1));
+    }
     cluster.sync();
 }
 
@@ -1617,15 +1809,17 @@ __global__ void __launch_bounds__(ST, 1) k_arrival_step(Work w, Seg seg, uint32_
     const uint32_t nt = *const_cast<volatile uint32_t *>(&P.ntiles);
     const bool mine = t < nt;
     if (mine && tid == 0) w.tile_seg[t] = 0;
-    if (mine) small_tile<ST, false>(w, t, S);
-    cluster.sync();
-    if (mine) {
-        small_check(w, t);
-        join_pairs<ST>(w, t, tid);
+    const bool linked = mine && small_tile<ST>(w, t, S);
+    if (mine && !linked) {   // clusters for the pairs of other tiles to be joined to, until any_order takes the step
+        for (uint32_t i = t * TILE + tid; i < min((t + 1) * TILE, g.n); i += ST) w.root_of[i] = t * TILE;
+        if (tid == 0) w.gpar[t * TILE] = t * TILE;
     }
+    cluster.sync();
+    if (mine) small_check(w, t, linked);
+    if (linked) join_pairs<ST>(w, t, tid);
     if (t == 0 && tid == 0) seg_close(g, P);
     cluster.sync();
-    if (tiles_left(w, nt)) any_order(w, t, nt, S);
+    if (tiles_left(w, nt)) any_order(w, t, nt, *reinterpret_cast<SortShared *>(a_raw));
     if (mine) root_tile<ST>(w, t, g.ss != nullptr);
     cluster.sync();
     if (mine) label_tile<ST>(w, t, g, reinterpret_cast<uint32_t *>(a_raw), s_cnt);

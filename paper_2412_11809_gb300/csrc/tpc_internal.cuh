@@ -156,7 +156,7 @@ struct ATile {
     uint32_t h0;               // positions from h0 on were looked at
     uint64_t lo;               // smallest ToA an earlier hit may have and join one of its hits
     uint64_t cmax[ACHUNKS];    // largest ToA of each quarter of its positions
-    uint32_t redo;             // to be joined with every earlier tile
+    uint32_t redo;             // not done: the step is taken in any order
 };
 
 // Feature sums of one tile cluster (at a cluster's root: of the cluster).
@@ -398,7 +398,7 @@ __device__ __forceinline__ void setup_seg(Seg &g, uint32_t &off, uint32_t &tile)
 // The step's state.  A stream that one step of a context could not be taken on
 // the arrival-order path for (disordered too far, too many hits within dt)
 // mostly goes on like that, and finding out again took 6 to 40 percent of each
-// step: after such a step the next 1, 3, 7, ... 63 start on the time-sorted
+// step: after such a step the next 3, 15 or 63 start on the time-sorted
 // path, until one tried in between is covered.
 __device__ __forceinline__ void setup_prob(Prob &p, uint32_t nsegs, uint32_t tiles, uint32_t positions, uint32_t arrival) {
     const uint32_t fail = p.raw_fail;
@@ -416,7 +416,7 @@ __device__ __forceinline__ void setup_prob(Prob &p, uint32_t nsegs, uint32_t til
     p.held = 0;
     if (arrival == RAW_TRY) {
         if (tried) {
-            p.hold = p.backoff = lost ? min(2u * p.backoff + 1u, HOLD_MOST) : 0u;
+            p.hold = p.backoff = lost ? min(4u * p.backoff + 3u, HOLD_MOST) : 0u;
             p.hold_as = fail;
         }
         if (p.hold) {
