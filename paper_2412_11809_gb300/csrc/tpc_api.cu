@@ -170,6 +170,10 @@ struct Workspace {
     cudaError_t ensure(size_t positions) {
         size_t need = grown(positions);
         if (w.seg && need == alloc_need) return cudaSuccess;
+        Prob p{};   // what it keeps from step to step (setup_prob) moves along
+        if (w.prob && (cudaMemcpyAsync(&p, w.prob, sizeof(Prob), cudaMemcpyDeviceToHost, mem.stream) != cudaSuccess ||
+                       cudaStreamSynchronize(mem.stream) != cudaSuccess))
+            p = Prob{};
         mem.release();   // freed after the steps already queued on the owner's stream
         alloc_need = need;
         pos_cap = need;
@@ -209,7 +213,6 @@ struct Workspace {
         w.atile = reinterpret_cast<ATile *>(w.hist);
         w.atmax = w.tile_base;
         if (e == cudaSuccess) {
-            Prob p{};
             p.tile_cap = (uint32_t)T;
             p.pos_cap = (uint32_t)P;
             e = cudaMemcpyAsync(w.prob, &p, sizeof(Prob), cudaMemcpyHostToDevice, mem.stream);

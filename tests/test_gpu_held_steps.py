@@ -75,6 +75,18 @@ def test_small_and_batched_steps_between():
                     base[c] += len(h)
 
 
+def test_growing_steps():
+    """The arrays grow between the steps, and what the context holds moves along."""
+    with Clusterer(256, 256, 200) as c:
+        base = 0
+        for k, n in enumerate([N, 150_000, 90_000, 400_000, 900_000]):
+            hits = _hits("unordered" if k < 3 else 0, k, n=n)
+            c.push(hits)
+            c.flush()
+            _check(c, hits, base, 200)
+            base += n
+
+
 def test_errors_in_held_steps():
     """A hit outside the sensor is reported by a step that starts on the time-sorted path."""
     with Clusterer(256, 256, 200) as c:
