@@ -1054,8 +1054,8 @@ static cudaError_t enqueue_variant(tpc_ctx *c, const Launch &L) {
 }
 
 // Variants (b) and (c): one graph, as the steps of (a).  (b) waits for it: if
-// a list of open edges overflowed, every hit's neighbours are looked at again
-// and the features summed anew.  As some fifty launches, with the host looking
+// a list of open edges overflowed, every hit's neighbours are looked at again,
+// the features' kernels having found no tiles.  As some fifty launches, with the host looking
 // at (b)'s flags after each round, a call with 10,000 hits took 1120 us ((b)) and
 // 1210 ((c)), mostly between kernels; 430 and 510 so.
 static int flush_variant(tpc_ctx *c, Tracer *tr) {
@@ -1105,7 +1105,6 @@ static int flush_variant(tpc_ctx *c, Tracer *tr) {
         }
         if (again) {
             launch_comp_parents(c->ws.w, c->vs.v, L);
-            launch_init_roots(c->ws.w, L);
             launch_features(c->ws.w, L, true);
             launch_outputs(c->ws.w, L);
         }

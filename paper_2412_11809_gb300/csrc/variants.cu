@@ -852,13 +852,14 @@ __device__ __forceinline__ bool gunion_last(uint32_t *parent, uint32_t *glast, u
 
 // Append the warp's open edges (a node of h's group, a node of its
 // neighbour's group, h's key) to list `out` (one atomic per warp); on
-// overflow the list is marked and the next round takes every hit again.
-__device__ __forceinline__ void push_edges(const VarWork &v, int out, unsigned long long *listed, uint32_t *flags, bool keep,
+// overflow the list is marked and the next round takes every hit again.  Whether
+// the list is full by now.
+__device__ __forceinline__ bool push_edges(const VarWork &v, int out, unsigned long long *listed, uint32_t *flags, bool keep,
                                            uint32_t a, uint32_t b, uint32_t key) {
     uint2 *list = pick(v.edges, out);
     uint32_t *keys = pick(v.ekey, out);
     const uint32_t m = __ballot_sync(0xffffffffu, keep);
-    if (!m) return;
+    if (!m) return false;
     const int lane = threadIdx.x & 31;
     unsigned long long base = 0;   // 64 bits: a full round can push more than 2^32 edges
     if (lane == __ffs(m) - 1) base = atomicAdd(listed, (unsigned long long)__popc(m));
@@ -872,6 +873,7 @@ __device__ __forceinline__ void push_edges(const VarWork &v, int out, unsigned l
             flags[1] = 1u;
         }
     }
+    return base >= v.edge_cap;
 }
 
 // The first entries at or after position s of G timelines [at, at + n)
@@ -912,6 +914,10 @@ __device__ __forceinline__ void lane_bounds(const uint32_t *tl, uint32_t (&at)[G
 // 1078 and 943 us (416 of them the searches).  Not kept: warp-wide searches of
 // four neighbours at once (1075), and second steps up, last keys and unions
 // also taken together (1066, with twice the edges listed).
+// A warp that finds the list full lists no more: on streams where nearly every
+// edge stays open the one counter's atomics took longer than all else (8 M hits
+// at 0.25 a tick, dt 128: 10.0 ms a call with three full rounds, 5.7 so; reading
+// the list's mark instead cost as much).
 constexpr int FIRST_THREADS = 128, FIRST_G = 8;
 
 __global__ void __launch_bounds__(FIRST_THREADS, 5) k_global_first(Work w, VarWork v) {
@@ -925,7 +931,7 @@ __global__ void __launch_bounds__(FIRST_THREADS, 5) k_global_first(Work w, VarWo
     const uint32_t *ps = v.pix_start;
     const int lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * (blockDim.x >> 5);
-    bool changed = false;
+    bool changed = false, full = false;   // full: the list was, when this warp last listed an edge
     for (uint32_t i0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32u; i0 < n; i0 += warps * 32u) {
         const uint32_t i = i0 + (uint32_t)lane;
         const bool valid = i < n;
@@ -954,7 +960,7 @@ __global__ void __launch_bounds__(FIRST_THREADS, 5) k_global_first(Work w, VarWo
                 }
             }
             changed |= r == 1;
-            push_edges(v, 0, v.ecount, v.changed, r == 2, rh, rl, me.w);
+            full |= push_edges(v, 0, v.ecount, v.changed, r == 2 && !full, rh, rl, me.w);
         };
         {   // its own pixel: the entry before
             const bool has = valid && i > ps[p];
@@ -1083,6 +1089,9 @@ __global__ void __launch_bounds__(256) k_global_rounds(Work w, VarWork v, uint32
         status[3] = exact;
         status[4] = open < v.edge_cap ? (uint32_t)open : v.edge_cap;
         status[5] = rounds == MAX_ROUNDS;
+        // with another full round to come, nothing for the features and outputs behind this one
+        w.prob->ntiles = over ? 0u : v.prob->ntiles;
+        w.prob->nsegs = over ? 0u : v.prob->nsegs;
     }
 }
 
