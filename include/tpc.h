@@ -418,7 +418,7 @@ void tpc_filler_destroy(tpc_filler *f);
    Asynchronous: returns after queueing.  TPC_ERR_ARG for n >
    TPC_STATIC_MAX_HITS, null pointers or a sensor larger than tpc_create
    allows.  Working memory is one fixed device array of the library
-   (about 3.7 MB per GPU that loads it, held until exit), shared by every
+   (about 4.9 MB per GPU that loads it, held until exit), shared by every
    call and keeping the last call's contents: calls whose work overlaps on
    the GPU race on it, so order them on one stream.  The first call on a
    device does set-up (looks up that array's device address with

@@ -1854,7 +1854,7 @@ cudaError_t init_arrival_attributes() {
         e = cudaFuncSetAttribute(k_arrival_tile<AT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMEM);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_arrival_step, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMALL_SMEM);
-    if (e == cudaSuccess)   // clusters of 16 (a GPC of this GPU has 16 SMs and more)
+    if (e == cudaSuccess)   // clusters of 16
         e = cudaFuncSetAttribute(k_arrival_step, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
 }
@@ -1880,23 +1880,45 @@ void launch_arrival_output(const Work &w, const Launch &L) {
     L.mark("k_arrival_emit");
 }
 
-// A small step of at most `tiles` tiles; seg: its segment, or null if w.seg
-// holds it already.
-cudaError_t launch_arrival_step(const Work &w, const Seg *seg, uint32_t tiles, uint32_t tile_cap, uint64_t *counts,
-                                uint32_t keep, const Launch &L) {
+uint32_t arrival_step_cluster(uint32_t tiles) {
     uint32_t ctas = 1;
     while (ctas < tiles) ctas *= 2;
+    return ctas;
+}
+
+static cudaLaunchConfig_t step_config(uint32_t ctas, cudaLaunchAttribute *a, cudaStream_t st) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(ctas);
     cfg.blockDim = dim3(ST);
     cfg.dynamicSmemBytes = A_SMALL_SMEM;
-    cfg.stream = L.stream;
-    cudaLaunchAttribute a{};
-    a.id = cudaLaunchAttributeClusterDimension;
-    a.val.clusterDim.x = ctas;
-    a.val.clusterDim.y = a.val.clusterDim.z = 1;
-    cfg.attrs = &a;
+    cfg.stream = st;
+    a->id = cudaLaunchAttributeClusterDimension;
+    a->val.clusterDim.x = ctas;
+    a->val.clusterDim.y = a->val.clusterDim.z = 1;
+    cfg.attrs = a;
     cfg.numAttrs = 1;
+    return cfg;
+}
+
+// A whole GPU holds clusters of SMALL_TILES CTAs of this size, one to an SM, in
+// a GPC; a part of one (fewer SMs of a GPC for the process) may not.
+int arrival_step_ctas() {
+    for (uint32_t ctas = SMALL_TILES; ctas; ctas /= 2) {
+        cudaLaunchAttribute a{};
+        const cudaLaunchConfig_t cfg = step_config(ctas, &a, nullptr);
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, k_arrival_step, &cfg) == cudaSuccess && clusters > 0) return (int)ctas;
+        cudaGetLastError();   // (too large is an answer)
+    }
+    return 0;
+}
+
+// A small step of at most `tiles` tiles; seg: its segment, or null if w.seg
+// holds it already.
+cudaError_t launch_arrival_step(const Work &w, const Seg *seg, uint32_t tiles, uint32_t tile_cap, uint64_t *counts,
+                                uint32_t keep, const Launch &L) {
+    cudaLaunchAttribute a{};
+    const cudaLaunchConfig_t cfg = step_config(arrival_step_cluster(tiles), &a, L.stream);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, k_arrival_step, w, seg ? *seg : Seg{}, seg ? 1u : 0u, tile_cap, counts, keep);
     L.mark("k_arrival_step");
     return e;

@@ -31,3 +31,11 @@ void ctx_sensor(tpc_ctx *c, uint32_t *width, uint32_t *height);
 int ctx_device(tpc_ctx *c);
 
 }  // namespace tpc
+
+// For tests, beside the interface: tpc_cluster_static() as on a device that
+// holds clusters of at most most_ctas CTAs, and a context on such a device
+// (before its first step).
+extern "C" int tpc_internal_static(const tpc_hit *hits, size_t n, uint32_t width, uint32_t height, uint64_t dt,
+                                   uint64_t *labels, tpc_cluster *records, size_t record_cap, uint64_t *counts,
+                                   void *stream, int most_ctas);
+extern "C" int tpc_internal_most_ctas(tpc_ctx *c, int most_ctas);

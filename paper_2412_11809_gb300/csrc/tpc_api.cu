@@ -18,6 +18,7 @@
 // a persistent grid over (segment, tile) work items, so no step waits for the
 // host and the sequence is captured once into a CUDA graph and replayed.
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -211,7 +212,6 @@ struct Workspace {
         w.xlist = reinterpret_cast<uint2 *>(w.lab_tmp);
         w.rkey = w.keys[0];
         w.atile = reinterpret_cast<ATile *>(w.hist);
-        w.atmax = w.tile_base;
         if (e == cudaSuccess) {
             p.tile_cap = (uint32_t)T;
             p.pos_cap = (uint32_t)P;
@@ -295,6 +295,15 @@ int num_sms(int dev) {
     return n > 0 ? n : 1;
 }
 
+// arrival_step_ctas() of a device (the current one), asked once.
+int step_ctas(int dev) {
+    static std::atomic<int> known[MAX_DEVICES];   // + 1
+    if (dev < 0 || dev >= MAX_DEVICES) return arrival_step_ctas();
+    int k = known[dev].load();
+    if (!k) known[dev].store(k = arrival_step_ctas() + 1);
+    return k - 1;
+}
+
 int map_err(uint32_t bits) {
     if (bits & E_RANGE) return TPC_ERR_RANGE;
     if (bits & E_SPAN) return TPC_ERR_SPAN;
@@ -328,6 +337,7 @@ struct tpc_ctx {
     uint64_t budget = 0;
     int ctas_per_sm = 0;
     int sms = 1;
+    int step_ctas = 0;             // largest cluster the device holds for a small step
     int64_t fail_alloc = 0;        // TPC_OPT_FAIL_ALLOC countdown (0: off)
 
     // non-streaming pending hits
@@ -645,10 +655,11 @@ cudaError_t run_step(tpc_ctx *owner, Workspace &ws, int nsegs, StepMode mode, cu
 }
 
 // The path of a step over these segments; positions: at least its hits.
-StepMode step_mode(const Seg *segs, int nsegs, size_t positions) {
+StepMode step_mode(const tpc_ctx *c, const Seg *segs, int nsegs, size_t positions) {
     for (int i = 0; i < nsegs; ++i)
         if (segs[i].link_general || segs[i].dt >= ARRIVAL_DT) return STEP_SORTED;
-    return nsegs == 1 && positions <= (size_t)SMALL_TILES * TILE ? STEP_SMALL : STEP_ARRIVAL;
+    return nsegs == 1 && positions <= (size_t)SMALL_TILES * TILE && c->step_ctas >= (int)SMALL_TILES ? STEP_SMALL
+                                                                                                       : STEP_ARRIVAL;
 }
 
 // Outputs of a one-shot step: the caller's bound buffers, else the
@@ -806,7 +817,7 @@ int stream_step(tpc_ctx *c, size_t n, bool close_all) {
     s.carry_cap = (uint32_t)c->carry_cap;
     s.n_new = (uint32_t)n;
     if (upload_segs(c, c->ws.w, &s, 1, c->stream) != cudaSuccess) return TPC_ERR_CUDA;
-    if (run_step(c, c->ws, 1, step_mode(&s, 1, positions), c->stream) != cudaSuccess) return TPC_ERR_CUDA;
+    if (run_step(c, c->ws, 1, step_mode(c, &s, 1, positions), c->stream) != cudaSuccess) return TPC_ERR_CUDA;
     c->scur = in;
     c->pushed += n;
     c->carry_ub = close_all ? 0 : positions;
@@ -890,6 +901,7 @@ int tpc_create(uint32_t width, uint32_t height, uint64_t dt, int variant, tpc_ct
     if (cudaGetDevice(&c->device) != cudaSuccess) { delete c; return TPC_ERR_CUDA; }
     c->sms = num_sms(c->device);
     if (init_kernel_attributes() != cudaSuccess) { delete c; return TPC_ERR_CUDA; }
+    c->step_ctas = ::step_ctas(c->device);
     bool ok = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) == cudaSuccess;
     c->own_stream = ok;
     bind_mem(c);
@@ -988,6 +1000,13 @@ int tpc_push(tpc_ctx *c, const tpc_hit *hits, size_t n, int where) {
         : cudaMemcpyAsync(c->in + c->pending, hits, n * sizeof(tpc_hit), cudaMemcpyDeviceToDevice, c->stream);
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? TPC_ERR_NOMEM : TPC_ERR_CUDA;
     c->pending += n;
+    return TPC_OK;
+}
+
+int tpc_internal_most_ctas(tpc_ctx *c, int most_ctas) {
+    if (!c) return TPC_ERR_ARG;
+    std::lock_guard<std::mutex> lk(c->mu);
+    c->step_ctas = std::min(c->step_ctas, most_ctas);
     return TPC_OK;
 }
 
@@ -1141,7 +1160,7 @@ static int flush_impl(tpc_ctx *c, Tracer *tr) {
     s.gidx_base = c->pushed;
     s.n_new = (uint32_t)n;
     if (upload_segs(c, c->ws.w, &s, 1, c->stream) != cudaSuccess) return TPC_ERR_CUDA;
-    if (run_step(c, c->ws, 1, step_mode(&s, 1, n), c->stream, tr) != cudaSuccess) return TPC_ERR_CUDA;
+    if (run_step(c, c->ws, 1, step_mode(c, &s, 1, n), c->stream, tr) != cudaSuccess) return TPC_ERR_CUDA;
     c->res_base = c->pushed;
     c->pushed += n;
     c->pending = 0;
@@ -1308,7 +1327,7 @@ int tpc::batch_step(tpc_ctx **ctxs, int n, bool consume) {
         segs[k] = s;
     }
     if (upload_segs(lead, lead->ws.w, segs.data(), n, lead->stream) != cudaSuccess) return TPC_ERR_CUDA;
-    if (run_step(lead, lead->ws, n, step_mode(segs.data(), n, positions), lead->stream) != cudaSuccess) return TPC_ERR_CUDA;
+    if (run_step(lead, lead->ws, n, step_mode(lead, segs.data(), n, positions), lead->stream) != cudaSuccess) return TPC_ERR_CUDA;
     if (cudaEventRecord(lead->done_ev, lead->stream) != cudaSuccess) return TPC_ERR_CUDA;
     for (int i = 0; i < n; ++i) {
         tpc_ctx *c = ctxs[i];

@@ -208,7 +208,6 @@ struct Work {
     uint2 *xlist;              // (lab_tmp) [tile][A_PAIRS] pairs across tiles: tile cluster, earlier hit's position
     uint32_t *rkey;            // (keys[0]) per position: ToA - the tile's base; may be null
     ATile *atile;              // (hist) per tile
-    uint32_t *atmax;           // (tile_base) per tile: largest key
 };
 static_assert(sizeof(ATile) <= RADIX * sizeof(uint32_t) && A_PAIRS * sizeof(uint2) <= TILE * sizeof(uint64_t) &&
               sizeof(RootSlot) <= sizeof(Slot), "arrival-order arrays fit the sorted path's");
@@ -555,6 +554,8 @@ void launch_arrival_link(const Work &w, cudaGraphConditionalHandle otherwise, bo
 void launch_arrival_output(const Work &w, const Launch &L);
 cudaError_t launch_arrival_step(const Work &w, const Seg *seg, uint32_t tiles, uint32_t tile_cap, uint64_t *counts,
                                 uint32_t keep, const Launch &L);
+uint32_t arrival_step_cluster(uint32_t tiles);   // CTAs launch_arrival_step takes for that many tiles
+int arrival_step_ctas();                         // the most that the current device holds in one cluster, 0: none
 void launch_seg_finalize(const Work &w, const Launch &L, cudaGraphConditionalHandle general = 0);
 void launch_make_keys(const Work &w, const Launch &L);
 void launch_sort_fast(const Work &w, const Launch &L);
