@@ -230,8 +230,9 @@ typedef struct tpc_tune_report {
    bucket floor(log2(hits)) of its pending hits, the number of contexts) or,
    if absent (or with TPC_TUNE_FORCE), time the pending batch itself, which
    stays pending: the defaults, then coordinate descent over the fields of
-   tpc_tuning, two passes, three timed runs per candidate, a change kept if
-   its median improves by more than 1 %.  Sets the choice on ctxs[0] and
+   tpc_tuning that its step reads (those of the time-sorted path only where
+   the step takes it), two passes, three timed runs per candidate, a change
+   kept if its median improves by more than 1 %.  Sets the choice on ctxs[0] and
    appends it to the cache file (cache_path NULL: no cache).  Work is
    ordered on ctxs[0]'s stream and waited for. */
 int tpc_tune_batch(tpc_ctx **ctxs, int n, const char *cache_path, int flags, tpc_tune_report *rep);

@@ -29,6 +29,7 @@ std::mutex &ctx_mutex(tpc_ctx *c);
 size_t ctx_pending(tpc_ctx *c);
 void ctx_sensor(tpc_ctx *c, uint32_t *width, uint32_t *height);
 int ctx_device(tpc_ctx *c);
+bool ctx_sorted_step(tpc_ctx *c);         // the last finished step of the context took the time-sorted path
 
 }  // namespace tpc
 

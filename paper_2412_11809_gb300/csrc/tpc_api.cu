@@ -1446,6 +1446,7 @@ void tpc::ctx_sensor(tpc_ctx *c, uint32_t *width, uint32_t *height) {
     *width = c->width;
     *height = c->height;
 }
+bool tpc::ctx_sorted_step(tpc_ctx *c) { return !c->h_info->arrival; }
 int tpc::ctx_device(tpc_ctx *c) { return c->device; }
 
 extern "C" {
