@@ -89,11 +89,13 @@ def path_bytes_per_hit(n_hits: int, n_clusters: int) -> float:
 
 
 # Device-code sources: every kernel of a processing step with its launch
-# configuration.  The launch order lives in the API file's capture_step(),
-# hashed on its own; the rest of that file (context bookkeeping, checkpoints)
+# configuration.  The launch order lives in the API file's LAUNCH_ORDER
+# functions, hashed on their own; the rest of that file (context bookkeeping, checkpoints)
 # and the host-side buffer filling are not part of any kernel.
 KERNEL_SOURCES = ("arrival.cu", "features.cu", "link.cu", "noalloc.cu", "prepare.cu", "radix.cu", "sortfast.cu",
                   "tpc_internal.cuh")   # variants.cu: (b)/(c) kernels, never launched by the step
+
+LAUNCH_ORDER = ("enqueue_general_sort", "enqueue_sorted", "capture_step")
 
 
 def kernel_source_sha() -> str:
@@ -105,8 +107,9 @@ def kernel_source_sha() -> str:
     for f in KERNEL_SOURCES:
         h.update(open(os.path.join(csrc, f), "rb").read())
     api = open(os.path.join(csrc, "tpc_api.cu")).read()
-    start = api.index("cudaError_t capture_step(")
-    h.update(api[start:api.index("\n}\n", start)].encode())
+    for name in LAUNCH_ORDER:
+        start = api.index(f" {name}(const Work &w")
+        h.update(api[start:api.index("\n}\n", start)].encode())
     return h.hexdigest()[:16]
 
 
