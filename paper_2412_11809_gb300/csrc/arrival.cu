@@ -1848,6 +1848,51 @@ __global__ void __launch_bounds__(ST, 1) k_arrival_step(Work w, Seg seg, uint32_
     }
 }
 
+// tpc_forest of a step on this path, whose union-find runs over tile clusters:
+// the (ToA, input) order by the radix sort of the kept keys, every hit's parent
+// its cluster's earliest hit.  What the step kept besides is written over: the
+// keys become relative to its smallest ToA, and the slots' place holds each
+// cluster's first sorted position and the parents.
+__global__ void __launch_bounds__(256) k_forest_keys(Work w) {
+    Prob &P = *w.prob;
+    const Seg &g = w.seg[0];
+    const uint32_t n = g.n, stride = gridDim.x * blockDim.x, i0 = blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t *first = reinterpret_cast<uint32_t *>(w.slot);
+    for (uint32_t i = i0; i < n; i += stride) {
+        w.keys[0][i] = (uint32_t)(w.atile[i / TILE].base + w.rkey[i] - g.toa_min);
+        w.vals[0][i] = i;
+    }
+    for (uint32_t c = i0; c < g.ntiles * TILE; c += stride) first[c] = 0xFFFFFFFFu;
+    if (i0 == 0) {
+        const uint64_t span = g.toa_max - g.toa_min;
+        P.npasses = span ? (64u - __clzll((long long)span) + RADIX_BITS - 1u) / RADIX_BITS : 0u;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_forest_first(Work w) {
+    const uint32_t *order = pick(w.vals, sorted_sel(*w.prob));
+    uint32_t *first = reinterpret_cast<uint32_t *>(w.slot);
+    for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < w.seg[0].n; s += gridDim.x * blockDim.x) {
+        uint32_t *f = first + w.gpar[w.root_of[order[s]]];
+        if (*reinterpret_cast<volatile uint32_t *>(f) > s) atomicMin(f, s);
+    }
+}
+
+__global__ void __launch_bounds__(256) k_forest_parents(Work w, uint32_t *parent) {
+    const uint32_t *order = pick(w.vals, sorted_sel(*w.prob));
+    const uint32_t *first = reinterpret_cast<const uint32_t *>(w.slot);
+    for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < w.seg[0].n; s += gridDim.x * blockDim.x)
+        parent[s] = first[w.gpar[w.root_of[order[s]]]];
+}
+
+// Leaves the order in vals[npasses % 2].
+void launch_forest(const Work &w, uint32_t *parent, const Launch &L) {
+    k_forest_keys<<<L.fit(k_forest_keys, 256, 0), 256, 0, L.stream>>>(w);
+    for (int pass = 0; pass < 4; ++pass) launch_radix_pass(w, pass, L);
+    k_forest_first<<<L.fit(k_forest_first, 256, 0), 256, 0, L.stream>>>(w);
+    k_forest_parents<<<L.fit(k_forest_parents, 256, 0), 256, 0, L.stream>>>(w, parent);
+}
+
 cudaError_t init_arrival_attributes() {
     cudaError_t e = cudaFuncSetAttribute(k_arrival_tile<AT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, A_SMEM);
     if (e == cudaSuccess)

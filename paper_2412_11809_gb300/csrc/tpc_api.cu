@@ -827,45 +827,6 @@ int stream_step(tpc_ctx *c, size_t n, bool close_all) {
     return TPC_OK;
 }
 
-// tpc_forest of a step on the arrival-order path, whose union-find runs over
-// tile clusters: the (ToA, input) order from the kept keys (a stable radix
-// sort on the host), every hit's parent its cluster's earliest hit.
-int forest_of_arrival(tpc_ctx *c, size_t n, uint32_t *parent, uint32_t *input_pos) {
-    const size_t tiles = (n + TILE - 1) / TILE;
-    const Work &w = c->ws.w;
-    try {
-        std::vector<uint32_t> cluster(n), key(n), gpar(tiles * TILE), a(n), first(tiles * TILE, 0xFFFFFFFFu);
-        std::vector<ATile> at(tiles);
-        std::vector<uint64_t> toa(n);
-        if (cudaMemcpy(cluster.data(), w.root_of, n * 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
-            cudaMemcpy(key.data(), w.rkey, n * 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
-            cudaMemcpy(gpar.data(), w.gpar, tiles * TILE * 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
-            cudaMemcpy(at.data(), w.atile, tiles * sizeof(ATile), cudaMemcpyDeviceToHost) != cudaSuccess)
-            return TPC_ERR_CUDA;
-        uint64_t lowest = ~0ull;
-        for (size_t i = 0; i < n; ++i) {
-            toa[i] = at[i / TILE].base + key[i];
-            lowest = std::min(lowest, toa[i]);
-            a[i] = (uint32_t)i;
-        }
-        for (int shift = 0; shift < 32; shift += 16) {   // a step's ToAs span less than 2^32 ticks
-            std::vector<size_t> start(65537, 0);
-            for (size_t i = 0; i < n; ++i) ++start[(((toa[i] - lowest) >> shift) & 0xFFFF) + 1];
-            for (int d = 0; d < 65536; ++d) start[d + 1] += start[d];
-            for (size_t i = 0; i < n; ++i) input_pos[start[((toa[a[i]] - lowest) >> shift) & 0xFFFF]++] = a[i];
-            std::copy(input_pos, input_pos + n, a.begin());
-        }
-        for (size_t s = 0; s < n; ++s) {
-            const size_t root = gpar[cluster[a[s]]];
-            if (first[root] == 0xFFFFFFFFu) first[root] = (uint32_t)s;
-            parent[s] = first[root];
-        }
-    } catch (const std::bad_alloc &) {
-        return TPC_ERR_NOMEM;
-    }
-    return TPC_OK;
-}
-
 int read_result(tpc_ctx *c, StepInfo &r) {
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return TPC_ERR_CUDA;
     if (!c->has_result) {
@@ -1367,11 +1328,26 @@ int tpc_forest(tpc_ctx *c, uint32_t *parent, uint32_t *input_pos, size_t cap, si
     if (n > cap) return TPC_ERR_CAP;
     if (!n) return TPC_OK;
     if (!parent || !input_pos) return TPC_ERR_ARG;
-    if (r.arrival) return forest_of_arrival(c, n, parent, input_pos);
-    // the sorted order lives in the buffer the step's last sort pass wrote
+    const uint32_t *from = c->ws.w.parent;
+    if (r.arrival) {   // built on the first call after the step
+        uint32_t *built = reinterpret_cast<uint32_t *>(c->ws.w.slot) + c->ws.pos_cap;
+        if (r.arrival != FOREST_BUILT) {
+            Launch L{grid_of(c), c->stream, nullptr, c->sms, c->ctas_per_sm};
+            launch_forest(c->ws.w, built, L);
+            if (cudaMemcpyAsync(&r.npasses, &c->ws.w.prob->npasses, sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream) !=
+                    cudaSuccess ||
+                cudaStreamSynchronize(c->stream) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
+                c->has_result = false;   // (its arrays are written over in part)
+                return TPC_ERR_CUDA;
+            }
+            c->h_info->npasses = r.npasses;
+            c->h_info->arrival = FOREST_BUILT;
+        }
+        from = built;
+    }
+    // the sorted order lives in the buffer the last sort pass wrote
     const uint32_t sel = r.npasses & 1u;
-    if (cudaMemcpy(parent, c->ws.w.parent + r.off, n * sizeof(uint32_t), cudaMemcpyDeviceToHost) !=
-            cudaSuccess ||
+    if (cudaMemcpy(parent, from + r.off, n * sizeof(uint32_t), cudaMemcpyDeviceToHost) != cudaSuccess ||
         cudaMemcpy(input_pos, c->ws.w.vals[sel] + r.off, n * sizeof(uint32_t), cudaMemcpyDeviceToHost) !=
             cudaSuccess)
         return TPC_ERR_CUDA;

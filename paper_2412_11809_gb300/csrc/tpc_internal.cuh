@@ -64,8 +64,10 @@ struct StepInfo {
     uint32_t n_final, n_clusters, n_open;
     uint32_t err;                             // ErrBits of the whole step
     uint32_t npasses;                         // time-sorted path: its sorted data is in buffer npasses % 2
-    uint32_t arrival;                         // the arrival-order path covered the step
+    uint32_t arrival;                         // the arrival-order path covered the step (the host: FOREST_BUILT)
 };
+
+constexpr uint32_t FOREST_BUILT = 2;          // its work arrays hold the step's forest in time order
 
 struct Seg {
     // ---- set by the host ----------------------------------------------
@@ -552,6 +554,7 @@ void launch_setup(const Work &w, int nsegs, const Launch &L, bool arrival = fals
 cudaError_t init_arrival_attributes();
 void launch_arrival_link(const Work &w, cudaGraphConditionalHandle otherwise, bool parts, const Launch &L);
 void launch_arrival_output(const Work &w, const Launch &L);
+void launch_forest(const Work &w, uint32_t *parent, const Launch &L);
 cudaError_t launch_arrival_step(const Work &w, const Seg *seg, uint32_t tiles, uint32_t tile_cap, uint64_t *counts,
                                 uint32_t keep, const Launch &L);
 uint32_t arrival_step_cluster(uint32_t tiles);   // CTAs launch_arrival_step takes for that many tiles
