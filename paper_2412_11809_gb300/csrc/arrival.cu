@@ -642,7 +642,8 @@ __device__ __forceinline__ uint32_t arrival_cut(const Seg &g, uint32_t j, uint64
 }
 
 // Bound by issue and shared-memory latency, not by bytes: 64 Mi hits (256x256)
-// take 2260 us at 16 B read and 4 B written each.  Of a tile's time the records
+// take 2260 us at 16 B read and 8 B written each (the cluster, and the key that
+// tpc_forest reads).  Of a tile's time the records
 // take 22 percent, cell numbers and heads 9, the walk over neighbour cells 17,
 // crowded cells 8, positions and ToTs 7, the forest and its roots 24, features
 // 10.  Two CTAs of 512 threads at 64 registers; one of 1024 takes 2906 (its

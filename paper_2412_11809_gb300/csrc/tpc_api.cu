@@ -12,6 +12,9 @@
 //   table link -> tile link (redo tiles) -> border fast -> border link ->
 //   accumulate (finds the roots) -> labels -> tile scan -> records ->
 //   stream compact -> stream end.
+// Steps of up to 65,536 hits are one kernel, in any order.  After a step that the
+// arrival-order path did not cover the next ones start on the time-sorted one
+// (setup_prob).
 // Streaming contexts also checkpoint and restore their open state here
 // (tpc_snapshot / tpc_restore).
 // Every size the kernels need is read from device memory and every kernel is
